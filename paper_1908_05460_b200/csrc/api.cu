@@ -2,6 +2,7 @@
 // approximation-schedule driver (paper Section 2.5).  Every step of the path runs in this library's
 // kernels; there is no CPU or library fallback.
 #include <atomic>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -171,6 +172,38 @@ ExactLayout exact_layout(const Geom& g, int math, int algo)
     return cache.get(plan_key(g, math, algo), [&] { return build_exact_layout(g, math, algo); });
 }
 
+// The channels-last kernel takes what the kernels above do not tile; ALGO_DIRECT, ALGO_TENSOR and the one-pass TF32
+// mode stay with them.
+struct ClRoute { bool use; ClPlan plan; size_t partial_off, x_off, dy_off, total; };
+ClRoute build_cl_route(const gaconv_conv_desc_t* desc, const Geom& g)
+{
+    ClRoute R{};
+    if (!tensor_maps_available() || !plan_cl(g, desc->dy_layout == GACONV_DY_NPQK, &R.plan)) return R;
+    gaconv_conv_desc_t native = *desc;
+    native.x_layout = GACONV_X_NHWC; native.dy_layout = GACONV_DY_NKPQ;
+    Geom gn;
+    if (make_geom(&native, &gn) != GACONV_OK) return R;
+    const ExactLayout L = exact_layout(gn, GACONV_MATH_DEFAULT, GACONV_ALGO_AUTO);
+    // Below ~4 million products the FP32-pipe kernel's one or two launches are as quick (8-9 us, 4x32x9x9 -> 48, 1x1)
+    const double products = (double)g.n * g.p * g.q * g.k * g.c * g.r * g.s;
+    R.use = !(L.tc_ok || L.stem_ok || direct_mma_supported(gn, L.dp)) && products > 4e6;
+#ifdef GACONV_TUNING
+    if (const char* e = getenv("GACONV_CL")) R.use = atoi(e) != 0;
+#endif
+    R.partial_off = kWsDataOffset;
+    R.x_off = align_up(R.partial_off + R.plan.partial_bytes, 256);
+    R.dy_off = R.x_off + R.plan.x_bytes;
+    R.total = R.dy_off + R.plan.dy_bytes;
+    return R;
+}
+bool cl_route(const gaconv_conv_desc_t* desc, const Geom& g, ClRoute* R)
+{
+    if (desc->math != GACONV_MATH_DEFAULT || desc->algo != GACONV_ALGO_AUTO) return false;
+    static PlanCache<ClRoute> cache;
+    *R = cache.get(plan_key(g, desc->dy_layout, 0), [&] { return build_cl_route(desc, g); });
+    return R->use;
+}
+
 // entries retained per map by the top-k method: desc->topk clamped to the map size; 0 = invalid
 int topk_of(const gaconv_conv_desc_t* d, const Geom& g)
 {
@@ -311,6 +344,99 @@ struct gaconv_schedule {
     bool* mask;   // SEEDED_FRACTION: layers in the approximated subset
 };
 
+gaconv_status_t gaconv::exact_workspace(const gaconv_conv_desc_t* desc, bool cl, size_t* bytes)
+{
+    Geom g;
+    gaconv_status_t st = make_geom(desc, &g);
+    if (st != GACONV_OK) return st;
+    ClRoute C;
+    if (cl && cl_route(desc, g, &C)) { *bytes = C.total; return GACONV_OK; }
+    const Relayout R = plan_relayout(desc, GACONV_METHOD_EXACT);      // operands that are transposed first: the inner call's scratch, then the copies
+    if (R.move_x || R.move_dy)
+        *bytes = align_up(R.inner_bytes, 256) + (R.move_x ? align_up(x_bytes_of(desc), 256) : 0) + (R.move_dy ? dy_bytes_of(g) : 0);
+    else
+        *bytes = exact_layout(g, desc->math, desc->algo).total;
+    return GACONV_OK;
+}
+
+gaconv_status_t gaconv::run_exact(const void* x, const void* dy, float* dw, const gaconv_conv_desc_t* desc, cudaStream_t stream, bool cl)
+{
+    Geom g;
+    gaconv_status_t st = make_geom(desc, &g);
+    if (st != GACONV_OK) return st;
+    if (x == nullptr || dy == nullptr || dw == nullptr) return GACONV_ERR_NULL_POINTER;
+    if (!aligned16(x) || !aligned16(dy) || !aligned16(dw)) return GACONV_ERR_MISALIGNED;
+    if (desc->math == GACONV_MATH_TF32 && g.bf16) return GACONV_ERR_BAD_DESC;
+    ClRoute C;
+    if (cl && cl_route(desc, g, &C)) {
+        st = check_ws(desc, C.total);
+        if (st != GACONV_OK) return st;
+        char* ws = static_cast<char*>(desc->workspace);
+        return launch_cl(x, dy, dw, reinterpret_cast<float*>(ws + C.partial_off), ws + C.x_off, ws + C.dy_off, reinterpret_cast<uint32_t*>(ws),
+                         C.plan, stream) == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
+    }
+    if (desc->dy_layout == GACONV_DY_NPQK && g.k > 1 && desc->algo != GACONV_ALGO_DIRECT) {
+        // Small maps: the tensor-core kernel's dY operand IS the channels-last order (its pre-pass would transpose an
+        // N x K x P x Q gradient into it), so a channels-last gradient is read where it lies; only X may have to move.
+        const Relayout R = plan_relayout(desc, GACONV_METHOD_EXACT);
+        Geom gi;
+        if (make_geom(&R.inner, &gi) == GACONV_OK) {
+            const ExactLayout Li = exact_layout(gi, desc->math, desc->algo);
+            if (Li.tc_ok && Li.tp.reads_transposed_dy) {
+                const size_t head = align_up(Li.total, 256);
+                st = check_ws(desc, head + (R.move_x ? x_bytes_of(desc) : 0));
+                if (st != GACONV_OK) return st;
+                char* ws = static_cast<char*>(desc->workspace);
+                const void* xs = x;
+                if (R.move_x) {
+                    if (launch_transpose_batched(x, ws + head, g.c, g.h * g.w, g.n, g.bf16, stream) != cudaSuccess)
+                        return GACONV_ERR_CUDA;
+                    xs = ws + head;
+                }
+                cudaError_t e = launch_tc(xs, nullptr, dw, reinterpret_cast<float*>(ws + Li.partial_off), const_cast<void*>(dy),
+                                          reinterpret_cast<uint32_t*>(ws + kWsCounterOffset), reinterpret_cast<uint32_t*>(ws), Li.tp,
+                                          stream);
+                return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
+            }
+        }
+    }
+    {
+        gaconv_conv_desc_t inner;
+        const void *xt = nullptr, *dyt = nullptr;
+        bool moved = false;
+        st = relayout_operands(x, dy, desc, GACONV_METHOD_EXACT, stream, &inner, &xt, &dyt, &moved);
+        if (st != GACONV_OK) return st;
+        if (moved) return run_exact(xt, dyt, dw, &inner, stream, false);
+    }
+    const ExactLayout L = exact_layout(g, desc->math, desc->algo);
+    const bool mma_ok = direct_mma_supported(g, L.dp);
+    if (desc->math == GACONV_MATH_TF32 && !mma_ok && !L.tc_ok) return GACONV_ERR_UNSUPPORTED;
+    if (desc->algo == GACONV_ALGO_TENSOR && !L.tc_ok) return GACONV_ERR_UNSUPPORTED;
+    st = check_ws(desc, L.total);
+    if (st != GACONV_OK) return st;
+    char* ws = static_cast<char*>(desc->workspace);
+    if (L.tc_ok && desc->algo != GACONV_ALGO_DIRECT) {
+        cudaError_t e = launch_tc(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off), ws + L.scratch_off,
+                                  reinterpret_cast<uint32_t*>(ws + kWsCounterOffset), reinterpret_cast<uint32_t*>(ws), L.tp,
+                                  stream);
+        return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
+    }
+    if (L.stem_ok && desc->algo != GACONV_ALGO_DIRECT && desc->math == GACONV_MATH_DEFAULT) {
+        cudaError_t e = launch_stem(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off), reinterpret_cast<uint32_t*>(ws), L.sp,
+                                    stream);
+        return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
+    }
+    if (mma_ok && (desc->algo != GACONV_ALGO_DIRECT || desc->math == GACONV_MATH_TF32)) {
+        cudaError_t e = launch_direct_mma(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off), reinterpret_cast<uint32_t*>(ws),
+                                          g, L.dp, desc->math != GACONV_MATH_TF32, stream);
+        return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
+    }
+    cudaError_t e = launch_direct(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off),
+                                  reinterpret_cast<uint32_t*>(ws), g, L.dp,
+                                  stream);
+    return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
+}
+
 extern "C" {
 
 const char* gaconv_status_string(gaconv_status_t s)
@@ -333,6 +459,7 @@ uint64_t gaconv_launch_count(void) { return g_launches.load(std::memory_order_re
 gaconv_status_t gaconv_workspace_size(const gaconv_conv_desc_t* desc, int32_t method, size_t* bytes)
 {
     if (bytes == nullptr) return GACONV_ERR_NULL_POINTER;
+    if (method == GACONV_METHOD_EXACT) return exact_workspace(desc, true, bytes);
     Geom g;
     gaconv_status_t st = make_geom(desc, &g);
     if (st != GACONV_OK) return st;
@@ -344,7 +471,6 @@ gaconv_status_t gaconv_workspace_size(const gaconv_conv_desc_t* desc, int32_t me
         }
     }
     switch (method) {
-        case GACONV_METHOD_EXACT: *bytes = exact_layout(g, desc->math, desc->algo).total; return GACONV_OK;
         case GACONV_METHOD_TOP1: *bytes = top1_layout(g).total; return GACONV_OK;
         case GACONV_METHOD_TOPK: {
             const int t = topk_of(desc, g);
@@ -369,72 +495,7 @@ gaconv_status_t gaconv_workspace_init(void* workspace, size_t bytes, void* strea
 
 gaconv_status_t gaconv_dw_exact(const void* x, const void* dy, float* dw, const gaconv_conv_desc_t* desc, void* stream)
 {
-    Geom g;
-    gaconv_status_t st = make_geom(desc, &g);
-    if (st != GACONV_OK) return st;
-    if (x == nullptr || dy == nullptr || dw == nullptr) return GACONV_ERR_NULL_POINTER;
-    if (!aligned16(x) || !aligned16(dy) || !aligned16(dw)) return GACONV_ERR_MISALIGNED;
-    if (desc->math == GACONV_MATH_TF32 && g.bf16) return GACONV_ERR_BAD_DESC;
-    if (desc->dy_layout == GACONV_DY_NPQK && g.k > 1 && desc->algo != GACONV_ALGO_DIRECT) {
-        // Small maps: the tensor-core kernel's dY operand IS the channels-last order (its pre-pass would transpose an
-        // N x K x P x Q gradient into it), so a channels-last gradient is read where it lies; only X may have to move.
-        const Relayout R = plan_relayout(desc, GACONV_METHOD_EXACT);
-        Geom gi;
-        if (make_geom(&R.inner, &gi) == GACONV_OK) {
-            const ExactLayout Li = exact_layout(gi, desc->math, desc->algo);
-            if (Li.tc_ok && Li.tp.reads_transposed_dy) {
-                const size_t head = align_up(Li.total, 256);
-                st = check_ws(desc, head + (R.move_x ? x_bytes_of(desc) : 0));
-                if (st != GACONV_OK) return st;
-                char* ws = static_cast<char*>(desc->workspace);
-                const void* xs = x;
-                if (R.move_x) {
-                    if (launch_transpose_batched(x, ws + head, g.c, g.h * g.w, g.n, g.bf16, static_cast<cudaStream_t>(stream)) != cudaSuccess)
-                        return GACONV_ERR_CUDA;
-                    xs = ws + head;
-                }
-                cudaError_t e = launch_tc(xs, nullptr, dw, reinterpret_cast<float*>(ws + Li.partial_off), const_cast<void*>(dy),
-                                          reinterpret_cast<uint32_t*>(ws + kWsCounterOffset), reinterpret_cast<uint32_t*>(ws), Li.tp,
-                                          static_cast<cudaStream_t>(stream));
-                return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
-            }
-        }
-    }
-    {
-        gaconv_conv_desc_t inner;
-        const void *xt = nullptr, *dyt = nullptr;
-        bool moved = false;
-        st = relayout_operands(x, dy, desc, GACONV_METHOD_EXACT, static_cast<cudaStream_t>(stream), &inner, &xt, &dyt, &moved);
-        if (st != GACONV_OK) return st;
-        if (moved) return gaconv_dw_exact(xt, dyt, dw, &inner, stream);
-    }
-    const ExactLayout L = exact_layout(g, desc->math, desc->algo);
-    const bool mma_ok = direct_mma_supported(g, L.dp);
-    if (desc->math == GACONV_MATH_TF32 && !mma_ok && !L.tc_ok) return GACONV_ERR_UNSUPPORTED;
-    if (desc->algo == GACONV_ALGO_TENSOR && !L.tc_ok) return GACONV_ERR_UNSUPPORTED;
-    st = check_ws(desc, L.total);
-    if (st != GACONV_OK) return st;
-    char* ws = static_cast<char*>(desc->workspace);
-    if (L.tc_ok && desc->algo != GACONV_ALGO_DIRECT) {
-        cudaError_t e = launch_tc(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off), ws + L.scratch_off,
-                                  reinterpret_cast<uint32_t*>(ws + kWsCounterOffset), reinterpret_cast<uint32_t*>(ws), L.tp,
-                                  static_cast<cudaStream_t>(stream));
-        return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
-    }
-    if (L.stem_ok && desc->algo != GACONV_ALGO_DIRECT && desc->math == GACONV_MATH_DEFAULT) {
-        cudaError_t e = launch_stem(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off), reinterpret_cast<uint32_t*>(ws), L.sp,
-                                    static_cast<cudaStream_t>(stream));
-        return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
-    }
-    if (mma_ok && (desc->algo != GACONV_ALGO_DIRECT || desc->math == GACONV_MATH_TF32)) {
-        cudaError_t e = launch_direct_mma(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off), reinterpret_cast<uint32_t*>(ws),
-                                          g, L.dp, desc->math != GACONV_MATH_TF32, static_cast<cudaStream_t>(stream));
-        return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
-    }
-    cudaError_t e = launch_direct(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off),
-                                  reinterpret_cast<uint32_t*>(ws), g, L.dp,
-                                  static_cast<cudaStream_t>(stream));
-    return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
+    return run_exact(x, dy, dw, desc, static_cast<cudaStream_t>(stream), true);
 }
 
 gaconv_status_t gaconv_dw_approx(int32_t method, const void* x, const void* dy, float* dw,

@@ -1,0 +1,926 @@
+// Exact filter gradient on tcgen05 for any map, channel count, stride and layout: an implicit GEMM whose two
+// operands are channels-last bf16 tensors, X as [n][h][w][c] and dY as [n][p][q][k].
+//
+//   dW[k, r, s, c] = alpha * sum_{n,p,q} dY[n,p,q,k] * Xz[n, p*st+r-pad, q*st+s-pad, c]         (Section 2.4)
+//
+// Why channels last for both: a pixel is then one row of shared memory (up to 64 channels = 128 bytes), both MMA
+// operands are MN-major, and the reduction index (pixels) walks over rows.  A filter shift is a descriptor offset of
+// whole rows, whatever the map's width, so no map size is special; the copy engine's zero fill supplies the padding,
+// the ragged edges and the channels past the end.  Operands that are not in that form are brought into it by one
+// packing pass into the workspace (pack_kernel): N x C x H x W activations, N x K x P x Q gradients, channel counts
+// that are no multiple of 8, and fp32 inputs, which become three bf16 planes x = x0 + x1 + x2 (8 + 8 + 8 bits).  The
+// fp32 product is then the six plane products of weight 2^-16 and more; what is left out is below 2^-23 of it.
+//
+// Reduction order inside a chunk (a few image rows, or several whole images), in k-steps of 16 pixels:
+//   flat    rows of pitch Wp = Q + halo columns, walked end to end; dY is loaded with the same pitch, its columns past
+//           Q reading as zeros.  Works for every Q; wastes (Wp - Q) / Q of the k-steps.
+//   paired  Q a multiple of 8: a k-step is 8 columns of two neighbouring rows (the stride between the two 8-pixel
+//           groups of a descriptor is one row), so that the halo columns are never multiplied.
+// A table of the plan holds the offsets of the k-steps of either order.
+//
+// Which operand is the MMA's M side:
+//   k-side  M = 128 output channels, N = consecutive column shifts x channels (up to 256).
+//   c-side  (few output channels) M = 128 = shifts x channels of X, N = output channels; M = 64 MMAs would take as
+//           long as M = 128 ones, so with K <= 64 this form is the faster one although one shift in four is unused.
+// The MMAs of one k-step differ only in the X offset and the accumulator columns; the list of them is part of the plan.
+//
+// CTA = one tile of dW (k-tile x c-tile x filter rows) and a contiguous range of chunks.  Its accumulator block goes to
+// the workspace as [column][128 lanes] (coalesced: a warp writes one column of 32 lanes per store) and cl_reduce_kernel
+// adds the splits in order, so results are the same from run to run.
+//
+// Every wait is bounded; on expiry the kernel raises the workspace status word, lets its copies land, frees its tensor
+// memory and returns.
+#include <cuda.h>
+
+#include <algorithm>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <type_traits>
+
+#include "gaconv_internal.h"
+#include "tma.cuh"
+#include "umma.cuh"
+
+// tuning builds: per CTA of the last launch, SM cycles of {entry, dependency, first data, issue done, accumulators done, exit},
+// and the cycles the issuer waited for data / the producer for a free stage
+#ifdef GACONV_TUNING
+__device__ long long gaconv_tuning_cl[512][8];
+#define GACONV_STAMP(slot, cond) do { if (cond) gaconv_tuning_cl[(blockIdx.y * gridDim.x + blockIdx.x) & 511][slot] = clock64(); } while (0)
+#define GACONV_TALLY(slot, v) do { gaconv_tuning_cl[(blockIdx.y * gridDim.x + blockIdx.x) & 511][slot] = (v); } while (0)
+#define GACONV_CLOCK() clock64()
+#else
+#define GACONV_STAMP(slot, cond) do { } while (0)
+#define GACONV_TALLY(slot, v) do { } while (0)
+#define GACONV_CLOCK() 0
+#endif
+
+namespace gaconv {
+namespace {
+
+constexpr int kMaxGroups = 16, kMaxKsteps = 128, kMaxStages = 8;
+
+struct ClGroup {            // one MMA of a k-step
+    int x_off;              // offset of its X rows inside the X region of a stage, 16-byte units
+    int r, s0, cnt, cbase;  // filter row, first column shift, atoms in use, first channel (relative to the c-tile)
+};
+
+struct ClParams {
+    int n, c, h, w, k, r, s, p, q, stride, pad_h, pad_w;
+    long long ws_k, ws_c, ws_r, ws_s;
+    float alpha;
+    int tiles_k, tiles_c, tiles_r, splits, chunk_base, chunk_rem, chunks;
+    int ci, bp, cpi;                // chunk = ci whole images, or bp output rows of one; chunks per image
+    int kt, rc, ct;                 // output channels, filter rows and channels per tile
+    int ka, katoms, ca, na;         // channels per atom (one shared-memory row) and atoms per tile, dY and X
+    int planes, nprod;              // bf16: 1, 1; fp32: 3, 6
+    int phases, row_tiles;          // X tiles per chunk and atom: column phases x filter rows (stride > 1), else 1 x 1
+    int dy_box, dy_alloc, x_box, x_alloc;       // bytes one copy writes, and the distance to the next tile
+    int x_region, x_plane, dy_plane, stage_bytes, stages;
+    uint32_t tx_bytes;
+    int paired, ksteps, x_pitch, dy_pitch, x_img, dy_img;
+    int c_side;                     // 1: X is the M side
+    int merged;                     // 1: the MN atoms of an X operand are channel atoms, 0: column shifts
+    int ngroups, nmma, cols, tmem_cols;
+    int epoch;                      // chunks of one issuer between two readings of its accumulators
+    uint32_t x_hi, dy_hi, x_lbo, dy_lbo, idesc;
+    ClGroup g[kMaxGroups];
+    uint2 k_off[kMaxKsteps];        // k-step -> offset of its X and dY rows, 16-byte units
+};
+
+// fp32 operands: which planes of X and dY each of the six products of a k-step takes
+__device__ constexpr uint32_t prod_x(int i) { return i == 1 ? 2u : (i == 2 || i == 4) ? 1u : 0u; }
+__device__ constexpr uint32_t prod_dy(int i) { return i == 0 ? 2u : (i == 2 || i == 3) ? 1u : 0u; }
+
+// Warps: 0 and 1 issue MMAs, 2 and 3 fill the stages, 4 to 11 hold the sums.
+//
+// The tensor core adds into its accumulators by truncation, so an accumulator's error grows with the number of additions
+// (~2e-8 of it each).  After every `epoch` chunks an issuer hands its accumulator set to the eight summing warps, which add
+// it to fp32 registers, and starts afresh: the error stays that of a short sum.  There are two sets and two issuers, which
+// take alternate chunks: while one waits (for data, for its set to be read, or merely for its own instructions), the other
+// keeps the tensor core busy.
+constexpr int kThreads = 384, kMaxCols = 192;
+
+template <int NG, bool F32, bool CSIDE>
+__global__ void __launch_bounds__(kThreads, 1)
+cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CUtensorMap map_x, float* __restrict__ dw,
+          float* __restrict__ partial, uint32_t* __restrict__ status, const __grid_constant__ ClParams P)
+{
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t bar_full[kMaxStages], bar_empty[kMaxStages], bar_acc[2], bar_free[2];
+    __shared__ uint32_t s_tmem_base;
+    __shared__ volatile int s_abort;
+    __shared__ int2 s_col[kMaxCols];        // column of the block -> {offset in dW, atoms in use}
+
+    const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tile = blockIdx.x, split = blockIdx.y;
+    const int r0 = (tile % P.tiles_r) * P.rc, kc = tile / P.tiles_r;
+    const int k0 = (kc / P.tiles_c) * P.kt, c0 = (kc % P.tiles_c) * P.ct;
+    const int ch_begin = split * P.chunk_base + min(split, P.chunk_rem);
+    const int nchunks = P.chunk_base + (split < P.chunk_rem ? 1 : 0);
+
+    GACONV_STAMP(0, threadIdx.x == 0);
+    pdl_release_next_grid();
+    // Rows behind the copied boxes that MMAs may touch: zeros, written once (no copy ever reaches them).  A zero dY row
+    // makes the reduction end where the chunk ends; the X rows opposite only have to be finite.
+    {
+        const int tiles_dy = P.planes * P.katoms, tiles_all = tiles_dy + P.planes * P.na * P.phases * P.row_tiles;
+        for (int t = warp; t < P.stages * tiles_all; t += kThreads / 32) {
+            const int st = t / tiles_all, i = t - st * tiles_all;
+            const bool is_dy = i < tiles_dy;
+            const int base = st * P.stage_bytes + (is_dy ? i * P.dy_alloc : P.x_region + (i - tiles_dy) * P.x_alloc);
+            const int from = is_dy ? P.dy_box : P.x_box, to = is_dy ? P.dy_alloc : P.x_alloc;
+            for (int o = from + lane * 16; o < to; o += 512)
+                asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(smem_base + base + o), "r"(0) : "memory");
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (threadIdx.x == 0) {
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&map_dy) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
+        for (int i = 0; i < P.stages; ++i) { mbar_init(smem_u32(&bar_full[i]), 1); mbar_init(smem_u32(&bar_empty[i]), 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&bar_acc[i]), 1); mbar_init(smem_u32(&bar_free[i]), 8); }
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"(P.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_base = s_tmem_base;
+    pdl_wait_prior_grid();
+    GACONV_STAMP(1, threadIdx.x == 0);
+
+    if (warp == 2 || warp == 3) {
+        // ------------------------------------------------------------------ TMA producers
+        // Each fills every other chunk; lane b issues copy b.  Filling a stage (wait, byte count, copies) takes a warp ~600
+        // cycles however large the copies are: one producer gave 33 bytes a cycle on 37 KB stages, two give 66.
+        const bool whole = P.cpi == 0;
+        constexpr int np = 2;
+        const int first = warp - 2, c_first = ch_begin + first;
+        int n0 = whole ? c_first * P.ci : c_first / P.cpi, p0 = whole ? 0 : (c_first % P.cpi) * P.bp;
+        // this lane's copy of every chunk (a plan has at most 32): where it goes, and its coordinates relative to the chunk's
+        const int x_tiles = P.na * P.phases * P.row_tiles, per_plane = P.katoms + x_tiles;
+        const int pl = lane / per_plane, i = lane - pl * per_plane, j = i - P.katoms, jt = j / P.na, rl = jt / P.phases;
+        const bool mine = lane < P.planes * per_plane, is_dy = i < P.katoms;
+        const CUtensorMap* map = is_dy ? &map_dy : &map_x;
+        const uint32_t dst = is_dy ? pl * P.dy_plane + i * P.dy_alloc : P.x_region + pl * P.x_plane + j * P.x_alloc;
+        const int ch = is_dy ? k0 + P.ka * i : c0 + P.ca * (j - jt * P.na), col = is_dy ? 0 : jt - rl * P.phases - P.pad_w;
+        const int row_mul = is_dy ? 1 : P.stride, row_add = is_dy ? 0 : r0 + rl - P.pad_h;
+        int st = first, ph = 0, it = first;
+        while (st >= P.stages) { st -= P.stages; ph ^= 1; }
+        for (; it < nchunks; it += np) {
+            const uint32_t full = smem_u32(&bar_full[st]);
+            if (it >= P.stages && !mbar_wait(smem_u32(&bar_empty[st]), ph ^ 1)) { s_abort = 1; atomicOr(status, 1u); }
+            if (__any_sync(0xffffffffu, s_abort)) break;
+            if (lane == 0) mbar_expect_tx(full, P.tx_bytes);
+            __syncwarp();
+            if (mine) tma_load_5d(smem_base + st * P.stage_bytes + dst, map, full, ch, col, p0 * row_mul + row_add, n0, pl);
+            if (whole) n0 += np * P.ci;
+            else for (p0 += np * P.bp; p0 >= P.cpi * P.bp; p0 -= P.cpi * P.bp) ++n0;
+            for (st += np; st >= P.stages; st -= P.stages) ph ^= 1;
+        }
+        if (lane == 0 && s_abort)      // let the copies already issued land (bounded)
+            for (int i = it - np; i >= first && i > it - np - P.stages; i -= np) mbar_wait(smem_u32(&bar_full[i % P.stages]), (i / P.stages) & 1);
+    } else if (warp < 2) {
+        // ------------------------------------------------------------------ MMA issuers
+        // The whole warp walks the chunks and one elected lane issues (elected rather than "lane 0": the compiler then knows
+        // that a single thread is active and moves descriptors to uniform registers without a loop over lanes; the lane
+        // test cost ~100 cycles per MMA).  An MMA holds its registers until the tensor core takes it, and a loop that
+        // comes round to the same registers waits for that, ~200 cycles; predicates computed per MMA cost ~100 each.
+        // Hence straight-line code of a dozen MMAs per iteration, entered in the middle for a remainder, the offsets of the
+        // k-steps in the parameter bank, and the one MMA that starts an accumulator issued apart.
+        constexpr int PER = NG * (F32 ? 6 : 1), U = PER >= 8 ? 1 : PER == 1 ? 12 : PER == 2 ? 6 : PER == 3 ? 4 : 2;
+        const uint32_t x_plane = (uint32_t)P.x_plane >> 4, dy_plane = (uint32_t)P.dy_plane >> 4;
+        const uint64_t x_hi = (uint64_t)P.x_hi << 32, dy_hi = (uint64_t)P.dy_hi << 32;
+        const int ksteps = P.ksteps, ngroups = P.ngroups;
+        const uint32_t nmma = P.nmma, idesc = P.idesc;
+        uint32_t off[NG];
+#pragma unroll
+        for (int g = 0; g < NG; ++g) off[g] = NG <= 9 || g < ngroups ? (uint32_t)P.g[g].x_off : 0u;
+        const uint32_t acc = tmem_base + warp * P.cols;
+        int st = warp, ph = 0, in_epoch = 0, free_ph = 0;       // (the number of stages is even: a stage is always the same issuer's)
+        long long waited = 0;          // (tuning builds)
+        for (int it = warp; it < nchunks; it += 2) {
+            if (in_epoch == P.epoch) {
+                if (elect_one()) umma_commit(smem_u32(&bar_acc[warp]));
+                if (!mbar_wait(smem_u32(&bar_free[warp]), free_ph)) { s_abort = 1; atomicOr(status, 1u); break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                free_ph ^= 1; in_epoch = 0;
+            }
+            const long long t0 = GACONV_CLOCK();
+            if (!mbar_wait(smem_u32(&bar_full[st]), ph)) { s_abort = 1; atomicOr(status, 1u); break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            waited += GACONV_CLOCK() - t0;
+            GACONV_STAMP(2, it == 0);
+            const bool fresh = in_epoch == 0;
+            if (elect_one()) {
+                const uint32_t sa = smem_base + st * P.stage_bytes;
+                const uint32_t dy_lo = P.dy_lbo | ((sa >> 4) & 0x3fffu), x_lo = P.x_lbo | (((sa + P.x_region) >> 4) & 0x3fffu);
+                auto step = [&](int k, bool starts) {
+                    const uint2 o = P.k_off[k];
+#pragma unroll
+                    for (int pr = 0; pr < (F32 ? 6 : 1); ++pr) {
+                        const uint64_t dyd = dy_hi | (dy_lo + o.y + (F32 ? prod_dy(pr) * dy_plane : 0u));
+                        const uint64_t xd = x_hi | (x_lo + o.x + (F32 ? prod_x(pr) * x_plane : 0u));
+#pragma unroll
+                        for (int g = 0; g < NG; ++g)
+                            if (NG <= 9 || g < ngroups) {          // (up to nine MMAs there is an instance for every count)
+                                const uint64_t ad = CSIDE ? xd + off[g] : dyd, bd = CSIDE ? dyd : xd + off[g];
+                                if (starts && pr == 0) umma_bf16(acc + g * nmma, ad, bd, idesc, 0u);
+                                else umma_bf16_acc(acc + g * nmma, ad, bd, idesc);
+                            }
+                    }
+                };
+                int k = 0;
+                if (fresh) step(k++, true);
+                switch ((ksteps - k) % U) {
+                    case 11: step(k++, false); [[fallthrough]];
+                    case 10: step(k++, false); [[fallthrough]];
+                    case 9: step(k++, false); [[fallthrough]];
+                    case 8: step(k++, false); [[fallthrough]];
+                    case 7: step(k++, false); [[fallthrough]];
+                    case 6: step(k++, false); [[fallthrough]];
+                    case 5: step(k++, false); [[fallthrough]];
+                    case 4: step(k++, false); [[fallthrough]];
+                    case 3: step(k++, false); [[fallthrough]];
+                    case 2: step(k++, false); [[fallthrough]];
+                    case 1: step(k++, false);
+                }
+                for (; k < ksteps; k += U) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) step(k + u, false);
+                }
+                umma_commit(smem_u32(&bar_empty[st]));
+            }
+            __syncwarp();
+            ++in_epoch;
+            for (st += 2; st >= P.stages; st -= P.stages) ph ^= 1;
+        }
+        if (warp < nchunks && elect_one()) {
+            umma_commit(smem_u32(&bar_acc[warp]));
+            GACONV_STAMP(3, warp == 0);
+            if (warp == 0) GACONV_TALLY(6, waited);
+        }
+        __syncwarp();
+    } else if (warp >= 4) {
+        // ------------------------------------------------------------------ summing warps
+        // Warps w and w + 4 read the same 32 lanes of tensor memory and take alternate 16-column pieces.
+        constexpr int NB = kMaxCols / 32;
+        const int sp = warp & 3, half = (warp - 4) >> 2, l128 = 32 * sp + lane, blocks = P.cols >> 4;
+        float sum[NB][16];
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+#pragma unroll
+            for (int e = 0; e < 16; ++e) sum[i][e] = 0.f;
+        bool ok = true;
+        for (int done = 0, ph = 0; done < nchunks && ok; done += 2 * P.epoch, ph ^= 1)
+            for (int set = 0; set < 2 && done + set < nchunks && ok; ++set) {
+                ok = mbar_wait(smem_u32(&bar_acc[set]), ph);
+                if (!ok) { s_abort = 1; atomicOr(status, 1u); }
+                ok = __all_sync(0xffffffffu, ok && !s_abort);        // warp-uniform: the tensor-memory loads are warp-wide
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (!ok) break;
+                const uint32_t src = tmem_base + set * P.cols + 16 * half + ((uint32_t)(32 * sp) << 16);
+#pragma unroll
+                for (int i = 0; i < NB; i += 2) {                    // two pieces in flight
+                    if (2 * i + half < blocks) {
+                        float v[2][16];
+                        const bool two = i + 1 < NB && 2 * (i + 1) + half < blocks;
+                        tmem_ld16_nowait(src + 32 * i, v[0]);
+                        if (two) tmem_ld16_nowait(src + 32 * (i + 1), v[1]);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) sum[i][e] += v[0][e];
+                        if (i + 1 < NB && two) {
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) sum[i + 1 < NB ? i + 1 : i][e] += v[1][e];
+                        }
+                    }
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_free[set])) : "memory");
+            }
+        GACONV_STAMP(4, threadIdx.x == 128);
+        // ------------------------------------------------------------------ block -> workspace, or dW
+        // Through shared memory, [column][128 lanes] (the stages are free: every copy has landed and every MMA has read).
+        // The workspace copy then is one bulk store per 16 columns; the only split of a tile writes dW itself, along the
+        // channels (one word of padding per column: lanes that read along the columns stay in different banks).
+        if (ok) {
+            const bool direct = P.splits == 1;
+            const int pitch = direct ? 129 : 128, t = threadIdx.x - 128;
+            float* blk = reinterpret_cast<float*>(smem_raw + (smem_base - smem_u32(smem_raw)));
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+                if (2 * i + half < blocks) {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) blk[(16 * (2 * i + half) + e) * pitch + l128] = sum[i][e];
+                }
+            if (direct)
+                for (int col = t; col < P.cols; col += 256) {
+                    const int g = col / P.nmma, j = col - g * P.nmma;
+                    const ClGroup& G = P.g[g];
+                    const int a = CSIDE ? 0 : P.merged ? 0 : j / P.ca, c = c0 + G.cbase + (CSIDE ? 0 : P.merged ? j : j - a * P.ca);
+                    const int k = CSIDE ? k0 + j : 0;
+                    const bool valid = r0 + G.r < P.r && (CSIDE ? k < P.k : c < P.c && a < G.cnt);
+                    s_col[col] = make_int2((int)(k * P.ws_k + c * P.ws_c + (r0 + G.r) * P.ws_r + (G.s0 + P.stride * a) * P.ws_s), valid ? G.cnt : 0);
+                }
+            else asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            if (!direct) {
+                float* out = partial + ((size_t)tile * P.splits + split) * P.cols * 128;
+                if (t < blocks) {
+                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(out + t * 2048), "r"(smem_base + t * 8192), "r"(8192) : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+                }
+            } else if (CSIDE) {
+                const int a = l128 / P.ca, cc = P.merged ? l128 : l128 - a * P.ca;          // this lane's atom and channel
+                float* d = dw + (P.merged ? 0 : (long long)P.stride * a * P.ws_s) + cc * P.ws_c;
+                if (c0 + cc < P.c) {
+#pragma unroll 8
+                    for (int col = half; col < P.cols; col += 2) {
+                        const int2 o = s_col[col];
+                        if (P.merged ? o.y > 0 : a < o.y) d[o.x] = P.alpha * blk[col * 129 + l128];
+                    }
+                }
+            } else {
+                int off[NB];                // this lane's columns, the same in every row; -1: none
+#pragma unroll
+                for (int u = 0; u < NB; ++u) {
+                    const int2 o = lane + 32 * u < P.cols ? s_col[lane + 32 * u] : make_int2(0, 0);
+                    off[u] = o.y > 0 ? o.x : -1;
+                }
+#pragma unroll 2
+                for (int l = warp - 4; l < 128; l += 8) {
+                    if (k0 + l >= P.k) break;
+                    float* d = dw + (k0 + l) * P.ws_k;
+#pragma unroll
+                    for (int u = 0; u < NB; ++u)
+                        if (off[u] >= 0) d[off[u]] = P.alpha * blk[(lane + 32 * u) * 129 + l];
+                }
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    GACONV_STAMP(5, threadIdx.x == 0);
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(P.tmem_cols) : "memory");
+    }
+}
+
+// Sum of the splits of every (tile, column), in split order: grid (column groups, tiles).  A warp adds one column's 128
+// lanes (a float4 each) over every W-th split; the W partial sums of a column meet in shared memory.  A block finishes
+// CB columns, so that where consecutive columns are consecutive channels of dW it writes CB of them in one piece.
+template <int CB>
+__global__ void __launch_bounds__(256)
+cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, const __grid_constant__ ClParams P)
+{
+    constexpr int W = 8 / CB;
+    __shared__ float s_sum[8][128];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tile = blockIdx.y, col0 = blockIdx.x * CB;
+    const int r0 = (tile % P.tiles_r) * P.rc, kc = tile / P.tiles_r;
+    const int k0 = (kc / P.tiles_c) * P.kt, c0 = (kc % P.tiles_c) * P.ct;
+    pdl_release_next_grid();
+    pdl_wait_prior_grid();
+    {
+        const int cb = warp % CB, sw = warp / CB, col = col0 + cb, g = col / P.nmma, j = col - g * P.nmma;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        bool live = col < P.cols && r0 + P.g[g].r < P.r;
+        if (live) {
+            if (P.c_side) live = k0 + j < P.k;
+            else live = c0 + P.g[g].cbase + (P.merged ? j : j % P.ca) < P.c;
+        }
+        if (live) {
+            const float4* src = reinterpret_cast<const float4*>(partial + ((size_t)tile * P.splits * P.cols + col) * 128) + lane;
+            const size_t step = (size_t)P.cols * 32;
+            for (int s = sw; s < P.splits; s += 8 * W) {
+                float4 u[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) u[i] = s + i * W < P.splits ? __ldcg(src + (size_t)(s + i * W) * step) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) { acc.x += u[i].x; acc.y += u[i].y; acc.z += u[i].z; acc.w += u[i].w; }
+            }
+        }
+        *reinterpret_cast<float4*>(&s_sum[sw * CB + cb][4 * lane]) = acc;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 128 * CB; e += 256) {
+        const int cb = P.c_side ? e / 128 : e % CB, l = P.c_side ? e % 128 : e / CB, col = col0 + cb;
+        if (col >= P.cols) continue;
+        float t = s_sum[cb][l];
+#pragma unroll
+        for (int w = 1; w < W; ++w) t += s_sum[w * CB + cb][l];
+        const int gi = col / P.nmma, j = col - gi * P.nmma, mn = P.c_side ? l : j, a = mn / P.ca;
+        const ClGroup& g = P.g[gi];
+        const int k = k0 + (P.c_side ? j : l), c = c0 + g.cbase + (P.merged ? mn : mn - a * P.ca);
+        const int r = r0 + g.r, s = P.merged ? g.s0 : g.s0 + P.stride * a;
+        if (k < P.k && c < P.c && r < P.r && (P.merged || a < g.cnt))
+            dw[k * P.ws_k + c * P.ws_c + r * P.ws_r + s * P.ws_s] = P.alpha * t;
+    }
+}
+
+// ---- packing: one operand -> channels-last bf16 planes, channels padded to a multiple of 8 with zeros -------------------
+struct PackOp {
+    const void* src;
+    __nv_bfloat16* dst;
+    int ch, chp, px, n;         // source: n images of px pixels and ch channels; destination rows of chp channels
+    int channels_last;          // source order: 1 [n][px][ch], 0 [n][ch][px]
+    int px_tiles, ch_tiles;     // tiles of an image (channels-first sources): kPackPx pixels x
+    int ch_tile;                // at most 64 channels, a multiple of 8
+    int blocks;                 // tiles in all
+    size_t plane;               // elements of a destination plane
+};
+
+__device__ __forceinline__ uint32_t bf16_pair(float a, float b) {
+    const __nv_bfloat162 t = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&t);
+}
+// two fp32 values -> their planes, packed pairwise: x0 = the upper 16 bits of x (no rounding, so nothing overflows),
+// x1 = bf16(x - x0), x2 = bf16(x - x0 - x1); both differences are exact
+__device__ __forceinline__ void split2(float u, float v, uint32_t (&w)[3]) {
+    const uint32_t a = __float_as_uint(u) & 0xffff0000u, b = __float_as_uint(v) & 0xffff0000u;
+    w[0] = (a >> 16) | b;
+    const float ru = u - __uint_as_float(a), rv = v - __uint_as_float(b);
+    w[1] = bf16_pair(ru, rv);
+    w[2] = bf16_pair(ru - __uint_as_float(w[1] << 16), rv - __uint_as_float(w[1] & 0xffff0000u));
+}
+// copies `bytes` (4, 8 or 16) to shared memory without a stop in registers; zeros instead when !in
+template <int BYTES>
+__device__ __forceinline__ void copy_async(uint32_t dst, const void* src, bool in) {
+    const int n = in ? BYTES : 0;
+    if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(BYTES), "r"(n) : "memory");
+}
+
+// Blocks [0, x.blocks) pack X, the others dY.  E: the element as a plain number of its size (float, or the 16 bits of a
+// bf16).  A block turns a tile of 64 channels x 128 pixels (64 of fp32, whose three planes take the room) of a channels-first source: rows of pixels arrive in shared memory
+// (asynchronous copies where rows start on 4-byte boundaries), ldmatrix.trans turns 8 x 8 blocks on the way out, and with its
+// row addresses ordered (0 1 8 9 16 17 24 25), (2 3 10 11 ...) ... a lane receives eight consecutive channels of a pixel, one
+// 16-byte store.  (Turning by single elements in registers was bound by instructions: 22 us on 13 MB of gradients and 8 MB of
+// activations.)  The 16-byte chunks of a row are permuted by the same order, so that the eight rows of a block sit in
+// different banks.
+template <typename E> constexpr int kPackPx = sizeof(E) == 4 ? 64 : 128;
+
+template <typename E>
+__global__ void __launch_bounds__(256)
+pack_kernel(const PackOp x, const PackOp dy)
+{
+    constexpr int NP = sizeof(E) == 4 ? 3 : 1, TPX = kPackPx<E>, ROW = 2 * TPX;       // planes; bytes of a tile row
+    __shared__ __align__(128) unsigned char s_tile[NP][64 * ROW];
+    pdl_release_next_grid();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool is_x = (int)blockIdx.x < x.blocks;
+    const PackOp& o = is_x ? x : dy;
+    const int blk = is_x ? blockIdx.x : blockIdx.x - x.blocks;
+    const E* src = static_cast<const E*>(o.src);
+    if (o.channels_last) {
+        const int g8 = o.chp >> 3;
+        const size_t items = (size_t)o.n * o.px * g8;
+        const bool vec = (o.ch & 7) == 0;
+        pdl_wait_prior_grid();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const size_t it = (size_t)blk * 1024 + i * 256 + threadIdx.x;
+            if (it >= items) return;
+            const size_t row = it / g8;
+            const int c = (int)(it - row * g8) * 8;
+            const E* p = src + row * o.ch + c;
+            alignas(16) E v[8];
+            if (vec) {
+                const uint4* q = reinterpret_cast<const uint4*>(p);
+#pragma unroll
+                for (int j = 0; j < (int)sizeof(E) / 2; ++j) reinterpret_cast<uint4*>(v)[j] = __ldg(q + j);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = c + j < o.ch ? __ldg(p + j) : E(0);
+            }
+            uint4* out = reinterpret_cast<uint4*>(o.dst + row * o.chp + c);
+            if constexpr (sizeof(E) == 4) {
+                uint32_t w[4][3];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) split2(v[2 * j], v[2 * j + 1], w[j]);
+#pragma unroll
+                for (int pl = 0; pl < 3; ++pl) out[pl * (o.plane / 8)] = make_uint4(w[0][pl], w[1][pl], w[2][pl], w[3][pl]);
+            } else {
+                *out = *reinterpret_cast<const uint4*>(v);
+            }
+        }
+        return;
+    }
+    const int per_img = o.px_tiles * o.ch_tiles, n = blk / per_img, rest = blk - n * per_img, ct = rest / o.px_tiles, c0 = ct * o.ch_tile;
+    const int p0 = (rest - ct * o.px_tiles) * TPX, rows = min(o.ch_tile, o.ch - c0), left = min(TPX, o.px - p0);
+    const E* base = src + ((size_t)n * o.ch + c0) * o.px + p0;
+    const uint32_t tile = smem_u32(s_tile);
+    auto at = [&](int row, int px) {          // byte offset of a pixel in its (permuted) row
+        const int sw = (((row >> 3) & 3) << 1) | (row & 1);
+        return row * ROW + ((((px >> 3) ^ sw) << 4) | ((px & 7) << 1));
+    };
+    pdl_wait_prior_grid();
+    if constexpr (sizeof(E) == 2) {
+        if ((o.px & 1) == 0) {
+            auto fill = [&](auto width) {
+                constexpr int V = decltype(width)::value;
+#pragma unroll
+                for (int i = 0; i < 32 / V; ++i) {
+                    const int e = (i * 256 + (int)threadIdx.x) * V, row = e >> 7, px = e & 127;
+                    const bool in = row < rows && px < left;
+                    copy_async<2 * V>(tile + at(row, px), in ? base + (size_t)row * o.px + px : src, in);
+                }
+            };
+            if ((o.px & 7) == 0) fill(std::integral_constant<int, 8>());
+            else if ((o.px & 3) == 0) fill(std::integral_constant<int, 4>());
+            else fill(std::integral_constant<int, 2>());
+            asm volatile("cp.async.wait_all;" ::: "memory");
+        } else {
+            // rows of odd length: 32-bit loads from the word that holds the row's first pixel; a row that starts in the middle
+            // of a word takes each pair of pixels from two neighbouring words
+#pragma unroll 4
+            for (int i = 0; i < 16; ++i) {
+                const int row = warp + 8 * (i >> 1), l = lane + 32 * (i & 1);
+                const E* q = base + (size_t)row * o.px;
+                const uint32_t* w = reinterpret_cast<const uint32_t*>(reinterpret_cast<uintptr_t>(q) & ~(uintptr_t)3);
+                const int odd = (int)((reinterpret_cast<uintptr_t>(q) >> 1) & 1);
+                auto word = [&](int k) -> uint32_t {             // (a word is read whole only if both halves lie in the row)
+                    const int first = 2 * k - odd;
+                    if (row >= rows || first >= left) return 0u;
+                    if (first + 1 < left && first >= 0) return __ldg(w + k);
+                    const unsigned short* h = reinterpret_cast<const unsigned short*>(w + k);
+                    return first < 0 ? (uint32_t)__ldg(h + 1) << 16 : (uint32_t)__ldg(h);
+                };
+                const uint32_t w0 = word(l), w1 = odd ? word(l + 1) : 0u;
+                *reinterpret_cast<uint32_t*>(&s_tile[0][at(row, 2 * l)]) = odd ? __funnelshift_r(w0, w1, 16) : w0;
+            }
+        }
+    } else {
+        const bool vec = (o.px & 3) == 0;
+#pragma unroll 4
+        for (int i = 0; i < TPX / 16; ++i) {
+            const int e = (i * 256 + (int)threadIdx.x) * 4, row = e / TPX, px = e % TPX;
+            const E* q = base + (size_t)row * o.px + px;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row < rows) {
+                if (vec) { if (px < left) v = __ldg(reinterpret_cast<const float4*>(q)); }
+                else {
+                    if (px < left) v.x = __ldg(q);
+                    if (px + 1 < left) v.y = __ldg(q + 1);
+                    if (px + 2 < left) v.z = __ldg(q + 2);
+                    if (px + 3 < left) v.w = __ldg(q + 3);
+                }
+            }
+            uint32_t w0[3], w1[3];
+            split2(v.x, v.y, w0); split2(v.z, v.w, w1);
+#pragma unroll
+            for (int pl = 0; pl < NP; ++pl) *reinterpret_cast<uint2*>(&s_tile[pl][at(row, px)]) = make_uint2(w0[pl], w1[pl]);
+        }
+    }
+    __syncthreads();
+    const int rho = lane & 7, m = lane >> 3, end = min(c0 + o.ch_tile, o.chp);
+#pragma unroll
+    for (int i = 0; i < TPX / 32; ++i) {
+        const int blk8 = warp * (TPX / 64) + (i >> 1), h = i & 1;        // eight pixels, half of the channels
+        const int row = h * 32 + 8 * (rho >> 1) + 2 * m + (rho & 1);
+        const int px = 8 * blk8 + (lane >> 2), c = c0 + h * 32 + 8 * (lane & 3);
+#pragma unroll
+        for (int pl = 0; pl < NP; ++pl) {
+            uint32_t r[4];
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(tile + pl * 64 * ROW + at(row, 8 * blk8)) : "memory");
+            if (px < left && c < end)
+                *reinterpret_cast<uint4*>(o.dst + pl * o.plane + ((size_t)n * o.px + p0 + px) * o.chp + c) = make_uint4(r[0], r[1], r[2], r[3]);
+        }
+    }
+}
+
+// ---------------------------------------------------------------- host side: the plan
+int round_up(int v, int m) { return (v + m - 1) / m * m; }
+int ceil_div(int a, int b) { return (a + b - 1) / b; }
+
+constexpr int kStageBudget = 216 * 1024;
+
+// What a candidate costs, in SM cycles, from rates measured with kernels of one kind each: an MMA of N columns takes N / 2
+// cycles; shared memory moves 128 bytes a cycle, the MMAs' operands, (128 + N) / 4 cycles, and what the copies write; copies
+// deliver ~80 bytes a cycle and one row (pixel) in no less than 1.4 cycles; a chunk costs its producer and its issuer ~940
+// cycles of instructions each (two of either work in turn); a CTA writes its block at ~21 bytes a cycle; start, first loads,
+// drain and the second kernel come to a few thousand.
+struct Cost { double cycles; int splits; };
+Cost cost_of(const ClParams& P, int sms, double block_share)
+{
+    const double mma = (double)P.ksteps * P.ngroups * P.nprod * P.nmma / 2.0;
+    const double shared = (double)P.ksteps * P.ngroups * P.nprod * ((128 + P.nmma) / 4.0 + 2) + P.tx_bytes / 128.0;
+    const double rows = (double)P.planes * (P.katoms * (P.dy_box / (P.ka * 2)) + P.na * P.phases * P.row_tiles * (P.x_box / (P.ca * 2)));
+    const double load = std::max(P.tx_bytes / 80.0, rows * 1.4);
+    const double chunk = std::max({mma * 1.03, shared, load, 470.0}) * (P.stages > 2 ? 1.0 : 1.2) + 40;
+    const int tiles = P.tiles_k * P.tiles_c * P.tiles_r;
+    const double block_bytes = (double)P.cols * 512 * block_share;
+    Cost best{1e30, 1};
+    const int most = std::max(1, std::min(P.chunks, sms / tiles));
+    for (int sp = most; sp >= 1; sp = sp > 8 ? sp * 7 / 8 : sp - 1) {
+        const int waves = ceil_div(tiles * sp, sms), per = ceil_div(P.chunks, sp);
+        const double main = waves * (4500 + load * std::min({per, P.stages, 4}) / 2 + per * chunk + block_bytes / 21);
+        const double red = sp == 1 ? 0.0 : 4000 + (double)tiles * sp * block_bytes / (25.0 * sms);
+        if (main + red < best.cycles) best = Cost{main + red, sp};
+    }
+    return best;
+}
+
+bool build_groups(ClParams& P)
+{
+    P.ngroups = 0;
+    const int rows = P.rc, st = P.stride, wt = P.x_pitch;
+    // atoms of one MMA on the X side: c-side exactly fills M = 128; k-side as many as N = 256 takes
+    const int atoms_max = P.c_side ? 128 / P.ca : 256 / P.ca;
+    int atoms = 0;
+    auto add = [&](int tile_i, int row_px, int r, int s0, int cnt, int cbase) {
+        if (P.ngroups == kMaxGroups) return false;
+        P.g[P.ngroups++] = ClGroup{(tile_i * P.x_alloc + row_px * P.ca * 2) >> 4, r, s0, cnt, cbase};
+        return true;
+    };
+    if (P.merged) atoms = P.na;
+    else {      // the shifts of a column phase are shared out evenly over as few MMAs as hold them
+        const int shifts = ceil_div(P.s, st);
+        atoms = P.c_side ? atoms_max : ceil_div(shifts, ceil_div(shifts, atoms_max));
+    }
+    for (int rl = 0; rl < rows; ++rl)
+        for (int ph = 0; ph < P.phases; ++ph) {
+            const int base_tile = st > 1 ? (rl * P.phases + ph) * P.na : 0, base_px = st > 1 ? 0 : rl * wt;
+            const int shifts = (P.s - ph + st - 1) / st;
+            if (P.merged) {
+                for (int i = 0; i < shifts; ++i)
+                    if (!add(base_tile, base_px + i, rl, ph + st * i, 1, 0)) return false;
+            } else {
+                for (int a = 0; a < P.na; ++a)
+                    for (int i = 0; i < shifts; i += atoms)
+                        if (!add(base_tile + a, base_px + i, rl, ph + st * i, std::min(atoms, shifts - i), a * P.ca)) return false;
+            }
+        }
+    P.nmma = P.c_side ? P.kt : atoms * P.ca;
+    P.cols = P.ngroups * P.nmma;
+    if (P.cols > kMaxCols) return false;
+    P.tmem_cols = 32;
+    while (P.tmem_cols < 2 * P.cols) P.tmem_cols *= 2;
+    return true;
+}
+
+// Fills the chunk-dependent fields; false when the candidate does not fit.
+bool shape_chunk(ClParams& P, int ci, int bp, bool paired)
+{
+    const int st = P.stride;
+    const bool whole = ci > 1 || bp >= P.p;
+    if (paired) bp = round_up(bp, 2);
+    P.ci = ci; P.bp = bp; P.paired = paired ? 1 : 0;
+    P.cpi = whole ? 0 : ceil_div(P.p, bp);
+    P.chunks = whole ? ceil_div(P.n, ci) : P.n * P.cpi;
+    const int wp = P.q + ceil_div(P.s, st) - 1, halo = st == 1 ? P.rc - 1 : 0;
+    const int x_rows = bp + halo, dy_rows = (!paired && ci > 1) ? bp + halo : bp, dy_w = paired ? P.q : wp;
+    if ((wp - 1) * st + 1 > 256 || (x_rows - 1) * st + 1 > 256 || dy_rows > 256 || ci > 256) return false;
+    P.x_pitch = wp; P.dy_pitch = dy_w; P.x_img = x_rows * wp; P.dy_img = dy_rows * dy_w;
+    P.ksteps = paired ? ci * (bp / 2) * (P.q / 8) : ceil_div(ci * dy_rows * dy_w, 16);
+    if (P.ksteps > kMaxKsteps) return false;
+    const int xb = P.ca * 2, db = P.ka * 2;
+    P.x_box = ci * x_rows * wp * xb;
+    P.dy_box = ci * dy_rows * dy_w * db;
+    // last X row an MMA touches: last k-step, last row and column shift, unused shifts of the c-side form
+    const int last = paired ? (ci - 1) * P.x_img + (bp - 1) * wp + P.q - 1 : P.ksteps * 16 - 1;
+    const int far = last + halo * wp + ceil_div(P.s, st) - 1 + (P.c_side ? 128 / P.ca : 256 / P.ca);
+    P.x_alloc = round_up(std::max(P.x_box, (far + 1) * xb), 1024);
+    P.dy_alloc = round_up(std::max(P.dy_box, paired ? 0 : P.ksteps * 16 * db), 1024);
+    P.x_plane = P.na * P.phases * P.row_tiles * P.x_alloc;
+    P.dy_plane = P.katoms * P.dy_alloc;
+    P.x_region = P.planes * P.dy_plane;
+    P.stage_bytes = P.x_region + P.planes * P.x_plane;
+    if (P.planes * (P.katoms + P.na * P.phases * P.row_tiles) > 32) return false;        // one copy per lane of a producer
+    P.stages = std::min(kMaxStages, kStageBudget / P.stage_bytes) & ~1;
+    P.epoch = std::max(1, (P.nprod > 1 ? 16 : 64) / P.ksteps);
+    if (P.stages < 2) return false;
+    P.tx_bytes = (uint32_t)(P.planes * (P.katoms * P.dy_box + P.na * P.phases * P.row_tiles * P.x_box));
+    if (P.tx_bytes >= (1u << 20)) return false;
+    const uint32_t x_sbo = paired ? wp * xb : 8 * xb, dy_sbo = paired ? dy_w * db : 8 * db;
+    const uint32_t x_swz = P.ca == 64 ? 2 : P.ca == 32 ? 4 : 6, dy_swz = P.ka == 64 ? 2 : P.ka == 32 ? 4 : 6;
+    P.x_hi = (x_sbo >> 4) | (1u << 14) | (x_swz << 29);
+    P.dy_hi = (dy_sbo >> 4) | (1u << 14) | (dy_swz << 29);
+    P.x_lbo = (uint32_t)((P.merged ? P.x_alloc : xb) >> 4) << 16;
+    P.dy_lbo = (uint32_t)((P.katoms > 1 ? P.dy_alloc : 0) >> 4) << 16;      // one atom: the upper half of M repeats the lower
+    for (int i = 0; i < P.ksteps; ++i) {
+        int xr = 16 * i, dr = 16 * i;
+        if (paired) {
+            const int j = i % (P.q / 8), t = i / (P.q / 8), pr = t % (bp / 2), im = t / (bp / 2);
+            xr = im * P.x_img + 2 * pr * wp + 8 * j;
+            dr = im * P.dy_img + 2 * pr * dy_w + 8 * j;
+        }
+        P.k_off[i] = make_uint2((unsigned)(xr * xb) >> 4, (unsigned)(dr * db) >> 4);
+    }
+    return build_groups(P);
+}
+
+struct ClHost {             // what ClPlan::opaque holds
+    ClParams p;
+    bool pack_x, pack_dy, f32, x_nhwc, dy_npqk;
+    int xch, dych;          // channels per pixel row of the operands the tensor maps describe
+    int cb;                 // columns per block of the second kernel
+};
+static_assert(sizeof(ClHost) <= sizeof(ClPlan::opaque), "ClPlan::opaque too small");
+
+PackOp pack_op(const void* src, void* dst, int ch, int px, int n, bool last, size_t plane, int tile_px)
+{
+    PackOp o{};
+    o.src = src; o.dst = static_cast<__nv_bfloat16*>(dst);
+    o.ch = ch; o.chp = round_up(ch, 8); o.px = px; o.n = n; o.channels_last = last ? 1 : 0; o.plane = plane;
+    o.px_tiles = ceil_div(px, tile_px); o.ch_tiles = ceil_div(ch, 64);
+    o.ch_tile = round_up(ceil_div(ch, o.ch_tiles), 8);
+    o.ch_tiles = ceil_div(ch, o.ch_tile);
+    o.blocks = last ? (int)(((size_t)n * px * (o.chp / 8) + 1023) / 1024) : n * o.px_tiles * o.ch_tiles;
+    return o;
+}
+
+typedef void (*ClKernel)(const CUtensorMap, const CUtensorMap, float*, float*, uint32_t*, const ClParams);
+ClKernel kernel_for(int ng, bool f32, bool c_side)
+{
+#define GACONV_CL_PICK(N) if (ng <= N) return f32 ? (c_side ? cl_kernel<N, true, true> : cl_kernel<N, true, false>) : (c_side ? cl_kernel<N, false, true> : cl_kernel<N, false, false>);
+    GACONV_CL_PICK(1) GACONV_CL_PICK(2) GACONV_CL_PICK(3) GACONV_CL_PICK(4) GACONV_CL_PICK(5) GACONV_CL_PICK(6) GACONV_CL_PICK(7) GACONV_CL_PICK(8)
+    GACONV_CL_PICK(9) GACONV_CL_PICK(16)
+#undef GACONV_CL_PICK
+    return nullptr;
+}
+
+}  // namespace
+
+bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
+{
+    if (g.stride_h != g.stride_w || g.r > 16 || g.s > 16) return false;
+    const bool nhwc = g.xs_c == 1 || g.c == 1;
+    ClHost H{};
+    H.f32 = !g.bf16;
+    H.x_nhwc = nhwc; H.dy_npqk = dy_npqk || g.k == 1;
+    H.pack_x = H.f32 || !nhwc || g.c % 8 != 0;
+    H.pack_dy = H.f32 || !H.dy_npqk || g.k % 8 != 0;
+    H.xch = round_up(g.c, 8); H.dych = round_up(g.k, 8);
+    const size_t x_el = (size_t)g.n * g.h * g.w * H.xch, dy_el = (size_t)g.n * g.p * g.q * H.dych;
+    if (x_el > ((size_t)1 << 31) || dy_el > ((size_t)1 << 31)) return false;
+
+    ClParams B{};
+    B.n = g.n; B.c = g.c; B.h = g.h; B.w = g.w; B.k = g.k; B.r = g.r; B.s = g.s; B.p = g.p; B.q = g.q;
+    B.stride = g.stride_h; B.pad_h = g.pad_h; B.pad_w = g.pad_w; B.alpha = g.alpha;
+    B.ws_k = g.ws_k; B.ws_c = g.ws_c; B.ws_r = g.ws_r; B.ws_s = g.ws_s;
+    B.planes = H.f32 ? 3 : 1; B.nprod = H.f32 ? 6 : 1;
+    B.phases = std::min(g.stride_h, g.s);
+    B.ca = g.c > 32 ? 64 : g.c > 16 ? 32 : 16;
+    const int sms = g.sm_budget > 0 ? std::min(g.sm_budget, device_sms()) : device_sms();
+
+    ClParams best{};
+    double best_cycles = 1e30;
+    for (int form = 0; form < 2; ++form) {
+        const int k16 = round_up(g.k, 16);
+        const int kts[4] = {form ? std::min(k16, 256) : 128, 128, 64, 32};
+        for (int ki = 0; ki < (form ? 4 : 1); ++ki) {
+            if (ki > 0 && (kts[ki] >= kts[0] || kts[ki] >= k16)) continue;
+            ClParams F = B;
+            F.c_side = form; F.kt = kts[ki];
+            const int kw = std::min(F.kt, k16);
+            F.ka = kw > 32 ? 64 : kw > 16 ? 32 : 16;
+            F.katoms = ceil_div(kw, F.ka);
+            F.tiles_k = ceil_div(g.k, F.kt);
+            for (int na = 1; na <= 4; na *= 2) {
+                if (na > 1 && (F.ca < 64 || (na - 1) * 64 >= g.c)) break;
+                if (form && na > 2) break;
+                if (!form && na > 2 && g.s > 1) break;
+                F.na = na; F.ct = na * F.ca;
+                F.merged = na > 1 && (form || g.s == 1) ? 1 : 0;
+                F.tiles_c = ceil_div(g.c, F.ct);
+                for (int rc = 1; rc <= g.r; ++rc) {
+                    F.rc = rc; F.tiles_r = ceil_div(g.r, rc);
+                    if (rc > 1 && ceil_div(g.r, rc) == ceil_div(g.r, rc - 1)) continue;
+                    F.row_tiles = F.stride > 1 ? rc : 1;
+                    if (F.stride == 1) F.phases = 1;
+                    // part of the accumulator block that stands for elements of dW
+                    const double share = (double)g.k * g.c * g.r * g.s / ((double)F.tiles_k * F.tiles_c * F.tiles_r * 128);
+                    for (int mode = 0; mode < 2; ++mode) {
+                        if (mode == 1 && g.q % 8 != 0) break;
+                        auto consider = [&](int ci, int bp) {
+                            ClParams C = F;
+                            if (!shape_chunk(C, ci, bp, mode == 1)) return false;
+#ifdef GACONV_TUNING
+                            if (const char* e = getenv("GACONV_CL_KS")) if (C.ksteps < atoi(e)) return true;
+                            if (const char* e = getenv("GACONV_CL_KSMAX")) if (C.ksteps > atoi(e)) return true;
+                            if (const char* e = getenv("GACONV_CL_FORM")) if (C.c_side != atoi(e)) return true;
+                            if (const char* e = getenv("GACONV_CL_RC")) if (C.rc != atoi(e)) return true;
+                            if (const char* e = getenv("GACONV_CL_KT")) if (C.kt != atoi(e)) return true;
+                            if (const char* e = getenv("GACONV_CL_NA")) if (C.na != atoi(e)) return true;
+#endif
+                            const Cost c = cost_of(C, sms, std::min(1.0, 1.3 * share / C.cols));
+                            if (c.cycles < best_cycles) { best_cycles = c.cycles; C.splits = c.splits; best = C; }
+                            return true;
+                        };
+                        int last_bp = 0;
+                        for (int parts = g.p; parts >= 1; --parts) {      // fewer and fewer, larger and larger bands
+                            int bp = ceil_div(g.p, parts);
+                            if (mode == 1) bp = round_up(bp, 2);
+                            if (bp == last_bp) continue;
+                            last_bp = bp;
+                            if (!consider(1, bp)) break;
+                        }
+                        for (int ci = 2; ci <= 64 && ci <= g.n; ci = ci < 4 ? ci + 1 : ci + ci / 2)
+                            if (!consider(ci, g.p)) break;
+                    }
+                }
+            }
+        }
+    }
+    if (best_cycles >= 1e30) return false;
+    best.chunk_base = best.chunks / best.splits;
+    best.chunk_rem = best.chunks - best.chunk_base * best.splits;
+    best.idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(best.nmma >> 3) << 17) | (8u << 24);
+    H.p = best;
+    H.cb = best.splits > 32 ? 1 : best.splits > 16 ? 2 : best.splits > 8 ? 4 : 8;
+    const int tiles = best.tiles_k * best.tiles_c * best.tiles_r;
+    if (tiles > 65535 || best.splits > 65535) return false;
+    out->cycles = best_cycles;
+    out->partial_bytes = best.splits == 1 ? 0 : (size_t)tiles * best.splits * best.cols * 512;
+    out->x_bytes = H.pack_x ? align_up(x_el * 2 * best.planes, 256) : 0;
+    out->dy_bytes = H.pack_dy ? align_up(dy_el * 2 * best.planes, 256) : 0;
+    memcpy(out->opaque, &H, sizeof(H));
+    return true;
+}
+
+cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, void* x_scratch, void* dy_scratch, uint32_t* status,
+                      const ClPlan& plan, cudaStream_t stream)
+{
+    ClHost H;
+    memcpy(&H, plan.opaque, sizeof(H));
+    const ClParams& P = H.p;
+    cudaError_t err;
+    const size_t x_el = (size_t)P.n * P.h * P.w * H.xch, dy_el = (size_t)P.n * P.p * P.q * H.dych;
+    if (H.pack_x || H.pack_dy) {
+        PackOp ox{}, od{};
+        const int tile_px = H.f32 ? kPackPx<float> : kPackPx<unsigned short>;
+        if (H.pack_x) ox = pack_op(x, x_scratch, P.c, P.h * P.w, P.n, H.x_nhwc, x_el, tile_px);
+        if (H.pack_dy) od = pack_op(dy, dy_scratch, P.k, P.p * P.q, P.n, H.dy_npqk, dy_el, tile_px);
+        const dim3 grid((unsigned)(ox.blocks + od.blocks));
+        err = H.f32 ? launch_kernel(pack_kernel<float>, grid, dim3(256), 0, stream, dim3(1, 1, 1), ox, od)
+                    : launch_kernel(pack_kernel<unsigned short>, grid, dim3(256), 0, stream, dim3(1, 1, 1), ox, od);
+        if (err != cudaSuccess) return err;
+        note_launch();
+        if (H.pack_x) x = x_scratch;
+        if (H.pack_dy) dy = dy_scratch;
+    }
+    // tensor maps over (channel, column, row, image, plane); box extents count the pixels stepped over at the conv stride
+    auto encode = [&](CUtensorMap* map, const void* base, int ch, int chp, int w, int h, size_t plane_el, int atom, int bw, int bh, int st) {
+        const cuuint64_t row = (cuuint64_t)chp * 2;
+        cuuint64_t dims[5] = {(cuuint64_t)ch, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)P.n, (cuuint64_t)P.planes};
+        cuuint64_t strides[4] = {row, row * w, row * w * h, (cuuint64_t)plane_el * 2};
+        cuuint32_t box[5] = {(cuuint32_t)atom, (cuuint32_t)((bw - 1) * st + 1), (cuuint32_t)((bh - 1) * st + 1), (cuuint32_t)P.ci, 1};
+        cuuint32_t es[5] = {1, (cuuint32_t)st, (cuuint32_t)st, 1, 1};
+        const CUtensorMapSwizzle swz = atom == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : atom == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
+        return encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    CUtensorMap map_dy, map_x;
+    if (!encode(&map_dy, dy, P.k, H.dych, P.q, P.p, dy_el, P.ka, P.dy_pitch, P.dy_img / P.dy_pitch, 1) ||
+        !encode(&map_x, x, P.c, H.xch, P.w, P.h, x_el, P.ca, P.x_pitch, P.x_img / P.x_pitch, P.stride))
+        return cudaErrorInvalidValue;
+    // the stages; at the end they hold the accumulator block
+    const size_t smem = std::max((size_t)P.stages * P.stage_bytes, (size_t)P.cols * 129 * 4) + 1024;
+    const dim3 grid((unsigned)(P.tiles_k * P.tiles_c * P.tiles_r), (unsigned)P.splits);
+    ClKernel kern = kernel_for(P.ngroups, H.f32, P.c_side != 0);
+    if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return err;
+    if ((err = launch_kernel(kern, grid, dim3(kThreads), smem, stream, dim3(1, 1, 1), map_dy, map_x, dw, partial, status, P)) != cudaSuccess) return err;
+    note_launch();
+    if (P.splits == 1) return cudaSuccess;
+    const dim3 rgrid((unsigned)ceil_div(P.cols, H.cb), grid.x);
+    err = H.cb == 1   ? launch_kernel(cl_reduce_kernel<1>, rgrid, dim3(256), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P)
+          : H.cb == 2 ? launch_kernel(cl_reduce_kernel<2>, rgrid, dim3(256), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P)
+          : H.cb == 4 ? launch_kernel(cl_reduce_kernel<4>, rgrid, dim3(256), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P)
+                      : launch_kernel(cl_reduce_kernel<8>, rgrid, dim3(256), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P);
+    if (err != cudaSuccess) return err;
+    note_launch();
+    return cudaSuccess;
+}
+
+}  // namespace gaconv
+
+#ifdef GACONV_TUNING
+extern "C" int gaconv_tuning_read_cl(long long* host) { return (int)cudaMemcpyFromSymbol(host, gaconv_tuning_cl, sizeof(gaconv_tuning_cl)); }
+// tuning builds: the plan of a problem, as launch_cl would use it
+extern "C" int gaconv_tuning_plan_cl(const int* v, int bf16, int x_nhwc, int npqk, int budget, void* out, int size)
+{
+    using namespace gaconv;
+    Geom g{};
+    g.n = v[0]; g.c = v[1]; g.h = v[2]; g.w = v[3]; g.k = v[4]; g.r = v[5]; g.s = v[6]; g.stride_h = g.stride_w = v[7]; g.pad_h = g.pad_w = v[8];
+    g.p = (g.h + 2 * g.pad_h - g.r) / g.stride_h + 1; g.q = (g.w + 2 * g.pad_w - g.s) / g.stride_w + 1;
+    g.xs_c = x_nhwc ? 1 : 2;
+    g.ws_c = 1; g.ws_s = g.c; g.ws_r = g.s * g.c; g.ws_k = g.r * g.s * g.c;
+    g.bf16 = bf16 != 0; g.alpha = 1.f; g.sm_budget = budget;
+    ClPlan P;
+    if (!plan_cl(g, npqk != 0, &P) || size < (int)sizeof(ClHost)) return -1;
+    memcpy(out, P.opaque, sizeof(ClHost));
+    return (int)P.cycles;
+}
+#endif

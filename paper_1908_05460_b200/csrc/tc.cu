@@ -50,6 +50,7 @@
 
 #include "gaconv_internal.h"
 #include "tma.cuh"
+#include "umma.cuh"
 
 // GACONV_TUNING builds carry clock64 stamps of CTA (0,0)'s phases (workspace bytes [64,128)) and read
 // planner overrides from the environment; the default build has neither.
@@ -67,14 +68,6 @@ __device__ __forceinline__ unsigned long long gaconv_globaltimer() { unsigned lo
 namespace gaconv {
 namespace {
 
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void umma_bf16_acc(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, 1, 1;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc) : "memory");
-}
 // 16 bytes from the same shared-memory offset in CTA `rank` of this cluster
 __device__ __forceinline__ float4 ld_dsmem_f4(uint32_t local_addr, uint32_t rank) {
     uint32_t remote;
@@ -88,20 +81,6 @@ __device__ __forceinline__ float4 ld_dsmem_f4(uint32_t local_addr, uint32_t rank
 __device__ __forceinline__ void umma_tf32(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
                  ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3, int c4) {
-    asm volatile("cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
-                 ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-// Issues the load only; the caller executes tcgen05.wait::ld before reading v.
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float (&v)[16]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
-                   "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
-                 : "r"(taddr));
 }
 struct TcParams {
     Geom g;
@@ -709,27 +688,13 @@ int env_int(const char* name, int dflt) { const char* e = getenv(name); return e
 constexpr int env_int(const char*, int dflt) { return dflt; }
 #endif
 
-// SMs of the current device (one CTA of this kernel fills an SM)
-int sm_count()
-{
-    static int cached[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
-    if (cached[dev] == 0) {
-        int n = 0;
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 148;
-        cached[dev] = n;
-    }
-    return cached[dev];
-}
-
 // How many clusters of `cl` CTAs of this kernel (one CTA per SM) the current device holds at once.
 int resident_clusters(int cl)
 {
     static int cached[64][5] = {};
-    if (cl <= 1) return sm_count();
+    if (cl <= 1) return device_sms();
     int dev = 0;
-    if (cl > 4 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return sm_count() / cl * 8 / 10;
+    if (cl > 4 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return device_sms() / cl * 8 / 10;
     if (cached[dev][cl] == 0) {
         int n = 0;
         cudaLaunchConfig_t cfg = {};
@@ -741,7 +706,7 @@ int resident_clusters(int cl)
         if (cudaFuncSetAttribute(exact_tc_kernel<0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess ||
             cudaOccupancyMaxActiveClusters(&n, exact_tc_kernel<0, 0>, &cfg) != cudaSuccess || n < 1) {
             (void)cudaGetLastError();
-            n = sm_count() / cl * 8 / 10;          // no answer: a cautious guess
+            n = device_sms() / cl * 8 / 10;          // no answer: a cautious guess
         }
         cached[dev][cl] = n;
     }
@@ -756,7 +721,7 @@ bool choose_splits(TcParams& P, const Geom& g, int tiles)
     // second kernel adds them up.  Larger clusters mean less workspace traffic, but fewer resident CTAs (clusters
     // are placed GPC by GPC: 148 CTAs fit as pairs, 135 as triples, 132 as quadruples).
     // SMs this launch may count on: all of them, or the caller's budget (layers sharing the GPU on several lanes)
-    const int sms = g.sm_budget > 0 ? std::min(g.sm_budget, sm_count()) : sm_count();
+    const int sms = g.sm_budget > 0 ? std::min(g.sm_budget, device_sms()) : device_sms();
     int max_splits = env_int("GACONV_TC_SPLITS", 0);
     if (max_splits <= 0) {
         max_splits = sms / tiles;
@@ -812,6 +777,22 @@ bool choose_splits(TcParams& P, const Geom& g, int tiles)
 }
 
 }  // namespace
+
+// SMs of the current device (one CTA of this kernel fills an SM)
+int device_sms()
+{
+    static int cached[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+    if (cached[dev] == 0) {
+        int n = 0;
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 148;
+        cached[dev] = n;
+    }
+    return cached[dev];
+}
+
+bool tensor_maps_available() { return encode_fn() != nullptr; }
 
 bool plan_tc(const Geom& g, TcPlan* out)
 {

@@ -1,0 +1,79 @@
+"""The channels-last tensor-core kernel (csrc/cl.cu) at the edges of its tiles, against the oracle: odd maps, channel
+counts off every tile size, strides, every packing path, several images per chunk, one split and many."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle
+from paper_1908_05460_b200 import binding as B
+from paper_1908_05460_b200 import inputs as I
+from paper_1908_05460_b200.layers import ConvLayer
+from helpers import GpuLayer, norm_err, oshape, to_f64, TOL_F32
+
+pytestmark = pytest.mark.gpu
+
+# (no other tensor-core kernel tiles these maps; each has more than the 4 million products the kernel is used from)
+SHAPES = [
+    ConvLayer("13x11 c19 k87", 5, 19, 13, 11, 87, 3, 3, 1, 1, dy_std=1.0),
+    ConvLayer("28x20 c72 k120", 3, 72, 28, 20, 120, 3, 3, 1, 1),
+    ConvLayer("7x7 maps, several images, c130 k260", 9, 130, 7, 7, 260, 3, 3, 1, 1),
+    ConvLayer("9x24 row pairs, odd rows", 4, 64, 9, 24, 64, 3, 3, 1, 1),
+    ConvLayer("stride 2, 27x27 -> 14x14", 4, 64, 27, 27, 100, 3, 3, 2, 1),
+    ConvLayer("stride 2, no padding, 5x5", 3, 40, 21, 17, 48, 5, 5, 2, 0),
+    ConvLayer("7x7 filter, stride 2, 3 channels", 6, 3, 33, 31, 64, 7, 7, 2, 3),
+    ConvLayer("7x7 filter c33", 2, 33, 19, 12, 30, 7, 7, 1, 3),
+    ConvLayer("1x1 c200 k72", 7, 200, 11, 5, 72, 1, 1, 1, 0),
+    ConvLayer("many splits, k8", 60, 20, 25, 19, 8, 3, 3, 1, 1),
+    ConvLayer("one output channel", 40, 48, 31, 15, 1, 3, 3, 1, 1),
+    ConvLayer("5x3 maps, more tiles than SMs", 3, 400, 5, 3, 530, 3, 3, 1, 1),
+    ConvLayer("3x5 filter", 6, 36, 18, 18, 44, 3, 5, 1, 1),
+]
+LAYOUTS = {"paper": {}, "nchw": dict(x_layout=B.X_NCHW, dw_layout=B.DW_KCRS),
+           "nhwc": dict(dy_layout=B.DY_NPQK, dw_layout=B.DW_KCRS), "rsck": dict(x_layout=B.X_NCHW, dy_layout=B.DY_NPQK, dw_layout=B.DW_RSCK)}
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
+@pytest.mark.parametrize("li", range(len(SHAPES)), ids=[l.name for l in SHAPES])
+def test_every_layout_matches_the_oracle(li, dtype):
+    layer = SHAPES[li]
+    x, dy = I.make_layer_inputs(layer, dtype, 11, li)
+    ref, dn = oracle.dw_exact(to_f64(x), to_f64(dy), oshape(layer), 0.5)
+    first = None
+    for name, kw in LAYOUTS.items():
+        g = GpuLayer(layer, dtype, x, dy, alpha=0.5, **kw)
+        before = B.gaconv_launch_count()
+        got = g.exact()
+        assert B.gaconv_launch_count() - before <= 3, name
+        assert norm_err(got, ref, dn) <= TOL_F32 / 2, name        # bf16 products are exact in fp32 as well
+        np.testing.assert_array_equal(got, g.exact())
+        first = got if first is None else first
+        np.testing.assert_array_equal(got, first)                # the same operands, however they were handed over
+        assert B.gaconv_poll_async_status(g.desc) == B.OK
+    few = GpuLayer(layer, dtype, x, dy, alpha=0.5, sm_budget=11)
+    assert norm_err(few.exact(), ref, dn) <= TOL_F32 / 2
+
+
+def test_long_sums_keep_fp32_accuracy():
+    """Tens of thousands of products per output and an activation with a mean: the tensor core's own additions truncate,
+    so without the periodic hand-over to fp32 registers the error would grow with the sum."""
+    layer = ConvLayer("long", 40, 16, 45, 47, 16, 3, 3, 1, 1, dy_std=1.0)
+    for dtype in (torch.float32, torch.bfloat16):
+        x, dy = I.make_layer_inputs(layer, dtype, 11, 50)
+        dy = (dy.float() + 0.5).to(dtype)
+        ref, dn = oracle.dw_exact(to_f64(x), to_f64(dy), oshape(layer))
+        g = GpuLayer(layer, dtype, x, dy, sm_budget=2)
+        assert norm_err(g.exact(), ref, dn) <= 2e-6
+
+
+def test_static_scratch_takes_the_kernels_that_fit():
+    """Scratch beyond the built-in array: gaconv_dw_exact_static falls back to the kernels that need less of it."""
+    layer = ConvLayer("packed copies of 12 MB", 40, 64, 30, 30, 64, 3, 3, 1, 1)
+    x, dy = I.make_layer_inputs(layer, torch.float32, 11, 51)
+    g = GpuLayer(layer, torch.float32, x, dy)
+    want = g.exact()
+    bare = B.make_desc(layer, torch.float32)
+    assert B.gaconv_workspace_size(bare, B.METHOD_EXACT) > B.gaconv_static_scratch_bytes()
+    g.dw.fill_(float("nan"))
+    B.gaconv_dw_exact_static(g.x, g.dy, g.dw, bare)
+    got = g.logical_dw()
+    assert np.max(np.abs(got - want)) <= 1e-4 * np.abs(want).max() and B.gaconv_poll_async_status_static() == B.OK
