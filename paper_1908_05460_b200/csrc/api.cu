@@ -342,6 +342,7 @@ struct gaconv_schedule {
     double fraction;
     uint64_t seed;
     bool* mask;   // SEEDED_FRACTION: layers in the approximated subset
+    struct StepCache* steps = nullptr;      // repeated steps as CUDA graphs, created on first use
 };
 
 gaconv_status_t gaconv::exact_workspace(const gaconv_conv_desc_t* desc, bool cl, size_t* bytes)
@@ -712,14 +713,19 @@ int32_t gaconv_schedule_method(const gaconv_schedule_t* s, int32_t layer, int64_
     return approx ? s->method : GACONV_METHOD_EXACT;
 }
 
+// seed of a random-gradient layer at a step
+static uint64_t layer_seed(const gaconv_schedule_t* s, int64_t step, int32_t layer)
+{
+    return splitmix64(s->seed ^ splitmix64((uint64_t)step * 0x100000001B3ull + (uint64_t)layer));
+}
+
 gaconv_status_t gaconv_schedule_run_layer(const gaconv_schedule_t* s, int32_t layer, int64_t step, const void* x,
                                           const void* dy, float* dw, const gaconv_conv_desc_t* desc, void* stream)
 {
     const int32_t m = gaconv_schedule_method(s, layer, step);
     if (m == -2) return GACONV_ERR_BAD_DESC;
     if (m == GACONV_METHOD_EXACT) return gaconv_dw_exact(x, dy, dw, desc, stream);
-    const uint64_t seed = splitmix64(s->seed ^ splitmix64((uint64_t)step * 0x100000001B3ull + (uint64_t)layer));
-    return gaconv_dw_approx(m, x, dy, dw, desc, seed, stream);
+    return gaconv_dw_approx(m, x, dy, dw, desc, layer_seed(s, step, layer), stream);
 }
 
 // ---- lanes: side streams on which the layers of a step run next to one another ----------------------
@@ -728,7 +734,9 @@ namespace {
 constexpr int kMaxLanes = 16, kMaxLaneDevices = 64;
 struct LanePool {
     bool ready = false;
+    int device = -1;
     cudaStream_t side[kMaxLanes - 1] = {};
+    cudaStream_t record = nullptr;                  // lane 0 of a step that is being recorded as a graph
     cudaEvent_t fork = nullptr, join[kMaxLanes - 1] = {};
 };
 std::mutex g_lane_mutex;
@@ -741,7 +749,9 @@ LanePool* lane_pool()
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxLaneDevices) return nullptr;
     LanePool& p = g_lanes[dev];
     if (!p.ready) {
-        if (cudaEventCreateWithFlags(&p.fork, cudaEventDisableTiming) != cudaSuccess) return nullptr;
+        p.device = dev;
+        if (cudaEventCreateWithFlags(&p.fork, cudaEventDisableTiming) != cudaSuccess ||
+            cudaStreamCreateWithFlags(&p.record, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
         for (int i = 0; i < kMaxLanes - 1; ++i)
             if (cudaStreamCreateWithFlags(&p.side[i], cudaStreamNonBlocking) != cudaSuccess ||
                 cudaEventCreateWithFlags(&p.join[i], cudaEventDisableTiming) != cudaSuccess) return nullptr;
@@ -751,6 +761,95 @@ LanePool* lane_pool()
 }
 
 }  // namespace
+
+// ---- repeated steps ------------------------------------------------------------------------------------------------
+// A step of a ResNet-20 is some fifty launches and event operations, 120-190 us of host time where the kernels take 40-80 us
+// at small batches.  A training program calls run_step with the same buffers, descriptors and methods over and over, so the
+// second time a schedule sees a step it is recorded as a CUDA graph, and from then on one graph launch enqueues it.  What the
+// graph does not fix are the seeds of random-gradient layers, which change every step: their nodes get new ones before each
+// launch.  A schedule keeps the kMaxSteps most recently used graphs; they go with it.
+constexpr int kMinGraphLayers = 6;
+struct StepKey {
+    std::vector<unsigned char> bytes;
+    void put(const void* p, size_t n) { const unsigned char* b = static_cast<const unsigned char*>(p); bytes.insert(bytes.end(), b, b + n); }
+};
+struct RandomNode { cudaGraphNode_t node; int32_t layer; int key_arg; };
+struct StepGraph {
+    std::vector<unsigned char> key;
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;        // nullptr: seen once
+    bool refused = false;                  // could not be recorded
+    int launches = 0;
+    int64_t step = -1;                     // whose seeds the graph holds
+    std::vector<RandomNode> random;
+    uint64_t used = 0;
+};
+struct StepCache {
+    static constexpr size_t kMaxSteps = 8;
+    std::vector<StepGraph> e;
+    uint64_t clock = 0;
+    static void drop(StepGraph& g)
+    {
+        if (g.exec != nullptr) cudaGraphExecDestroy(g.exec);      // (a graph still running is freed when it completes)
+        if (g.graph != nullptr) cudaGraphDestroy(g.graph);
+    }
+    ~StepCache() { for (StepGraph& g : e) drop(g); }
+};
+
+// enqueues the layers of a step on the lanes; with `random`, notes the graph nodes of random-gradient layers (while capturing)
+static gaconv_status_t enqueue_step(const gaconv_schedule_t* s, int64_t step, int32_t num_layers, const void* const* x, const void* const* dy,
+                                    float* const* dw, const gaconv_conv_desc_t* const* descs, int32_t lanes, cudaStream_t main_stream,
+                                    LanePool* pool, std::vector<RandomNode>* random)
+{
+    const int used = lanes < num_layers ? lanes : num_layers;
+    // fork: the side streams start after everything already enqueued on the caller's stream
+    if (used > 1) {
+        if (cudaEventRecord(pool->fork, main_stream) != cudaSuccess) return GACONV_ERR_CUDA;
+        for (int i = 0; i < used - 1; ++i)
+            if (cudaStreamWaitEvent(pool->side[i], pool->fork, 0) != cudaSuccess) return GACONV_ERR_CUDA;
+    }
+    gaconv_status_t result = GACONV_OK;
+    for (int l = 0; l < num_layers && result == GACONV_OK; ++l) {
+        const int lane = l % used;
+        cudaStream_t st = lane == 0 ? main_stream : pool->side[lane - 1];
+        result = gaconv_schedule_run_layer(s, l, step, x[l], dy[l], dw[l], descs[l], st);
+        if (result == GACONV_OK && random != nullptr && gaconv_schedule_method(s, l, step) == GACONV_METHOD_RANDOM) {
+            cudaStreamCaptureStatus status;
+            const cudaGraphNode_t* deps = nullptr;
+            const cudaGraphEdgeData* edges = nullptr;
+            cudaGraph_t graph;
+            size_t n = 0;
+            Geom g;
+            if (cudaStreamGetCaptureInfo_v3(st, &status, nullptr, &graph, &deps, &edges, &n) != cudaSuccess || n != 1 || make_geom(descs[l], &g) != GACONV_OK)
+                result = GACONV_ERR_CUDA;
+            else
+                random->push_back(RandomNode{deps[0], l, random_key_arg(g)});
+        }
+    }
+    // join (also after an error, so that the side streams never stay forked from a capturing stream)
+    for (int i = 0; i < used - 1; ++i)
+        if (cudaEventRecord(pool->join[i], pool->side[i]) != cudaSuccess || cudaStreamWaitEvent(main_stream, pool->join[i], 0) != cudaSuccess)
+            return GACONV_ERR_CUDA;
+    return result;
+}
+
+// gives the random-gradient layers of a recorded step the seeds of `step`
+static bool set_seeds(const gaconv_schedule_t* s, StepGraph& g, int64_t step)
+{
+    for (const RandomNode& r : g.random) {
+        cudaKernelNodeParams p;
+        if (cudaGraphKernelNodeGetParams(r.node, &p) != cudaSuccess) return false;
+        const uint64_t seed = layer_seed(s, step, r.layer);
+        uint32_t key0 = (uint32_t)seed, key1 = (uint32_t)(seed >> 32);
+        void* args[8];
+        for (int i = 0; i < r.key_arg + 3; ++i) args[i] = p.kernelParams[i];      // (the keys are followed by one more argument)
+        args[r.key_arg] = &key0; args[r.key_arg + 1] = &key1;
+        p.kernelParams = args;
+        if (cudaGraphExecKernelNodeSetParams(g.exec, r.node, &p) != cudaSuccess) return false;
+    }
+    g.step = step;
+    return true;
+}
 
 gaconv_status_t gaconv_schedule_run_step(const gaconv_schedule_t* s, int64_t step, int32_t num_layers, const void* const* x,
                                          const void* const* dy, float* const* dw, const gaconv_conv_desc_t* const* descs,
@@ -766,36 +865,83 @@ gaconv_status_t gaconv_schedule_run_step(const gaconv_schedule_t* s, int64_t ste
                 if (descs[o]->workspace == descs[l]->workspace) return GACONV_ERR_BAD_DESC;
     }
     cudaStream_t main_stream = static_cast<cudaStream_t>(stream);
-    if (lanes == 1 || num_layers == 1) {
-        for (int l = 0; l < num_layers; ++l) {
-            const gaconv_status_t st = gaconv_schedule_run_layer(s, l, step, x[l], dy[l], dw[l], descs[l], stream);
-            if (st != GACONV_OK) return st;
-        }
-        return GACONV_OK;
-    }
     std::lock_guard<std::mutex> lock(g_lane_mutex);          // one set of lanes per device: enqueueing is serialised
     LanePool* pool = lane_pool();
     if (pool == nullptr) return GACONV_ERR_CUDA;
-    const int used = lanes < num_layers ? lanes : num_layers;
-    // fork: the side streams start after everything already enqueued on the caller's stream
-    if (cudaEventRecord(pool->fork, main_stream) != cudaSuccess) return GACONV_ERR_CUDA;
-    for (int i = 0; i < used - 1; ++i)
-        if (cudaStreamWaitEvent(pool->side[i], pool->fork, 0) != cudaSuccess) return GACONV_ERR_CUDA;
-    gaconv_status_t result = GACONV_OK;
-    for (int l = 0; l < num_layers && result == GACONV_OK; ++l) {
-        const int lane = l % used;
-        result = gaconv_schedule_run_layer(s, l, step, x[l], dy[l], dw[l], descs[l], lane == 0 ? stream : static_cast<void*>(pool->side[lane - 1]));
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    // Few layers: their launches cost the host less (~6 us a layer) than a graph's start and end cost the GPU between two steps
+    // (two layers of the two-layer CNN at N = 256: 49 us launched, 65 us as a graph).  A capture in progress records the
+    // launches themselves.
+    if (num_layers < kMinGraphLayers || cudaStreamIsCapturing(main_stream, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone)
+        return enqueue_step(s, step, num_layers, x, dy, dw, descs, lanes, main_stream, pool, nullptr);
+
+    // everything the recorded launches depend on
+    StepKey key;
+    key.bytes.reserve((size_t)num_layers * (sizeof(gaconv_conv_desc_t) + 3 * sizeof(void*) + 4) + 64);
+    const int32_t head[3] = {pool->device, lanes, num_layers};
+    key.put(head, sizeof(head));
+    for (int l = 0; l < num_layers; ++l) {
+        const int32_t method = gaconv_schedule_method(s, l, step);
+        const void* ptrs[3] = {x[l], dy[l], dw[l]};
+        key.put(&method, sizeof(method)); key.put(ptrs, sizeof(ptrs)); key.put(descs[l], sizeof(*descs[l]));
     }
-    // join (also after an error, so that the side streams never stay forked from a capturing stream)
-    for (int i = 0; i < used - 1; ++i)
-        if (cudaEventRecord(pool->join[i], pool->side[i]) != cudaSuccess || cudaStreamWaitEvent(main_stream, pool->join[i], 0) != cudaSuccess)
-            return GACONV_ERR_CUDA;
-    return result;
+    if (s->steps == nullptr) const_cast<gaconv_schedule*>(s)->steps = new (std::nothrow) StepCache;
+    StepCache* cache = s->steps;
+    StepGraph* g = nullptr;
+    if (cache != nullptr) {
+        for (StepGraph& c : cache->e)
+            if (c.key == key.bytes) { g = &c; break; }
+        if (g != nullptr) g->used = ++cache->clock;
+    }
+    if (g == nullptr || g->refused) {
+        const gaconv_status_t st = enqueue_step(s, step, num_layers, x, dy, dw, descs, lanes, main_stream, pool, nullptr);
+        if (st == GACONV_OK && g == nullptr && cache != nullptr) {      // a step that may come again
+            if (cache->e.size() >= StepCache::kMaxSteps) {
+                size_t oldest = 0;
+                for (size_t i = 1; i < cache->e.size(); ++i)
+                    if (cache->e[i].used < cache->e[oldest].used) oldest = i;
+                StepCache::drop(cache->e[oldest]);
+                cache->e.erase(cache->e.begin() + oldest);
+            }
+            cache->e.emplace_back();
+            cache->e.back().key = std::move(key.bytes);
+            cache->e.back().used = ++cache->clock;
+        }
+        return st;
+    }
+    if (g->exec == nullptr) {
+        const uint64_t before = gaconv_launch_count();
+        gaconv_status_t st = GACONV_ERR_CUDA;
+        g->random.clear();
+        if (cudaStreamBeginCapture(pool->record, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+            st = enqueue_step(s, step, num_layers, x, dy, dw, descs, lanes, pool->record, pool, &g->random);
+            if (cudaStreamEndCapture(pool->record, &g->graph) != cudaSuccess) st = GACONV_ERR_CUDA;
+        }
+        if (st == GACONV_OK && cudaGraphInstantiate(&g->exec, g->graph, 0) != cudaSuccess) { g->exec = nullptr; st = GACONV_ERR_CUDA; }
+        g->launches = (int)(gaconv_launch_count() - before);
+        note_launch(-g->launches);              // recorded, not launched
+        g->step = step;
+        if (st != GACONV_OK) {
+            (void)cudaGetLastError();
+            StepCache::drop(*g);
+            g->graph = nullptr; g->exec = nullptr; g->refused = true;
+            return enqueue_step(s, step, num_layers, x, dy, dw, descs, lanes, main_stream, pool, nullptr);
+        }
+    }
+    if (g->step != step && !set_seeds(s, *g, step)) {
+        (void)cudaGetLastError();
+        g->refused = true;
+        return enqueue_step(s, step, num_layers, x, dy, dw, descs, lanes, main_stream, pool, nullptr);
+    }
+    if (cudaGraphLaunch(g->exec, main_stream) != cudaSuccess) return GACONV_ERR_CUDA;
+    note_launch(g->launches);
+    return GACONV_OK;
 }
 
 void gaconv_schedule_destroy(gaconv_schedule_t* s)
 {
     if (s == nullptr) return;
+    delete s->steps;
     delete[] s->mask;
     delete s;
 }

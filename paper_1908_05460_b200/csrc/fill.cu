@@ -133,10 +133,17 @@ cudaError_t launch_zero(float* dw, size_t count, cudaStream_t stream)
     return launch_kernel(zero_kernel, dim3((unsigned)blocks), dim3(256), 0, stream, dim3(1, 1, 1), dw, count);
 }
 
+static bool stored_in_logical_order(const Geom& g)
+{
+    return g.ws_s == 1 && g.ws_r == g.s && g.ws_c == (long long)g.r * g.s && g.ws_k == (long long)g.c * g.r * g.s;
+}
+
+int random_key_arg(const Geom& g) { return stored_in_logical_order(g) ? 2 : 3; }
+
 cudaError_t launch_random(float* dw, const Geom& g, uint64_t seed, float std, cudaStream_t stream)
 {
     const size_t count = (size_t)g.k * g.c * g.r * g.s;
-    const bool contiguous = (g.ws_s == 1 && g.ws_r == g.s && g.ws_c == (long long)g.r * g.s && g.ws_k == (long long)g.c * g.r * g.s);
+    const bool contiguous = stored_in_logical_order(g);
     const uint32_t key0 = (uint32_t)seed, key1 = (uint32_t)(seed >> 32);
     note_launch();
     if (contiguous) {

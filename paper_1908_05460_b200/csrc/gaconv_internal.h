@@ -98,6 +98,7 @@ cudaError_t launch_top1_fused(const void* x, const void* dy, float* dw, const Ge
 // ---- zero / random gradient ----
 cudaError_t launch_zero(float* dw, size_t count, cudaStream_t stream);
 cudaError_t launch_random(float* dw, const Geom& g, uint64_t seed, float std, cudaStream_t stream);
+int random_key_arg(const Geom& g);     // position of the first of the two key words among the kernel's arguments
 
 // ---- exact filter gradient, direct FP32 kernel (any shape, any layout) ----
 struct DirectPlan {
