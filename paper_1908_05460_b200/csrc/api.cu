@@ -172,8 +172,33 @@ ExactLayout exact_layout(const Geom& g, int math, int algo)
     return cache.get(plan_key(g, math, algo), [&] { return build_exact_layout(g, math, algo); });
 }
 
-// The channels-last kernel takes what the kernels above do not tile; ALGO_DIRECT, ALGO_TENSOR and the one-pass TF32
-// mode stay with them.
+// Which problems the channels-last kernel takes: those the kernels above do not tile, and of the others those on which it
+// measured faster (in microseconds, the older kernel first; N = 128 unless said).  `reordered`: X or dY comes in the other
+// order than N x H x W x C / N x K x P x Q, which costs the older kernels a transposing pass and this one none or a cheaper one.
+// ALGO_DIRECT, ALGO_TENSOR and the one-pass TF32 mode stay with the older kernels.
+bool prefer_cl(const Geom& g, const ExactLayout& L, bool reordered)
+{
+    const double products = (double)g.n * g.p * g.q * g.k * g.c * g.r * g.s;
+    const bool shared = g.sm_budget > 0;            // other layers run beside this one
+    // (below 30 million products the order of the operands does not change the kernel, nor the result's last bits)
+    reordered = reordered && products > 3e7;
+    if (g.bf16) {
+        if (L.tc_ok) {
+            if (L.tp.reads_transposed_dy || products < 3e7) return false;       // maps under 64 pixels: 512->512 on 2x2 11.5 / 18.2
+            if (reordered) return true;                             // 128->128 on 16x16, dY channels last 28.4 / 17.8
+            if (g.c <= 16 || (g.c < 64 && shared)) return false;    // 16->16 on 32x32 11.9 / 12.5; on 18 SMs 28 / 38
+            return g.r < 5;                                         // 5x5 64->64 on 16x16 16.1 / 17.8, 3x3 64->64 on 32x32 24.1 / 22.5
+        }
+        if (L.stem_ok) return reordered || (!shared && g.r * g.s * g.c > 32);       // 5x5 3->64 26.4 / 22.6, 3x3 3->16 10.4 / 14.8
+    } else {
+        if (L.stem_ok) return false;                                // 3->64 on 32x32 28 / 53
+        if (L.tc_ok)                                                // 128->128 on 16x16 92 / 53, 64->64 on 8x8 17.1 / 18.1, on 18 SMs 44 / 40
+            return reordered || (g.c >= 128 ? products > 4e8 : g.c >= 64 && (shared || products > 3e9));
+        if (direct_mma_supported(g, L.dp))                          // 16->16 on 32x32 19 / 40, 48->96 on 16x16 (N = 64) 31 / 23
+            return g.c >= 64 || (g.c >= 24 && g.stride_h == 1 && !shared);
+    }
+    return products > 4e6;          // FP32 pipes: below this their one or two launches are as quick (8-9)
+}
 struct ClRoute { bool use; ClPlan plan; size_t partial_off, x_off, dy_off, total; };
 ClRoute build_cl_route(const gaconv_conv_desc_t* desc, const Geom& g)
 {
@@ -184,9 +209,7 @@ ClRoute build_cl_route(const gaconv_conv_desc_t* desc, const Geom& g)
     Geom gn;
     if (make_geom(&native, &gn) != GACONV_OK) return R;
     const ExactLayout L = exact_layout(gn, GACONV_MATH_DEFAULT, GACONV_ALGO_AUTO);
-    // Below ~4 million products the FP32-pipe kernel's one or two launches are as quick (8-9 us, 4x32x9x9 -> 48, 1x1)
-    const double products = (double)g.n * g.p * g.q * g.k * g.c * g.r * g.s;
-    R.use = !(L.tc_ok || L.stem_ok || direct_mma_supported(gn, L.dp)) && products > 4e6;
+    R.use = prefer_cl(gn, L, (desc->x_layout == GACONV_X_NCHW && g.c > 1) || (desc->dy_layout == GACONV_DY_NPQK && g.k > 1));
 #ifdef GACONV_TUNING
     if (const char* e = getenv("GACONV_CL")) R.use = atoi(e) != 0;
 #endif

@@ -16,7 +16,10 @@
 //           Q reading as zeros.  Works for every Q; wastes (Wp - Q) / Q of the k-steps.
 //   paired  Q a multiple of 8: a k-step is 8 columns of two neighbouring rows (the stride between the two 8-pixel
 //           groups of a descriptor is one row), so that the halo columns are never multiplied.
-// A table of the plan holds the offsets of the k-steps of either order.
+// pixels  dY as it lies, N x K x P x Q (K-major rows of 64 pixels, Q a multiple of 8): a k-step is 16 consecutive pixels of an
+//           image, no halo columns and no packing of dY.  Its two groups of 8 X pixels lie 8 pixels apart, or a row's end further,
+//           so the X descriptor's stride belongs to the k-step.
+// A table of the plan holds the offsets of the k-steps of every order.
 //
 // Which operand is the MMA's M side:
 //   k-side  M = 128 output channels, N = consecutive column shifts x channels (up to 256).
@@ -60,6 +63,9 @@ namespace {
 
 constexpr int kMaxGroups = 16, kMaxKsteps = 128, kMaxStages = 8;
 
+// order of the reduction inside a chunk, see above
+enum { kFlat = 0, kPaired = 1, kPixels = 2 };
+
 struct ClGroup {            // one MMA of a k-step
     int x_off;              // offset of its X rows inside the X region of a stage, 16-byte units
     int r, s0, cnt, cbase;  // filter row, first column shift, atoms in use, first channel (relative to the c-tile)
@@ -78,14 +84,15 @@ struct ClParams {
     int dy_box, dy_alloc, x_box, x_alloc;       // bytes one copy writes, and the distance to the next tile
     int x_region, x_plane, dy_plane, stage_bytes, stages;
     uint32_t tx_bytes;
-    int paired, ksteps, x_pitch, dy_pitch, x_img, dy_img;
+    int order, ksteps, x_pitch, dy_pitch, x_img, dy_img;
+    int dy_subs;                    // kPixels: 64-pixel boxes of dY per image of a chunk
     int c_side;                     // 1: X is the M side
     int merged;                     // 1: the MN atoms of an X operand are channel atoms, 0: column shifts
     int ngroups, nmma, cols, tmem_cols;
     int epoch;                      // chunks of one issuer between two readings of its accumulators
-    uint32_t x_hi, dy_hi, x_lbo, dy_lbo, idesc;
+    uint32_t dy_hi, x_lbo, dy_lbo, idesc;
     ClGroup g[kMaxGroups];
-    uint2 k_off[kMaxKsteps];        // k-step -> offset of its X and dY rows, 16-byte units
+    uint4 k_off[kMaxKsteps];        // k-step -> offsets of its X and dY rows (16-byte units), upper word of its X descriptor
 };
 
 // fp32 operands: which planes of X and dY each of the six products of a k-step takes
@@ -169,6 +176,8 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
         const bool mine = lane < P.planes * per_plane, is_dy = i < P.katoms;
         const CUtensorMap* map = is_dy ? &map_dy : &map_x;
         const uint32_t dst = is_dy ? pl * P.dy_plane + i * P.dy_alloc : P.x_region + pl * P.x_plane + j * P.x_alloc;
+        const bool pixels = is_dy && P.order == kPixels;          // box i: 64 pixels of image i / dy_subs, K-major
+        const int dy_img = pixels ? i / P.dy_subs : 0, dy_px = 64 * (i - dy_img * P.dy_subs);
         const int ch = is_dy ? k0 + P.ka * i : c0 + P.ca * (j - jt * P.na), col = is_dy ? 0 : jt - rl * P.phases - P.pad_w;
         const int row_mul = is_dy ? 1 : P.stride, row_add = is_dy ? 0 : r0 + rl - P.pad_h;
         int st = first, ph = 0, it = first;
@@ -179,7 +188,8 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
             if (__any_sync(0xffffffffu, s_abort)) break;
             if (lane == 0) mbar_expect_tx(full, P.tx_bytes);
             __syncwarp();
-            if (mine) tma_load_5d(smem_base + st * P.stage_bytes + dst, map, full, ch, col, p0 * row_mul + row_add, n0, pl);
+            if (pixels) { if (mine) tma_load_3d(smem_base + st * P.stage_bytes + dst, map, full, p0 * P.q + dy_px, k0, n0 + dy_img); }
+            else if (mine) tma_load_5d(smem_base + st * P.stage_bytes + dst, map, full, ch, col, p0 * row_mul + row_add, n0, pl);
             if (whole) n0 += np * P.ci;
             else for (p0 += np * P.bp; p0 >= P.cpi * P.bp; p0 -= P.cpi * P.bp) ++n0;
             for (st += np; st >= P.stages; st -= P.stages) ph ^= 1;
@@ -196,7 +206,7 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
         // k-steps in the parameter bank, and the one MMA that starts an accumulator issued apart.
         constexpr int PER = NG * (F32 ? 6 : 1), U = PER >= 8 ? 1 : PER == 1 ? 12 : PER == 2 ? 6 : PER == 3 ? 4 : 2;
         const uint32_t x_plane = (uint32_t)P.x_plane >> 4, dy_plane = (uint32_t)P.dy_plane >> 4;
-        const uint64_t x_hi = (uint64_t)P.x_hi << 32, dy_hi = (uint64_t)P.dy_hi << 32;
+        const uint64_t dy_hi = (uint64_t)P.dy_hi << 32;
         const int ksteps = P.ksteps, ngroups = P.ngroups;
         const uint32_t nmma = P.nmma, idesc = P.idesc;
         uint32_t off[NG];
@@ -222,7 +232,8 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
                 const uint32_t sa = smem_base + st * P.stage_bytes;
                 const uint32_t dy_lo = P.dy_lbo | ((sa >> 4) & 0x3fffu), x_lo = P.x_lbo | (((sa + P.x_region) >> 4) & 0x3fffu);
                 auto step = [&](int k, bool starts) {
-                    const uint2 o = P.k_off[k];
+                    const uint4 o = P.k_off[k];
+                    const uint64_t x_hi = (uint64_t)o.z << 32;
 #pragma unroll
                     for (int pr = 0; pr < (F32 ? 6 : 1); ++pr) {
                         const uint64_t dyd = dy_hi | (dy_lo + o.y + (F32 ? prod_dy(pr) * dy_plane : 0u));
@@ -376,55 +387,68 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
     }
 }
 
-// Sum of the splits of every (tile, column), in split order: grid (column groups, tiles).  A warp adds one column's 128
-// lanes (a float4 each) over every W-th split; the W partial sums of a column meet in shared memory.  A block finishes
-// CB columns, so that where consecutive columns are consecutive channels of dW it writes CB of them in one piece.
-template <int CB>
-__global__ void __launch_bounds__(256)
-cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, const __grid_constant__ ClParams P)
+// Sum of the splits of every (tile, column), in a fixed order: grid (column blocks, tiles), 32 * CB * G threads.  Warp (g, c)
+// adds the 128 lanes (a float4 each) of column c over the splits g, g + G, ...; the G partial sums meet in shared memory.  G is
+// chosen so that a warp's loads are all in flight at once (eight, then a second round), CB so that the grid covers the GPU;
+// where consecutive columns are consecutive channels of dW a block writes CB of them in one piece.  Latency-bound: what an
+// element is, and where it goes, is worked out before the wait for the sums.
+__global__ void __launch_bounds__(1024)
+cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, const __grid_constant__ ClParams P, int log_cb, int G)
 {
-    constexpr int W = 8 / CB;
-    __shared__ float s_sum[8][128];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tile = blockIdx.y, col0 = blockIdx.x * CB;
-    const int r0 = (tile % P.tiles_r) * P.rc, kc = tile / P.tiles_r;
-    const int k0 = (kc / P.tiles_c) * P.kt, c0 = (kc % P.tiles_c) * P.ct;
+    __shared__ float s_sum[32][128];
+    __shared__ int2 s_col[16];               // column -> {offset in dW, atoms in use (0: not an element)}
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, CB = 1 << log_cb;
+    const int tile = blockIdx.y, col0 = blockIdx.x << log_cb;
     pdl_release_next_grid();
-    pdl_wait_prior_grid();
-    {
-        const int cb = warp % CB, sw = warp / CB, col = col0 + cb, g = col / P.nmma, j = col - g * P.nmma;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        bool live = col < P.cols && r0 + P.g[g].r < P.r;
-        if (live) {
-            if (P.c_side) live = k0 + j < P.k;
-            else live = c0 + P.g[g].cbase + (P.merged ? j : j % P.ca) < P.c;
+    const int tr = tile / P.tiles_r, r0 = (tile - tr * P.tiles_r) * P.rc, tk = tr / P.tiles_c;
+    const int k0 = tk * P.kt, c0 = (tr - tk * P.tiles_c) * P.ct;
+    const int ca_shift = 31 - __clz(P.ca), mn_mask = P.merged ? 127 : P.ca - 1;
+    if ((int)threadIdx.x < CB) {
+        const int col = col0 + threadIdx.x;
+        int2 o = make_int2(0, 0);
+        if (col < P.cols) {
+            const int gi = col / P.nmma, j = col - gi * P.nmma;
+            const ClGroup& g = P.g[gi];
+            const int a = P.c_side || P.merged ? 0 : j >> ca_shift, k = P.c_side ? k0 + j : 0;
+            const int c = c0 + g.cbase + (P.c_side ? 0 : P.merged ? j : j & mn_mask);
+            const bool valid = r0 + g.r < P.r && (P.c_side ? k < P.k : c < P.c && a < g.cnt);
+            o = make_int2((int)(k * P.ws_k + c * P.ws_c + (r0 + g.r) * P.ws_r + (g.s0 + P.stride * a) * P.ws_s), valid ? g.cnt : 0);
         }
-        if (live) {
-            const float4* src = reinterpret_cast<const float4*>(partial + ((size_t)tile * P.splits * P.cols + col) * 128) + lane;
-            const size_t step = (size_t)P.cols * 32;
-            for (int s = sw; s < P.splits; s += 8 * W) {
-                float4 u[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) u[i] = s + i * W < P.splits ? __ldcg(src + (size_t)(s + i * W) * step) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) { acc.x += u[i].x; acc.y += u[i].y; acc.z += u[i].z; acc.w += u[i].w; }
-            }
-        }
-        *reinterpret_cast<float4*>(&s_sum[sw * CB + cb][4 * lane]) = acc;
+        s_col[threadIdx.x] = o;
     }
+    const int cb = warp & (CB - 1), grp = warp >> log_cb;
+    const float4* src = reinterpret_cast<const float4*>(partial + ((size_t)tile * P.splits * P.cols + col0 + cb) * 128) + lane;
+    const size_t step = (size_t)P.cols * 32;
     __syncthreads();
-    for (int e = threadIdx.x; e < 128 * CB; e += 256) {
-        const int cb = P.c_side ? e / 128 : e % CB, l = P.c_side ? e % 128 : e / CB, col = col0 + cb;
-        if (col >= P.cols) continue;
-        float t = s_sum[cb][l];
+    const bool live = s_col[cb].y > 0;
+    pdl_wait_prior_grid();
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (live)
+        for (int s = grp; s < P.splits; s += 8 * G) {
+            float4 u[8];
 #pragma unroll
-        for (int w = 1; w < W; ++w) t += s_sum[w * CB + cb][l];
-        const int gi = col / P.nmma, j = col - gi * P.nmma, mn = P.c_side ? l : j, a = mn / P.ca;
-        const ClGroup& g = P.g[gi];
-        const int k = k0 + (P.c_side ? j : l), c = c0 + g.cbase + (P.merged ? mn : mn - a * P.ca);
-        const int r = r0 + g.r, s = P.merged ? g.s0 : g.s0 + P.stride * a;
-        if (k < P.k && c < P.c && r < P.r && (P.merged || a < g.cnt))
-            dw[k * P.ws_k + c * P.ws_c + r * P.ws_r + s * P.ws_s] = P.alpha * t;
+            for (int i = 0; i < 8; ++i) u[i] = s + i * G < P.splits ? __ldcg(src + (size_t)(s + i * G) * step) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) { acc.x += u[i].x; acc.y += u[i].y; acc.z += u[i].z; acc.w += u[i].w; }
+        }
+    *reinterpret_cast<float4*>(&s_sum[warp][4 * lane]) = acc;
+    __syncthreads();
+    for (int e = threadIdx.x; e < CB << 7; e += blockDim.x) {
+        const int c = P.c_side ? e >> 7 : e & (CB - 1), l = P.c_side ? e & 127 : e >> log_cb;
+        const int2 o = s_col[c];
+        bool valid; long long off = o.x;
+        if (P.c_side) {
+            const int a = P.merged ? 0 : l >> ca_shift, ch = l & mn_mask;
+            valid = a < o.y && c0 + ch < P.c;
+            off += ch * P.ws_c + P.stride * a * P.ws_s;
+        } else {
+            valid = o.y > 0 && k0 + l < P.k;
+            off += (k0 + l) * P.ws_k;
+        }
+        if (!valid) continue;
+        float t = s_sum[c][l];
+        for (int w = 1; w < G; ++w) t += s_sum[(w << log_cb) + c][l];
+        dw[off] = P.alpha * t;
     }
 }
 
@@ -616,7 +640,7 @@ Cost cost_of(const ClParams& P, int sms, double block_share)
 {
     const double mma = (double)P.ksteps * P.ngroups * P.nprod * P.nmma / 2.0;
     const double shared = (double)P.ksteps * P.ngroups * P.nprod * ((128 + P.nmma) / 4.0 + 2) + P.tx_bytes / 128.0;
-    const double rows = (double)P.planes * (P.katoms * (P.dy_box / (P.ka * 2)) + P.na * P.phases * P.row_tiles * (P.x_box / (P.ca * 2)));
+    const double rows = (double)P.planes * (P.katoms * (P.dy_box / (P.order == kPixels ? 128 : P.ka * 2)) + P.na * P.phases * P.row_tiles * (P.x_box / (P.ca * 2)));
     const double load = std::max(P.tx_bytes / 80.0, rows * 1.4);
     const double chunk = std::max({mma * 1.03, shared, load, 470.0}) * (P.stages > 2 ? 1.0 : 1.2) + 40;
     const int tiles = P.tiles_k * P.tiles_c * P.tiles_r;
@@ -671,52 +695,68 @@ bool build_groups(ClParams& P)
 }
 
 // Fills the chunk-dependent fields; false when the candidate does not fit.
-bool shape_chunk(ClParams& P, int ci, int bp, bool paired)
+bool shape_chunk(ClParams& P, int ci, int bp, int order)
 {
     const int st = P.stride;
     const bool whole = ci > 1 || bp >= P.p;
-    if (paired) bp = round_up(bp, 2);
-    P.ci = ci; P.bp = bp; P.paired = paired ? 1 : 0;
+    if (order == kPaired) bp = round_up(bp, 2);
+    if (order == kPixels && !whole && bp * P.q % 16 != 0) return false;         // k-steps do not cross chunks
+    P.ci = ci; P.bp = bp; P.order = order;
     P.cpi = whole ? 0 : ceil_div(P.p, bp);
     P.chunks = whole ? ceil_div(P.n, ci) : P.n * P.cpi;
     const int wp = P.q + ceil_div(P.s, st) - 1, halo = st == 1 ? P.rc - 1 : 0;
-    const int x_rows = bp + halo, dy_rows = (!paired && ci > 1) ? bp + halo : bp, dy_w = paired ? P.q : wp;
+    const int x_rows = bp + halo, dy_rows = (order == kFlat && ci > 1) ? bp + halo : bp, dy_w = order == kFlat ? wp : P.q;
     if ((wp - 1) * st + 1 > 256 || (x_rows - 1) * st + 1 > 256 || dy_rows > 256 || ci > 256) return false;
     P.x_pitch = wp; P.dy_pitch = dy_w; P.x_img = x_rows * wp; P.dy_img = dy_rows * dy_w;
-    P.ksteps = paired ? ci * (bp / 2) * (P.q / 8) : ceil_div(ci * dy_rows * dy_w, 16);
+    const int steps_img = order == kPaired ? (bp / 2) * (P.q / 8) : ceil_div(bp * P.q, 16);
+    P.ksteps = order == kFlat ? ceil_div(ci * dy_rows * dy_w, 16) : ci * steps_img;
     if (P.ksteps > kMaxKsteps) return false;
     const int xb = P.ca * 2, db = P.ka * 2;
     P.x_box = ci * x_rows * wp * xb;
-    P.dy_box = ci * dy_rows * dy_w * db;
+    if (order == kPixels) {          // one box per 64 pixels: rows of 128 bytes, one per output channel
+        P.dy_subs = ceil_div(bp * P.q, 64);
+        P.katoms = ci * P.dy_subs;
+        P.dy_box = std::min(P.kt, P.k) * 128;
+        P.dy_alloc = round_up(P.kt * 128, 1024);
+    } else {
+        P.dy_box = ci * dy_rows * dy_w * db;
+        P.dy_alloc = round_up(std::max(P.dy_box, order == kPaired ? 0 : P.ksteps * 16 * db), 1024);
+    }
     // last X row an MMA touches: last k-step, last row and column shift, unused shifts of the c-side form
-    const int last = paired ? (ci - 1) * P.x_img + (bp - 1) * wp + P.q - 1 : P.ksteps * 16 - 1;
+    const int last = order == kFlat ? P.ksteps * 16 - 1 : (ci - 1) * P.x_img + (bp - 1) * wp + P.q - 1 + (order == kPixels ? 8 : 0);
     const int far = last + halo * wp + ceil_div(P.s, st) - 1 + (P.c_side ? 128 / P.ca : 256 / P.ca);
     P.x_alloc = round_up(std::max(P.x_box, (far + 1) * xb), 1024);
-    P.dy_alloc = round_up(std::max(P.dy_box, paired ? 0 : P.ksteps * 16 * db), 1024);
-    P.x_plane = P.na * P.phases * P.row_tiles * P.x_alloc;
+    const int x_tiles = P.na * P.phases * P.row_tiles;
+    P.x_plane = x_tiles * P.x_alloc;
     P.dy_plane = P.katoms * P.dy_alloc;
     P.x_region = P.planes * P.dy_plane;
     P.stage_bytes = P.x_region + P.planes * P.x_plane;
-    if (P.planes * (P.katoms + P.na * P.phases * P.row_tiles) > 32) return false;        // one copy per lane of a producer
+    if (P.planes * (P.katoms + x_tiles) > 32) return false;        // one copy per lane of a producer
     P.stages = std::min(kMaxStages, kStageBudget / P.stage_bytes) & ~1;
     P.epoch = std::max(1, (P.nprod > 1 ? 16 : 64) / P.ksteps);
     if (P.stages < 2) return false;
-    P.tx_bytes = (uint32_t)(P.planes * (P.katoms * P.dy_box + P.na * P.phases * P.row_tiles * P.x_box));
+    P.tx_bytes = (uint32_t)(P.planes * (P.katoms * P.dy_box + x_tiles * P.x_box));
     if (P.tx_bytes >= (1u << 20)) return false;
-    const uint32_t x_sbo = paired ? wp * xb : 8 * xb, dy_sbo = paired ? dy_w * db : 8 * db;
-    const uint32_t x_swz = P.ca == 64 ? 2 : P.ca == 32 ? 4 : 6, dy_swz = P.ka == 64 ? 2 : P.ka == 32 ? 4 : 6;
-    P.x_hi = (x_sbo >> 4) | (1u << 14) | (x_swz << 29);
+    const uint32_t x_swz = P.ca == 64 ? 2 : P.ca == 32 ? 4 : 6, dy_swz = order == kPixels || P.ka == 64 ? 2 : P.ka == 32 ? 4 : 6;
+    const uint32_t dy_sbo = order == kPixels ? 8 * 128 : order == kPaired ? dy_w * db : 8 * db;
     P.dy_hi = (dy_sbo >> 4) | (1u << 14) | (dy_swz << 29);
     P.x_lbo = (uint32_t)((P.merged ? P.x_alloc : xb) >> 4) << 16;
-    P.dy_lbo = (uint32_t)((P.katoms > 1 ? P.dy_alloc : 0) >> 4) << 16;      // one atom: the upper half of M repeats the lower
+    // (one atom: the upper half of M repeats the lower)
+    P.dy_lbo = order == kPixels ? 1u << 16 : (uint32_t)((P.katoms > 1 ? P.dy_alloc : 0) >> 4) << 16;
     for (int i = 0; i < P.ksteps; ++i) {
-        int xr = 16 * i, dr = 16 * i;
-        if (paired) {
+        int x_row = 16 * i, dy_off = 16 * i * db, x_sbo = 8;          // X row, dY bytes, X rows between the two 8-pixel groups
+        if (order == kPaired) {
             const int j = i % (P.q / 8), t = i / (P.q / 8), pr = t % (bp / 2), im = t / (bp / 2);
-            xr = im * P.x_img + 2 * pr * wp + 8 * j;
-            dr = im * P.dy_img + 2 * pr * dy_w + 8 * j;
+            x_row = im * P.x_img + 2 * pr * wp + 8 * j;
+            dy_off = (im * P.dy_img + 2 * pr * dy_w + 8 * j) * db;
+            x_sbo = wp;
+        } else if (order == kPixels) {
+            const int im = i / steps_img, j = 16 * (i % steps_img), p = j / P.q, q = j % P.q;
+            x_row = im * P.x_img + p * wp + q;
+            dy_off = (im * P.dy_subs + j / 64) * P.dy_alloc + (j % 64) * 2;
+            x_sbo = q + 8 < P.q ? 8 : wp - P.q + 8;
         }
-        P.k_off[i] = make_uint2((unsigned)(xr * xb) >> 4, (unsigned)(dr * db) >> 4);
+        P.k_off[i] = make_uint4((unsigned)(x_row * xb) >> 4, (unsigned)dy_off >> 4, (unsigned)(x_sbo * xb) >> 4 | (1u << 14) | (x_swz << 29), 0u);
     }
     return build_groups(P);
 }
@@ -725,7 +765,7 @@ struct ClHost {             // what ClPlan::opaque holds
     ClParams p;
     bool pack_x, pack_dy, f32, x_nhwc, dy_npqk;
     int xch, dych;          // channels per pixel row of the operands the tensor maps describe
-    int cb;                 // columns per block of the second kernel
+    int log_cb, groups;     // second kernel: columns per block, split groups per column
 };
 static_assert(sizeof(ClHost) <= sizeof(ClPlan::opaque), "ClPlan::opaque too small");
 
@@ -802,11 +842,12 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
                     if (F.stride == 1) F.phases = 1;
                     // part of the accumulator block that stands for elements of dW
                     const double share = (double)g.k * g.c * g.r * g.s / ((double)F.tiles_k * F.tiles_c * F.tiles_r * 128);
-                    for (int mode = 0; mode < 2; ++mode) {
-                        if (mode == 1 && g.q % 8 != 0) break;
+                    for (int mode = kFlat; mode <= kPixels; ++mode) {
+                        if (mode != kFlat && g.q % 8 != 0) break;
+                        if (mode == kPixels && (H.f32 || H.dy_npqk)) break;
                         auto consider = [&](int ci, int bp) {
                             ClParams C = F;
-                            if (!shape_chunk(C, ci, bp, mode == 1)) return false;
+                            if (!shape_chunk(C, ci, bp, mode)) return mode == kPixels && bp * C.q % 16 != 0;
 #ifdef GACONV_TUNING
                             if (const char* e = getenv("GACONV_CL_KS")) if (C.ksteps < atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_KSMAX")) if (C.ksteps > atoi(e)) return true;
@@ -815,14 +856,16 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
                             if (const char* e = getenv("GACONV_CL_KT")) if (C.kt != atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_NA")) if (C.na != atoi(e)) return true;
 #endif
-                            const Cost c = cost_of(C, sms, std::min(1.0, 1.3 * share / C.cols));
+                            Cost c = cost_of(C, sms, std::min(1.0, 1.3 * share / C.cols));
+                            // a packing pass of dY: its launch, and its bytes twice
+                            if (mode != kPixels && H.pack_dy) c.cycles += 3500 + (double)dy_el * 2 * (1 + C.planes) / (16.0 * sms);
                             if (c.cycles < best_cycles) { best_cycles = c.cycles; C.splits = c.splits; best = C; }
                             return true;
                         };
                         int last_bp = 0;
                         for (int parts = g.p; parts >= 1; --parts) {      // fewer and fewer, larger and larger bands
                             int bp = ceil_div(g.p, parts);
-                            if (mode == 1) bp = round_up(bp, 2);
+                            if (mode == kPaired) bp = round_up(bp, 2);
                             if (bp == last_bp) continue;
                             last_bp = bp;
                             if (!consider(1, bp)) break;
@@ -837,9 +880,16 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
     if (best_cycles >= 1e30) return false;
     best.chunk_base = best.chunks / best.splits;
     best.chunk_rem = best.chunks - best.chunk_base * best.splits;
+    // fp32 accumulators, bf16 operands, both MN-major (dY K-major where it is read as it lies), N, M = 128
     best.idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(best.nmma >> 3) << 17) | (8u << 24);
+    if (best.order == kPixels) { best.idesc &= ~(best.c_side ? 1u << 16 : 1u << 15); H.pack_dy = false; }
     H.p = best;
-    H.cb = best.splits > 32 ? 1 : best.splits > 16 ? 2 : best.splits > 8 ? 4 : 8;
+    // second kernel: at most eight loads a thread, a block of at most 32 warps, and as many blocks as there are SMs where the
+    // columns allow it
+    H.groups = 1;
+    while (H.groups < 32 && H.groups * 8 < best.splits) H.groups *= 2;
+    H.log_cb = 4;
+    while (H.log_cb > 0 && ((H.groups << H.log_cb) > 32 || best.tiles_k * best.tiles_c * best.tiles_r * ceil_div(best.cols, 1 << H.log_cb) < sms)) --H.log_cb;
     const int tiles = best.tiles_k * best.tiles_c * best.tiles_r;
     if (tiles > 65535 || best.splits > 65535) return false;
     out->cycles = best_cycles;
@@ -883,7 +933,14 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
                            swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
     CUtensorMap map_dy, map_x;
-    if (!encode(&map_dy, dy, P.k, H.dych, P.q, P.p, dy_el, P.ka, P.dy_pitch, P.dy_img / P.dy_pitch, 1) ||
+    auto encode_pixels = [&](CUtensorMap* map) {              // dY as (pixel, channel, image)
+        const cuuint64_t pq = (cuuint64_t)P.p * P.q;
+        cuuint64_t dims[3] = {pq, (cuuint64_t)P.k, (cuuint64_t)P.n}, strides[2] = {pq * 2, pq * P.k * 2};
+        cuuint32_t box[3] = {64, (cuuint32_t)std::min(P.kt, P.k), 1}, es[3] = {1, 1, 1};
+        return encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(dy), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    if (!(P.order == kPixels ? encode_pixels(&map_dy) : encode(&map_dy, dy, P.k, H.dych, P.q, P.p, dy_el, P.ka, P.dy_pitch, P.dy_img / P.dy_pitch, 1)) ||
         !encode(&map_x, x, P.c, H.xch, P.w, P.h, x_el, P.ca, P.x_pitch, P.x_img / P.x_pitch, P.stride))
         return cudaErrorInvalidValue;
     // the stages; at the end they hold the accumulator block
@@ -894,11 +951,9 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
     if ((err = launch_kernel(kern, grid, dim3(kThreads), smem, stream, dim3(1, 1, 1), map_dy, map_x, dw, partial, status, P)) != cudaSuccess) return err;
     note_launch();
     if (P.splits == 1) return cudaSuccess;
-    const dim3 rgrid((unsigned)ceil_div(P.cols, H.cb), grid.x);
-    err = H.cb == 1   ? launch_kernel(cl_reduce_kernel<1>, rgrid, dim3(256), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P)
-          : H.cb == 2 ? launch_kernel(cl_reduce_kernel<2>, rgrid, dim3(256), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P)
-          : H.cb == 4 ? launch_kernel(cl_reduce_kernel<4>, rgrid, dim3(256), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P)
-                      : launch_kernel(cl_reduce_kernel<8>, rgrid, dim3(256), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P);
+    const dim3 rgrid((unsigned)ceil_div(P.cols, 1 << H.log_cb), grid.x);
+    err = launch_kernel(cl_reduce_kernel, rgrid, dim3(32u * H.groups << H.log_cb), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P,
+                        H.log_cb, H.groups);
     if (err != cudaSuccess) return err;
     note_launch();
     return cudaSuccess;

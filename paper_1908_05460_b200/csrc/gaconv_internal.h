@@ -149,7 +149,7 @@ cudaError_t launch_tc(const void* x, const void* dy, float* dw, float* partial, 
 struct ClPlan {
     double cycles;                          // the planner's estimate of the two kernels, SM cycles
     size_t partial_bytes, x_bytes, dy_bytes;    // workspace: accumulator blocks, packed copies of the operands (0: read in place)
-    alignas(8) unsigned char opaque[2048];  // kernel parameters, private to cl.cu
+    alignas(8) unsigned char opaque[3072];  // kernel parameters, private to cl.cu
 };
 bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* plan);
 cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, void* x_scratch, void* dy_scratch, uint32_t* status,

@@ -38,7 +38,7 @@ def test_every_layout_matches_the_oracle(li, dtype):
     layer = SHAPES[li]
     x, dy = I.make_layer_inputs(layer, dtype, 11, li)
     ref, dn = oracle.dw_exact(to_f64(x), to_f64(dy), oshape(layer), 0.5)
-    first = None
+    first = {}
     for name, kw in LAYOUTS.items():
         g = GpuLayer(layer, dtype, x, dy, alpha=0.5, **kw)
         before = B.gaconv_launch_count()
@@ -46,8 +46,10 @@ def test_every_layout_matches_the_oracle(li, dtype):
         assert B.gaconv_launch_count() - before <= 3, name
         assert norm_err(got, ref, dn) <= TOL_F32 / 2, name        # bf16 products are exact in fp32 as well
         np.testing.assert_array_equal(got, g.exact())
-        first = got if first is None else first
-        np.testing.assert_array_equal(got, first)                # the same operands, however they were handed over
+        # the same operands, however they were handed over; only a bf16 gradient on rows of whole 16-byte pieces is read as it
+        # lies, so that its pixels are summed in another order when it comes channels last
+        order = kw.get("dy_layout", B.DY_NKPQ) if dtype == torch.bfloat16 and layer.q % 8 == 0 else None
+        np.testing.assert_array_equal(got, first.setdefault(order, got))
         assert B.gaconv_poll_async_status(g.desc) == B.OK
     few = GpuLayer(layer, dtype, x, dy, alpha=0.5, sm_budget=11)
     assert norm_err(few.exact(), ref, dn) <= TOL_F32 / 2
