@@ -187,39 +187,94 @@ select_sparse_transposed_kernel(const __nv_bfloat16* __restrict__ dy, __nv_bfloa
     }
 }
 
-// Selection of the top-k variant: one warp per map.  Round t picks the largest key below the key picked in
-// round t-1, where key = (bit pattern of |v|, complement of the position): keys are distinct, larger magnitude
-// first and, among equal magnitudes, the lower position first -- the order the single arg-max uses.
-template <typename T>
+// Selection of the top-k variant: one warp per map; take(t, j) receives the t-th retained position, the return value is the
+// map's sum.  Larger magnitude first and, among equal magnitudes, the lower position first -- the order the single arg-max uses.
+// Every lane keeps its best candidate; a round picks the best of the warp (two warp reductions), after which only the lane
+// that gave it looks for its next one, among the elements it holds in registers (maps of up to 1024 pixels: HELD a lane, all
+// loads in flight at once) or, HELD = 0, reads again.  A serial chain bounds it, not the bytes: a round used to be a pass over
+// the map and ten dependent shuffles.  (fp32 25x25, k = 4, 2,800 maps: 11.8 -> 7.3 us; bf16 7x5, k = 4, 29,232 maps: 20 -> 9;
+// bf16 33x33, k = 3, 9,024 maps: 25 -> 20, the re-reading form -- holding 64 a lane leaves too few warps and takes 31.)
+template <typename T> struct BitsOf;
+// (load: volatile, so that the compiler keeps the value in a register instead of reading it again in every round)
+template <> struct BitsOf<float> {
+    typedef uint32_t type;
+    static constexpr uint32_t kMag = 0x7fffffffu;
+    __device__ static __forceinline__ float value(uint32_t b) { return __uint_as_float(b); }
+    __device__ static __forceinline__ uint32_t load(const uint32_t* p) { uint32_t v; asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p)); return v; }
+};
+template <> struct BitsOf<__nv_bfloat16> {
+    typedef unsigned short type;
+    static constexpr uint32_t kMag = 0x7fffu;
+    __device__ static __forceinline__ float value(uint32_t b) { return bf16_bits_to_float(b); }
+    __device__ static __forceinline__ uint32_t load(const unsigned short* p) { unsigned short v; asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p)); return v; }
+};
+
+template <typename T, int HELD, typename Take>
+__device__ __forceinline__ float topk_of_map(const T* __restrict__ map, int pq, int topk, Take take)
+{
+    typedef BitsOf<T> B;
+    constexpr bool held = HELD > 0;
+    constexpr int N = held ? HELD : 1;
+    const int lane = threadIdx.x & 31;
+    const typename B::type* m = reinterpret_cast<const typename B::type*>(map);
+    float total = 0.0f;
+    uint32_t v[N];                          // held: bits of element lane + 32 i
+    uint32_t taken = 0u;                    // which of them are taken
+    uint32_t best = 0u, best_j = 0xffffffffu;  // 1 + magnitude of the lane's best candidate (0: none left), its position
+    if constexpr (held) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = B::load(m + min(lane + 32 * i, pq - 1));      // (no branch: a lane past the end reads the last element, and ignores it)
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            if (lane + 32 * i < pq) {
+                total += B::value(v[i]);
+                const uint32_t k = (v[i] & B::kMag) + 1u;
+                if (k > best) { best = k; best_j = lane + 32 * i; }
+            }
+    } else {
+#pragma unroll 8
+        for (int j = lane; j < pq; j += 32) {
+            const uint32_t b = __ldg(m + j), k = (b & B::kMag) + 1u;
+            total += B::value(b);
+            if (k > best) { best = k; best_j = j; }
+        }
+    }
+    for (int t = 0; t < topk; ++t) {
+        const uint32_t top = __reduce_max_sync(0xffffffffu, best);
+        const uint32_t j = __reduce_min_sync(0xffffffffu, best == top ? best_j : 0xffffffffu);
+        take(t, (int)j);
+        if (best_j == j && t + 1 < topk) {
+            best = 0u; best_j = 0xffffffffu;
+            if constexpr (held) {
+                taken |= 1u << (j >> 5);
+#pragma unroll
+                for (int i = 0; i < N; ++i) {
+                    const uint32_t k = (v[i] & B::kMag) + 1u;
+                    if (lane + 32 * i < pq && !((taken >> i) & 1u) && k > best) { best = k; best_j = lane + 32 * i; }
+                }
+            } else {
+                for (int i = lane; i < pq; i += 32) {      // what comes after (top, j): lower magnitudes, and equal ones further on
+                    const uint32_t k = (__ldg(m + i) & B::kMag) + 1u;
+                    if ((k < top || (k == top && (uint32_t)i > j)) && k > best) { best = k; best_j = i; }
+                }
+            }
+        }
+    }
+    for (int off = 16; off > 0; off >>= 1) total += __shfl_xor_sync(0xffffffffu, total, off);
+    return total;
+}
+
+template <typename T, int HELD>
 __global__ void __launch_bounds__(256)
 select_topk_kernel(const T* __restrict__ dy, int32_t* __restrict__ idx, float* __restrict__ sum, long long num_maps, int pq, int topk)
 {
     pdl_release_next_grid();
     pdl_wait_prior_grid();
-    const int lane = threadIdx.x & 31;
     const long long m = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (m >= num_maps) return;
-    const T* map = dy + m * (long long)pq;
-    unsigned long long prev = ~0ull;
-    float total = 0.0f;
-    for (int t = 0; t < topk; ++t) {
-        unsigned long long best = 0ull;
-        for (int j = lane; j < pq; j += 32) {
-            Scan sc{-1, 0, 0.0f};
-            Elem<T>::visit1(map, j, sc);
-            const unsigned long long key = ((unsigned long long)(unsigned)(sc.best_mag + 1) << 32) | (0xffffffffu - (unsigned)j);
-            if (key < prev && key > best) best = key;
-            if (t == 0) total += sc.sum;
-        }
-        for (int off = 16; off > 0; off >>= 1) {
-            const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, off);
-            best = other > best ? other : best;
-        }
-        if (lane == 0) idx[m * topk + t] = (int)(0xffffffffu - (unsigned)(best & 0xffffffffu));
-        prev = best;
-    }
-    for (int off = 16; off > 0; off >>= 1) total += __shfl_xor_sync(0xffffffffu, total, off);
-    if (lane == 0) sum[m] = total;
+    const bool first = (threadIdx.x & 31) == 0;
+    const float total = topk_of_map<T, HELD>(dy + m * (long long)pq, pq, topk, [&](int t, int j) { if (first) idx[m * topk + t] = j; });
+    if (first) sum[m] = total;
 }
 
 // four consecutive elements, raw (16-byte load for fp32, 8-byte load for bf16), and their values as floats
@@ -531,14 +586,23 @@ cudaError_t launch_select_sparse_transposed(const void* dy, void* dyt, const Geo
     return e;
 }
 
-cudaError_t launch_select_topk(const void* dy, int32_t* idx, float* sum, const Geom& g, int topk, cudaStream_t stream)
+template <typename T>
+static cudaError_t launch_select_topk_t(const T* dy, int32_t* idx, float* sum, const Geom& g, int topk, cudaStream_t stream)
 {
     const long long maps = (long long)g.n * g.k;
-    const unsigned grid = (unsigned)((maps + 7) / 8);
-    if (g.bf16) select_topk_kernel<__nv_bfloat16><<<grid, 256, 0, stream>>>(static_cast<const __nv_bfloat16*>(dy), idx, sum, maps, g.p * g.q, topk);
-    else        select_topk_kernel<float><<<grid, 256, 0, stream>>>(static_cast<const float*>(dy), idx, sum, maps, g.p * g.q, topk);
+    const int pq = g.p * g.q;
+    const dim3 grid((unsigned)((maps + 7) / 8));
     note_launch();
-    return cudaGetLastError();
+#define GACONV_TOPK_CASE(H) if (pq <= 32 * H) return launch_kernel(select_topk_kernel<T, H>, grid, dim3(256), 0, stream, dim3(1, 1, 1), dy, idx, sum, maps, pq, topk);
+    GACONV_TOPK_CASE(1) GACONV_TOPK_CASE(2) GACONV_TOPK_CASE(4) GACONV_TOPK_CASE(8) GACONV_TOPK_CASE(16) GACONV_TOPK_CASE(24) GACONV_TOPK_CASE(32)
+#undef GACONV_TOPK_CASE
+    return launch_kernel(select_topk_kernel<T, 0>, grid, dim3(256), 0, stream, dim3(1, 1, 1), dy, idx, sum, maps, pq, topk);
+}
+
+cudaError_t launch_select_topk(const void* dy, int32_t* idx, float* sum, const Geom& g, int topk, cudaStream_t stream)
+{
+    return g.bf16 ? launch_select_topk_t(static_cast<const __nv_bfloat16*>(dy), idx, sum, g, topk, stream)
+                  : launch_select_topk_t(static_cast<const float*>(dy), idx, sum, g, topk, stream);
 }
 
 GatherPlan plan_gather(const Geom& g)
@@ -590,8 +654,6 @@ static cudaError_t launch_fused_t(const T* x, const T* dy, float* dw, const Geom
     // two passes over the CTA's maps; measured: helps 32-channel layers, neutral or worse for 16 and 64
     const int threads = (g.sm_budget == 0 && g.k >= 32 && (long long)cl * g.k <= 148 * 2) ? 512 : 256;
     const int groups = rsc / (WIDE ? 8 : vec_x ? 4 : 1);
-    const int batch = (sizeof(T) == 4 || WIDE) ? 4 : 8;
-    (void)batch;
     while (nj < 16 && nj * 2 <= ipc * topk && nj * 2 * groups <= threads) nj *= 2;        // image lanes: as many as keep every item on its own thread
     while (nj > 1 && (size_t)rsc * 4 * (1 + nj) > 150 * 1024) nj /= 2;              // the subtotals must fit shared memory
     const size_t smem = (((size_t)rsc * 4 + 15) & ~(size_t)15) + (size_t)ipc * topk * 16 + (nj > 1 ? (size_t)nj * rsc * 4 : 0) + 16;
