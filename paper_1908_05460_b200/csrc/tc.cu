@@ -859,8 +859,8 @@ bool plan_tc(const Geom& g, TcPlan* out)
     P.b_swz = swz_code(ct * 2);
     // wide tile: stride 1, whole rows per chunk, k-steps inside a row (Q a multiple of 16) or exactly two rows (Q = 8)
     P.wide = (env_int("GACONV_TC_WIDE", 1) && !small_map && g.stride_h == 1 && (g.q % 16 == 0 || g.q == 8) && 64 % g.q == 0) ? 1 : 0;
-    // small maps, one filter row per CTA: the (pixel, image) ordering with a single haloed X tile
-    const bool tiny2 = tiny && P.rc == 1 && g.stride_h == 1 && g.q % 2 == 0 && g.n >= 8 && env_int("GACONV_TC_TINY2", 1);
+    // small maps, one filter row per CTA: the (pixel, image) ordering with a single haloed X tile (of 128-byte rows)
+    const bool tiny2 = tiny && ct == 64 && P.rc == 1 && g.stride_h == 1 && g.q % 2 == 0 && g.n >= 8 && env_int("GACONV_TC_TINY2", 1);
     P.tiny2 = tiny2 ? 1 : 0;
     P.b_tiles = (P.wide || tiny2) ? 1 : halo ? g.s : P.rc * g.s;
 
