@@ -87,6 +87,7 @@ struct ClParams {
     int order, ksteps, x_pitch, dy_pitch, x_img, dy_img;
     int dy_subs;                    // kPixels: 64-pixel boxes of dY per image of a chunk
     int c_side;                     // 1: X is the M side
+    int s_inner;                    // 1: column shifts lie next to one another in dW (K x C x R x S): columns are written shift by shift
     int merged;                     // 1: the MN atoms of an X operand are channel atoms, 0: column shifts
     int ngroups, nmma, cols, tmem_cols;
     int epoch;                      // chunks of one issuer between two readings of its accumulators
@@ -98,6 +99,15 @@ struct ClParams {
 // fp32 operands: which planes of X and dY each of the six products of a k-step takes
 __device__ constexpr uint32_t prod_x(int i) { return i == 1 ? 2u : (i == 2 || i == 4) ? 1u : 0u; }
 __device__ constexpr uint32_t prod_dy(int i) { return i == 0 ? 2u : (i == 2 || i == 3) ? 1u : 0u; }
+
+// The e-th column of a k-side block in the order of dW: where the shifts of a channel are neighbours in memory, shift by shift,
+// so that a store of 32 lanes touches 13 sectors instead of 32 (K x C x R x S, 512->512 on 2x2 maps: the stores were 12 of 24 us).
+__device__ __forceinline__ int written_column(const ClParams& P, int e)
+{
+    if (!P.s_inner) return e;
+    const int g = e / P.nmma, j = e - g * P.nmma, atoms = P.nmma / P.ca, c = j / atoms;
+    return g * P.nmma + (j - c * atoms) * P.ca + c;
+}
 
 // Warps: 0 and 1 issue MMAs, 2 and 3 fill the stages, 4 to 11 hold the sums.
 //
@@ -321,16 +331,18 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
         // ------------------------------------------------------------------ block -> workspace, or dW
         // Through shared memory, [column][128 lanes] (the stages are free: every copy has landed and every MMA has read).
         // The workspace copy then is one bulk store per 16 columns; the only split of a tile writes dW itself, along the
-        // channels (one word of padding per column: lanes that read along the columns stay in different banks).
+        // channels, or along the shifts of a channel (padding per column and per shift: lanes that read along the columns stay in
+        // different banks).
         if (ok) {
             const bool direct = P.splits == 1;
-            const int pitch = direct ? 129 : 128, t = threadIdx.x - 128;
+            const int t = threadIdx.x - 128, ca_log = 31 - __clz(P.ca);
+            auto at = [&](int col) { return direct ? col * 129 + 11 * (col >> ca_log) : col * 128; };
             float* blk = reinterpret_cast<float*>(smem_raw + (smem_base - smem_u32(smem_raw)));
 #pragma unroll
             for (int i = 0; i < NB; ++i)
                 if (2 * i + half < blocks) {
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) blk[(16 * (2 * i + half) + e) * pitch + l128] = sum[i][e];
+                    for (int e = 0; e < 16; ++e) blk[at(16 * (2 * i + half) + e) + l128] = sum[i][e];
                 }
             if (direct)
                 for (int col = t; col < P.cols; col += 256) {
@@ -357,15 +369,17 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
 #pragma unroll 8
                     for (int col = half; col < P.cols; col += 2) {
                         const int2 o = s_col[col];
-                        if (P.merged ? o.y > 0 : a < o.y) d[o.x] = P.alpha * blk[col * 129 + l128];
+                        if (P.merged ? o.y > 0 : a < o.y) d[o.x] = P.alpha * blk[at(col) + l128];
                     }
                 }
             } else {
-                int off[NB];                // this lane's columns, the same in every row; -1: none
+                int off[NB], pos[NB];       // this lane's columns, the same in every row; -1: none
 #pragma unroll
                 for (int u = 0; u < NB; ++u) {
-                    const int2 o = lane + 32 * u < P.cols ? s_col[lane + 32 * u] : make_int2(0, 0);
+                    const int e = lane + 32 * u, col = e < P.cols ? written_column(P, e) : 0;
+                    const int2 o = e < P.cols ? s_col[col] : make_int2(0, 0);
                     off[u] = o.y > 0 ? o.x : -1;
+                    pos[u] = at(col);
                 }
 #pragma unroll 2
                 for (int l = warp - 4; l < 128; l += 8) {
@@ -373,7 +387,7 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
                     float* d = dw + (k0 + l) * P.ws_k;
 #pragma unroll
                     for (int u = 0; u < NB; ++u)
-                        if (off[u] >= 0) d[off[u]] = P.alpha * blk[(lane + 32 * u) * 129 + l];
+                        if (off[u] >= 0) d[off[u]] = P.alpha * blk[pos[u] + l];
                 }
             }
         }
@@ -404,9 +418,10 @@ cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, cons
     const int k0 = tk * P.kt, c0 = (tr - tk * P.tiles_c) * P.ct;
     const int ca_shift = 31 - __clz(P.ca), mn_mask = P.merged ? 127 : P.ca - 1;
     if ((int)threadIdx.x < CB) {
-        const int col = col0 + threadIdx.x;
+        int col = col0 + threadIdx.x;
         int2 o = make_int2(0, 0);
         if (col < P.cols) {
+            if (!P.c_side) col = written_column(P, col);
             const int gi = col / P.nmma, j = col - gi * P.nmma;
             const ClGroup& g = P.g[gi];
             const int a = P.c_side || P.merged ? 0 : j >> ca_shift, k = P.c_side ? k0 + j : 0;
@@ -417,7 +432,8 @@ cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, cons
         s_col[threadIdx.x] = o;
     }
     const int cb = warp & (CB - 1), grp = warp >> log_cb;
-    const float4* src = reinterpret_cast<const float4*>(partial + ((size_t)tile * P.splits * P.cols + col0 + cb) * 128) + lane;
+    const int src_col = P.c_side || col0 + cb >= P.cols ? col0 + cb : written_column(P, col0 + cb);
+    const float4* src = reinterpret_cast<const float4*>(partial + ((size_t)tile * P.splits * P.cols + src_col) * 128) + lane;
     const size_t step = (size_t)P.cols * 32;
     __syncthreads();
     const bool live = s_col[cb].y > 0;
@@ -434,7 +450,9 @@ cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, cons
     *reinterpret_cast<float4*>(&s_sum[warp][4 * lane]) = acc;
     __syncthreads();
     for (int e = threadIdx.x; e < CB << 7; e += blockDim.x) {
-        const int c = P.c_side ? e >> 7 : e & (CB - 1), l = P.c_side ? e & 127 : e >> log_cb;
+        const int c = P.c_side ? e >> 7 : e & (CB - 1);
+        int l = P.c_side ? e & 127 : e >> log_cb;
+        if (P.c_side && P.s_inner) { const int t_shift = 7 - ca_shift; l = ((l & ((1 << t_shift) - 1)) << ca_shift) + (l >> t_shift); }
         const int2 o = s_col[c];
         bool valid; long long off = o.x;
         if (P.c_side) {
@@ -687,6 +705,7 @@ bool build_groups(ClParams& P)
             }
         }
     P.nmma = P.c_side ? P.kt : atoms * P.ca;
+    P.s_inner = !P.merged && P.s > 1 && P.ws_s < P.ws_c;
     P.cols = P.ngroups * P.nmma;
     if (P.cols > kMaxCols) return false;
     P.tmem_cols = 32;
@@ -944,7 +963,7 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
         !encode(&map_x, x, P.c, H.xch, P.w, P.h, x_el, P.ca, P.x_pitch, P.x_img / P.x_pitch, P.stride))
         return cudaErrorInvalidValue;
     // the stages; at the end they hold the accumulator block
-    const size_t smem = std::max((size_t)P.stages * P.stage_bytes, (size_t)P.cols * 129 * 4) + 1024;
+    const size_t smem = std::max((size_t)P.stages * P.stage_bytes, (size_t)(P.cols * 129 + 12 * 11) * 4) + 1024;
     const dim3 grid((unsigned)(P.tiles_k * P.tiles_c * P.tiles_r), (unsigned)P.splits);
     ClKernel kern = kernel_for(P.ngroups, H.f32, P.c_side != 0);
     if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return err;
