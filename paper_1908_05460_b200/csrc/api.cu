@@ -184,7 +184,8 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, bool reordered)
     reordered = reordered && products > 3e7;
     if (g.bf16) {
         if (L.tc_ok) {
-            if (L.tp.reads_transposed_dy || products < 3e7) return false;       // maps under 64 pixels: 512->512 on 2x2 11.5 / 18.2
+            if (L.tp.reads_transposed_dy) return products > 5e6;        // maps under 64 pixels: 512->512 on 4x4, N = 256 31.1 / 27.0
+            if (products < 3e7) return false;
             if (reordered) return true;                             // 128->128 on 16x16, dY channels last 28.4 / 17.8
             if (g.c <= 16 || (g.c < 64 && shared)) return false;    // 16->16 on 32x32 11.9 / 12.5; on 18 SMs 28 / 38
             return g.r < 5;                                         // 5x5 64->64 on 16x16 16.1 / 17.8, 3x3 64->64 on 32x32 24.1 / 22.5

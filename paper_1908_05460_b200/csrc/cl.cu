@@ -19,6 +19,10 @@
 // pixels  dY as it lies, N x K x P x Q (K-major rows of 64 pixels, Q a multiple of 8): a k-step is 16 consecutive pixels of an
 //           image, no halo columns and no packing of dY.  Its two groups of 8 X pixels lie 8 pixels apart, or a row's end further,
 //           so the X descriptor's stride belongs to the k-step.
+//   images  (small or odd maps, many images) rows ordered (pixel, image): tensor maps with permuted dimensions deliver, for every
+//           pixel of a band, the rows of `ci` images.  A column shift is then ci rows; a k-step is 16 images of a pixel (ci = 8:
+//           of two pixels), no halo column is ever multiplied, and filter rows that fall outside the map are skipped.  The k-side
+//           form at stride 1 does not even load halo columns: at the edge of the map its MMAs take fewer column shifts.
 // A table of the plan holds the offsets of the k-steps of every order.
 //
 // Which operand is the MMA's M side:
@@ -28,8 +32,9 @@
 // The MMAs of one k-step differ only in the X offset and the accumulator columns; the list of them is part of the plan.
 //
 // CTA = one tile of dW (k-tile x c-tile x filter rows) and a contiguous range of chunks.  Its accumulator block goes to
-// the workspace as [column][128 lanes] (coalesced: a warp writes one column of 32 lanes per store) and cl_reduce_kernel
-// adds the splits in order, so results are the same from run to run.
+// the workspace as [column][128 lanes] and cl_reduce_kernel adds the splits in order, so results are the same from run to run.
+// (Adding them over a thread-block cluster's shared memory instead costs more: reads from other SMs came to ~10 bytes a cycle,
+// where the workspace takes 21, and clusters of six leave SMs idle: 256->256 on 8x8, N = 128 19.1 us against 18.8.)
 //
 // Every wait is bounded; on expiry the kernel raises the workspace status word, lets its copies land, frees its tensor
 // memory and returns.
@@ -64,7 +69,7 @@ namespace {
 constexpr int kMaxGroups = 16, kMaxKsteps = 128, kMaxStages = 8;
 
 // order of the reduction inside a chunk, see above
-enum { kFlat = 0, kPaired = 1, kPixels = 2 };
+enum { kFlat = 0, kPaired = 1, kPixels = 2, kImages = 3 };
 
 struct ClGroup {            // one MMA of a k-step
     int x_off;              // offset of its X rows inside the X region of a stage, 16-byte units
@@ -86,14 +91,20 @@ struct ClParams {
     uint32_t tx_bytes;
     int order, ksteps, x_pitch, dy_pitch, x_img, dy_img;
     int dy_subs;                    // kPixels: 64-pixel boxes of dY per image of a chunk
+    int px_rows;                    // kImages: rows of a pixel (images); else 1
+    int x_pre;                      // bytes of zeros before an X tile (kImages without halo columns; else 0)
+    int skip;                       // kImages, whole maps, one filter row a tile: k-steps per map row, to leave out rows opposite the padding
     int c_side;                     // 1: X is the M side
     int s_inner;                    // 1: column shifts lie next to one another in dW (K x C x R x S): columns are written shift by shift
     int merged;                     // 1: the MN atoms of an X operand are channel atoms, 0: column shifts
     int ngroups, nmma, cols, tmem_cols;
+    int mma_cols;                   // columns of all MMAs of a chunk and product
     int epoch;                      // chunks of one issuer between two readings of its accumulators
     uint32_t dy_hi, x_lbo, dy_lbo, idesc;
     ClGroup g[kMaxGroups];
-    uint4 k_off[kMaxKsteps];        // k-step -> offsets of its X and dY rows (16-byte units), upper word of its X descriptor
+    // k-step -> offsets of its X and dY rows (16-byte units), upper word of its X descriptor, and, with one k-side MMA a k-step,
+    // the first column of that MMA | its N in the instruction descriptor's place (0 << 17 in idesc)
+    uint4 k_off[kMaxKsteps];
 };
 
 // fp32 operands: which planes of X and dY each of the six products of a k-step takes
@@ -104,9 +115,22 @@ __device__ constexpr uint32_t prod_dy(int i) { return i == 0 ? 2u : (i == 2 || i
 // so that a store of 32 lanes touches 13 sectors instead of 32 (K x C x R x S, 512->512 on 2x2 maps: the stores were 12 of 24 us).
 __device__ __forceinline__ int written_column(const ClParams& P, int e)
 {
-    if (!P.s_inner) return e;
+    if (P.c_side || !P.s_inner) return e;
     const int g = e / P.nmma, j = e - g * P.nmma, atoms = P.nmma / P.ca, c = j / atoms;
     return g * P.nmma + (j - c * atoms) * P.ca + c;
+}
+// Element (column, lane) of a block that goes to dW directly, in words: [column][128], the lanes of a column exchanged by a key, so that neither a column's
+// lanes, nor a lane's columns, nor the shifts of a channel meet in one bank.
+__device__ __forceinline__ int block_key(int col, int ca_log) { return (col + 11 * (col >> ca_log)) & 31; }
+// Column -> {offset in dW, atoms in use (0: not an element)}
+__device__ __forceinline__ int2 column_target(const ClParams& P, int col, int k0, int c0, int r0)
+{
+    const int gi = col / P.nmma, j = col - gi * P.nmma;
+    const ClGroup& g = P.g[gi];
+    const int a = P.c_side || P.merged ? 0 : j / P.ca, k = P.c_side ? k0 + j : 0;
+    const int c = c0 + g.cbase + (P.c_side ? 0 : P.merged ? j : j - a * P.ca);
+    const bool valid = r0 + g.r < P.r && (P.c_side ? k < P.k : c < P.c && a < g.cnt);
+    return make_int2((int)(k * P.ws_k + c * P.ws_c + (r0 + g.r) * P.ws_r + (g.s0 + P.stride * a) * P.ws_s), valid ? g.cnt : 0);
 }
 
 // Warps: 0 and 1 issue MMAs, 2 and 3 fill the stages, 4 to 11 hold the sums.
@@ -127,7 +151,7 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
     __shared__ __align__(8) uint64_t bar_full[kMaxStages], bar_empty[kMaxStages], bar_acc[2], bar_free[2];
     __shared__ uint32_t s_tmem_base;
     __shared__ volatile int s_abort;
-    __shared__ int2 s_col[kMaxCols];        // column of the block -> {offset in dW, atoms in use}
+    __shared__ int2 s_col[kMaxCols];        // column_target of every column
 
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -147,9 +171,11 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
             const int st = t / tiles_all, i = t - st * tiles_all;
             const bool is_dy = i < tiles_dy;
             const int base = st * P.stage_bytes + (is_dy ? i * P.dy_alloc : P.x_region + (i - tiles_dy) * P.x_alloc);
-            const int from = is_dy ? P.dy_box : P.x_box, to = is_dy ? P.dy_alloc : P.x_alloc;
-            for (int o = from + lane * 16; o < to; o += 512)
-                asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(smem_base + base + o), "r"(0) : "memory");
+            const int from = is_dy ? P.dy_box : P.x_pre + P.x_box, to = is_dy ? P.dy_alloc : P.x_alloc;
+            auto zero = [&](int o) { asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(smem_base + base + o), "r"(0) : "memory"); };
+            for (int o = from + lane * 16; o < to; o += 512) zero(o);
+            if (!is_dy)
+                for (int o = lane * 16; o < P.x_pre; o += 512) zero(o);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -161,6 +187,8 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (P.splits == 1)
+        for (int col = threadIdx.x; col < P.cols; col += kThreads) s_col[col] = column_target(P, col, k0, c0, r0);
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"(P.tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -179,16 +207,16 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
         const bool whole = P.cpi == 0;
         constexpr int np = 2;
         const int first = warp - 2, c_first = ch_begin + first;
-        int n0 = whole ? c_first * P.ci : c_first / P.cpi, p0 = whole ? 0 : (c_first % P.cpi) * P.bp;
+        int n0 = (whole ? c_first : c_first / P.cpi) * P.ci, p0 = whole ? 0 : (c_first % P.cpi) * P.bp;
         // this lane's copy of every chunk (a plan has at most 32): where it goes, and its coordinates relative to the chunk's
         const int x_tiles = P.na * P.phases * P.row_tiles, per_plane = P.katoms + x_tiles;
         const int pl = lane / per_plane, i = lane - pl * per_plane, j = i - P.katoms, jt = j / P.na, rl = jt / P.phases;
         const bool mine = lane < P.planes * per_plane, is_dy = i < P.katoms;
         const CUtensorMap* map = is_dy ? &map_dy : &map_x;
-        const uint32_t dst = is_dy ? pl * P.dy_plane + i * P.dy_alloc : P.x_region + pl * P.x_plane + j * P.x_alloc;
-        const bool pixels = is_dy && P.order == kPixels;          // box i: 64 pixels of image i / dy_subs, K-major
+        const uint32_t dst = is_dy ? pl * P.dy_plane + i * P.dy_alloc : P.x_region + pl * P.x_plane + j * P.x_alloc + P.x_pre;
+        const bool images = P.order == kImages, pixels = is_dy && P.order == kPixels;          // box i: 64 pixels of image i / dy_subs, K-major
         const int dy_img = pixels ? i / P.dy_subs : 0, dy_px = 64 * (i - dy_img * P.dy_subs);
-        const int ch = is_dy ? k0 + P.ka * i : c0 + P.ca * (j - jt * P.na), col = is_dy ? 0 : jt - rl * P.phases - P.pad_w;
+        const int ch = is_dy ? k0 + P.ka * i : c0 + P.ca * (j - jt * P.na), col = is_dy || P.x_pre ? 0 : jt - rl * P.phases - P.pad_w;
         const int row_mul = is_dy ? 1 : P.stride, row_add = is_dy ? 0 : r0 + rl - P.pad_h;
         int st = first, ph = 0, it = first;
         while (st >= P.stages) { st -= P.stages; ph ^= 1; }
@@ -199,9 +227,12 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
             if (lane == 0) mbar_expect_tx(full, P.tx_bytes);
             __syncwarp();
             if (pixels) { if (mine) tma_load_3d(smem_base + st * P.stage_bytes + dst, map, full, p0 * P.q + dy_px, k0, n0 + dy_img); }
-            else if (mine) tma_load_5d(smem_base + st * P.stage_bytes + dst, map, full, ch, col, p0 * row_mul + row_add, n0, pl);
+            else if (mine) {
+                const int row = p0 * row_mul + row_add;
+                tma_load_5d(smem_base + st * P.stage_bytes + dst, map, full, ch, images ? n0 : col, images ? col : row, images ? row : n0, pl);
+            }
             if (whole) n0 += np * P.ci;
-            else for (p0 += np * P.bp; p0 >= P.cpi * P.bp; p0 -= P.cpi * P.bp) ++n0;
+            else for (p0 += np * P.bp; p0 >= P.cpi * P.bp; p0 -= P.cpi * P.bp) n0 += P.ci;
             for (st += np; st >= P.stages; st -= P.stages) ph ^= 1;
         }
         if (lane == 0 && s_abort)      // let the copies already issued land (bounded)
@@ -217,7 +248,12 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
         constexpr int PER = NG * (F32 ? 6 : 1), U = PER >= 8 ? 1 : PER == 1 ? 12 : PER == 2 ? 6 : PER == 3 ? 4 : 2;
         const uint32_t x_plane = (uint32_t)P.x_plane >> 4, dy_plane = (uint32_t)P.dy_plane >> 4;
         const uint64_t dy_hi = (uint64_t)P.dy_hi << 32;
-        const int ksteps = P.ksteps, ngroups = P.ngroups;
+        const int ngroups = P.ngroups;
+        int k_first = 0, ksteps = P.ksteps;
+        if (P.skip) {       // output rows whose input row r0 lies inside the map
+            const int lo = max(0, (P.pad_h - r0 + P.stride - 1) / P.stride), hi = min(P.p, (P.h - 1 + P.pad_h - r0) / P.stride + 1);
+            if (lo < hi) { k_first = lo * P.skip; ksteps = hi * P.skip; }       // (none: multiply the zeros)
+        }
         const uint32_t nmma = P.nmma, idesc = P.idesc;
         uint32_t off[NG];
 #pragma unroll
@@ -252,12 +288,14 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
                         for (int g = 0; g < NG; ++g)
                             if (NG <= 9 || g < ngroups) {          // (up to nine MMAs there is an instance for every count)
                                 const uint64_t ad = CSIDE ? xd + off[g] : dyd, bd = CSIDE ? dyd : xd + off[g];
-                                if (starts && pr == 0) umma_bf16(acc + g * nmma, ad, bd, idesc, 0u);
-                                else umma_bf16_acc(acc + g * nmma, ad, bd, idesc);
+                                const uint32_t d = acc + (NG == 1 && !CSIDE ? o.w & 0xffffu : g * nmma);
+                                const uint32_t id = NG == 1 && !CSIDE ? idesc | (o.w & 0xffff0000u) : idesc;
+                                if (starts && pr == 0) umma_bf16(d, ad, bd, id, 0u);
+                                else umma_bf16_acc(d, ad, bd, id);
                             }
                     }
                 };
-                int k = 0;
+                int k = k_first;
                 if (fresh) step(k++, true);
                 switch ((ksteps - k) % U) {
                     case 11: step(k++, false); [[fallthrough]];
@@ -328,77 +366,112 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_free[set])) : "memory");
             }
         GACONV_STAMP(4, threadIdx.x == 128);
-        // ------------------------------------------------------------------ block -> workspace, or dW
-        // Through shared memory, [column][128 lanes] (the stages are free: every copy has landed and every MMA has read).
-        // The workspace copy then is one bulk store per 16 columns; the only split of a tile writes dW itself, along the
-        // channels, or along the shifts of a channel (padding per column and per shift: lanes that read along the columns stay in
-        // different banks).
-        if (ok) {
-            const bool direct = P.splits == 1;
-            const int t = threadIdx.x - 128, ca_log = 31 - __clz(P.ca);
-            auto at = [&](int col) { return direct ? col * 129 + 11 * (col >> ca_log) : col * 128; };
+        // The only split of a tile, channels innermost in dW: from the registers, eight channels (a sector) a store.
+        const bool sectors = !CSIDE && P.splits == 1 && P.ws_c == 1 && (P.c & 7) == 0 && (reinterpret_cast<uintptr_t>(dw) & 31) == 0;
+        if (ok && sectors) {
+            float* d = dw + (k0 + l128) * P.ws_k;
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+                if (2 * i + half < blocks && k0 + l128 < P.k) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int2 o = s_col[16 * (2 * i + half) + 8 * h];
+                        const float* v = sum[i] + 8 * h;
+                        const float a = P.alpha;
+                        if (o.y > 0)
+                            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d + o.x), "f"(a * v[0]), "f"(a * v[1]),
+                                         "f"(a * v[2]), "f"(a * v[3]), "f"(a * v[4]), "f"(a * v[5]), "f"(a * v[6]), "f"(a * v[7]) : "memory");
+                    }
+                }
+        } else if (ok) {        // the block (the stages are free: every copy has landed and every MMA has read)
             float* blk = reinterpret_cast<float*>(smem_raw + (smem_base - smem_u32(smem_raw)));
+            const int ca_log = 31 - __clz(P.ca);
+            const bool keyed = P.splits == 1;
 #pragma unroll
             for (int i = 0; i < NB; ++i)
                 if (2 * i + half < blocks) {
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) blk[at(16 * (2 * i + half) + e) + l128] = sum[i][e];
+                    for (int e = 0; e < 16; ++e) {
+                        const int col = 16 * (2 * i + half) + e;
+                        if (keyed) blk[col * 128 + (l128 ^ block_key(col, ca_log))] = sum[i][e];
+                        else blk[col * 128 + l128] = sum[i][e];
+                    }
                 }
-            if (direct)
-                for (int col = t; col < P.cols; col += 256) {
-                    const int g = col / P.nmma, j = col - g * P.nmma;
-                    const ClGroup& G = P.g[g];
-                    const int a = CSIDE ? 0 : P.merged ? 0 : j / P.ca, c = c0 + G.cbase + (CSIDE ? 0 : P.merged ? j : j - a * P.ca);
-                    const int k = CSIDE ? k0 + j : 0;
-                    const bool valid = r0 + G.r < P.r && (CSIDE ? k < P.k : c < P.c && a < G.cnt);
-                    s_col[col] = make_int2((int)(k * P.ws_k + c * P.ws_c + (r0 + G.r) * P.ws_r + (G.s0 + P.stride * a) * P.ws_s), valid ? G.cnt : 0);
-                }
-            else asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            asm volatile("bar.sync 1, 256;" ::: "memory");
-            if (!direct) {
-                float* out = partial + ((size_t)tile * P.splits + split) * P.cols * 128;
+            if (P.splits > 1) {      // to the workspace, one bulk store per 16 columns
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                asm volatile("bar.sync 1, 256;" ::: "memory");
+                const int t = threadIdx.x - 128;
                 if (t < blocks) {
+                    float* out = partial + ((size_t)tile * P.splits + split) * P.cols * 128;
                     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(out + t * 2048), "r"(smem_base + t * 8192), "r"(8192) : "memory");
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-                }
-            } else if (CSIDE) {
-                const int a = l128 / P.ca, cc = P.merged ? l128 : l128 - a * P.ca;          // this lane's atom and channel
-                float* d = dw + (P.merged ? 0 : (long long)P.stride * a * P.ws_s) + cc * P.ws_c;
-                if (c0 + cc < P.c) {
-#pragma unroll 8
-                    for (int col = half; col < P.cols; col += 2) {
-                        const int2 o = s_col[col];
-                        if (P.merged ? o.y > 0 : a < o.y) d[o.x] = P.alpha * blk[at(col) + l128];
-                    }
-                }
-            } else {
-                int off[NB], pos[NB];       // this lane's columns, the same in every row; -1: none
-#pragma unroll
-                for (int u = 0; u < NB; ++u) {
-                    const int e = lane + 32 * u, col = e < P.cols ? written_column(P, e) : 0;
-                    const int2 o = e < P.cols ? s_col[col] : make_int2(0, 0);
-                    off[u] = o.y > 0 ? o.x : -1;
-                    pos[u] = at(col);
-                }
-#pragma unroll 2
-                for (int l = warp - 4; l < 128; l += 8) {
-                    if (k0 + l >= P.k) break;
-                    float* d = dw + (k0 + l) * P.ws_k;
-#pragma unroll
-                    for (int u = 0; u < NB; ++u)
-                        if (off[u] >= 0) d[off[u]] = P.alpha * blk[pos[u] + l];
                 }
             }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    GACONV_STAMP(5, threadIdx.x == 0);
+    GACONV_STAMP(7, threadIdx.x == 0);
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(P.tmem_cols) : "memory");
     }
+    // ---------------------------------------------------------------------- the only split of a tile: all warps, block -> dW
+    const bool sectors = !CSIDE && P.ws_c == 1 && (P.c & 7) == 0 && (reinterpret_cast<uintptr_t>(dw) & 31) == 0;        // (written already)
+    if (P.splits == 1 && !sectors && !s_abort) {
+        const float* blk = reinterpret_cast<const float*>(smem_raw + (smem_base - smem_u32(smem_raw)));
+        const int cols = P.cols;
+        const int ca_log = 31 - __clz(P.ca);
+        if (CSIDE) {
+            const int third = threadIdx.x >> 7;
+            int l = threadIdx.x & 127;
+            if (P.s_inner) l = ((l & ((1 << (7 - ca_log)) - 1)) << ca_log) + (l >> (7 - ca_log));
+            const int a = P.merged ? 0 : l >> ca_log, cc = P.merged ? l : l & (P.ca - 1);          // this lane's atom and channel
+            float* d = dw + P.stride * a * P.ws_s + cc * P.ws_c;
+            if (c0 + cc < P.c) {
+#pragma unroll 4
+                for (int col = third; col < cols; col += 3) {
+                    const int2 o = s_col[col];
+                    if (a < o.y) d[o.x] = P.alpha * blk[col * 128 + (l ^ block_key(col, ca_log))];
+                }
+            }
+        } else if (P.ws_c == 1 && (P.c & 3) == 0) {
+            // a warp takes four rows x 32 columns: four lines of 128 bytes a store
+            const int cgs = (cols + 31) >> 5, cq = (lane & 7) << 2;
+#pragma unroll 2
+            for (int t = warp; t < 32 * cgs; t += kThreads / 32) {
+                const int cg = t >> 5, l = ((t & 31) << 2) + (lane >> 3), col = (cg << 5) + cq;
+                if (col < cols && k0 + l < P.k) {
+                    const int2 o = s_col[col];
+                    float v[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) v[i] = P.alpha * blk[(col + i) * 128 + (l ^ block_key(col + i, ca_log))];
+                    if (o.y > 0) *reinterpret_cast<float4*>(dw + (k0 + l) * P.ws_k + o.x) = make_float4(v[0], v[1], v[2], v[3]);
+                }
+            }
+        } else {
+            for (int cb = 0; cb < cols; cb += 64) {        // two columns a lane
+                int off[2], pos[2], key[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int e = cb + lane + 32 * u, col = e < cols ? written_column(P, e) : 0;
+                    const int2 o = s_col[col];
+                    off[u] = e < cols && o.y > 0 ? o.x : -1;
+                    pos[u] = col * 128; key[u] = block_key(col, ca_log);
+                }
+#pragma unroll 4
+                for (int l = warp; l < 128; l += kThreads / 32) {
+                    if (k0 + l >= P.k) break;
+                    float* d = dw + (k0 + l) * P.ws_k;
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+                        if (off[u] >= 0) d[off[u]] = P.alpha * blk[pos[u] + (l ^ key[u])];
+                }
+            }
+        }
+    }
+    GACONV_STAMP(5, threadIdx.x == 0);
 }
 
 // Sum of the splits of every (tile, column), in a fixed order: grid (column blocks, tiles), 32 * CB * G threads.  Warp (g, c)
@@ -410,7 +483,7 @@ __global__ void __launch_bounds__(1024)
 cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, const __grid_constant__ ClParams P, int log_cb, int G)
 {
     __shared__ float s_sum[32][128];
-    __shared__ int2 s_col[16];               // column -> {offset in dW, atoms in use (0: not an element)}
+    __shared__ int2 s_col[16];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, CB = 1 << log_cb;
     const int tile = blockIdx.y, col0 = blockIdx.x << log_cb;
     pdl_release_next_grid();
@@ -418,21 +491,13 @@ cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, cons
     const int k0 = tk * P.kt, c0 = (tr - tk * P.tiles_c) * P.ct;
     const int ca_shift = 31 - __clz(P.ca), mn_mask = P.merged ? 127 : P.ca - 1;
     if ((int)threadIdx.x < CB) {
-        int col = col0 + threadIdx.x;
+        const int e = col0 + threadIdx.x;
         int2 o = make_int2(0, 0);
-        if (col < P.cols) {
-            if (!P.c_side) col = written_column(P, col);
-            const int gi = col / P.nmma, j = col - gi * P.nmma;
-            const ClGroup& g = P.g[gi];
-            const int a = P.c_side || P.merged ? 0 : j >> ca_shift, k = P.c_side ? k0 + j : 0;
-            const int c = c0 + g.cbase + (P.c_side ? 0 : P.merged ? j : j & mn_mask);
-            const bool valid = r0 + g.r < P.r && (P.c_side ? k < P.k : c < P.c && a < g.cnt);
-            o = make_int2((int)(k * P.ws_k + c * P.ws_c + (r0 + g.r) * P.ws_r + (g.s0 + P.stride * a) * P.ws_s), valid ? g.cnt : 0);
-        }
+        if (e < P.cols) o = column_target(P, written_column(P, e), k0, c0, r0);
         s_col[threadIdx.x] = o;
     }
     const int cb = warp & (CB - 1), grp = warp >> log_cb;
-    const int src_col = P.c_side || col0 + cb >= P.cols ? col0 + cb : written_column(P, col0 + cb);
+    const int src_col = col0 + cb < P.cols ? written_column(P, col0 + cb) : 0;
     const float4* src = reinterpret_cast<const float4*>(partial + ((size_t)tile * P.splits * P.cols + src_col) * 128) + lane;
     const size_t step = (size_t)P.cols * 32;
     __syncthreads();
@@ -478,6 +543,7 @@ struct PackOp {
     int channels_last;          // source order: 1 [n][px][ch], 0 [n][ch][px]
     int px_tiles, ch_tiles;     // tiles of an image (channels-first sources): kPackPx pixels x
     int ch_tile;                // at most 64 channels, a multiple of 8
+    int slab;                   // images per block, where an image's channels of a block are taken as one piece (0: by rows of pixels)
     int blocks;                 // tiles in all
     size_t plane;               // elements of a destination plane
 };
@@ -517,7 +583,7 @@ __global__ void __launch_bounds__(256)
 pack_kernel(const PackOp x, const PackOp dy)
 {
     constexpr int NP = sizeof(E) == 4 ? 3 : 1, TPX = kPackPx<E>, ROW = 2 * TPX;       // planes; bytes of a tile row
-    __shared__ __align__(128) unsigned char s_tile[NP][64 * ROW];
+    __shared__ __align__(128) unsigned char s_tile[NP][64 * ROW];       // (a slab: at most 64 x 64 elements and their padding)
     pdl_release_next_grid();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool is_x = (int)blockIdx.x < x.blocks;
@@ -550,6 +616,40 @@ pack_kernel(const PackOp x, const PackOp dy)
                 uint32_t w[4][3];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) split2(v[2 * j], v[2 * j + 1], w[j]);
+#pragma unroll
+                for (int pl = 0; pl < 3; ++pl) out[pl * (o.plane / 8)] = make_uint4(w[0][pl], w[1][pl], w[2][pl], w[3][pl]);
+            } else {
+                *out = *reinterpret_cast<const uint4*>(v);
+            }
+        }
+        return;
+    }
+    if (o.slab) {
+        // Maps under 64 pixels: 64 channels of an image are one piece of memory, read as such (rows of pixels would be short and
+        // mostly outside the tile) and picked apart on the way out; eight channels' pixels are followed by 16 bytes of padding.
+        constexpr int V = 16 / sizeof(E);
+        const int ng = blk / o.ch_tiles, c0 = (blk - ng * o.ch_tiles) * 64, n0 = ng * o.slab, imgs = min(o.slab, o.n - n0);
+        const int rows = min(64, o.ch - c0), vecs = rows * o.px / V, grp = 8 * o.px / V, img_vecs = 8 * (grp + 1);
+        float4* tile = reinterpret_cast<float4*>(s_tile);
+        pdl_wait_prior_grid();
+#pragma unroll 4
+        for (int e = threadIdx.x; e < imgs * vecs; e += 256) {
+            const int i = e / vecs, v = e - i * vecs;
+            tile[i * img_vecs + v + v / grp] = __ldg(reinterpret_cast<const float4*>(src + ((size_t)(n0 + i) * o.ch + c0) * o.px) + v);
+        }
+        __syncthreads();
+        const int q8 = min(8, (o.chp - c0) >> 3), items = imgs * o.px * q8;
+        for (int e = threadIdx.x; e < items; e += 256) {
+            const int ip = e / q8, q = e - ip * q8, i = ip / o.px, j = ip - i * o.px;
+            const E* p = reinterpret_cast<const E*>(tile + i * img_vecs + q * (grp + 1)) + j;
+            alignas(16) E v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = 8 * q + u < rows ? p[u * o.px] : E(0);
+            uint4* out = reinterpret_cast<uint4*>(o.dst + ((size_t)(n0 + i) * o.px + j) * o.chp + c0 + 8 * q);
+            if constexpr (sizeof(E) == 4) {
+                uint32_t w[4][3];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) split2(v[2 * u], v[2 * u + 1], w[u]);
 #pragma unroll
                 for (int pl = 0; pl < 3; ++pl) out[pl * (o.plane / 8)] = make_uint4(w[0][pl], w[1][pl], w[2][pl], w[3][pl]);
             } else {
@@ -649,48 +749,63 @@ int ceil_div(int a, int b) { return (a + b - 1) / b; }
 constexpr int kStageBudget = 216 * 1024;
 
 // What a candidate costs, in SM cycles, from rates measured with kernels of one kind each: an MMA of N columns takes N / 2
-// cycles; shared memory moves 128 bytes a cycle, the MMAs' operands, (128 + N) / 4 cycles, and what the copies write; copies
-// deliver ~80 bytes a cycle and one row (pixel) in no less than 1.4 cycles; a chunk costs its producer and its issuer ~940
-// cycles of instructions each (two of either work in turn); a CTA writes its block at ~21 bytes a cycle; start, first loads,
-// drain and the second kernel come to a few thousand.
+// cycles; shared memory moves 128 bytes a cycle (147 of a mix), the MMAs' operands, (128 + N) / 4 cycles, and what the copies write; copies
+// deliver ~80 bytes a cycle and one row (pixel) in no less than 1.4 cycles; a chunk costs its producer and its issuer ~1200
+// cycles of instructions each (two of either work in turn); a CTA writes its block at ~21 bytes a cycle to the workspace and at
+// ~18 to dW; start, first loads, drain and the second kernel come to a few thousand.
 struct Cost { double cycles; int splits; };
 Cost cost_of(const ClParams& P, int sms, double block_share)
 {
-    const double mma = (double)P.ksteps * P.ngroups * P.nprod * P.nmma / 2.0;
-    const double shared = (double)P.ksteps * P.ngroups * P.nprod * ((128 + P.nmma) / 4.0 + 2) + P.tx_bytes / 128.0;
+    double ksteps = P.ksteps;
+    if (P.skip) {       // the tile with the fewest rows left out decides
+        int most = 0;
+        for (int r = 0; r < P.r; ++r)
+            most = std::max(most, std::min(P.p, (P.h - 1 + P.pad_h - r) / P.stride + 1) - std::max(0, (P.pad_h - r + P.stride - 1) / P.stride));
+        ksteps = std::max(1, most) * P.skip;
+    }
+    const double mma = ksteps / P.ksteps * P.mma_cols * P.nprod / 2.0;
+    const double shared = ksteps / P.ksteps * P.nprod * (P.mma_cols / 4.0 + P.ksteps * P.ngroups * (128 / 4.0 + 2)) + P.tx_bytes / 128.0;
     const double rows = (double)P.planes * (P.katoms * (P.dy_box / (P.order == kPixels ? 128 : P.ka * 2)) + P.na * P.phases * P.row_tiles * (P.x_box / (P.ca * 2)));
     const double load = std::max(P.tx_bytes / 80.0, rows * 1.4);
-    const double chunk = std::max({mma * 1.03, shared, load, 470.0}) * (P.stages > 2 ? 1.0 : 1.2) + 40;
+    const double chunk = std::max({mma * 1.03, shared * 0.87, load, 600.0}) * (P.stages > 2 ? 1.0 : 1.2) + 40;
     const int tiles = P.tiles_k * P.tiles_c * P.tiles_r;
     const double block_bytes = (double)P.cols * 512 * block_share;
     Cost best{1e30, 1};
     const int most = std::max(1, std::min(P.chunks, sms / tiles));
     for (int sp = most; sp >= 1; sp = sp > 8 ? sp * 7 / 8 : sp - 1) {
         const int waves = ceil_div(tiles * sp, sms), per = ceil_div(P.chunks, sp);
-        const double main = waves * (4500 + load * std::min({per, P.stages, 4}) / 2 + per * chunk + block_bytes / 21);
+        const double main = waves * (4500 + load * std::min({per, P.stages, 4}) / 2 + per * chunk + block_bytes / (sp == 1 ? 18 : 21));
         const double red = sp == 1 ? 0.0 : 4000 + (double)tiles * sp * block_bytes / (25.0 * sms);
         if (main + red < best.cycles) best = Cost{main + red, sp};
     }
     return best;
 }
 
+// column shifts that one MMA covers (not merged)
+int shifts_of(const ClParams& P)
+{
+    const int most = P.c_side ? 128 / P.ca : 256 / P.ca, shifts = ceil_div(P.s, P.stride);
+    return P.c_side ? most : ceil_div(shifts, ceil_div(shifts, most));
+}
+// the last column shift that an MMA touches, in use or not
+int far_shift(const ClParams& P)
+{
+    const int shifts = ceil_div(P.s, P.stride), atoms = P.merged ? 1 : shifts_of(P);
+    return ceil_div(shifts, atoms) * atoms - 1;
+}
+
 bool build_groups(ClParams& P)
 {
     P.ngroups = 0;
     const int rows = P.rc, st = P.stride, wt = P.x_pitch;
-    // atoms of one MMA on the X side: c-side exactly fills M = 128; k-side as many as N = 256 takes
-    const int atoms_max = P.c_side ? 128 / P.ca : 256 / P.ca;
-    int atoms = 0;
+    // atoms of one MMA on the X side: c-side exactly fills M = 128; k-side as many as N = 256 takes, the shifts of a column phase
+    // shared out evenly over as few MMAs as hold them
+    const int atoms = P.merged ? P.na : shifts_of(P);
     auto add = [&](int tile_i, int row_px, int r, int s0, int cnt, int cbase) {
         if (P.ngroups == kMaxGroups) return false;
-        P.g[P.ngroups++] = ClGroup{(tile_i * P.x_alloc + row_px * P.ca * 2) >> 4, r, s0, cnt, cbase};
+        P.g[P.ngroups++] = ClGroup{(tile_i * P.x_alloc + row_px * P.px_rows * P.ca * 2) >> 4, r, s0, cnt, cbase};
         return true;
     };
-    if (P.merged) atoms = P.na;
-    else {      // the shifts of a column phase are shared out evenly over as few MMAs as hold them
-        const int shifts = ceil_div(P.s, st);
-        atoms = P.c_side ? atoms_max : ceil_div(shifts, ceil_div(shifts, atoms_max));
-    }
     for (int rl = 0; rl < rows; ++rl)
         for (int ph = 0; ph < P.phases; ++ph) {
             const int base_tile = st > 1 ? (rl * P.phases + ph) * P.na : 0, base_px = st > 1 ? 0 : rl * wt;
@@ -713,22 +828,25 @@ bool build_groups(ClParams& P)
     return true;
 }
 
-// Fills the chunk-dependent fields; false when the candidate does not fit.
-bool shape_chunk(ClParams& P, int ci, int bp, int order)
+// Fills the chunk-dependent fields; false when the candidate does not fit.  bare: kImages without halo columns.
+bool shape_chunk(ClParams& P, int ci, int bp, int order, bool bare = false)
 {
     const int st = P.stride;
-    const bool whole = ci > 1 || bp >= P.p;
+    const bool images = order == kImages, whole = images ? bp >= P.p : ci > 1 || bp >= P.p;
     if (order == kPaired) bp = round_up(bp, 2);
     if (order == kPixels && !whole && bp * P.q % 16 != 0) return false;         // k-steps do not cross chunks
     P.ci = ci; P.bp = bp; P.order = order;
     P.cpi = whole ? 0 : ceil_div(P.p, bp);
-    P.chunks = whole ? ceil_div(P.n, ci) : P.n * P.cpi;
-    const int wp = P.q + ceil_div(P.s, st) - 1, halo = st == 1 ? P.rc - 1 : 0;
+    P.mma_cols = 0;
+    P.chunks = whole ? ceil_div(P.n, ci) : ceil_div(P.n, ci) * P.cpi;
+    P.px_rows = images ? ci : 1;
+    P.skip = images && !bare && whole && P.rc == 1 && P.q * ci % 16 == 0 ? P.q * ci / 16 : 0;
+    const int wp = bare ? P.w : P.q + ceil_div(P.s, st) - 1, halo = st == 1 ? P.rc - 1 : 0;
     const int x_rows = bp + halo, dy_rows = (order == kFlat && ci > 1) ? bp + halo : bp, dy_w = order == kFlat ? wp : P.q;
     if ((wp - 1) * st + 1 > 256 || (x_rows - 1) * st + 1 > 256 || dy_rows > 256 || ci > 256) return false;
     P.x_pitch = wp; P.dy_pitch = dy_w; P.x_img = x_rows * wp; P.dy_img = dy_rows * dy_w;
     const int steps_img = order == kPaired ? (bp / 2) * (P.q / 8) : ceil_div(bp * P.q, 16);
-    P.ksteps = order == kFlat ? ceil_div(ci * dy_rows * dy_w, 16) : ci * steps_img;
+    P.ksteps = order == kFlat ? ceil_div(ci * dy_rows * dy_w, 16) : images ? ceil_div(bp * P.q * ci, 16) : ci * steps_img;
     if (P.ksteps > kMaxKsteps) return false;
     const int xb = P.ca * 2, db = P.ka * 2;
     P.x_box = ci * x_rows * wp * xb;
@@ -742,9 +860,11 @@ bool shape_chunk(ClParams& P, int ci, int bp, int order)
         P.dy_alloc = round_up(std::max(P.dy_box, order == kPaired ? 0 : P.ksteps * 16 * db), 1024);
     }
     // last X row an MMA touches: last k-step, last row and column shift, unused shifts of the c-side form
-    const int last = order == kFlat ? P.ksteps * 16 - 1 : (ci - 1) * P.x_img + (bp - 1) * wp + P.q - 1 + (order == kPixels ? 8 : 0);
-    const int far = last + halo * wp + ceil_div(P.s, st) - 1 + (P.c_side ? 128 / P.ca : 256 / P.ca);
-    P.x_alloc = round_up(std::max(P.x_box, (far + 1) * xb), 1024);
+    // (kImages: in whole pixels, one more where the last k-step is half a k-step)
+    const int last = order == kFlat ? P.ksteps * 16 - 1 : ((images ? 1 : ci) - 1) * P.x_img + (bp - 1) * wp + P.q - 1 + (order == kPixels ? 8 : 0) + (images && ci % 16 != 0 ? 1 : 0);
+    P.x_pre = bare ? round_up(std::max(P.pad_w, 1) * ci * xb, 1024) : 0;
+    const int far = last + halo * wp + (images ? far_shift(P) : ceil_div(P.s, st) - 1 + (P.c_side ? 128 / P.ca : 256 / P.ca));
+    P.x_alloc = P.x_pre + round_up(bare ? P.x_box : std::max(P.x_box, (far + 1) * P.px_rows * xb), 1024);
     const int x_tiles = P.na * P.phases * P.row_tiles;
     P.x_plane = x_tiles * P.x_alloc;
     P.dy_plane = P.katoms * P.dy_alloc;
@@ -759,25 +879,44 @@ bool shape_chunk(ClParams& P, int ci, int bp, int order)
     const uint32_t x_swz = P.ca == 64 ? 2 : P.ca == 32 ? 4 : 6, dy_swz = order == kPixels || P.ka == 64 ? 2 : P.ka == 32 ? 4 : 6;
     const uint32_t dy_sbo = order == kPixels ? 8 * 128 : order == kPaired ? dy_w * db : 8 * db;
     P.dy_hi = (dy_sbo >> 4) | (1u << 14) | (dy_swz << 29);
-    P.x_lbo = (uint32_t)((P.merged ? P.x_alloc : xb) >> 4) << 16;
+    P.x_lbo = (uint32_t)((P.merged ? P.x_alloc : P.px_rows * xb) >> 4) << 16;
     // (one atom: the upper half of M repeats the lower)
     P.dy_lbo = order == kPixels ? 1u << 16 : (uint32_t)((P.katoms > 1 ? P.dy_alloc : 0) >> 4) << 16;
     for (int i = 0; i < P.ksteps; ++i) {
+        int s_lo = 0, s_hi = 0;                                        // bare: column shifts of the k-step
         int x_row = 16 * i, dy_off = 16 * i * db, x_sbo = 8;          // X row, dY bytes, X rows between the two 8-pixel groups
         if (order == kPaired) {
             const int j = i % (P.q / 8), t = i / (P.q / 8), pr = t % (bp / 2), im = t / (bp / 2);
             x_row = im * P.x_img + 2 * pr * wp + 8 * j;
             dy_off = (im * P.dy_img + 2 * pr * dy_w + 8 * j) * db;
             x_sbo = wp;
+        } else if (images) {
+            const int px = 16 * i / ci, p = px / P.q, q = px % P.q;
+            x_row = (p * wp + q) * ci + 16 * i % ci;
+            if (bare) {
+                // the shifts whose column lies in the map; pixel 0 takes all of them, those to the left from the zeros before the
+                // tile, so that the MMA that starts an accumulator writes every column of it
+                if (px > 0) { s_lo = std::max(0, P.pad_w - q); s_hi = std::min(P.s, P.w + P.pad_w - q); }
+                x_row += (s_lo - P.pad_w) * ci + P.x_pre / xb;
+            }
+            if (ci == 8 && q + 1 == P.q && px + 1 < bp * P.q) x_sbo = 8 * (wp - P.q + 1);       // the second pixel starts the next row
         } else if (order == kPixels) {
             const int im = i / steps_img, j = 16 * (i % steps_img), p = j / P.q, q = j % P.q;
             x_row = im * P.x_img + p * wp + q;
             dy_off = (im * P.dy_subs + j / 64) * P.dy_alloc + (j % 64) * 2;
             x_sbo = q + 8 < P.q ? 8 : wp - P.q + 8;
         }
-        P.k_off[i] = make_uint4((unsigned)(x_row * xb) >> 4, (unsigned)dy_off >> 4, (unsigned)(x_sbo * xb) >> 4 | (1u << 14) | (x_swz << 29), 0u);
+        P.k_off[i] = make_uint4((unsigned)(x_row * xb) >> 4, (unsigned)dy_off >> 4, (unsigned)(x_sbo * xb) >> 4 | (1u << 14) | (x_swz << 29),
+                                (unsigned)(s_lo * P.ca) | (unsigned)((bare ? (s_hi - s_lo) * P.ca : 0) >> 3) << 17);
     }
-    return build_groups(P);
+    if (!build_groups(P)) return false;
+    if (!P.c_side && P.ngroups == 1)
+        for (int i = 0; i < P.ksteps; ++i) {
+            if (!bare || P.k_off[i].w >> 17 == 0) P.k_off[i].w = (unsigned)(P.nmma >> 3) << 17;
+            P.mma_cols += (P.k_off[i].w >> 17) * 8;
+        }
+    else P.mma_cols = P.ksteps * P.ngroups * P.nmma;
+    return true;
 }
 
 struct ClHost {             // what ClPlan::opaque holds
@@ -796,6 +935,14 @@ PackOp pack_op(const void* src, void* dst, int ch, int px, int n, bool last, siz
     o.px_tiles = ceil_div(px, tile_px); o.ch_tiles = ceil_div(ch, 64);
     o.ch_tile = round_up(ceil_div(ch, o.ch_tiles), 8);
     o.ch_tiles = ceil_div(ch, o.ch_tile);
+    // a slab: 16-byte pieces, up to 64 pixels of 64 channels; images enough for every thread to have work, blocks enough for every SM
+    const int vec = tile_px == kPackPx<float> ? 4 : 8;
+    if (!last && px < 64 && (long long)ch * px % vec == 0) {
+        o.ch_tile = 64; o.ch_tiles = ceil_div(ch, 64);
+        o.slab = std::max(1, std::min(64 / px, n * o.ch_tiles / 296));
+        o.blocks = ceil_div(n, o.slab) * o.ch_tiles;
+        return o;
+    }
     o.blocks = last ? (int)(((size_t)n * px * (o.chp / 8) + 1023) / 1024) : n * o.px_tiles * o.ch_tiles;
     return o;
 }
@@ -861,18 +1008,21 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
                     if (F.stride == 1) F.phases = 1;
                     // part of the accumulator block that stands for elements of dW
                     const double share = (double)g.k * g.c * g.r * g.s / ((double)F.tiles_k * F.tiles_c * F.tiles_r * 128);
-                    for (int mode = kFlat; mode <= kPixels; ++mode) {
-                        if (mode != kFlat && g.q % 8 != 0) break;
-                        if (mode == kPixels && (H.f32 || H.dy_npqk)) break;
-                        auto consider = [&](int ci, int bp) {
+                    for (int mode = kFlat; mode <= kImages; ++mode) {
+                        if ((mode == kPaired || mode == kPixels) && g.q % 8 != 0) continue;
+                        // (small maps: one order for every layout of dY, so that its results do not depend on it either)
+                        if (mode == kPixels && (H.f32 || H.dy_npqk || g.p * g.q < 64)) continue;
+                        if (mode == kImages && g.n < 5) continue;
+                        auto consider = [&](int ci, int bp, bool bare) {
                             ClParams C = F;
-                            if (!shape_chunk(C, ci, bp, mode)) return mode == kPixels && bp * C.q % 16 != 0;
+                            if (!shape_chunk(C, ci, bp, mode, bare)) return mode == kPixels && bp * C.q % 16 != 0;
 #ifdef GACONV_TUNING
                             if (const char* e = getenv("GACONV_CL_KS")) if (C.ksteps < atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_KSMAX")) if (C.ksteps > atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_FORM")) if (C.c_side != atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_RC")) if (C.rc != atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_KT")) if (C.kt != atoi(e)) return true;
+                            if (const char* e = getenv("GACONV_CL_BARE")) if ((C.x_pre > 0) != (atoi(e) != 0)) return true;
                             if (const char* e = getenv("GACONV_CL_NA")) if (C.na != atoi(e)) return true;
 #endif
                             Cost c = cost_of(C, sms, std::min(1.0, 1.3 * share / C.cols));
@@ -881,16 +1031,38 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
                             if (c.cycles < best_cycles) { best_cycles = c.cycles; C.splits = c.splits; best = C; }
                             return true;
                         };
+                        if (mode == kImages) {
+                            for (int ci = 8; ci <= 64 && ci < 2 * g.n; ci *= 2) {
+                                int last_bp = 0;
+                                for (int parts = g.p; parts >= 1; --parts) {
+                                    const int bp = ceil_div(g.p, parts);
+                                    if (bp == last_bp) continue;
+                                    last_bp = bp;
+                                    if (!consider(ci, bp, false)) break;
+                                }
+                                // no halo columns: one MMA a k-step, of shifts alone, and a first pixel with every shift inside or to the left
+                                if (form == 0 && ci >= 16 && na == 1 && rc == 1 && F.stride == 1 && g.s > 1 && g.s * F.ca <= kMaxCols && g.w >= g.s - g.pad_w && g.pad_w < g.w) {
+                                    last_bp = 0;
+                                    for (int parts = g.p; parts >= 1; --parts) {
+                                        const int bp = ceil_div(g.p, parts);
+                                        if (bp == last_bp) continue;
+                                        last_bp = bp;
+                                        if (!consider(ci, bp, true)) break;
+                                    }
+                                }
+                            }
+                            continue;
+                        }
                         int last_bp = 0;
                         for (int parts = g.p; parts >= 1; --parts) {      // fewer and fewer, larger and larger bands
                             int bp = ceil_div(g.p, parts);
                             if (mode == kPaired) bp = round_up(bp, 2);
                             if (bp == last_bp) continue;
                             last_bp = bp;
-                            if (!consider(1, bp)) break;
+                            if (!consider(1, bp, false)) break;
                         }
                         for (int ci = 2; ci <= 64 && ci <= g.n; ci = ci < 4 ? ci + 1 : ci + ci / 2)
-                            if (!consider(ci, g.p)) break;
+                            if (!consider(ci, g.p, false)) break;
                     }
                 }
             }
@@ -900,7 +1072,7 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
     best.chunk_base = best.chunks / best.splits;
     best.chunk_rem = best.chunks - best.chunk_base * best.splits;
     // fp32 accumulators, bf16 operands, both MN-major (dY K-major where it is read as it lies), N, M = 128
-    best.idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(best.nmma >> 3) << 17) | (8u << 24);
+    best.idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | (best.c_side || best.ngroups > 1 ? (uint32_t)(best.nmma >> 3) << 17 : 0u) | (8u << 24);
     if (best.order == kPixels) { best.idesc &= ~(best.c_side ? 1u << 16 : 1u << 15); H.pack_dy = false; }
     H.p = best;
     // second kernel: at most eight loads a thread, a block of at most 32 warps, and as many blocks as there are SMs where the
@@ -940,13 +1112,16 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
         if (H.pack_x) x = x_scratch;
         if (H.pack_dy) dy = dy_scratch;
     }
-    // tensor maps over (channel, column, row, image, plane); box extents count the pixels stepped over at the conv stride
+    // tensor maps over (channel, column, row, image, plane), the rows of a box in the order of the reduction; box extents count the pixels stepped over at the conv stride
     auto encode = [&](CUtensorMap* map, const void* base, int ch, int chp, int w, int h, size_t plane_el, int atom, int bw, int bh, int st) {
         const cuuint64_t row = (cuuint64_t)chp * 2;
         cuuint64_t dims[5] = {(cuuint64_t)ch, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)P.n, (cuuint64_t)P.planes};
         cuuint64_t strides[4] = {row, row * w, row * w * h, (cuuint64_t)plane_el * 2};
         cuuint32_t box[5] = {(cuuint32_t)atom, (cuuint32_t)((bw - 1) * st + 1), (cuuint32_t)((bh - 1) * st + 1), (cuuint32_t)P.ci, 1};
         cuuint32_t es[5] = {1, (cuuint32_t)st, (cuuint32_t)st, 1, 1};
+        if (P.order == kImages) {        // (channel, image, column, row, plane)
+            for (int i : {2, 1}) { std::swap(dims[i], dims[i + 1]); std::swap(strides[i - 1], strides[i]); std::swap(box[i], box[i + 1]); std::swap(es[i], es[i + 1]); }
+        }
         const CUtensorMapSwizzle swz = atom == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : atom == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
         return encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                            swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -963,7 +1138,7 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
         !encode(&map_x, x, P.c, H.xch, P.w, P.h, x_el, P.ca, P.x_pitch, P.x_img / P.x_pitch, P.stride))
         return cudaErrorInvalidValue;
     // the stages; at the end they hold the accumulator block
-    const size_t smem = std::max((size_t)P.stages * P.stage_bytes, (size_t)(P.cols * 129 + 12 * 11) * 4) + 1024;
+    const size_t smem = std::max((size_t)P.stages * P.stage_bytes, (size_t)P.cols * 512) + 1024;
     const dim3 grid((unsigned)(P.tiles_k * P.tiles_c * P.tiles_r), (unsigned)P.splits);
     ClKernel kern = kernel_for(P.ngroups, H.f32, P.c_side != 0);
     if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return err;
