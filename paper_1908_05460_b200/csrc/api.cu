@@ -115,21 +115,25 @@ bool top1_dense_route(const Geom& g, TcPlan* tp)
     return g.bf16 && ((g.p * g.q <= 16 && g.c >= 128) || (g.p * g.q <= 64 && g.c >= 256)) && plan_tc(g, tp);
 }
 
-struct Top1Layout { size_t idx_off, sum_off, partial_off, sparse_off, scratch_off, total; GatherPlan gp; TcPlan tp; bool dense; };
+struct Top1Layout { size_t idx_off, sum_off, partial_off, sparse_off, scratch_off, total; GatherPlan gp; TcPlan tp; ClPlan cp; bool dense, cl; };
 Top1Layout build_top1_layout(const Geom& g)
 {
     Top1Layout L;
     L.gp = plan_gather(g);
     L.dense = top1_dense_route(g, &L.tp);
+    // the contraction: by the channels-last kernel, which reads either form of the sparse tensor (256->256 on 8x8, N = 256:
+    // 37 us with the other kernel, 32)
+    L.cl = L.dense && tensor_maps_available() && plan_cl(g, L.tp.reads_transposed_dy, &L.cp);
+    const size_t cl_scratch = L.cl ? L.cp.x_bytes + L.cp.dy_bytes : 0;
     const size_t maps = (size_t)g.n * g.k;
     L.idx_off = kWsDataOffset;
     L.sum_off = align_up(L.idx_off + maps * sizeof(int32_t), 256);
     L.partial_off = align_up(L.sum_off + maps * sizeof(float), 256);
     size_t partial = L.gp.partial_bytes;
-    if (L.dense && L.tp.partial_bytes > partial) partial = L.tp.partial_bytes;
+    if (L.dense) partial = std::max(partial, L.cl ? L.cp.partial_bytes : L.tp.partial_bytes);
     L.sparse_off = align_up(L.partial_off + partial, 256);
     L.scratch_off = align_up(L.sparse_off + (L.dense ? maps * g.p * g.q * 2 : 0), 256);
-    L.total = align_up(L.scratch_off + (L.dense ? L.tp.scratch_bytes : 0), 256);
+    L.total = align_up(L.scratch_off + (L.dense ? L.tp.scratch_bytes + cl_scratch : 0), 256);
     return L;
 }
 
@@ -579,6 +583,11 @@ gaconv_status_t gaconv_dw_approx(int32_t method, const void* x, const void* dy, 
             if (launch_select_sparse_transposed(dy, ws + L.scratch_off, g, cs) != cudaSuccess) return GACONV_ERR_CUDA;
             sparse = nullptr;
         } else if (launch_select(dy, idx, sum, sparse, g, cs) != cudaSuccess) return GACONV_ERR_CUDA;
+        if (L.cl) {
+            char* packed = ws + L.scratch_off + L.tp.scratch_bytes;
+            return launch_cl(x, sparse != nullptr ? sparse : ws + L.scratch_off, dw, reinterpret_cast<float*>(ws + L.partial_off), packed,
+                             packed + L.cp.x_bytes, reinterpret_cast<uint32_t*>(ws), L.cp, cs) == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
+        }
         return launch_tc(x, sparse, dw, reinterpret_cast<float*>(ws + L.partial_off), ws + L.scratch_off,
                          reinterpret_cast<uint32_t*>(ws + kWsCounterOffset), reinterpret_cast<uint32_t*>(ws), L.tp,
                          cs) == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
