@@ -197,6 +197,9 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, bool reordered)
         if (L.stem_ok) return reordered || (!shared && g.r * g.s * g.c > 32);       // 5x5 3->64 26.4 / 22.6, 3x3 3->16 10.4 / 14.8
     } else {
         if (L.stem_ok) return false;                                // 3->64 on 32x32 28 / 53
+        // (the tensor core truncates as it adds, 1e-8 for each MMA of the other kernel's CTA: where that has more than 1,500 of them
+        // its results are over 1.4e-5 away from this one's, and stay what they have been)
+        if (L.tc_ok && L.tp.chain > 1500) return false;
         if (L.tc_ok)                                                // 128->128 on 16x16 92 / 53, 64->64 on 8x8 17.1 / 18.1, on 18 SMs 44 / 40
             return reordered || (g.c >= 128 ? products > 4e8 : g.c >= 64 && (shared || products > 3e9));
         if (direct_mma_supported(g, L.dp))                          // 16->16 on 32x32 19 / 40, 48->96 on 16x16 (N = 64) 31 / 23

@@ -1031,6 +1031,7 @@ bool plan_tc_f32(const Geom& g, int passes, TcPlan* out)
     // the two planes of each operand, [plane][elements]
     out->scratch_bytes = passes == 3 ? 2 * ((size_t)g.n * g.c * g.h * g.w + (size_t)g.n * g.k * pq) * 4 : 0;
     out->reads_transposed_dy = false;
+    out->chain = (int)((long long)P.chunks * P.ksteps * passes / P.splits);
     out->stacked_rows = P.stack != 0;
     memcpy(out->opaque, &P, sizeof(P));
     return encode_fn() != nullptr;
