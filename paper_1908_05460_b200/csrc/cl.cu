@@ -541,8 +541,10 @@ struct PackOp {
     __nv_bfloat16* dst;
     int ch, chp, px, n;         // source: n images of px pixels and ch channels; destination rows of chp channels
     int channels_last;          // source order: 1 [n][px][ch], 0 [n][ch][px]
-    int px_tiles, ch_tiles;     // tiles of an image (channels-first sources): kPackPx pixels x
+    int px_tiles, ch_tiles;     // tiles of an image (channels-first sources): tile_px pixels x
     int ch_tile;                // at most 64 channels, a multiple of 8
+    int tile_px;                // pixels of a tile
+    int gather;                 // rows of pixels that do not lie on 16-byte boundaries, or few channels
     int slab;                   // images per block, where an image's channels of a block are taken as one piece (0: by rows of pixels)
     int blocks;                 // tiles in all
     size_t plane;               // elements of a destination plane
@@ -561,29 +563,42 @@ __device__ __forceinline__ void split2(float u, float v, uint32_t (&w)[3]) {
     w[1] = bf16_pair(ru, rv);
     w[2] = bf16_pair(ru - __uint_as_float(w[1] << 16), rv - __uint_as_float(w[1] & 0xffff0000u));
 }
-// copies `bytes` (4, 8 or 16) to shared memory without a stop in registers; zeros instead when !in
-template <int BYTES>
-__device__ __forceinline__ void copy_async(uint32_t dst, const void* src, bool in) {
-    const int n = in ? BYTES : 0;
-    if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
-    else asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(BYTES), "r"(n) : "memory");
+// copies the first n <= 16 bytes of a 16-byte piece to shared memory without a stop in registers; zeros behind them
+__device__ __forceinline__ void copy_async(uint32_t dst, const void* src, int n) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
 }
 
 // Blocks [0, x.blocks) pack X, the others dY.  E: the element as a plain number of its size (float, or the 16 bits of a
 // bf16).  A block turns a tile of 64 channels x 128 pixels (64 of fp32, whose three planes take the room) of a channels-first source: rows of pixels arrive in shared memory
-// (asynchronous copies where rows start on 4-byte boundaries), ldmatrix.trans turns 8 x 8 blocks on the way out, and with its
+// by asynchronous copies, ldmatrix.trans turns 8 x 8 blocks on the way out, and with its
 // row addresses ordered (0 1 8 9 16 17 24 25), (2 3 10 11 ...) ... a lane receives eight consecutive channels of a pixel, one
 // 16-byte store.  (Turning by single elements in registers was bound by instructions: 22 us on 13 MB of gradients and 8 MB of
 // activations.)  The 16-byte chunks of a row are permuted by the same order, so that the eight rows of a block sit in
 // different banks.
 template <typename E> constexpr int kPackPx = sizeof(E) == 4 ? 64 : 128;
 
+// eight channels of a pixel -> 16 bytes of every plane
+template <typename E>
+__device__ __forceinline__ void store8(const E (&v)[8], __nv_bfloat16* dst, size_t plane) {
+    uint4* out = reinterpret_cast<uint4*>(dst);
+    if constexpr (sizeof(E) == 4) {
+        uint32_t w[4][3];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) split2(v[2 * j], v[2 * j + 1], w[j]);
+#pragma unroll
+        for (int pl = 0; pl < 3; ++pl) out[pl * (plane / 8)] = make_uint4(w[0][pl], w[1][pl], w[2][pl], w[3][pl]);
+    } else {
+        *out = make_uint4(v[0] | (uint32_t)v[1] << 16, v[2] | (uint32_t)v[3] << 16, v[4] | (uint32_t)v[5] << 16, v[6] | (uint32_t)v[7] << 16);
+    }
+}
+
 template <typename E>
 __global__ void __launch_bounds__(256)
 pack_kernel(const PackOp x, const PackOp dy)
 {
     constexpr int NP = sizeof(E) == 4 ? 3 : 1, TPX = kPackPx<E>, ROW = 2 * TPX;       // planes; bytes of a tile row
-    __shared__ __align__(128) unsigned char s_tile[NP][64 * ROW];       // (a slab: at most 64 x 64 elements and their padding)
+    constexpr int kTile = 64 * ROW, kBytes = NP * kTile > 17664 ? NP * kTile : 17664;         // (slabs and gathered rows: at most 17,664)
+    __shared__ __align__(128) unsigned char s_tile[kBytes];
     pdl_release_next_grid();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool is_x = (int)blockIdx.x < x.blocks;
@@ -592,16 +607,16 @@ pack_kernel(const PackOp x, const PackOp dy)
     const E* src = static_cast<const E*>(o.src);
     if (o.channels_last) {
         const int g8 = o.chp >> 3;
-        const size_t items = (size_t)o.n * o.px * g8;
+        const unsigned items = (unsigned)o.n * o.px * g8;            // (an operand has at most 2^31 elements)
         const bool vec = (o.ch & 7) == 0;
         pdl_wait_prior_grid();
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const size_t it = (size_t)blk * 1024 + i * 256 + threadIdx.x;
+            const unsigned it = blk * 1024u + i * 256 + threadIdx.x;
             if (it >= items) return;
-            const size_t row = it / g8;
+            const unsigned row = it / (unsigned)g8;
             const int c = (int)(it - row * g8) * 8;
-            const E* p = src + row * o.ch + c;
+            const E* p = src + (size_t)row * o.ch + c;
             alignas(16) E v[8];
             if (vec) {
                 const uint4* q = reinterpret_cast<const uint4*>(p);
@@ -611,16 +626,7 @@ pack_kernel(const PackOp x, const PackOp dy)
 #pragma unroll
                 for (int j = 0; j < 8; ++j) v[j] = c + j < o.ch ? __ldg(p + j) : E(0);
             }
-            uint4* out = reinterpret_cast<uint4*>(o.dst + row * o.chp + c);
-            if constexpr (sizeof(E) == 4) {
-                uint32_t w[4][3];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) split2(v[2 * j], v[2 * j + 1], w[j]);
-#pragma unroll
-                for (int pl = 0; pl < 3; ++pl) out[pl * (o.plane / 8)] = make_uint4(w[0][pl], w[1][pl], w[2][pl], w[3][pl]);
-            } else {
-                *out = *reinterpret_cast<const uint4*>(v);
-            }
+            store8(v, o.dst + (size_t)row * o.chp + c, o.plane);
         }
         return;
     }
@@ -645,83 +651,85 @@ pack_kernel(const PackOp x, const PackOp dy)
             alignas(16) E v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) v[u] = 8 * q + u < rows ? p[u * o.px] : E(0);
-            uint4* out = reinterpret_cast<uint4*>(o.dst + ((size_t)(n0 + i) * o.px + j) * o.chp + c0 + 8 * q);
-            if constexpr (sizeof(E) == 4) {
-                uint32_t w[4][3];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) split2(v[2 * u], v[2 * u + 1], w[u]);
-#pragma unroll
-                for (int pl = 0; pl < 3; ++pl) out[pl * (o.plane / 8)] = make_uint4(w[0][pl], w[1][pl], w[2][pl], w[3][pl]);
-            } else {
-                *out = *reinterpret_cast<const uint4*>(v);
-            }
+            store8(v, o.dst + ((size_t)(n0 + i) * o.px + j) * o.chp + c0 + 8 * q, o.plane);
         }
         return;
     }
     const int per_img = o.px_tiles * o.ch_tiles, n = blk / per_img, rest = blk - n * per_img, ct = rest / o.px_tiles, c0 = ct * o.ch_tile;
-    const int p0 = (rest - ct * o.px_tiles) * TPX, rows = min(o.ch_tile, o.ch - c0), left = min(TPX, o.px - p0);
+    const int p0 = (rest - ct * o.px_tiles) * o.tile_px, rows = min(o.ch_tile, o.ch - c0), left = min(o.tile_px, o.px - p0);
     const E* base = src + ((size_t)n * o.ch + c0) * o.px + p0;
     const uint32_t tile = smem_u32(s_tile);
+    if (o.gather) {
+        // The 16-byte pieces that hold a row, each row with its own offset from the boundary; eight elements per store are then
+        // picked from eight rows (16 bytes between groups of eight rows keep their banks apart).  (30 MB of 23x23 maps: copied by
+        // words into the order that ldmatrix wants 39 us, this way 18; bound by the instructions that pick.)
+        const int pitch = o.tile_px * (int)sizeof(E) + 16, row_bytes = o.px * (int)sizeof(E), bytes = left * (int)sizeof(E);
+        const char* first = reinterpret_cast<const char*>(base);
+        const char* end = reinterpret_cast<const char*>(src + (size_t)o.n * o.ch * o.px);
+        const int first_off = (int)(reinterpret_cast<uintptr_t>(base) & 15);
+        pdl_wait_prior_grid();
+#pragma unroll 4
+        for (int row = warp; row < rows; row += 8) {
+            const int off = (first_off + row * row_bytes) & 15;
+            const char* piece = first + (size_t)row * row_bytes - off;
+            const uint32_t dst = tile + row * pitch + (row >> 3) * 16;
+            for (int k = 16 * lane; k < bytes + off; k += 512) copy_async(dst + k, piece + k, (int)min((ptrdiff_t)16, end - (piece + k)));
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        // a thread keeps its eight rows and walks over pixels
+        const int q8 = min(o.ch_tile, o.chp - c0) >> 3, log_q = 32 - __clz(q8 - 1), q = threadIdx.x & ((1 << log_q) - 1), r8 = 8 * q;
+        if (q >= q8) return;
+        const unsigned char* at[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) at[u] = s_tile + (r8 + u) * pitch + q * 16 + ((first_off + (r8 + u) * row_bytes) & 15);
+        const int valid = rows - r8;
+        __nv_bfloat16* d = o.dst + ((size_t)n * o.px + p0) * o.chp + c0 + r8;
+#pragma unroll 2
+        for (int j = threadIdx.x >> log_q; j < left; j += 256 >> log_q) {
+            alignas(16) E v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = *reinterpret_cast<const E*>(at[u] + j * sizeof(E));
+            if (valid < 8) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) if (u >= valid) v[u] = E(0);
+            }
+            store8(v, d + (size_t)j * o.chp, o.plane);
+        }
+        return;
+    }
     auto at = [&](int row, int px) {          // byte offset of a pixel in its (permuted) row
         const int sw = (((row >> 3) & 3) << 1) | (row & 1);
         return row * ROW + ((((px >> 3) ^ sw) << 4) | ((px & 7) << 1));
     };
     pdl_wait_prior_grid();
     if constexpr (sizeof(E) == 2) {
-        if ((o.px & 1) == 0) {
-            auto fill = [&](auto width) {
-                constexpr int V = decltype(width)::value;
+        if ((o.px & 7) == 0) {
 #pragma unroll
-                for (int i = 0; i < 32 / V; ++i) {
-                    const int e = (i * 256 + (int)threadIdx.x) * V, row = e >> 7, px = e & 127;
-                    const bool in = row < rows && px < left;
-                    copy_async<2 * V>(tile + at(row, px), in ? base + (size_t)row * o.px + px : src, in);
-                }
-            };
-            if ((o.px & 7) == 0) fill(std::integral_constant<int, 8>());
-            else if ((o.px & 3) == 0) fill(std::integral_constant<int, 4>());
-            else fill(std::integral_constant<int, 2>());
-            asm volatile("cp.async.wait_all;" ::: "memory");
+            for (int i = 0; i < 4; ++i) {
+                const int e = (i * 256 + (int)threadIdx.x) * 8, row = e >> 7, px = e & 127;
+                const bool in = row < rows && px < left;
+                copy_async(tile + at(row, px), in ? base + (size_t)row * o.px + px : src, in ? 16 : 0);
+            }
         } else {
-            // rows of odd length: 32-bit loads from the word that holds the row's first pixel; a row that starts in the middle
-            // of a word takes each pair of pixels from two neighbouring words
-#pragma unroll 4
-            for (int i = 0; i < 16; ++i) {
-                const int row = warp + 8 * (i >> 1), l = lane + 32 * (i & 1);
-                const E* q = base + (size_t)row * o.px;
-                const uint32_t* w = reinterpret_cast<const uint32_t*>(reinterpret_cast<uintptr_t>(q) & ~(uintptr_t)3);
-                const int odd = (int)((reinterpret_cast<uintptr_t>(q) >> 1) & 1);
-                auto word = [&](int k) -> uint32_t {             // (a word is read whole only if both halves lie in the row)
-                    const int first = 2 * k - odd;
-                    if (row >= rows || first >= left) return 0u;
-                    if (first + 1 < left && first >= 0) return __ldg(w + k);
-                    const unsigned short* h = reinterpret_cast<const unsigned short*>(w + k);
-                    return first < 0 ? (uint32_t)__ldg(h + 1) << 16 : (uint32_t)__ldg(h);
-                };
-                const uint32_t w0 = word(l), w1 = odd ? word(l + 1) : 0u;
-                *reinterpret_cast<uint32_t*>(&s_tile[0][at(row, 2 * l)]) = odd ? __funnelshift_r(w0, w1, 16) : w0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int e = (i * 256 + (int)threadIdx.x) * 4, row = e >> 7, px = e & 127;
+                const bool in = row < rows && px < left;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(tile + at(row, px)), "l"(in ? base + (size_t)row * o.px + px : src), "r"(in ? 8 : 0) : "memory");
             }
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
     } else {
-        const bool vec = (o.px & 3) == 0;
 #pragma unroll 4
         for (int i = 0; i < TPX / 16; ++i) {
             const int e = (i * 256 + (int)threadIdx.x) * 4, row = e / TPX, px = e % TPX;
-            const E* q = base + (size_t)row * o.px + px;
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (row < rows) {
-                if (vec) { if (px < left) v = __ldg(reinterpret_cast<const float4*>(q)); }
-                else {
-                    if (px < left) v.x = __ldg(q);
-                    if (px + 1 < left) v.y = __ldg(q + 1);
-                    if (px + 2 < left) v.z = __ldg(q + 2);
-                    if (px + 3 < left) v.w = __ldg(q + 3);
-                }
-            }
+            if (row < rows && px < left) v = __ldg(reinterpret_cast<const float4*>(base + (size_t)row * o.px + px));
             uint32_t w0[3], w1[3];
             split2(v.x, v.y, w0); split2(v.z, v.w, w1);
 #pragma unroll
-            for (int pl = 0; pl < NP; ++pl) *reinterpret_cast<uint2*>(&s_tile[pl][at(row, px)]) = make_uint2(w0[pl], w1[pl]);
+            for (int pl = 0; pl < NP; ++pl) *reinterpret_cast<uint2*>(&s_tile[pl * kTile + at(row, px)]) = make_uint2(w0[pl], w1[pl]);
         }
     }
     __syncthreads();
@@ -932,11 +940,16 @@ PackOp pack_op(const void* src, void* dst, int ch, int px, int n, bool last, siz
     PackOp o{};
     o.src = src; o.dst = static_cast<__nv_bfloat16*>(dst);
     o.ch = ch; o.chp = round_up(ch, 8); o.px = px; o.n = n; o.channels_last = last ? 1 : 0; o.plane = plane;
-    o.px_tiles = ceil_div(px, tile_px); o.ch_tiles = ceil_div(ch, 64);
+    const int vec = tile_px == kPackPx<float> ? 4 : 8;
+    o.ch_tiles = ceil_div(ch, 64);
     o.ch_tile = round_up(ceil_div(ch, o.ch_tiles), 8);
     o.ch_tiles = ceil_div(ch, o.ch_tile);
+    o.gather = px % 4 != 0 || ch <= 16;
+    o.tile_px = tile_px;
+    if (o.gather)                      // (few channels: more pixels, the same number of bytes)
+        for (int c = o.ch_tile; c <= 32; c *= 2) o.tile_px *= 2;
+    o.px_tiles = ceil_div(px, o.tile_px);
     // a slab: 16-byte pieces, up to 64 pixels of 64 channels; images enough for every thread to have work, blocks enough for every SM
-    const int vec = tile_px == kPackPx<float> ? 4 : 8;
     if (!last && px < 64 && (long long)ch * px % vec == 0) {
         o.ch_tile = 64; o.ch_tiles = ceil_div(ch, 64);
         o.slab = std::max(1, std::min(64 / px, n * o.ch_tiles / 296));

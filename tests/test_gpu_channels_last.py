@@ -27,6 +27,8 @@ SHAPES = [
     ConvLayer("one output channel", 40, 48, 31, 15, 1, 3, 3, 1, 1),
     ConvLayer("5x3 maps, more tiles than SMs", 3, 400, 5, 3, 530, 3, 3, 1, 1),
     ConvLayer("3x5 filter", 6, 36, 18, 18, 44, 3, 5, 1, 1),
+    ConvLayer("odd pixels past a tile, 3 and 70 channels", 3, 3, 33, 35, 70, 3, 3, 1, 1),
+    ConvLayer("odd pixels, 24 and 12 channels", 9, 24, 21, 15, 12, 5, 5, 1, 2),
 ]
 LAYOUTS = {"paper": {}, "nchw": dict(x_layout=B.X_NCHW, dw_layout=B.DW_KCRS),
            "nhwc": dict(dy_layout=B.DY_NPQK, dw_layout=B.DW_KCRS), "rsck": dict(x_layout=B.X_NCHW, dy_layout=B.DY_NPQK, dw_layout=B.DW_RSCK)}
