@@ -200,10 +200,10 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, bool reordered)
         // (the tensor core truncates as it adds, 1e-8 for each MMA of the other kernel's CTA: where that has more than 1,500 of them
         // its results are over 1.4e-5 away from this one's, and stay what they have been)
         if (L.tc_ok && L.tp.chain > 1500) return false;
-        if (L.tc_ok)                                                // 128->128 on 16x16 92 / 53, 64->64 on 8x8 17.1 / 18.1, on 18 SMs 44 / 40
-            return reordered || (g.c >= 128 ? products > 4e8 : g.c >= 64 && (shared || products > 3e9));
+        if (L.tc_ok)                                                // 128->128 on 16x16 92 / 53, 64->64 on 8x8 17.1 / 18.3, on 18 SMs 44 / 32
+            return reordered || products > (g.c >= 128 ? 4e8 : shared ? 1e8 : g.c >= 64 ? 1e9 : 2e8);      // 32->32 on 16x16 18.3 / 17.1, on 18 SMs 42 / 35
         if (direct_mma_supported(g, L.dp))                          // 16->16 on 32x32 19 / 40, 48->96 on 16x16 (N = 64) 31 / 23
-            return g.c >= 64 || (g.c >= 24 && g.stride_h == 1 && !shared);
+            return g.c >= 64 || (g.c >= 24 && g.stride_h == 1 && !shared && products > 3e8);       // (N = 16) 24->16 on 32x32 10 / 14
     }
     return products > 4e6;          // FP32 pipes: below this their one or two launches are as quick (8-9)
 }

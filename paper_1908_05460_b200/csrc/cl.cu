@@ -29,6 +29,10 @@
 //   k-side  M = 128 output channels, N = consecutive column shifts x channels (up to 256).
 //   c-side  (few output channels) M = 128 = shifts x channels of X, N = output channels; M = 64 MMAs would take as
 //           long as M = 128 ones, so with K <= 64 this form is the faster one although one shift in four is unused.
+//   stack   (at most 64 output channels, stride 1) M = 128 = filter rows x output channels: the reduction walks over rows of X, and
+//           the channel atoms of the dY operand lie one map row apart, so that atom j is the gradient row that meets this X row
+//           in filter row r_hi - j.  One MMA does the work of two to eight whose M would be mostly idle.
+//           (Bound by the tensor core: fp32 5x5 64->64 on 16x16, N = 128 53 -> 42 us, bf16 5x5 144->16 on 63x63, N = 16 43 -> 21.)
 // The MMAs of one k-step differ only in the X offset and the accumulator columns; the list of them is part of the plan.
 //
 // CTA = one tile of dW (k-tile x c-tile x filter rows) and a contiguous range of chunks.  Its accumulator block goes to
@@ -95,6 +99,8 @@ struct ClParams {
     int x_pre;                      // bytes of zeros before an X tile (kImages without halo columns; else 0)
     int skip;                       // kImages, whole maps, one filter row a tile: k-steps per map row, to leave out rows opposite the padding
     int c_side;                     // 1: X is the M side
+    int slack;                      // bytes behind the last stage that MMAs may read
+    int stack;                      // 1: filter rows x output channels are the M side; chunks are bands of X rows
     int s_inner;                    // 1: column shifts lie next to one another in dW (K x C x R x S): columns are written shift by shift
     int merged;                     // 1: the MN atoms of an X operand are channel atoms, 0: column shifts
     int ngroups, nmma, cols, tmem_cols;
@@ -123,6 +129,7 @@ __device__ __forceinline__ int written_column(const ClParams& P, int e)
 // lanes, nor a lane's columns, nor the shifts of a channel meet in one bank.
 __device__ __forceinline__ int block_key(int col, int ca_log) { return (col + 11 * (col >> ca_log)) & 31; }
 // Column -> {offset in dW, atoms in use (0: not an element)}
+// (stack: without the filter row, which belongs to the lane)
 __device__ __forceinline__ int2 column_target(const ClParams& P, int col, int k0, int c0, int r0)
 {
     const int gi = col / P.nmma, j = col - gi * P.nmma;
@@ -130,7 +137,15 @@ __device__ __forceinline__ int2 column_target(const ClParams& P, int col, int k0
     const int a = P.c_side || P.merged ? 0 : j / P.ca, k = P.c_side ? k0 + j : 0;
     const int c = c0 + g.cbase + (P.c_side ? 0 : P.merged ? j : j - a * P.ca);
     const bool valid = r0 + g.r < P.r && (P.c_side ? k < P.k : c < P.c && a < g.cnt);
-    return make_int2((int)(k * P.ws_k + c * P.ws_c + (r0 + g.r) * P.ws_r + (g.s0 + P.stride * a) * P.ws_s), valid ? g.cnt : 0);
+    return make_int2((int)(k * P.ws_k + c * P.ws_c + (P.stack ? 0 : r0 + g.r) * P.ws_r + (g.s0 + P.stride * a) * P.ws_s), valid ? g.cnt : 0);
+}
+
+// k-side: lane -> offset in dW, -1: not an element
+__device__ __forceinline__ int lane_target(const ClParams& P, int l, int k0, int r0)
+{
+    if (!P.stack) return k0 + l < P.k ? (int)((k0 + l) * P.ws_k) : -1;
+    const int j = l >> (31 - __clz(P.ka)), k = l & (P.ka - 1), r = r0 + P.rc - 1 - j;
+    return j < P.rc && r < P.r && k < P.k ? (int)(k * P.ws_k + r * P.ws_r) : -1;
 }
 
 // Warps: 0 and 1 issue MMAs, 2 and 3 fill the stages, 4 to 11 hold the sums.
@@ -217,7 +232,8 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
         const bool images = P.order == kImages, pixels = is_dy && P.order == kPixels;          // box i: 64 pixels of image i / dy_subs, K-major
         const int dy_img = pixels ? i / P.dy_subs : 0, dy_px = 64 * (i - dy_img * P.dy_subs);
         const int ch = is_dy ? k0 + P.ka * i : c0 + P.ca * (j - jt * P.na), col = is_dy || P.x_pre ? 0 : jt - rl * P.phases - P.pad_w;
-        const int row_mul = is_dy ? 1 : P.stride, row_add = is_dy ? 0 : r0 + rl - P.pad_h;
+        const int row_mul = is_dy ? 1 : P.stride;
+        const int row_add = P.stack ? (is_dy ? P.pad_h - (r0 + P.rc - 1) : 0) : is_dy ? 0 : r0 + rl - P.pad_h;
         int st = first, ph = 0, it = first;
         while (st >= P.stages) { st -= P.stages; ph ^= 1; }
         for (; it < nchunks; it += np) {
@@ -369,10 +385,11 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
         // The only split of a tile, channels innermost in dW: from the registers, eight channels (a sector) a store.
         const bool sectors = !CSIDE && P.splits == 1 && P.ws_c == 1 && (P.c & 7) == 0 && (reinterpret_cast<uintptr_t>(dw) & 31) == 0;
         if (ok && sectors) {
-            float* d = dw + (k0 + l128) * P.ws_k;
+            const int lane_off = lane_target(P, l128, k0, r0);
+            float* d = dw + lane_off;
 #pragma unroll
             for (int i = 0; i < NB; ++i)
-                if (2 * i + half < blocks && k0 + l128 < P.k) {
+                if (2 * i + half < blocks && lane_off >= 0) {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const int2 o = s_col[16 * (2 * i + half) + 8 * h];
@@ -442,12 +459,13 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
 #pragma unroll 2
             for (int t = warp; t < 32 * cgs; t += kThreads / 32) {
                 const int cg = t >> 5, l = ((t & 31) << 2) + (lane >> 3), col = (cg << 5) + cq;
-                if (col < cols && k0 + l < P.k) {
+                const int lane_off = lane_target(P, l, k0, r0);
+                if (col < cols && lane_off >= 0) {
                     const int2 o = s_col[col];
                     float v[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) v[i] = P.alpha * blk[(col + i) * 128 + (l ^ block_key(col + i, ca_log))];
-                    if (o.y > 0) *reinterpret_cast<float4*>(dw + (k0 + l) * P.ws_k + o.x) = make_float4(v[0], v[1], v[2], v[3]);
+                    if (o.y > 0) *reinterpret_cast<float4*>(dw + lane_off + o.x) = make_float4(v[0], v[1], v[2], v[3]);
                 }
             }
         } else {
@@ -462,8 +480,9 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
                 }
 #pragma unroll 4
                 for (int l = warp; l < 128; l += kThreads / 32) {
-                    if (k0 + l >= P.k) break;
-                    float* d = dw + (k0 + l) * P.ws_k;
+                    const int lane_off = lane_target(P, l, k0, r0);
+                    if (lane_off < 0) continue;
+                    float* d = dw + lane_off;
 #pragma unroll
                     for (int u = 0; u < 2; ++u)
                         if (off[u] >= 0) d[off[u]] = P.alpha * blk[pos[u] + (l ^ key[u])];
@@ -525,8 +544,9 @@ cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, cons
             valid = a < o.y && c0 + ch < P.c;
             off += ch * P.ws_c + P.stride * a * P.ws_s;
         } else {
-            valid = o.y > 0 && k0 + l < P.k;
-            off += (k0 + l) * P.ws_k;
+            const int lane_off = lane_target(P, l, k0, r0);
+            valid = o.y > 0 && lane_off >= 0;
+            off += lane_off;
         }
         if (!valid) continue;
         float t = s_sum[c][l];
@@ -805,7 +825,7 @@ int far_shift(const ClParams& P)
 bool build_groups(ClParams& P)
 {
     P.ngroups = 0;
-    const int rows = P.rc, st = P.stride, wt = P.x_pitch;
+    const int rows = P.stack ? 1 : P.rc, st = P.stride, wt = P.x_pitch;
     // atoms of one MMA on the X side: c-side exactly fills M = 128; k-side as many as N = 256 takes, the shifts of a column phase
     // shared out evenly over as few MMAs as hold them
     const int atoms = P.merged ? P.na : shifts_of(P);
@@ -840,21 +860,23 @@ bool build_groups(ClParams& P)
 bool shape_chunk(ClParams& P, int ci, int bp, int order, bool bare = false)
 {
     const int st = P.stride;
-    const bool images = order == kImages, whole = images ? bp >= P.p : ci > 1 || bp >= P.p;
+    const int all_rows = P.stack ? P.h : P.p;
+    const bool images = order == kImages, whole = images ? bp >= all_rows : ci > 1 || bp >= all_rows;
     if (order == kPaired) bp = round_up(bp, 2);
     if (order == kPixels && !whole && bp * P.q % 16 != 0) return false;         // k-steps do not cross chunks
     P.ci = ci; P.bp = bp; P.order = order;
-    P.cpi = whole ? 0 : ceil_div(P.p, bp);
+    P.cpi = whole ? 0 : ceil_div(all_rows, bp);
     P.mma_cols = 0;
     P.chunks = whole ? ceil_div(P.n, ci) : ceil_div(P.n, ci) * P.cpi;
     P.px_rows = images ? ci : 1;
-    P.skip = images && !bare && whole && P.rc == 1 && P.q * ci % 16 == 0 ? P.q * ci / 16 : 0;
-    const int wp = bare ? P.w : P.q + ceil_div(P.s, st) - 1, halo = st == 1 ? P.rc - 1 : 0;
-    const int x_rows = bp + halo, dy_rows = (order == kFlat && ci > 1) ? bp + halo : bp, dy_w = order == kFlat ? wp : P.q;
+    P.skip = images && !bare && !P.stack && whole && P.rc == 1 && P.q * ci % 16 == 0 ? P.q * ci / 16 : 0;
+    const int wp = bare ? P.w : P.q + ceil_div(P.s, st) - 1, above = P.stack ? P.rc - 1 : 0, halo = st == 1 && !P.stack ? P.rc - 1 : 0;
+    const bool same = order == kFlat && ci > 1;          // (images of both operands at the same distance)
+    const int x_rows = bp + halo + (same ? above : 0), dy_rows = bp + above + (same ? halo : 0), dy_w = order == kFlat ? wp : P.q;
     if ((wp - 1) * st + 1 > 256 || (x_rows - 1) * st + 1 > 256 || dy_rows > 256 || ci > 256) return false;
     P.x_pitch = wp; P.dy_pitch = dy_w; P.x_img = x_rows * wp; P.dy_img = dy_rows * dy_w;
     const int steps_img = order == kPaired ? (bp / 2) * (P.q / 8) : ceil_div(bp * P.q, 16);
-    P.ksteps = order == kFlat ? ceil_div(ci * dy_rows * dy_w, 16) : images ? ceil_div(bp * P.q * ci, 16) : ci * steps_img;
+    P.ksteps = order == kFlat ? ceil_div(ci > 1 ? ci * dy_rows * dy_w : bp * dy_w, 16) : images ? ceil_div(bp * P.q * ci, 16) : ci * steps_img;
     if (P.ksteps > kMaxKsteps) return false;
     const int xb = P.ca * 2, db = P.ka * 2;
     P.x_box = ci * x_rows * wp * xb;
@@ -865,21 +887,25 @@ bool shape_chunk(ClParams& P, int ci, int bp, int order, bool bare = false)
         P.dy_alloc = round_up(P.kt * 128, 1024);
     } else {
         P.dy_box = ci * dy_rows * dy_w * db;
-        P.dy_alloc = round_up(std::max(P.dy_box, order == kPaired ? 0 : P.ksteps * 16 * db), 1024);
+        P.dy_alloc = round_up(std::max(P.dy_box, order == kPaired ? 0 : (P.ksteps * 16 + above * dy_w * P.px_rows) * db), 1024);
     }
     // last X row an MMA touches: last k-step, last row and column shift, unused shifts of the c-side form
     // (kImages: in whole pixels, one more where the last k-step is half a k-step)
     const int last = order == kFlat ? P.ksteps * 16 - 1 : ((images ? 1 : ci) - 1) * P.x_img + (bp - 1) * wp + P.q - 1 + (order == kPixels ? 8 : 0) + (images && ci % 16 != 0 ? 1 : 0);
+    const int zeros = P.stack && images && ci == 8 && bp * P.q % 2 != 0 ? P.x_img + 1 + far_shift(P) : 0;      // pixels, see below
     P.x_pre = bare ? round_up(std::max(P.pad_w, 1) * ci * xb, 1024) : 0;
     const int far = last + halo * wp + (images ? far_shift(P) : ceil_div(P.s, st) - 1 + (P.c_side ? 128 / P.ca : 256 / P.ca));
-    P.x_alloc = P.x_pre + round_up(bare ? P.x_box : std::max(P.x_box, (far + 1) * P.px_rows * xb), 1024);
+    P.x_alloc = P.x_pre + round_up(bare ? P.x_box : std::max(P.x_box, std::max(far + 1, zeros) * P.px_rows * xb), 1024);
     const int x_tiles = P.na * P.phases * P.row_tiles;
     P.x_plane = x_tiles * P.x_alloc;
     P.dy_plane = P.katoms * P.dy_alloc;
     P.x_region = P.planes * P.dy_plane;
     P.stage_bytes = P.x_region + P.planes * P.x_plane;
     if (P.planes * (P.katoms + x_tiles) > 32) return false;        // one copy per lane of a producer
-    P.stages = std::min(kMaxStages, kStageBudget / P.stage_bytes) & ~1;
+    // (stack: idle atoms of the last stage read on past their rows; what they read is multiplied into rows that nobody reads)
+    const int reach = P.stack ? (P.planes - 1) * P.dy_plane + (P.ksteps * 16 + (ci - 1) * P.dy_img + 128 / P.ka * dy_w * P.px_rows + 2 * dy_w) * db : 0;
+    P.slack = std::max(0, reach - P.stage_bytes);
+    P.stages = std::min(kMaxStages, (kStageBudget - P.slack) / P.stage_bytes) & ~1;
     P.epoch = std::max(1, (P.nprod > 1 ? 16 : 64) / P.ksteps);
     if (P.stages < 2) return false;
     P.tx_bytes = (uint32_t)(P.planes * (P.katoms * P.dy_box + x_tiles * P.x_box));
@@ -889,7 +915,7 @@ bool shape_chunk(ClParams& P, int ci, int bp, int order, bool bare = false)
     P.dy_hi = (dy_sbo >> 4) | (1u << 14) | (dy_swz << 29);
     P.x_lbo = (uint32_t)((P.merged ? P.x_alloc : P.px_rows * xb) >> 4) << 16;
     // (one atom: the upper half of M repeats the lower)
-    P.dy_lbo = order == kPixels ? 1u << 16 : (uint32_t)((P.katoms > 1 ? P.dy_alloc : 0) >> 4) << 16;
+    P.dy_lbo = P.stack ? (uint32_t)(dy_w * P.px_rows * db >> 4) << 16 : order == kPixels ? 1u << 16 : (uint32_t)((P.katoms > 1 ? P.dy_alloc : 0) >> 4) << 16;
     for (int i = 0; i < P.ksteps; ++i) {
         int s_lo = 0, s_hi = 0;                                        // bare: column shifts of the k-step
         int x_row = 16 * i, dy_off = 16 * i * db, x_sbo = 8;          // X row, dY bytes, X rows between the two 8-pixel groups
@@ -901,6 +927,8 @@ bool shape_chunk(ClParams& P, int ci, int bp, int order, bool bare = false)
         } else if (images) {
             const int px = 16 * i / ci, p = px / P.q, q = px % P.q;
             x_row = (p * wp + q) * ci + 16 * i % ci;
+            // (the other half of a last half k-step: in the stack form dY has rows there, so X must read zeros, those behind the tile)
+            if (P.stack && ci == 8 && px + 1 == bp * P.q) x_sbo = P.x_img * ci - x_row;
             if (bare) {
                 // the shifts whose column lies in the map; pixel 0 takes all of them, those to the left from the zeros before the
                 // tile, so that the MMA that starts an accumulator writes every column of it
@@ -996,25 +1024,29 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
 
     ClParams best{};
     double best_cycles = 1e30;
-    for (int form = 0; form < 2; ++form) {
-        const int k16 = round_up(g.k, 16);
-        const int kts[4] = {form ? std::min(k16, 256) : 128, 128, 64, 32};
-        for (int ki = 0; ki < (form ? 4 : 1); ++ki) {
+    for (int form = 0; form < 3; ++form) {           // k-side, c-side, stack
+        if (form == 2 && (g.k > 64 || g.r == 1 || g.stride_h != 1)) break;
+        const int k16 = round_up(g.k, 16), all_rows = form == 2 ? g.h : g.p;
+        const int kts[4] = {form == 2 ? (g.k > 32 ? 64 : k16) : form ? std::min(k16, 256) : 128, 128, 64, 32};
+        for (int ki = 0; ki < (form == 1 ? 4 : 1); ++ki) {
             if (ki > 0 && (kts[ki] >= kts[0] || kts[ki] >= k16)) continue;
             ClParams F = B;
-            F.c_side = form; F.kt = kts[ki];
+            F.c_side = form == 1; F.stack = form == 2; F.kt = kts[ki];
             const int kw = std::min(F.kt, k16);
             F.ka = kw > 32 ? 64 : kw > 16 ? 32 : 16;
             F.katoms = ceil_div(kw, F.ka);
             F.tiles_k = ceil_div(g.k, F.kt);
+            // (stack: with wide filters fewer channels a tile, so that all shifts fit one MMA and the accumulators)
+            for (int ca = B.ca; ca >= (form == 2 && g.s > 3 ? 16 : B.ca); ca /= 2)
             for (int na = 1; na <= 4; na *= 2) {
+                F.ca = ca;
                 if (na > 1 && (F.ca < 64 || (na - 1) * 64 >= g.c)) break;
-                if (form && na > 2) break;
-                if (!form && na > 2 && g.s > 1) break;
+                if (form == 1 && na > 2) break;
+                if (form != 1 && na > 2 && g.s > 1) break;
                 F.na = na; F.ct = na * F.ca;
-                F.merged = na > 1 && (form || g.s == 1) ? 1 : 0;
+                F.merged = na > 1 && (form == 1 || g.s == 1) ? 1 : 0;
                 F.tiles_c = ceil_div(g.c, F.ct);
-                for (int rc = 1; rc <= g.r; ++rc) {
+                for (int rc = form == 2 ? 2 : 1; rc <= (form == 2 ? std::min(g.r, 128 / F.ka) : g.r); ++rc) {
                     F.rc = rc; F.tiles_r = ceil_div(g.r, rc);
                     if (rc > 1 && ceil_div(g.r, rc) == ceil_div(g.r, rc - 1)) continue;
                     F.row_tiles = F.stride > 1 ? rc : 1;
@@ -1024,7 +1056,7 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
                     for (int mode = kFlat; mode <= kImages; ++mode) {
                         if ((mode == kPaired || mode == kPixels) && g.q % 8 != 0) continue;
                         // (small maps: one order for every layout of dY, so that its results do not depend on it either)
-                        if (mode == kPixels && (H.f32 || H.dy_npqk || g.p * g.q < 64)) continue;
+                        if (mode == kPixels && (form == 2 || H.f32 || H.dy_npqk || g.p * g.q < 64)) continue;
                         if (mode == kImages && g.n < 5) continue;
                         auto consider = [&](int ci, int bp, bool bare) {
                             ClParams C = F;
@@ -1035,10 +1067,12 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
                             if (const char* e = getenv("GACONV_CL_FORM")) if (C.c_side != atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_RC")) if (C.rc != atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_KT")) if (C.kt != atoi(e)) return true;
+                            if (const char* e = getenv("GACONV_CL_STACK")) if (C.stack != atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_BARE")) if ((C.x_pre > 0) != (atoi(e) != 0)) return true;
                             if (const char* e = getenv("GACONV_CL_NA")) if (C.na != atoi(e)) return true;
 #endif
                             Cost c = cost_of(C, sms, std::min(1.0, 1.3 * share / C.cols));
+                            if (form == 2) c.cycles *= 1.07;          // (by a few per cent the other forms are as quick or quicker)
                             // a packing pass of dY: its launch, and its bytes twice
                             if (mode != kPixels && H.pack_dy) c.cycles += 3500 + (double)dy_el * 2 * (1 + C.planes) / (16.0 * sms);
                             if (c.cycles < best_cycles) { best_cycles = c.cycles; C.splits = c.splits; best = C; }
@@ -1047,17 +1081,17 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
                         if (mode == kImages) {
                             for (int ci = 8; ci <= 64 && ci < 2 * g.n; ci *= 2) {
                                 int last_bp = 0;
-                                for (int parts = g.p; parts >= 1; --parts) {
-                                    const int bp = ceil_div(g.p, parts);
+                                for (int parts = all_rows; parts >= 1; --parts) {
+                                    const int bp = ceil_div(all_rows, parts);
                                     if (bp == last_bp) continue;
                                     last_bp = bp;
                                     if (!consider(ci, bp, false)) break;
                                 }
                                 // no halo columns: one MMA a k-step, of shifts alone, and a first pixel with every shift inside or to the left
-                                if (form == 0 && ci >= 16 && na == 1 && rc == 1 && F.stride == 1 && g.s > 1 && g.s * F.ca <= kMaxCols && g.w >= g.s - g.pad_w && g.pad_w < g.w) {
+                                if (form != 1 && ci >= 16 && na == 1 && (rc == 1 || form == 2) && F.stride == 1 && g.s > 1 && g.s * F.ca <= kMaxCols && g.w >= g.s - g.pad_w && g.pad_w < g.w) {
                                     last_bp = 0;
-                                    for (int parts = g.p; parts >= 1; --parts) {
-                                        const int bp = ceil_div(g.p, parts);
+                                    for (int parts = all_rows; parts >= 1; --parts) {
+                                        const int bp = ceil_div(all_rows, parts);
                                         if (bp == last_bp) continue;
                                         last_bp = bp;
                                         if (!consider(ci, bp, true)) break;
@@ -1067,15 +1101,15 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
                             continue;
                         }
                         int last_bp = 0;
-                        for (int parts = g.p; parts >= 1; --parts) {      // fewer and fewer, larger and larger bands
-                            int bp = ceil_div(g.p, parts);
+                        for (int parts = all_rows; parts >= 1; --parts) {      // fewer and fewer, larger and larger bands
+                            int bp = ceil_div(all_rows, parts);
                             if (mode == kPaired) bp = round_up(bp, 2);
                             if (bp == last_bp) continue;
                             last_bp = bp;
                             if (!consider(1, bp, false)) break;
                         }
                         for (int ci = 2; ci <= 64 && ci <= g.n; ci = ci < 4 ? ci + 1 : ci + ci / 2)
-                            if (!consider(ci, g.p, false)) break;
+                            if (!consider(ci, all_rows, false)) break;
                     }
                 }
             }
@@ -1151,7 +1185,7 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
         !encode(&map_x, x, P.c, H.xch, P.w, P.h, x_el, P.ca, P.x_pitch, P.x_img / P.x_pitch, P.stride))
         return cudaErrorInvalidValue;
     // the stages; at the end they hold the accumulator block
-    const size_t smem = std::max((size_t)P.stages * P.stage_bytes, (size_t)P.cols * 512) + 1024;
+    const size_t smem = std::max((size_t)P.stages * P.stage_bytes + P.slack, (size_t)P.cols * 512) + 1024;
     const dim3 grid((unsigned)(P.tiles_k * P.tiles_c * P.tiles_r), (unsigned)P.splits);
     ClKernel kern = kernel_for(P.ngroups, H.f32, P.c_side != 0);
     if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return err;

@@ -27,6 +27,10 @@ SHAPES = [
     ConvLayer("one output channel", 40, 48, 31, 15, 1, 3, 3, 1, 1),
     ConvLayer("5x3 maps, more tiles than SMs", 3, 400, 5, 3, 530, 3, 3, 1, 1),
     ConvLayer("3x5 filter", 6, 36, 18, 18, 44, 3, 5, 1, 1),
+    ConvLayer("stacked filter rows, 5x5, two row tiles", 12, 72, 17, 11, 40, 5, 5, 1, 2),
+    ConvLayer("13 outputs, no padding", 30, 100, 12, 9, 13, 3, 3, 1, 0),
+    ConvLayer("stacked filter rows, (pixel, image) order, odd pixels", 30, 130, 5, 9, 40, 5, 5, 1, 2),
+    ConvLayer("7x3 filter", 9, 70, 12, 16, 64, 7, 3, 1, 1),
     ConvLayer("odd pixels past a tile, 3 and 70 channels", 3, 3, 33, 35, 70, 3, 3, 1, 1),
     ConvLayer("odd pixels, 24 and 12 channels", 9, 24, 21, 15, 12, 5, 5, 1, 2),
 ]
