@@ -104,6 +104,15 @@ private:
     std::vector<std::pair<PlanKey, L>> e_;
 };
 
+// A large dW with short sums, split over CTAs, on a GPU of its own: the channels-last kernel writes as many partial blocks as it has
+// CTAs and reads them again, the older kernel adds them inside clusters (256->256 on 8x8, N = 64 16.9 / 14.6 us, N = 128
+// 20.1 / 19.9, N = 256 26.5 / 27.1; 256->512 on 4x4, N = 128 21.0 / 19.4; 128->256 on 8x8, N = 128 15.9 / 16.6).
+bool short_sums(const Geom& g, const ClPlan& plan)
+{
+    const double elements = (double)g.k * g.c * g.r * g.s;
+    return g.sm_budget == 0 && plan.partial_bytes > 0 && elements > 4e5 && (double)g.n * g.p * g.q < 0.015 * elements;
+}
+
 // Small maps with many channels (up to 4x4 pixels from 128 channels, up to 8x8 from 256): the N*K patch accumulations (N*K*R*S*C FMAs on the FP32 pipes,
 // the same number of bytes gathered from L2) cost more than the dense contraction on tensor cores, and with so few
 // pixels per map the sparse tensor is not that sparse (1 - 1/(PQ), Section 2.3).  Then the method is run
@@ -123,7 +132,7 @@ Top1Layout build_top1_layout(const Geom& g)
     L.dense = top1_dense_route(g, &L.tp);
     // the contraction: by the channels-last kernel, which reads either form of the sparse tensor (256->256 on 8x8, N = 256:
     // 37 us with the other kernel, 32)
-    L.cl = L.dense && tensor_maps_available() && plan_cl(g, L.tp.reads_transposed_dy, &L.cp);
+    L.cl = L.dense && tensor_maps_available() && plan_cl(g, L.tp.reads_transposed_dy, &L.cp) && !short_sums(g, L.cp);
     const size_t cl_scratch = L.cl ? L.cp.x_bytes + L.cp.dy_bytes : 0;
     const size_t maps = (size_t)g.n * g.k;
     L.idx_off = kWsDataOffset;
@@ -180,7 +189,7 @@ ExactLayout exact_layout(const Geom& g, int math, int algo)
 // measured faster (in microseconds, the older kernel first; N = 128 unless said).  `reordered`: X or dY comes in the other
 // order than N x H x W x C / N x K x P x Q, which costs the older kernels a transposing pass and this one none or a cheaper one.
 // ALGO_DIRECT, ALGO_TENSOR and the one-pass TF32 mode stay with the older kernels.
-bool prefer_cl(const Geom& g, const ExactLayout& L, bool reordered)
+bool prefer_cl(const Geom& g, const ExactLayout& L, const ClPlan& plan, bool reordered)
 {
     const double products = (double)g.n * g.p * g.q * g.k * g.c * g.r * g.s;
     const bool shared = g.sm_budget > 0;            // other layers run beside this one
@@ -188,6 +197,7 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, bool reordered)
     reordered = reordered && products > 3e7;
     if (g.bf16) {
         if (L.tc_ok) {
+            if (!reordered && short_sums(g, plan)) return false;
             if (L.tp.reads_transposed_dy) return products > 5e6;        // maps under 64 pixels: 512->512 on 4x4, N = 256 31.1 / 27.0
             if (products < 3e7) return false;
             if (reordered) return true;                             // 128->128 on 16x16, dY channels last 28.4 / 17.8
@@ -217,7 +227,7 @@ ClRoute build_cl_route(const gaconv_conv_desc_t* desc, const Geom& g)
     Geom gn;
     if (make_geom(&native, &gn) != GACONV_OK) return R;
     const ExactLayout L = exact_layout(gn, GACONV_MATH_DEFAULT, GACONV_ALGO_AUTO);
-    R.use = prefer_cl(gn, L, (desc->x_layout == GACONV_X_NCHW && g.c > 1) || (desc->dy_layout == GACONV_DY_NPQK && g.k > 1));
+    R.use = prefer_cl(gn, L, R.plan, (desc->x_layout == GACONV_X_NCHW && g.c > 1) || (desc->dy_layout == GACONV_DY_NPQK && g.k > 1));
 #ifdef GACONV_TUNING
     if (const char* e = getenv("GACONV_CL")) R.use = atoi(e) != 0;
 #endif

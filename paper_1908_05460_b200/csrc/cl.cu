@@ -799,7 +799,10 @@ Cost cost_of(const ClParams& P, int sms, double block_share)
     const int tiles = P.tiles_k * P.tiles_c * P.tiles_r;
     const double block_bytes = (double)P.cols * 512 * block_share;
     Cost best{1e30, 1};
-    const int most = std::max(1, std::min(P.chunks, sms / tiles));
+    int most = std::max(1, std::min(P.chunks, sms / tiles));
+#ifdef GACONV_TUNING
+    if (const char* e = getenv("GACONV_CL_SP")) most = std::min(most, atoi(e));
+#endif
     for (int sp = most; sp >= 1; sp = sp > 8 ? sp * 7 / 8 : sp - 1) {
         const int waves = ceil_div(tiles * sp, sms), per = ceil_div(P.chunks, sp);
         const double main = waves * (4500 + load * std::min({per, P.stages, 4}) / 2 + per * chunk + block_bytes / (sp == 1 ? 18 : 21));
@@ -1067,6 +1070,7 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
                             if (const char* e = getenv("GACONV_CL_FORM")) if (C.c_side != atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_RC")) if (C.rc != atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_KT")) if (C.kt != atoi(e)) return true;
+                            if (const char* e = getenv("GACONV_CL_MODE")) if (mode != atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_STACK")) if (C.stack != atoi(e)) return true;
                             if (const char* e = getenv("GACONV_CL_BARE")) if ((C.x_pre > 0) != (atoi(e) != 0)) return true;
                             if (const char* e = getenv("GACONV_CL_NA")) if (C.na != atoi(e)) return true;
