@@ -43,10 +43,11 @@ typedef enum {
 } gaconv_status_t;
 
 typedef enum { GACONV_F32 = 0, GACONV_BF16 = 1 } gaconv_dtype_t;            /* of x and dy            */
-typedef enum { GACONV_X_NHWC = 0, GACONV_X_NCHW = 1 } gaconv_x_layout_t;    /* NHWC: Section 2.4; NCHW is transposed once
-                                                                               into the workspace where a fast kernel applies */
+typedef enum { GACONV_X_NHWC = 0, GACONV_X_NCHW = 1 } gaconv_x_layout_t;    /* NHWC: Section 2.4; NCHW is brought into
+                                                                               channels-last order once, in the workspace, where a fast kernel applies */
 typedef enum { GACONV_DY_NKPQ = 0, GACONV_DY_NPQK = 1 } gaconv_dy_layout_t;  /* NKPQ = N C_o H W (Section 2.4); NPQK (channels
-                                                                               last) is transposed once into the workspace.
+                                                                               last) is read in place by the exact method's channels-last
+                                                                               kernel, else transposed once into the workspace.
                                                                                The selection-only entry points take NKPQ only */
 /* KRSC = C_o K K C_i (the layout of the paper's kernel, Section 2.4), KCRS = the frameworks' filter
  * layout, RSCK = K K C_i C_o (the order in which Section 2.4 first writes df) */
@@ -115,12 +116,13 @@ gaconv_status_t gaconv_dw_exact(const void *x, const void *dy, float *dw,
  * Some callers cannot give the library a workspace because they may not call cudaMalloc where they
  * run: a host framework's plugin that is handed only its inputs and outputs, a loop that was promised
  * "no allocation after warm-up", a process whose device memory pool belongs to someone else.  This
- * variant computes exactly what gaconv_dw_exact computes, with the same kernels, but keeps the scratch
+ * variant computes what gaconv_dw_exact computes, with the same kernels as far as their scratch fits (a call whose
+ * repacked operands do not fit takes the kernels that need none), but keeps the scratch
  * (split partial sums, control words) in a fixed array inside the library: gaconv_static_scratch_bytes()
  * bytes (8 MiB) that every GPU loading the library holds until the process exits.  desc->workspace and
  * desc->workspace_bytes are ignored.  The call allocates nothing (no cudaMalloc, cudaFree or
  * allocating library routine).
- *   - Limit: a problem whose gaconv_workspace_size(desc, GACONV_METHOD_EXACT) exceeds
+ *   - Limit: a problem whose scratch, without repacked operands, exceeds
  *     gaconv_static_scratch_bytes() is rejected with GACONV_ERR_WORKSPACE_TOO_SMALL and nothing is
  *     enqueued; use gaconv_dw_exact with a caller-owned workspace for those.
  *   - The first call on each device resolves the array's device address and clears its control words
@@ -220,7 +222,9 @@ gaconv_status_t gaconv_schedule_run_layer(const gaconv_schedule_t *sched, int32_
  * layer's result is bit for bit that of gaconv_schedule_run_layer with the same descriptor.  lanes in 1..16; with lanes > 1 the
  * descriptors must carry distinct workspaces (GACONV_ERR_BAD_DESC otherwise).  x, dy, dw, descs: host arrays
  * of num_layers device pointers / descriptor pointers.  Calls on one device share the lanes: enqueueing from
- * several host threads is serialised. */
+ * several host threads is serialised.  A step of six layers or more that is repeated with the same arguments (its number and
+ * the random method's seeds may change) is launched as one CUDA graph; the library keeps up to eight of them and drops the
+ * one least recently used. */
 gaconv_status_t gaconv_schedule_run_step(const gaconv_schedule_t *sched, int64_t step, int32_t num_layers,
                                          const void *const *x, const void *const *dy, float *const *dw,
                                          const gaconv_conv_desc_t *const *descs, int32_t lanes, void *stream);
