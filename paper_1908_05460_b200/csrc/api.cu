@@ -213,9 +213,11 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, const ClPlan& plan, bool reo
         if (L.tc_ok)                                                // 128->128 on 16x16 92 / 53, 64->64 on 8x8 17.1 / 18.3, on 18 SMs 44 / 32
             return reordered || products > (g.c >= 128 ? 4e8 : shared ? 1e8 : g.c >= 64 ? 1e9 : 2e8);      // 32->32 on 16x16 18.3 / 17.1, on 18 SMs 42 / 35
         if (direct_mma_supported(g, L.dp))                          // 16->16 on 32x32 19 / 40, 48->96 on 16x16 (N = 64) 31 / 23
-            return g.c >= 64 || (g.c >= 24 && g.stride_h == 1 && !shared && products > 3e8);       // (N = 16) 24->16 on 32x32 10 / 14
+            return (g.c >= 64 && products > 4e6) || (g.c >= 24 && g.stride_h == 1 && !shared && products > 3e8);       // (N = 16) 24->16 on 32x32 10 / 14
     }
-    return products > 4e6;          // FP32 pipes: below this their one or two launches are as quick (8-9)
+    // FP32 pipes: their one or two launches are as quick while the work is small -- longer with 3x3 filters of fp32 layers, whose
+    // operands must be packed (16->64 on 6x6, N = 30 10.3 / 12.3 us; 1x1 80->22 on 6x6, N = 105 27 / 12), and with three channels
+    return products > (!g.bf16 && g.r * g.s >= 9 ? 2e7 : g.c <= 4 ? 1e7 : 4e6);
 }
 struct ClRoute { bool use; ClPlan plan; size_t partial_off, x_off, dy_off, total; };
 ClRoute build_cl_route(const gaconv_conv_desc_t* desc, const Geom& g)
