@@ -198,7 +198,9 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, const ClPlan& plan, bool reo
     if (g.bf16) {
         if (L.tc_ok) {
             if (!reordered && short_sums(g, plan)) return false;
-            if (L.tp.reads_transposed_dy) return products > 5e6;        // maps under 64 pixels: 512->512 on 4x4, N = 256 31.1 / 27.0
+            // maps under 64 pixels: 512->512 on 4x4, N = 256 31.1 / 27.0, 128->16 on 4x8, N = 100 12.5 / 10.7; many input and few output
+            // channels (partial blocks of mostly idle lanes) 192->16 on 4x8, N = 23 8.9 / 11.6, 256->16 on 4x4, N = 200 13.3 / 15.0
+            if (L.tp.reads_transposed_dy) return products > 5e6 && (g.k > 32 || g.c <= 128);
             if (products < 3e7) return false;
             if (reordered) return true;                             // 128->128 on 16x16, dY channels last 28.4 / 17.8
             if (g.c <= 16 || (g.c < 64 && shared)) return false;    // 16->16 on 32x32 11.9 / 12.5; on 18 SMs 28 / 38
