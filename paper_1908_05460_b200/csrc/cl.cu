@@ -876,7 +876,7 @@ bool shape_chunk(ClParams& P, int ci, int bp, int order, bool bare = false)
     const int wp = bare ? P.w : P.q + ceil_div(P.s, st) - 1, above = P.stack ? P.rc - 1 : 0, halo = st == 1 && !P.stack ? P.rc - 1 : 0;
     const bool same = order == kFlat && ci > 1;          // (images of both operands at the same distance)
     const int x_rows = bp + halo + (same ? above : 0), dy_rows = bp + above + (same ? halo : 0), dy_w = order == kFlat ? wp : P.q;
-    if ((wp - 1) * st + 1 > 256 || (x_rows - 1) * st + 1 > 256 || dy_rows > 256 || ci > 256) return false;
+    if ((wp - 1) * st + 1 > kMaxMapBox || (x_rows - 1) * st + 1 > kMaxMapBox || dy_rows > kMaxMapBox || ci > kMaxMapBox) return false;
     P.x_pitch = wp; P.dy_pitch = dy_w; P.x_img = x_rows * wp; P.dy_img = dy_rows * dy_w;
     const int steps_img = order == kPaired ? (bp / 2) * (P.q / 8) : ceil_div(bp * P.q, 16);
     P.ksteps = order == kFlat ? ceil_div(ci > 1 ? ci * dy_rows * dy_w : bp * dy_w, 16) : images ? ceil_div(bp * P.q * ci, 16) : ci * steps_img;
@@ -1005,7 +1005,7 @@ ClKernel kernel_for(int ng, bool f32, bool c_side)
 
 bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
 {
-    if (g.stride_h != g.stride_w || g.r > 16 || g.s > 16) return false;
+    if (g.stride_h != g.stride_w || g.stride_h > kMaxMapStep || g.r > 16 || g.s > 16) return false;
     const bool nhwc = g.xs_c == 1 || g.c == 1;
     ClHost H{};
     H.f32 = !g.bf16;

@@ -798,7 +798,7 @@ bool plan_tc(const Geom& g, TcPlan* out)
 {
     if (!g.bf16) return false;
     if (g.xs_c != 1 || g.c % 8 != 0) return false;                       // NHWC with 16-byte pixel rows
-    if (g.stride_h != g.stride_w) return false;
+    if (g.stride_h != g.stride_w || g.stride_h > kMaxMapStep) return false;
     const int pq = g.p * g.q;
     // maps under 64 pixels: K-major rows of dY would be 32 or 64 bytes (or too short for TMA at all) and the
     // copy engine's cost is per row, so A is taken from a transposed copy with 128-byte rows instead
@@ -898,6 +898,7 @@ bool plan_tc(const Geom& g, TcPlan* out)
         if (bp == g.p && P.wide && P.rc == 1)
             while (ci * 2 <= 8 && ci * 2 <= g.n && stage_bytes(ci * 2, bp, &a_subs, &tb, &ts) <= budget) ci *= 2;
     }
+    if (g.stride_h > 1 && std::max(bp, g.q) * g.stride_h > kMaxMapBox) return false;      // (a box spans the pixels stepped over)
     P.ci = ci; P.bp = bp;
     P.stage_bytes = stage_bytes(ci, bp, &a_subs, &tb, &ts);
     if (tiny2) {                                        // A: [pixel][image][64 k] per atom; B: [row][column + halo][image][64 c]

@@ -53,6 +53,9 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
 }
 
 // ---------------------------------------------------------------- host: cuTensorMapEncodeTiled without linking libcuda
+// What a tensor map can step over and how far a box reaches; a planner refuses what is beyond (the encoder would)
+constexpr int kMaxMapStep = 8, kMaxMapBox = 256;
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

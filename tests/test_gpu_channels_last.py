@@ -85,3 +85,26 @@ def test_static_scratch_takes_the_kernels_that_fit():
     B.gaconv_dw_exact_static(g.x, g.dy, g.dw, bare)
     got = g.logical_dw()
     assert np.max(np.abs(got - want)) <= 1e-4 * np.abs(want).max() and B.gaconv_poll_async_status_static() == B.OK
+
+
+# strides and boxes beyond what a tensor map steps over (8 pixels, 256 a side): other kernels take them
+FAR = [
+    ConvLayer("stride 9", 20, 64, 40, 37, 96, 3, 3, 9, 1),
+    ConvLayer("stride 12, 12x12 patches", 8, 3, 60, 48, 200, 12, 12, 12, 0),
+    ConvLayer("stride 9, 8x8 outputs", 2, 16, 72, 72, 16, 3, 3, 9, 1),
+    ConvLayer("stride 8, the largest step", 20, 64, 40, 37, 96, 3, 3, 8, 1),
+    ConvLayer("stride 5, rows of 64 outputs", 2, 16, 20, 320, 16, 3, 3, 5, 1),
+    ConvLayer("stride 5, 64 rows of one output", 2, 16, 320, 1, 16, 1, 1, 5, 0),
+]
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
+@pytest.mark.parametrize("li", range(len(FAR)), ids=[l.name for l in FAR])
+def test_large_strides(li, dtype):
+    layer = FAR[li]
+    x, dy = I.make_layer_inputs(layer, dtype, 16, li)
+    ref, dn = oracle.dw_exact(to_f64(x), to_f64(dy), oshape(layer), 0.5)
+    for name, kw in LAYOUTS.items():
+        g = GpuLayer(layer, dtype, x, dy, alpha=0.5, **kw)
+        assert norm_err(g.exact(), ref, dn) <= TOL_F32, name
+        assert B.gaconv_poll_async_status(g.desc) == B.OK
