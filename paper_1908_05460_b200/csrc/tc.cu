@@ -161,7 +161,11 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constan
                 uint32_t* __restrict__ status, const TcParams P)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bar_full[kMaxStages], bar_empty[kMaxStages], bar_acc;
+    // Two "full" barriers a stage, taken in turn (barrier it % (2 * stages) for chunk it).  With two issuers on alternate chunks and an
+    // odd number of stages, a stage's chunks belong to the issuers in turn; an issuer that saw only every other phase of one
+    // barrier would take the phase of the same parity two laps back for its own -- and multiply a stage that is still being
+    // filled -- whenever a chunk lands before the one in front of it.
+    __shared__ __align__(8) uint64_t bar_full[2 * kMaxStages], bar_empty[kMaxStages], bar_acc;
     __shared__ uint32_t s_tmem_base;
     __shared__ volatile int s_abort;
     // for quad column cq of the CTA's block: offset of its first element within a dW row block, and how many of
@@ -199,7 +203,8 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constan
         // the tensor maps are kernel parameters: fetching them does not depend on the previous kernel
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_dy) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
-        for (int i = 0; i < P.stages; ++i) { mbar_init(smem_u32(&bar_full[i]), 1); mbar_init(smem_u32(&bar_empty[i]), P.dual ? 1 : P.issuers); }
+        for (int i = 0; i < 2 * P.stages; ++i) mbar_init(smem_u32(&bar_full[i]), 1);
+        for (int i = 0; i < P.stages; ++i) mbar_init(smem_u32(&bar_empty[i]), P.dual ? 1 : P.issuers);
         mbar_init(smem_u32(&bar_acc), P.issuers);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -245,9 +250,9 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constan
         // what copy `lane` is: image and box of an A copy, or filter row and column shift of a B copy
         const int a_img = (P.tiny || P.by_image) ? 0 : lane / P.a_subs_img, a_sub = (P.tiny || P.by_image) ? 0 : lane - a_img * P.a_subs_img;
         const int b_idx = lane - n_a, b_rr = b_idx > 0 ? b_idx / g.s : 0, b_ss = b_idx > 0 ? b_idx - b_rr * g.s : 0;
-        int issued = 0, st = 0, ph = 0;
+        int issued = 0, st = 0, ph = 0;                          // ph: parity of the lap
         for (int it = 0; it < nchunks; ++it) {
-            const uint32_t full = smem_u32(&bar_full[st]);
+            const uint32_t full = smem_u32(&bar_full[st + (ph ? P.stages : 0)]);
             int ok = 1;
             if (lane == 0) {
                 if (it >= P.stages && !mbar_wait(smem_u32(&bar_empty[st]), ph ^ 1)) { s_abort = 1; atomicOr(status, 1u); }
@@ -305,7 +310,7 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constan
             if (++st == P.stages) { st = 0; ph ^= 1; }
         }
         if (lane == 0 && s_abort) {   // drain: wait (bounded) for the copies already issued
-            for (int it = max(0, issued - P.stages); it < issued; ++it) mbar_wait(smem_u32(&bar_full[it % P.stages]), (it / P.stages) & 1);
+            for (int it = max(0, issued - P.stages); it < issued; ++it) mbar_wait(smem_u32(&bar_full[it % (2 * P.stages)]), (it / (2 * P.stages)) & 1);
         }
     } else if (warp >= 1 && warp <= 3 && warp - 1 < P.issuers && lane == 0) {
         const int issuer = warp - 1;
@@ -347,11 +352,11 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constan
         const uint32_t idesc = P.idesc;
         const int mine = P.dual ? issuer : 0, it_step_mask = P.dual ? 1 : 0;
         const uint32_t a_small = (uint32_t)P.a_plane_bytes >> 4, b_small = (uint32_t)P.b_plane_bytes >> 4;      // fp32, three passes
-        int st = 0, ph = 0;
+        int st = 0, lap = 0;
         bool fresh = true;            // the next k-step starts the accumulation (overwrites TMEM)
         for (int it = 0; it < nchunks; ++it) {
             if ((it & it_step_mask) == mine) {
-                if (!mbar_wait(smem_u32(&bar_full[st]), ph)) { s_abort = 1; atomicOr(status, 1u); break; }
+                if (!mbar_wait(smem_u32(&bar_full[st + (lap & 1 ? P.stages : 0)]), (lap >> 1) & 1)) { s_abort = 1; atomicOr(status, 1u); break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 GACONV_TL(1, it == 0 && issuer == 0);
                 const uint32_t sa = smem_base + st * P.stage_bytes;
@@ -394,7 +399,7 @@ exact_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constan
                 }
                 umma_commit(smem_u32(&bar_empty[st]));   // frees the stage once these MMAs have read it
             }
-            if (++st == P.stages) { st = 0; ph ^= 1; }
+            if (++st == P.stages) { st = 0; ++lap; }
         }
         umma_commit(smem_u32(&bar_acc));             // accumulators complete
         GACONV_TL(2, issuer == 0);
