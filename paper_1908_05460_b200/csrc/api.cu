@@ -204,6 +204,11 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, const ClPlan& plan, bool reo
             if (products < 3e7) return false;
             if (reordered) return true;                             // 128->128 on 16x16, dY channels last 28.4 / 17.8
             if (g.c <= 16 || (g.c < 64 && shared)) return false;    // 16->16 on 32x32 11.9 / 12.5; on 18 SMs 28 / 38
+            // 64 channels on few SMs: the older kernel's M = 64 fits, this one's 128 lanes are half idle or its tiles shared, until the
+            // main loop outweighs the rest (on 12 lanes beside copies of itself, us a layer: 64->64 on 8x8, N = 32 1.84 / 1.96,
+            // N = 128 2.69 / 2.93, N = 200 3.38 / 3.45, N = 512 6.3 / 5.8; 64->40 on 16x16, N = 64 3.0 / 3.8; not with 16 outputs,
+            // 64->16 on 16x16 3.8 / 3.4, nor at stride 2, 64->64 on 16x16 4.1 / 2.8; exact phase of a ResNet-20 step 77 / 80)
+            if (shared && g.c <= 64 && g.k > 16 && g.k <= 64 && g.stride_h == 1 && products < 5e8) return false;
             return g.r < 5;                                         // 5x5 64->64 on 16x16 16.1 / 17.8, 3x3 64->64 on 32x32 24.1 / 22.5
         }
         if (L.stem_ok) return reordered || (!shared && g.r * g.s * g.c > 32);       // 5x5 3->64 26.4 / 22.6, 3x3 3->16 10.4 / 14.8
