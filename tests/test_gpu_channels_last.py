@@ -8,30 +8,30 @@ from oracle import oracle
 from paper_1908_05460_b200 import binding as B
 from paper_1908_05460_b200 import inputs as I
 from paper_1908_05460_b200.layers import ConvLayer
-from helpers import GpuLayer, norm_err, oshape, to_f64, TOL_F32
+from helpers import GpuLayer, kernel_names, norm_err, oshape, to_f64, TOL_F32
 
 pytestmark = pytest.mark.gpu
 
-# (no other tensor-core kernel tiles these maps; each has more than the 4 million products the kernel is used from)
+# (no other tensor-core kernel tiles these maps; each has more products than the kernel is used from, in both types)
 SHAPES = [
-    ConvLayer("13x11 c19 k87", 5, 19, 13, 11, 87, 3, 3, 1, 1, dy_std=1.0),
+    ConvLayer("13x11 c19 k87", 15, 19, 13, 11, 87, 3, 3, 1, 1, dy_std=1.0),
     ConvLayer("28x20 c72 k120", 3, 72, 28, 20, 120, 3, 3, 1, 1),
     ConvLayer("7x7 maps, several images, c130 k260", 9, 130, 7, 7, 260, 3, 3, 1, 1),
     ConvLayer("9x24 row pairs, odd rows", 4, 64, 9, 24, 64, 3, 3, 1, 1),
     ConvLayer("stride 2, 27x27 -> 14x14", 4, 64, 27, 27, 100, 3, 3, 2, 1),
-    ConvLayer("stride 2, no padding, 5x5", 3, 40, 21, 17, 48, 5, 5, 2, 0),
-    ConvLayer("7x7 filter, stride 2, 3 channels", 6, 3, 33, 31, 64, 7, 7, 2, 3),
+    ConvLayer("stride 2, no padding, 5x5", 8, 40, 21, 17, 48, 5, 5, 2, 0),
+    ConvLayer("7x7 filter, stride 2, 3 channels", 11, 3, 33, 31, 64, 7, 7, 2, 3),
     ConvLayer("7x7 filter c33", 2, 33, 19, 12, 30, 7, 7, 1, 3),
     ConvLayer("1x1 c200 k72", 7, 200, 11, 5, 72, 1, 1, 1, 0),
     ConvLayer("many splits, k8", 60, 20, 25, 19, 8, 3, 3, 1, 1),
-    ConvLayer("one output channel", 40, 48, 31, 15, 1, 3, 3, 1, 1),
+    ConvLayer("one output channel", 102, 48, 31, 15, 1, 3, 3, 1, 1),
     ConvLayer("5x3 maps, more tiles than SMs", 3, 400, 5, 3, 530, 3, 3, 1, 1),
     ConvLayer("3x5 filter", 6, 36, 18, 18, 44, 3, 5, 1, 1),
     ConvLayer("stacked filter rows, 5x5, two row tiles", 12, 72, 17, 11, 40, 5, 5, 1, 2),
     ConvLayer("13 outputs, no padding", 30, 100, 12, 9, 13, 3, 3, 1, 0),
     ConvLayer("stacked filter rows, (pixel, image) order, odd pixels", 30, 130, 5, 9, 40, 5, 5, 1, 2),
     ConvLayer("7x3 filter", 9, 70, 12, 16, 64, 7, 3, 1, 1),
-    ConvLayer("odd pixels past a tile, 3 and 70 channels", 3, 3, 33, 35, 70, 3, 3, 1, 1),
+    ConvLayer("odd pixels past a tile, 3 and 70 channels", 15, 3, 33, 35, 70, 3, 3, 1, 1),
     ConvLayer("odd pixels, 24 and 12 channels", 9, 24, 21, 15, 12, 5, 5, 1, 2),
 ]
 LAYOUTS = {"paper": {}, "nchw": dict(x_layout=B.X_NCHW, dw_layout=B.DW_KCRS),
@@ -50,6 +50,7 @@ def test_every_layout_matches_the_oracle(li, dtype):
         before = B.gaconv_launch_count()
         got = g.exact()
         assert B.gaconv_launch_count() - before <= 3, name
+        assert any("cl_kernel" in k for k in kernel_names(lambda: B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc))), name
         assert norm_err(got, ref, dn) <= TOL_F32 / 2, name        # bf16 products are exact in fp32 as well
         np.testing.assert_array_equal(got, g.exact())
         # the same operands, however they were handed over; only a bf16 gradient on rows of whole 16-byte pieces is read as it
@@ -108,3 +109,6 @@ def test_large_strides(li, dtype):
         g = GpuLayer(layer, dtype, x, dy, alpha=0.5, **kw)
         assert norm_err(g.exact(), ref, dn) <= TOL_F32, name
         assert B.gaconv_poll_async_status(g.desc) == B.OK
+        if li in (0, 3):
+            names = kernel_names(lambda: B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc))
+            assert any("cl_kernel" in k for k in names) == (layer.stride <= 8), names
