@@ -107,8 +107,12 @@ gaconv_status_t gaconv_workspace_init(void *workspace, size_t bytes, void *strea
  *   dw[k,c,r,s] = alpha * sum_{n,p,q} Xz[n,c,p*stride_h+r-pad_h,q*stride_w+s-pad_w] * dy[n,k,p,q]
  * with Xz = x, zero outside the image; cross-correlation, no filter flip.
  * x: n*c*h*w elements of in_dtype in x_layout; dy: n*k*p*q elements in dy_layout; dw: k*c*r*s floats
- * in dw_layout (written).  Errors: NULL_POINTER, BAD_DESC, MISALIGNED, UNSUPPORTED,
- * WORKSPACE_TOO_SMALL, CUDA. */
+ * in dw_layout (written).
+ * Values that are not finite: where the channels-last tensor-core kernel takes the call, an element is NaN if a NaN or infinities
+ * of both signs are among its products, an infinity if infinities of one sign are, and no other element is
+ * touched; a product of the padding (a zero) with an Inf or NaN of dy counts as NaN or not at all.  The other kernels may
+ * give NaN for an infinity, and in further elements that the value's channel takes part in.
+ * Errors: NULL_POINTER, BAD_DESC, MISALIGNED, UNSUPPORTED, WORKSPACE_TOO_SMALL, CUDA. */
 gaconv_status_t gaconv_dw_exact(const void *x, const void *dy, float *dw,
                                 const gaconv_conv_desc_t *desc, void *stream);
 

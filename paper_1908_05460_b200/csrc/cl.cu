@@ -40,6 +40,12 @@
 // (Adding them over a thread-block cluster's shared memory instead costs more: reads from other SMs came to ~10 bytes a cycle,
 // where the workspace takes 21, and clusters of six leave SMs idle: 256->256 on 8x8, N = 128 19.1 us against 18.8.)
 //
+// Values that are not finite.  An Inf has no planes to split into (x - x0 = Inf - Inf), and the zero dY rows that end a chunk meet
+// real X rows, so that an Inf or NaN there reaches elements it has no part in.  But nothing is hidden: what has an infinite or
+// NaN product among those it should have comes out of the tensor core not finite.  So the writers look at every element, and
+// those that are not finite are summed anew, product by product from the operands as they were handed over (cl_repair).
+// (What may be missing are products of the padding with an Inf or NaN in dY: the orders and forms that skip the padding skip them.)
+//
 // Every wait is bounded; on expiry the kernel raises the workspace status word, lets its copies land, frees its tensor
 // memory and returns.
 #include <cuda.h>
@@ -148,6 +154,58 @@ __device__ __forceinline__ int lane_target(const ClParams& P, int l, int k0, int
     return j < P.rc && r < P.r && k < P.k ? (int)(k * P.ws_k + r * P.ws_r) : -1;
 }
 
+// The operands as the caller has them
+struct ClSource { const void *x, *dy; int f32, x_last, dy_last; };        // *_last: channels last
+
+__device__ __forceinline__ double cl_load(const void* p, size_t i, int f32)
+{
+    return f32 ? static_cast<const float*>(p)[i] : __bfloat162float(static_cast<const __nv_bfloat16*>(p)[i]);
+}
+// Element (column, lane) of a tile
+struct ClElement { int k, c, r, s; bool valid; };
+__device__ __forceinline__ ClElement cl_element(const ClParams& P, int tile, int col, int l)
+{
+    const int tr = tile / P.tiles_r, r0 = (tile - tr * P.tiles_r) * P.rc, tk = tr / P.tiles_c, k0 = tk * P.kt, c0 = (tr - tk * P.tiles_c) * P.ct;
+    const int gi = col / P.nmma, j = col - gi * P.nmma, ca_log = 31 - __clz(P.ca), ka_log = 31 - __clz(P.ka);
+    const ClGroup& g = P.g[gi];
+    const int mn = P.c_side ? l : j, a = P.merged ? 0 : mn >> ca_log;
+    ClElement e;
+    e.c = c0 + g.cbase + (P.merged ? mn : mn & (P.ca - 1)); e.s = g.s0 + P.stride * a;
+    e.k = P.c_side ? k0 + j : P.stack ? l & (P.ka - 1) : k0 + l;
+    e.r = r0 + (P.stack ? P.rc - 1 - (l >> ka_log) : g.r);
+    e.valid = e.k < P.k && e.c < P.c && a < g.cnt && e.r >= r0 && e.r < P.r;
+    return e;
+}
+// A warp sums the elements of the lanes in `left` anew, one by one, its lanes the output pixels in turn.  The padding counts as
+// zeros that are multiplied.  In double, so that finite sums do not depend on the order; a NaN ends the sum.
+// Never called on finite data, so that its speed is no matter.
+__device__ __noinline__ void cl_repair(const ClParams& P, const ClSource& S, float* dw, int tile, int col, int l, uint32_t left)
+{
+    const int lane = threadIdx.x & 31, px = P.p * P.q, all = P.n * px;
+    const ClElement mine = cl_element(P, tile, col, l);
+    while (left != 0) {
+        const int owner = __ffs(left) - 1;
+        left &= left - 1;
+        const int k = __shfl_sync(0xffffffffu, mine.k, owner), c = __shfl_sync(0xffffffffu, mine.c, owner);
+        const int r = __shfl_sync(0xffffffffu, mine.r, owner), s = __shfl_sync(0xffffffffu, mine.s, owner);
+        double sum = 0;
+        for (int base = 0; base < all; base += 32) {
+            const int i = base + lane;
+            if (i < all) {
+                const int n = i / px, p = (i - n * px) / P.q, q = i - n * px - p * P.q;
+                const int h = p * P.stride + r - P.pad_h, w = q * P.stride + s - P.pad_w;
+                const bool in = h >= 0 && h < P.h && w >= 0 && w < P.w;
+                const size_t xi = S.x_last ? (((size_t)n * P.h + h) * P.w + w) * P.c + c : (((size_t)n * P.c + c) * P.h + h) * P.w + w;
+                const size_t yi = S.dy_last ? (size_t)i * P.k + k : ((size_t)n * P.k + k) * px + (i - n * px);
+                sum += (in ? cl_load(S.x, xi, S.f32) : 0.0) * cl_load(S.dy, yi, S.f32);
+            }
+            if (__any_sync(0xffffffffu, isnan(sum))) break;
+        }
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) dw[k * P.ws_k + c * P.ws_c + r * P.ws_r + s * P.ws_s] = P.alpha * (float)sum;
+    }
+}
+
 // Warps: 0 and 1 issue MMAs, 2 and 3 fill the stages, 4 to 11 hold the sums.
 //
 // The tensor core adds into its accumulators by truncation, so an accumulator's error grows with the number of additions
@@ -160,7 +218,7 @@ constexpr int kThreads = 384, kMaxCols = 192;
 template <int NG, bool F32, bool CSIDE>
 __global__ void __launch_bounds__(kThreads, 1)
 cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CUtensorMap map_x, float* __restrict__ dw,
-          float* __restrict__ partial, uint32_t* __restrict__ status, const __grid_constant__ ClParams P)
+          float* __restrict__ partial, uint32_t* __restrict__ status, const __grid_constant__ ClParams P, const __grid_constant__ ClSource S)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[kMaxStages], bar_empty[kMaxStages], bar_acc[2], bar_free[2];
@@ -212,6 +270,7 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = s_tmem_base;
+    float finite = 0.f;         // NaN as soon as this thread has written an element that is not finite
     pdl_wait_prior_grid();
     GACONV_STAMP(1, threadIdx.x == 0);
 
@@ -395,9 +454,12 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
                         const int2 o = s_col[16 * (2 * i + half) + 8 * h];
                         const float* v = sum[i] + 8 * h;
                         const float a = P.alpha;
-                        if (o.y > 0)
+                        if (o.y > 0) {
+#pragma unroll
+                            for (int u = 0; u < 8; ++u) finite = fmaf(v[u], 0.f, finite);
                             asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d + o.x), "f"(a * v[0]), "f"(a * v[1]),
                                          "f"(a * v[2]), "f"(a * v[3]), "f"(a * v[4]), "f"(a * v[5]), "f"(a * v[6]), "f"(a * v[7]) : "memory");
+                        }
                     }
                 }
         } else if (ok) {        // the block (the stages are free: every copy has landed and every MMA has read)
@@ -450,7 +512,8 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
 #pragma unroll 4
                 for (int col = third; col < cols; col += 3) {
                     const int2 o = s_col[col];
-                    if (a < o.y) d[o.x] = P.alpha * blk[col * 128 + (l ^ block_key(col, ca_log))];
+                    const float v = blk[col * 128 + (l ^ block_key(col, ca_log))];
+                    if (a < o.y) { d[o.x] = P.alpha * v; finite = fmaf(v, 0.f, finite); }
                 }
             }
         } else if (P.ws_c == 1 && (P.c & 3) == 0) {
@@ -465,7 +528,11 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
                     float v[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) v[i] = P.alpha * blk[(col + i) * 128 + (l ^ block_key(col + i, ca_log))];
-                    if (o.y > 0) *reinterpret_cast<float4*>(dw + lane_off + o.x) = make_float4(v[0], v[1], v[2], v[3]);
+                    if (o.y > 0) {
+                        *reinterpret_cast<float4*>(dw + lane_off + o.x) = make_float4(v[0], v[1], v[2], v[3]);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) finite = fmaf(v[i], 0.f, finite);
+                    }
                 }
             }
         } else {
@@ -485,11 +552,22 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
                     float* d = dw + lane_off;
 #pragma unroll
                     for (int u = 0; u < 2; ++u)
-                        if (off[u] >= 0) d[off[u]] = P.alpha * blk[pos[u] + (l ^ key[u])];
+                        if (off[u] >= 0) {
+                            const float v = blk[pos[u] + (l ^ key[u])];
+                            d[off[u]] = P.alpha * v;
+                            finite = fmaf(v, 0.f, finite);
+                        }
                 }
             }
         }
     }
+    if (P.splits == 1 && __syncthreads_or(isnan(finite)) && !s_abort)
+        for (int e = warp; e < 4 * P.cols; e += kThreads / 32) {
+            const int col = e >> 2, l = 32 * (e & 3) + lane;
+            const ClElement el = cl_element(P, tile, col, l);
+            const uint32_t left = __ballot_sync(0xffffffffu, el.valid && !isfinite(__ldcg(dw + (el.k * P.ws_k + el.c * P.ws_c + el.r * P.ws_r + el.s * P.ws_s))));
+            if (left != 0) cl_repair(P, S, dw, tile, col, l, left);
+        }
     GACONV_STAMP(5, threadIdx.x == 0);
 }
 
@@ -498,8 +576,12 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
 // chosen so that a warp's loads are all in flight at once (eight, then a second round), CB so that the grid covers the GPU;
 // where consecutive columns are consecutive channels of dW a block writes CB of them in one piece.  Latency-bound: what an
 // element is, and where it goes, is worked out before the wait for the sums.
-__global__ void __launch_bounds__(1024)
-cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, const __grid_constant__ ClParams P, int log_cb, int G)
+// SHARED, for launches that share the GPU: registers for two blocks an SM.  On a GPU of its own there are no more blocks than SMs, and
+// with 64 registers instead of 32 all eight loads of a thread are in flight (fp32 64->128 stride 2 on 28x28, N = 64, whole
+// call: 32.7 -> 31.3 us); beside other layers that costs more than it gives (step of ResNet-20 150 -> 154).
+template <bool SHARED>
+__global__ void __launch_bounds__(1024, SHARED ? 2 : 1)
+cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, const __grid_constant__ ClParams P, const __grid_constant__ ClSource S, int log_cb, int G)
 {
     __shared__ float s_sum[32][128];
     __shared__ int2 s_col[16];
@@ -548,10 +630,14 @@ cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, cons
             valid = o.y > 0 && lane_off >= 0;
             off += lane_off;
         }
-        if (!valid) continue;
-        float t = s_sum[c][l];
-        for (int w = 1; w < G; ++w) t += s_sum[(w << log_cb) + c][l];
-        dw[off] = P.alpha * t;
+        float t = 0.f;
+        if (valid) {
+            t = s_sum[c][l];
+            for (int w = 1; w < G; ++w) t += s_sum[(w << log_cb) + c][l];
+            dw[off] = P.alpha * t;
+        }
+        const uint32_t left = __ballot_sync(0xffffffffu, !isfinite(t));        // (a warp's lanes come and go together: CB * 128 elements)
+        if (left != 0) cl_repair(P, S, dw, tile, written_column(P, min(col0 + c, P.cols - 1)), l, left);
     }
 }
 
@@ -963,6 +1049,7 @@ struct ClHost {             // what ClPlan::opaque holds
     bool pack_x, pack_dy, f32, x_nhwc, dy_npqk;
     int xch, dych;          // channels per pixel row of the operands the tensor maps describe
     int log_cb, groups;     // second kernel: columns per block, split groups per column
+    bool shared;            // other layers run beside this one
 };
 static_assert(sizeof(ClHost) <= sizeof(ClPlan::opaque), "ClPlan::opaque too small");
 
@@ -991,7 +1078,7 @@ PackOp pack_op(const void* src, void* dst, int ch, int px, int n, bool last, siz
     return o;
 }
 
-typedef void (*ClKernel)(const CUtensorMap, const CUtensorMap, float*, float*, uint32_t*, const ClParams);
+typedef void (*ClKernel)(const CUtensorMap, const CUtensorMap, float*, float*, uint32_t*, const ClParams, const ClSource);
 ClKernel kernel_for(int ng, bool f32, bool c_side)
 {
 #define GACONV_CL_PICK(N) if (ng <= N) return f32 ? (c_side ? cl_kernel<N, true, true> : cl_kernel<N, true, false>) : (c_side ? cl_kernel<N, false, true> : cl_kernel<N, false, false>);
@@ -1009,6 +1096,7 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
     const bool nhwc = g.xs_c == 1 || g.c == 1;
     ClHost H{};
     H.f32 = !g.bf16;
+    H.shared = g.sm_budget > 0;
     H.x_nhwc = nhwc; H.dy_npqk = dy_npqk || g.k == 1;
     H.pack_x = H.f32 || !nhwc || g.c % 8 != 0;
     H.pack_dy = H.f32 || !H.dy_npqk || g.k % 8 != 0;
@@ -1149,6 +1237,7 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
     memcpy(&H, plan.opaque, sizeof(H));
     const ClParams& P = H.p;
     cudaError_t err;
+    const ClSource src{x, dy, H.f32, H.x_nhwc, H.dy_npqk};
     const size_t x_el = (size_t)P.n * P.h * P.w * H.xch, dy_el = (size_t)P.n * P.p * P.q * H.dych;
     if (H.pack_x || H.pack_dy) {
         PackOp ox{}, od{};
@@ -1193,12 +1282,12 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
     const dim3 grid((unsigned)(P.tiles_k * P.tiles_c * P.tiles_r), (unsigned)P.splits);
     ClKernel kern = kernel_for(P.ngroups, H.f32, P.c_side != 0);
     if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return err;
-    if ((err = launch_kernel(kern, grid, dim3(kThreads), smem, stream, dim3(1, 1, 1), map_dy, map_x, dw, partial, status, P)) != cudaSuccess) return err;
+    if ((err = launch_kernel(kern, grid, dim3(kThreads), smem, stream, dim3(1, 1, 1), map_dy, map_x, dw, partial, status, P, src)) != cudaSuccess) return err;
     note_launch();
     if (P.splits == 1) return cudaSuccess;
     const dim3 rgrid((unsigned)ceil_div(P.cols, 1 << H.log_cb), grid.x);
-    err = launch_kernel(cl_reduce_kernel, rgrid, dim3(32u * H.groups << H.log_cb), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P,
-                        H.log_cb, H.groups);
+    err = launch_kernel(H.shared ? cl_reduce_kernel<true> : cl_reduce_kernel<false>, rgrid, dim3(32u * H.groups << H.log_cb), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P,
+                        src, H.log_cb, H.groups);
     if (err != cudaSuccess) return err;
     note_launch();
     return cudaSuccess;

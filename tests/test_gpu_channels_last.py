@@ -112,3 +112,47 @@ def test_large_strides(li, dtype):
         if li in (0, 3):
             names = kernel_names(lambda: B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc))
             assert any("cl_kernel" in k for k in names) == (layer.stride <= 8), names
+
+
+def _without_padding(x, dy, layer, k):
+    """dW[k] with the products of the padding left out (they are zeros unless dY is not finite there)."""
+    l, out = layer, np.zeros((layer.c, layer.r, layer.s))
+    for r in range(l.r):
+        for s in range(l.s):
+            ps = [p for p in range(l.p) if 0 <= p * l.stride + r - l.pad < l.h]
+            qs = [q for q in range(l.q) if 0 <= q * l.stride + s - l.pad < l.w]
+            xs = x[:, :, [p * l.stride + r - l.pad for p in ps]][:, :, :, [q * l.stride + s - l.pad for q in qs]]
+            out[:, r, s] = (xs * dy[:, k:k + 1][:, :, ps][:, :, :, qs]).sum(axis=(0, 2, 3))
+    return out
+
+
+def _alike(got, ref, bound):
+    with np.errstate(invalid="ignore"):
+        return (np.isnan(got) & np.isnan(ref)) | (got == ref) | (np.abs(got - ref) <= bound)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
+@pytest.mark.parametrize("li", range(len(SHAPES)), ids=[l.name for l in SHAPES])
+def test_values_that_are_not_finite(li, dtype):
+    """Infinities and NaNs reach the elements that they are part of, and no others; an infinite product stays infinite."""
+    layer = SHAPES[li]
+    l = layer
+    x, dy = I.make_layer_inputs(layer, dtype, 18, li)
+    inf, nan = float("inf"), float("nan")
+    x[0, 0, 0, 0], x[1, l.c // 2, l.h - 1, l.w - 1], x[l.n - 1, l.c - 1, l.h // 2, l.w // 2] = inf, -inf, nan
+    if l.k > 2:
+        dy[0, 0, l.p // 2, l.q // 2], dy[l.n - 1, l.k // 2, 0, 0], dy[1, l.k - 1, l.p - 1, l.q - 1] = inf, -inf, nan
+    xd, dyd = to_f64(x), to_f64(dy)
+    with np.errstate(invalid="ignore"):
+        ref, _ = oracle.dw_exact(xd, dyd, oshape(layer), 0.5)
+        bare = ref.copy()
+        for k in {0, l.k // 2, l.k - 1}:
+            bare[k] = 0.5 * _without_padding(xd, dyd, layer, k)
+        _, dn = oracle.dw_exact(np.where(np.isfinite(xd), xd, 0.0), np.where(np.isfinite(dyd), dyd, 0.0), oshape(layer), 0.5)
+    assert np.isinf(ref).any() and np.isnan(ref).any()
+    for kw in (LAYOUTS["paper"], LAYOUTS["rsck"], dict(sm_budget=1), dict(LAYOUTS["nchw"], sm_budget=1)):       # (one SM: one split)
+        g = GpuLayer(layer, dtype, x, dy, alpha=0.5, **kw)
+        got = g.exact()
+        ok = _alike(got, ref, TOL_F32 * dn) | _alike(got, bare, TOL_F32 * dn)
+        assert ok.all(), (kw, int((~ok).sum()), np.argwhere(~ok)[:3].tolist())
+        np.testing.assert_array_equal(got, g.exact())
