@@ -1092,7 +1092,7 @@ ClKernel kernel_for(int ng, bool f32, bool c_side)
 
 bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
 {
-    if (g.stride_h != g.stride_w || g.stride_h > kMaxMapStep || g.r > 16 || g.s > 16) return false;
+    if (g.stride_h != g.stride_w || g.stride_h > kMaxMapStep || g.r > 16 || g.s > 16 || !dw_offsets_fit(g)) return false;
     const bool nhwc = g.xs_c == 1 || g.c == 1;
     ClHost H{};
     H.f32 = !g.bf16;

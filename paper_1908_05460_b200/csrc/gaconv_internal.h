@@ -65,6 +65,9 @@ struct Geom {
     int sm_budget;                      // 0: plan for the whole GPU; n > 0: for about n SMs
 };
 
+// the tcgen05 kernels keep offsets in dW as 32-bit numbers
+inline bool dw_offsets_fit(const Geom& g) { return (long long)g.k * g.c * g.r * g.s <= 0x7fffffffll; }
+
 // ---- out[b][j][i] = in[b][i][j], i < rows, j < cols: N x C x H x W activations -> N x H x W x C, N x P x Q x K gradients -> N x K x P x Q ----
 cudaError_t launch_transpose_batched(const void* in, void* out, int rows, int cols, int batch, bool bf16, cudaStream_t stream);
 

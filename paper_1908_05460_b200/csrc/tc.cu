@@ -801,7 +801,7 @@ bool tensor_maps_available() { return encode_fn() != nullptr; }
 
 bool plan_tc(const Geom& g, TcPlan* out)
 {
-    if (!g.bf16) return false;
+    if (!g.bf16 || !dw_offsets_fit(g)) return false;
     if (g.xs_c != 1 || g.c % 8 != 0) return false;                       // NHWC with 16-byte pixel rows
     if (g.stride_h != g.stride_w || g.stride_h > kMaxMapStep) return false;
     const int pq = g.p * g.q;
@@ -962,7 +962,7 @@ bool plan_tc(const Geom& g, TcPlan* out)
 // output pixels.  passes = 3 (fp32 accuracy through split operands) or 1 (plain TF32).
 bool plan_tc_f32(const Geom& g, int passes, TcPlan* out)
 {
-    if (g.bf16 || g.xs_c != 1 || g.c % 32 != 0) return false;
+    if (g.bf16 || g.xs_c != 1 || g.c % 32 != 0 || !dw_offsets_fit(g)) return false;
     if (g.stride_h != 1 || g.stride_w != 1 || g.r > 7 || g.s > 7 || g.s * 32 > 256) return false;
     const int pq = g.p * g.q;
     if (pq % 32 != 0 || g.q % 8 != 0 || 32 % g.q != 0) return false;          // a 32-pixel box is whole rows, a k-step lies in a row

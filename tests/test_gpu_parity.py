@@ -714,3 +714,22 @@ def test_autograd_module_matches_the_frameworks_filter_gradient_and_follows_the_
             got = conv2.weight.grad.double().cpu().numpy()
             assert norm_err(got, ref, dn) <= 1e-4        # torch's forward runs in TF32/fp32: the activations differ in the last bits
             assert not torch.allclose(conv2.weight.grad, w2.grad, rtol=1e-2, atol=1e-3)
+
+
+def test_results_of_more_than_two_gigaelements():
+    """Offsets in dW that do not fit 32 bits: the tcgen05 kernels, which keep them so, leave the call to one that does not."""
+    n, c, k = 64, 46400, 46400
+    layer, dtype = ConvLayer("huge dW", n, c, 1, 1, k, 1, 1, 1, 0), torch.bfloat16
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x, dy = (torch.randn(n, ch, generator=g, device="cuda").to(dtype) for ch in (c, k))
+    desc = B.make_desc(layer, dtype)
+    ws = B.attach_workspace(desc, methods=(B.METHOD_EXACT,))
+    dw = torch.full((k, c), float("nan"), device="cuda")
+    B.gaconv_dw_exact(x, dy, dw, desc)
+    worst = 0.0
+    for k0 in range(0, k, 2900):
+        want, norm = (a[:, k0:k0 + 2900].double().t() @ b.double() for a, b in ((dy, x), (dy.abs(), x.abs())))
+        worst = max(worst, float(((dw[k0:k0 + 2900] - want).abs() / norm).nan_to_num(nan=1e30).max()))
+    assert worst <= TOL_F32 and B.gaconv_poll_async_status(desc) == B.OK
+    del dw, ws
+    torch.cuda.empty_cache()
