@@ -125,14 +125,14 @@ bool top1_dense_route(const Geom& g, TcPlan* tp)
 }
 
 struct Top1Layout { size_t idx_off, sum_off, partial_off, sparse_off, scratch_off, total; GatherPlan gp; TcPlan tp; ClPlan cp; bool dense, cl; };
-Top1Layout build_top1_layout(const Geom& g)
+Top1Layout build_top1_layout(const Geom& g, bool cl)
 {
     Top1Layout L;
     L.gp = plan_gather(g);
     L.dense = top1_dense_route(g, &L.tp);
     // the contraction: by the channels-last kernel, which reads either form of the sparse tensor (256->256 on 8x8, N = 256:
     // 37 us with the other kernel, 32)
-    L.cl = L.dense && tensor_maps_available() && plan_cl(g, L.tp.reads_transposed_dy, &L.cp) && !short_sums(g, L.cp);
+    L.cl = cl && L.dense && tensor_maps_available() && plan_cl(g, L.tp.reads_transposed_dy, &L.cp) && !short_sums(g, L.cp);
     const size_t cl_scratch = L.cl ? L.cp.x_bytes + L.cp.dy_bytes : 0;
     const size_t maps = (size_t)g.n * g.k;
     L.idx_off = kWsDataOffset;
@@ -146,10 +146,11 @@ Top1Layout build_top1_layout(const Geom& g)
     return L;
 }
 
-Top1Layout top1_layout(const Geom& g)
+// cl = false: without the channels-last kernel (workspaces that its packed operand does not fit)
+Top1Layout top1_layout(const Geom& g, bool cl)
 {
     static PlanCache<Top1Layout> cache;
-    return cache.get(plan_key(g, 0, 0), [&] { return build_top1_layout(g); });
+    return cache.get(plan_key(g, cl, 0), [&] { return build_top1_layout(g, cl); });
 }
 
 struct ExactLayout { size_t partial_off, scratch_off, total; DirectPlan dp; TcPlan tp; StemPlan sp; bool tc_ok, stem_ok; };
@@ -303,12 +304,13 @@ size_t x_bytes_of(const gaconv_conv_desc_t* d) { return (size_t)d->n * d->c * d-
 size_t dy_bytes_of(const Geom& g) { return (size_t)g.n * g.k * g.p * g.q * (g.bf16 ? 2 : 4); }
 
 // workspace of a call in the kernels' own dY layout (x in either layout); 0 with *ok = false when the descriptor is bad
-size_t native_ws_bytes(const gaconv_conv_desc_t* desc, const Geom& g, int32_t method, bool* ok)
+// (cl: with the channels-last kernel in the dense route of top-1; the exact method's takes every layout and is not asked here)
+size_t native_ws_bytes(const gaconv_conv_desc_t* desc, const Geom& g, int32_t method, bool cl, bool* ok)
 {
     *ok = true;
     switch (method) {
         case GACONV_METHOD_EXACT: return exact_layout(g, desc->math, desc->algo).total;
-        case GACONV_METHOD_TOP1: return top1_layout(g).total;
+        case GACONV_METHOD_TOP1: return top1_layout(g, cl).total;
         case GACONV_METHOD_TOPK: {
             const int t = topk_of(desc, g);
             if (t < 1) { *ok = false; return 0; }
@@ -322,7 +324,7 @@ size_t native_ws_bytes(const gaconv_conv_desc_t* desc, const Geom& g, int32_t me
 }
 
 // which operands move, and the inner call's workspace size; move_x == move_dy == false: the call runs as it is
-Relayout plan_relayout(const gaconv_conv_desc_t* desc, int32_t method)
+Relayout plan_relayout(const gaconv_conv_desc_t* desc, int32_t method, bool cl)
 {
     Relayout R{};
     R.inner = *desc;
@@ -331,28 +333,34 @@ Relayout plan_relayout(const gaconv_conv_desc_t* desc, int32_t method)
     R.move_dy = desc->dy_layout == GACONV_DY_NPQK && desc->k > 1;          // (one output channel: the two orders coincide)
     R.inner.dy_layout = GACONV_DY_NKPQ;
     if (desc->x_layout == GACONV_X_NCHW && desc->c >= 2 && desc->algo != GACONV_ALGO_DIRECT) {
-        gaconv_conv_desc_t cl = R.inner;
-        cl.x_layout = GACONV_X_NHWC;
+        gaconv_conv_desc_t nhwc = R.inner;
+        nhwc.x_layout = GACONV_X_NHWC;
         Geom gi;
-        if (make_geom(&cl, &gi) == GACONV_OK) {
+        if (make_geom(&nhwc, &gi) == GACONV_OK) {
             if (method == GACONV_METHOD_EXACT) {
                 const ExactLayout L = exact_layout(gi, desc->math, desc->algo);
                 R.move_x = L.tc_ok || L.stem_ok || direct_mma_supported(gi, L.dp);
             } else if (method == GACONV_METHOD_TOP1) {
-                R.move_x = top1_layout(gi).dense || (top1_fused_supported(gi) && gi.c % 4 == 0);
+                R.move_x = top1_layout(gi, cl).dense || (top1_fused_supported(gi) && gi.c % 4 == 0);
             } else {
                 R.move_x = topk_of(desc, gi) >= 1 && top1_fused_supported(gi) && gi.c % 4 == 0;
             }
-            if (R.move_x) R.inner = cl;
+            if (R.move_x) R.inner = nhwc;
         }
     }
     if (R.move_x || R.move_dy) {
         Geom gi;
         bool ok = false;
-        if (make_geom(&R.inner, &gi) == GACONV_OK) R.inner_bytes = native_ws_bytes(&R.inner, gi, method, &ok);
+        if (make_geom(&R.inner, &gi) == GACONV_OK) R.inner_bytes = native_ws_bytes(&R.inner, gi, method, cl, &ok);
         if (!ok) { R.move_x = R.move_dy = false; R.inner = *desc; R.inner_bytes = 0; }
     }
     return R;
+}
+
+// the inner call's scratch, then the transposed copies
+size_t moved_ws_bytes(const gaconv_conv_desc_t* desc, const Geom& g, const Relayout& R)
+{
+    return align_up(R.inner_bytes, 256) + (R.move_x ? align_up(x_bytes_of(desc), 256) : 0) + (R.move_dy ? dy_bytes_of(g) : 0);
 }
 
 // Transposes what has to move into the workspace tail and hands back the inner descriptor and operand pointers.
@@ -360,15 +368,16 @@ Relayout plan_relayout(const gaconv_conv_desc_t* desc, int32_t method)
 gaconv_status_t relayout_operands(const void* x, const void* dy, const gaconv_conv_desc_t* desc, int32_t method, cudaStream_t cs,
                                   gaconv_conv_desc_t* inner, const void** x_out, const void** dy_out, bool* moved)
 {
-    const Relayout R = plan_relayout(desc, method);
+    Relayout R = plan_relayout(desc, method, true);
     *moved = R.move_x || R.move_dy;
     if (!*moved) return GACONV_OK;
     Geom g;
     gaconv_status_t st = make_geom(desc, &g);
     if (st != GACONV_OK) return st;
+    if (desc->workspace_bytes < moved_ws_bytes(desc, g, R)) R = plan_relayout(desc, method, false);
     const size_t head = align_up(R.inner_bytes, 256);
     const size_t x_tail = R.move_x ? align_up(x_bytes_of(desc), 256) : 0;
-    st = check_ws(desc, head + x_tail + (R.move_dy ? dy_bytes_of(g) : 0));
+    st = check_ws(desc, moved_ws_bytes(desc, g, R));
     if (st != GACONV_OK) return st;
     char* ws = static_cast<char*>(desc->workspace);
     *x_out = x; *dy_out = dy;
@@ -395,18 +404,19 @@ struct gaconv_schedule {
     struct StepCache* steps = nullptr;      // repeated steps as CUDA graphs, created on first use
 };
 
-gaconv_status_t gaconv::exact_workspace(const gaconv_conv_desc_t* desc, bool cl, size_t* bytes)
+gaconv_status_t gaconv::method_workspace(const gaconv_conv_desc_t* desc, int32_t method, bool cl, size_t* bytes)
 {
     Geom g;
     gaconv_status_t st = make_geom(desc, &g);
     if (st != GACONV_OK) return st;
     ClRoute C;
-    if (cl && cl_route(desc, g, &C)) { *bytes = C.total; return GACONV_OK; }
-    const Relayout R = plan_relayout(desc, GACONV_METHOD_EXACT);      // operands that are transposed first: the inner call's scratch, then the copies
-    if (R.move_x || R.move_dy)
-        *bytes = align_up(R.inner_bytes, 256) + (R.move_x ? align_up(x_bytes_of(desc), 256) : 0) + (R.move_dy ? dy_bytes_of(g) : 0);
-    else
-        *bytes = exact_layout(g, desc->math, desc->algo).total;
+    if (cl && method == GACONV_METHOD_EXACT && cl_route(desc, g, &C)) { *bytes = C.total; return GACONV_OK; }
+    const Relayout R = plan_relayout(desc, method, cl);
+    if (R.move_x || R.move_dy) { *bytes = moved_ws_bytes(desc, g, R); return GACONV_OK; }
+    bool ok = false;
+    const size_t need = native_ws_bytes(desc, g, method, cl, &ok);
+    if (!ok) return GACONV_ERR_BAD_DESC;
+    *bytes = need;
     return GACONV_OK;
 }
 
@@ -419,7 +429,8 @@ gaconv_status_t gaconv::run_exact(const void* x, const void* dy, float* dw, cons
     if (!aligned16(x) || !aligned16(dy) || !aligned16(dw)) return GACONV_ERR_MISALIGNED;
     if (desc->math == GACONV_MATH_TF32 && g.bf16) return GACONV_ERR_BAD_DESC;
     ClRoute C;
-    if (cl && cl_route(desc, g, &C)) {
+    // (a workspace without room for the packed operands: the kernels that need none, as far as it goes)
+    if (cl && cl_route(desc, g, &C) && (desc->workspace == nullptr || desc->workspace_bytes >= C.total)) {
         st = check_ws(desc, C.total);
         if (st != GACONV_OK) return st;
         char* ws = static_cast<char*>(desc->workspace);
@@ -429,7 +440,7 @@ gaconv_status_t gaconv::run_exact(const void* x, const void* dy, float* dw, cons
     if (desc->dy_layout == GACONV_DY_NPQK && g.k > 1 && desc->algo != GACONV_ALGO_DIRECT) {
         // Small maps: the tensor-core kernel's dY operand IS the channels-last order (its pre-pass would transpose an
         // N x K x P x Q gradient into it), so a channels-last gradient is read where it lies; only X may have to move.
-        const Relayout R = plan_relayout(desc, GACONV_METHOD_EXACT);
+        const Relayout R = plan_relayout(desc, GACONV_METHOD_EXACT, false);
         Geom gi;
         if (make_geom(&R.inner, &gi) == GACONV_OK) {
             const ExactLayout Li = exact_layout(gi, desc->math, desc->algo);
@@ -510,29 +521,7 @@ uint64_t gaconv_launch_count(void) { return g_launches.load(std::memory_order_re
 gaconv_status_t gaconv_workspace_size(const gaconv_conv_desc_t* desc, int32_t method, size_t* bytes)
 {
     if (bytes == nullptr) return GACONV_ERR_NULL_POINTER;
-    if (method == GACONV_METHOD_EXACT) return exact_workspace(desc, true, bytes);
-    Geom g;
-    gaconv_status_t st = make_geom(desc, &g);
-    if (st != GACONV_OK) return st;
-    {   // operands that are transposed first: the inner call's scratch, then the transposed copies
-        const Relayout R = plan_relayout(desc, method);
-        if (R.move_x || R.move_dy) {
-            *bytes = align_up(R.inner_bytes, 256) + (R.move_x ? align_up(x_bytes_of(desc), 256) : 0) + (R.move_dy ? dy_bytes_of(g) : 0);
-            return GACONV_OK;
-        }
-    }
-    switch (method) {
-        case GACONV_METHOD_TOP1: *bytes = top1_layout(g).total; return GACONV_OK;
-        case GACONV_METHOD_TOPK: {
-            const int t = topk_of(desc, g);
-            if (t < 1) return GACONV_ERR_BAD_DESC;
-            *bytes = topk_layout(g, t).total;
-            return GACONV_OK;
-        }
-        case GACONV_METHOD_ZERO:
-        case GACONV_METHOD_RANDOM: *bytes = kWsDataOffset; return GACONV_OK;
-    }
-    return GACONV_ERR_BAD_DESC;
+    return method_workspace(desc, method, true, bytes);
 }
 
 gaconv_status_t gaconv_workspace_init(void* workspace, size_t bytes, void* stream)
@@ -593,7 +582,8 @@ gaconv_status_t gaconv_dw_approx(int32_t method, const void* x, const void* dy, 
             return GACONV_ERR_CUDA;
         return GACONV_OK;
     }
-    const Top1Layout L = top1_layout(g);
+    Top1Layout L = top1_layout(g, true);
+    if (L.cl && desc->workspace_bytes < L.total) L = top1_layout(g, false);
     st = check_ws(desc, L.total);       // required by every route, so that behaviour does not depend on the kernel picked
     if (st != GACONV_OK) return st;
     char* ws = static_cast<char*>(desc->workspace);
@@ -668,7 +658,8 @@ static gaconv_status_t dw_from_host(int32_t method, const void* x_host, const vo
         if (!aligned16(x_dev) || !aligned16(dy_dev)) return GACONV_ERR_MISALIGNED;
         if (method == GACONV_METHOD_EXACT && desc->math == GACONV_MATH_TF32 && g.bf16) return GACONV_ERR_BAD_DESC;
         size_t need = 0;
-        st = gaconv_workspace_size(desc, method, &need);
+        st = method_workspace(desc, method, true, &need);
+        if (st == GACONV_OK && desc->workspace_bytes < need) st = method_workspace(desc, method, false, &need);
         if (st != GACONV_OK) return st;
         st = check_ws(desc, need);
         if (st != GACONV_OK) return st;

@@ -162,8 +162,8 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
 int device_sms();       // SMs of the current device
 bool tensor_maps_available();       // the driver's tensor-map encoder was found
 
-// gaconv_dw_exact and its workspace; cl = false: without the channels-last kernel (callers whose scratch it does not fit)
-gaconv_status_t exact_workspace(const gaconv_conv_desc_t* desc, bool cl, size_t* bytes);
+// gaconv_workspace_size and gaconv_dw_exact; cl = false: without the channels-last kernel (callers whose scratch it does not fit)
+gaconv_status_t method_workspace(const gaconv_conv_desc_t* desc, int32_t method, bool cl, size_t* bytes);
 gaconv_status_t run_exact(const void* x, const void* dy, float* dw, const gaconv_conv_desc_t* desc, cudaStream_t stream, bool cl);
 
 }  // namespace gaconv

@@ -156,3 +156,44 @@ def test_values_that_are_not_finite(li, dtype):
         ok = _alike(got, ref, TOL_F32 * dn) | _alike(got, bare, TOL_F32 * dn)
         assert ok.all(), (kw, int((~ok).sum()), np.argwhere(~ok)[:3].tolist())
         np.testing.assert_array_equal(got, g.exact())
+
+
+@pytest.mark.parametrize("method", ["exact", "host", "top1"])
+@pytest.mark.parametrize("layer,dtype,kw", [
+    (ConvLayer("packed planes", 24, 64, 30, 30, 64, 3, 3, 1, 1), torch.float32, {}),
+    (ConvLayer("packed gradient", 20, 72, 28, 20, 120, 3, 3, 1, 1), torch.bfloat16, {}),
+    (ConvLayer("packed, channels first", 20, 72, 28, 20, 120, 3, 3, 1, 1), torch.bfloat16, dict(x_layout=B.X_NCHW)),
+    (ConvLayer("top-1 by the dense route", 20, 256, 8, 8, 100, 3, 3, 1, 1), torch.bfloat16, dict(x_layout=B.X_NCHW, dy_layout=B.DY_NPQK)),
+], ids=lambda v: v.name if isinstance(v, ConvLayer) else None)
+def test_smaller_workspaces(layer, dtype, kw, method):
+    """Without room for packed operands the older kernels take the call; what is accepted stays within the bytes it was given."""
+    x, dy = I.make_layer_inputs(layer, dtype, 19, 0)
+    ref, dn = oracle.dw_top1(to_f64(x), to_f64(dy), oshape(layer)) if method == "top1" else oracle.dw_exact(to_f64(x), to_f64(dy), oshape(layer))
+    tol = 2.0 ** -8 + 1e-4 if method == "top1" and dtype == torch.bfloat16 else TOL_F32          # (the dense route rounds a map's sum once)
+    g = GpuLayer(layer, dtype, x, dy, **kw)
+    which = {"exact": B.METHOD_EXACT, "host": B.METHOD_EXACT, "top1": B.METHOD_TOP1}[method]
+    full, accepted = B.gaconv_workspace_size(g.desc, which), []
+    x_host, dy_host, dw_host = g.x.cpu().pin_memory(), g.dy.cpu().pin_memory(), g.dw.cpu().pin_memory()
+    ws = torch.empty(full + 4096, dtype=torch.uint8, device="cuda")
+    for size in [full, full - 16] + [max(17024, full * i // 32) for i in range(30, 0, -3)]:
+        ws.fill_(0x5a)
+        B.gaconv_workspace_init(ws, size)
+        g.desc.workspace, g.desc.workspace_bytes = ws.data_ptr(), size
+        try:
+            if method == "host":
+                dw_host.fill_(float("nan"))
+                B.gaconv_dw_from_host(B.METHOD_EXACT, x_host, dy_host, dw_host, g.x, g.dy, g.dw, g.desc)
+                got = g.logical_dw()
+                np.testing.assert_array_equal(dw_host.numpy(), g.dw.cpu().numpy())
+            else:
+                got = g.exact() if method == "exact" else g.approx(B.METHOD_TOP1)
+        except B.GaconvError as e:
+            assert e.status == B.ERR_WORKSPACE_TOO_SMALL
+            continue
+        assert norm_err(got, ref, dn) <= tol
+        assert bool((ws[size:] == 0x5a).all()), size
+        assert B.gaconv_poll_async_status(g.desc) == B.OK
+        accepted.append(size)
+    assert accepted[0] == full
+    if method != "top1" and "packed" in layer.name:
+        assert len(accepted) > 1, (full, accepted)
