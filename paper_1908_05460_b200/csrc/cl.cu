@@ -76,7 +76,8 @@ __device__ long long gaconv_tuning_cl[512][8];
 namespace gaconv {
 namespace {
 
-constexpr int kMaxGroups = 16, kMaxKsteps = 128, kMaxStages = 8;
+constexpr int kMaxCols = 192;                   // accumulator columns of a CTA
+constexpr int kMaxGroups = kMaxCols / 16, kMaxKsteps = 128, kMaxStages = 8;
 
 // order of the reduction inside a chunk, see above
 enum { kFlat = 0, kPaired = 1, kPixels = 2, kImages = 3 };
@@ -213,7 +214,7 @@ __device__ __noinline__ void cl_repair(const ClParams& P, const ClSource& S, flo
 // it to fp32 registers, and starts afresh: the error stays that of a short sum.  There are two sets and two issuers, which
 // take alternate chunks: while one waits (for data, for its set to be read, or merely for its own instructions), the other
 // keeps the tensor core busy.
-constexpr int kThreads = 384, kMaxCols = 192;
+constexpr int kThreads = 384;
 
 template <int NG, bool F32, bool CSIDE>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -1083,7 +1084,7 @@ ClKernel kernel_for(int ng, bool f32, bool c_side)
 {
 #define GACONV_CL_PICK(N) if (ng <= N) return f32 ? (c_side ? cl_kernel<N, true, true> : cl_kernel<N, true, false>) : (c_side ? cl_kernel<N, false, true> : cl_kernel<N, false, false>);
     GACONV_CL_PICK(1) GACONV_CL_PICK(2) GACONV_CL_PICK(3) GACONV_CL_PICK(4) GACONV_CL_PICK(5) GACONV_CL_PICK(6) GACONV_CL_PICK(7) GACONV_CL_PICK(8)
-    GACONV_CL_PICK(9) GACONV_CL_PICK(16)
+    GACONV_CL_PICK(9) GACONV_CL_PICK(kMaxGroups)
 #undef GACONV_CL_PICK
     return nullptr;
 }
