@@ -34,6 +34,9 @@ if ROOT not in sys.path:
 METRIC = "dW-conv us/layer"
 UNIT = "us/layer"
 WORKLOADS = {0: "vgg19+resnet20+cnn2_cifar10_n128", 2: "resnet20_cifar10_n128", 3: "cnn2_cifar10_n128", 4: "vgg19_cifar10_n128"}
+# the kernels that do the arithmetic of an exact or top-1 call, one a call (the others transpose, pack, select or reduce)
+MAIN_KERNELS = ("cl_kernel", "exact_tc_kernel", "direct_mma_kernel", "stem_mma_kernel", "direct_tiled_kernel", "direct_element_kernel",
+                "top1_fused_kernel", "gather_kernel")
 ORACLE_SAMPLE_IMAGES = 128    # images per distinct layer shape that both oracle legs time (the whole batch at N = 128): ~6 s of CPU work
 
 
@@ -366,6 +369,7 @@ def main():
     from paper_1908_05460_b200 import build as build_mod
 
     from paper_1908_05460_b200 import dist_util
+    from paper_1908_05460_b200.graph_names import kernel_names
     rank, world, local = dist_util.env_rank()
     if rank == 0:
         build_mod.build()
@@ -555,6 +559,8 @@ def main():
                 row[name + "_us"] = streamed_us(s, m, args.layer_iters)
             for name, m in methods[:2]:
                 row[name + "_isolated_us"] = isolated_us(lambda: run_one(s, m, 2), 5)
+                launched = kernel_names(lambda: run_one(s, m, 2))
+                row[name + "_kernel"] = next(k for k in MAIN_KERNELS if any(k in n for n in launched))
             seen[key] = row
         row = dict(seen[key])
         row.update({"layer": l.name, "net": s.net, "index": s.li, "dtype": s.dname})
@@ -590,14 +596,14 @@ def main():
         t = sum_us["top1"]
         fams["top1"] = {"bound": "hbm", "achieved": sum(r["top1_bytes"] for r in table) / t / 1e3, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                         "frac": sum(r["top1_bytes"] for r in table) / (peaks["hbm_gbs"] * 1e3) / t, "layers": len(table), "sum_us": t}
-        # the dominant kernel first (the exact families are both mostly exact_tc_kernel launches, as in the ncu launch
-        # list of the step), then that kernel's larger family
-        kernel_of = {"exact_tensor_bound": "exact_tc_kernel", "exact_hbm_bound": "exact_tc_kernel", "top1": "top1_fused_kernel"}
-        per_kernel = {}
-        for f, v in fams.items():
-            per_kernel[kernel_of[f]] = per_kernel.get(kernel_of[f], 0.0) + v["sum_us"]
-        kernel = max(per_kernel, key=per_kernel.get)
-        dom = max((f for f in fams if kernel_of[f] == kernel), key=lambda f: fams[f]["sum_us"])
+        # time by (family, the kernel that the layer's call was seen to launch); the dominant kernel first, then its larger family
+        share = {("exact_" + b + "_bound", k): sum(r["exact_us"] for r in table if r["exact_bound"] == b and r["exact_kernel"] == k)
+                 for b in ("tensor", "hbm") for k in MAIN_KERNELS}
+        share.update({("top1", k): sum(r["top1_us"] for r in table if r["top1_kernel"] == k) for k in MAIN_KERNELS})
+        for f in fams:
+            fams[f]["kernels_us"] = {k: t for (g, k), t in share.items() if g == f and t > 0}
+        kernel = max(MAIN_KERNELS, key=lambda k: sum(t for (_, g), t in share.items() if g == k))
+        dom = max(fams, key=lambda f: share[f, kernel])
         roof = {k: fams[dom][k] for k in ("bound", "achieved", "peak", "unit", "frac")}
         roof.update({"kernel": kernel, "family": dom, "peak_source": peaks["source"], "families": fams,
                      "traffic": traffic_from_profiles(kernel, dom)})
