@@ -22,11 +22,12 @@ constexpr size_t kWsDataOffset    = kWsCounterOffset + sizeof(uint32_t) * kWsNum
 void note_launch(int count = 1);   // bookkeeping behind gaconv_launch_count()
 
 // ---- programmatic dependent launch ------------------------------------------------------------
-// Every kernel of the library is launched with programmatic stream serialization allowed and starts
-// with pdl_release_next_grid(): the next kernel in the stream may then be scheduled while this one is
-// still running, and do its own set-up (barrier init, tensor-memory allocation) early.  Before its
-// first access to global memory every kernel executes pdl_wait_prior_grid(), which returns only when
-// the previous kernel has completed and its writes are visible -- so results never depend on it.
+// Kernels are launched with programmatic stream serialization allowed (direct_element_kernel excepted), and most start with
+// pdl_release_next_grid(): the next kernel in the stream may then be scheduled while this one is still running, and do its own
+// set-up (barrier init, tensor-memory allocation) early.  (direct_tiled_kernel, direct_mma_kernel, stem_mma_kernel, top1_fused_kernel and
+// the two reductions of reduce.cu do not: what follows them starts when they end.)  Before its first access to global memory every
+// kernel executes pdl_wait_prior_grid(), which returns only when the previous kernel has completed and its writes are
+// visible -- so results never depend on it.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_release_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
