@@ -60,7 +60,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-inline EncodeTiledFn encode_fn()
+inline EncodeTiledFn driver_encode_fn()
 {
     static EncodeTiledFn fn = [] {
         void* p = nullptr;
@@ -70,6 +70,19 @@ inline EncodeTiledFn encode_fn()
     }();
     return fn;
 }
+// A driver call needs a context, which the runtime gives a thread only with its first launch: a thread's first call of the library
+// may come here before that.
+inline CUresult encode_in_context(CUtensorMap* map, CUtensorMapDataType type, cuuint32_t rank, void* base, const cuuint64_t* dims, const cuuint64_t* strides,
+                                  const cuuint32_t* box, const cuuint32_t* steps, CUtensorMapInterleave il, CUtensorMapSwizzle swz, CUtensorMapL2promotion l2,
+                                  CUtensorMapFloatOOBfill oob)
+{
+    CUresult r = driver_encode_fn()(map, type, rank, base, dims, strides, box, steps, il, swz, l2, oob);
+    int dev = 0;
+    if (r != CUDA_SUCCESS && cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess)
+        r = driver_encode_fn()(map, type, rank, base, dims, strides, box, steps, il, swz, l2, oob);
+    return r;
+}
+inline EncodeTiledFn encode_fn() { return driver_encode_fn() != nullptr ? encode_in_context : nullptr; }
 
 
 }  // namespace gaconv

@@ -1,5 +1,7 @@
 """The channels-last tensor-core kernel (csrc/cl.cu) at the edges of its tiles, against the oracle: odd maps, channel
 counts off every tile size, strides, every packing path, several images per chunk, one split and many."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -197,3 +199,30 @@ def test_smaller_workspaces(layer, dtype, kw, method):
     assert accepted[0] == full
     if method != "top1" and "packed" in layer.name:
         assert len(accepted) > 1, (full, accepted)
+
+
+@pytest.mark.parametrize("layer,dtype,kernel", [
+    (ConvLayer("channels last, nothing packed", 4, 64, 9, 24, 64, 3, 3, 1, 1), torch.bfloat16, "cl_kernel"),
+    (ConvLayer("older tensor-core kernel", 8, 16, 32, 32, 16, 3, 3, 1, 1), torch.bfloat16, "exact_tc_kernel"),
+    (ConvLayer("mma.sync", 6, 16, 32, 32, 16, 3, 3, 1, 1), torch.float32, "direct_mma_kernel"),
+    (ConvLayer("stem", 5, 3, 32, 32, 16, 3, 3, 1, 1), torch.float32, "stem_mma_kernel"),
+], ids=lambda v: v.name if isinstance(v, ConvLayer) else "")
+def test_first_call_of_a_thread(layer, dtype, kernel):
+    """A thread that has not touched the GPU yet, so that it has no context when the tensor maps are made."""
+    c = GpuLayer(layer, dtype, *I.make_layer_inputs(layer, dtype, 20, 0))
+    alone, errors, stream = c.exact(), [], torch.cuda.Stream().cuda_stream
+    assert any(kernel in k for k in kernel_names(lambda: B.gaconv_dw_exact(c.x, c.dy, c.dw, c.desc)))
+    c.dw.fill_(float("nan"))
+    torch.cuda.synchronize()
+
+    def work():
+        try:
+            B.gaconv_dw_exact(c.x, c.dy, c.dw, c.desc, stream)
+        except B.GaconvError as e:
+            errors.append(e)
+
+    t = threading.Thread(target=work)
+    t.start()
+    t.join()
+    assert not errors, errors[0]
+    np.testing.assert_array_equal(c.logical_dw(), alone)
