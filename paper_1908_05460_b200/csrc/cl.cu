@@ -1282,7 +1282,8 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
     const size_t smem = std::max((size_t)P.stages * P.stage_bytes + P.slack, (size_t)P.cols * 512) + 1024;
     const dim3 grid((unsigned)(P.tiles_k * P.tiles_c * P.tiles_r), (unsigned)P.splits);
     ClKernel kern = kernel_for(P.ngroups, H.f32, P.c_side != 0);
-    if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return err;
+    static std::atomic<unsigned long long> ready[kMaxGroups][2][2];
+    if ((err = allow_shared_memory((const void*)kern, ready[P.ngroups > 9 ? kMaxGroups - 1 : P.ngroups - 1][H.f32][P.c_side])) != cudaSuccess) return err;
     if ((err = launch_kernel(kern, grid, dim3(kThreads), smem, stream, dim3(1, 1, 1), map_dy, map_x, dw, partial, status, P, src)) != cudaSuccess) return err;
     note_launch();
     if (P.splits == 1) return cudaSuccess;

@@ -320,8 +320,9 @@ cudaError_t launch_t(const T* x, const T* dy, float* dw, float* partial, uint32_
 #define GACONV_DIRECT_LAUNCH(ST, RR, A, B, C, D)                                                                                 \
     {                                                                                                                            \
         auto kern = direct_tiled_kernel<T, ST, RR, RR, A, B, C, D>;                                                              \
-        if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);                \
-        launch_err = launch_kernel(kern, grid, dim3(kThreads), smem, stream, dim3(1, 1, 1), x, dy, dw, partial, status, map_dy, map_x, g, pl); \
+        static std::atomic<unsigned long long> ready{0};                                                                         \
+        launch_err = smem > 48 * 1024 ? allow_shared_memory((const void*)kern, ready) : cudaSuccess;                             \
+        if (launch_err == cudaSuccess) launch_err = launch_kernel(kern, grid, dim3(kThreads), smem, stream, dim3(1, 1, 1), x, dy, dw, partial, status, map_dy, map_x, g, pl); \
     }
 #define GACONV_DIRECT_CASE(RR, A, B, C, D)                                                                     \
     if (!done && g.r == RR && v.tkt == A && v.tct == B && v.otk == C && v.otc == D) {                          \

@@ -208,8 +208,9 @@ cudaError_t launch_direct_mma(const void* x, const void* dy, float* dw, float* p
 #define GACONV_MMA_CASE(RR, TP)                                                                                          \
     if (g.r == RR && three_pass == TP) {                                                                                 \
         auto kern = direct_mma_kernel<RR, RR, TP>;                                                                       \
-        if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);        \
-        launch_err = launch_kernel(kern, grid, dim3(kThreads), smem, stream, dim3(1, 1, 1), dw, partial, status, map_dy, map_x, g, pl); \
+        static std::atomic<unsigned long long> ready{0};                                                                 \
+        launch_err = smem > 48 * 1024 ? allow_shared_memory((const void*)kern, ready) : cudaSuccess;                     \
+        if (launch_err == cudaSuccess) launch_err = launch_kernel(kern, grid, dim3(kThreads), smem, stream, dim3(1, 1, 1), dw, partial, status, map_dy, map_x, g, pl); \
     }
     GACONV_MMA_CASE(1, true)
     GACONV_MMA_CASE(1, false)

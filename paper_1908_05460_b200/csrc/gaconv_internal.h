@@ -7,6 +7,7 @@
 
 #include "gaconv.h"
 
+#include <atomic>
 #include <utility>
 
 namespace gaconv {
@@ -51,6 +52,23 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
     }
     cfg.attrs = attr; cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+// Lets a kernel have all the dynamic shared memory that a block can get: once per (kernel, device), and always to the same value.
+// (The attribute belongs to the kernel, not to a launch.  Set to what each launch needs, a thread's call could lower it between
+// another thread's setting and launch, and a graph held nodes above what was set by the time it ran.)  `devices`: those done.
+inline cudaError_t allow_shared_memory(const void* kernel, std::atomic<unsigned long long>& devices)
+{
+    int dev = 0, most = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    if (dev < 64 && (devices.load(std::memory_order_acquire) >> dev & 1)) return cudaSuccess;
+    cudaFuncAttributes attr;
+    if ((err = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return err;
+    if ((err = cudaFuncGetAttributes(&attr, kernel)) != cudaSuccess) return err;
+    if ((err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)attr.sharedSizeBytes)) != cudaSuccess) return err;
+    if (dev < 64) devices.fetch_or(1ull << dev, std::memory_order_release);
+    return cudaSuccess;
 }
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }

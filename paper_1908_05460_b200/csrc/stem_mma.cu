@@ -257,8 +257,9 @@ cudaError_t launch_t(const void* x, const void* dy, float* dw, float* partial, u
 #define GACONV_STEM_CASE(N)                                                                                        \
     if (P.nt == N) {                                                                                               \
         auto kern = stem_mma_kernel<T, N>;                                                                         \
-        if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);  \
-        err = launch_kernel(kern, grid, dim3(kThreads), smem, stream, dim3(1, 1, 1), dw, partial, status, map_dy, map_x, P); \
+        static std::atomic<unsigned long long> ready{0};                                                           \
+        err = smem > 48 * 1024 ? allow_shared_memory((const void*)kern, ready) : cudaSuccess;                      \
+        if (err == cudaSuccess) err = launch_kernel(kern, grid, dim3(kThreads), smem, stream, dim3(1, 1, 1), dw, partial, status, map_dy, map_x, P); \
     }
     GACONV_STEM_CASE(1) GACONV_STEM_CASE(2) GACONV_STEM_CASE(3) GACONV_STEM_CASE(4) GACONV_STEM_CASE(5)
     GACONV_STEM_CASE(6) GACONV_STEM_CASE(7) GACONV_STEM_CASE(8) GACONV_STEM_CASE(9) GACONV_STEM_CASE(10)

@@ -708,7 +708,8 @@ int resident_clusters(int cl)
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = cl; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
-        if (cudaFuncSetAttribute(exact_tc_kernel<0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess ||
+        static std::atomic<unsigned long long> ready{0};
+        if (allow_shared_memory((const void*)exact_tc_kernel<0, 0>, ready) != cudaSuccess ||
             cudaOccupancyMaxActiveClusters(&n, exact_tc_kernel<0, 0>, &cfg) != cudaSuccess || n < 1) {
             (void)cudaGetLastError();
             n = device_sms() / cl * 8 / 10;          // no answer: a cautious guess
@@ -1131,17 +1132,11 @@ cudaError_t launch_tc(const void* x, const void* dy, float* dw, float* partial, 
     smem += 1024 + (size_t)P.m * 128;
     dim3 grid(P.tiles_k * P.tiles_c * (P.rsplit ? g.r : 1), P.splits);
     const int ks = P.a_sub_px / (P.f32 ? 8 : 16);
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
     cudaError_t err = cudaErrorInvalidValue;
 #define GACONV_TC_CASE(RR, KK)                                                                                     \
     if (err == cudaErrorInvalidValue && (RR == 0 || (P.rc == RR && ks == KK))) {                                     \
-        static size_t configured[64] = {};           /* the attribute is per device */                            \
-        err = cudaSuccess;                                                                                         \
-        if (dev < 0 || dev >= 64 || smem > configured[dev]) {                                                      \
-            err = cudaFuncSetAttribute(exact_tc_kernel<RR, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-            if (err == cudaSuccess && dev >= 0 && dev < 64) configured[dev] = smem;                                \
-        }                                                                                                          \
+        static std::atomic<unsigned long long> ready{0};                                                           \
+        err = allow_shared_memory((const void*)exact_tc_kernel<RR, KK>, ready);                                    \
         if (err == cudaSuccess) {                                                                                  \
             err = launch_kernel(exact_tc_kernel<RR, KK>, grid, dim3(256), smem, stream, dim3(1, P.cl, 1), map_dy, map_x, dw, \
                                 partial, counters, status, P);                                                    \

@@ -657,13 +657,10 @@ static cudaError_t launch_fused_t(const T* x, const T* dy, float* dw, const Geom
     while (nj < 16 && nj * 2 <= ipc * topk && nj * 2 * groups <= threads) nj *= 2;        // image lanes: as many as keep every item on its own thread
     while (nj > 1 && (size_t)rsc * 4 * (1 + nj) > 150 * 1024) nj /= 2;              // the subtotals must fit shared memory
     const size_t smem = (((size_t)rsc * 4 + 15) & ~(size_t)15) + (size_t)ipc * topk * 16 + (nj > 1 ? (size_t)nj * rsc * 4 : 0) + 16;
-    static size_t configured[64] = {};           // per device: the attribute belongs to the device's copy of the kernel
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (smem > 48 * 1024 && smem > configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(top1_fused_kernel<T, VEC, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static std::atomic<unsigned long long> ready{0};
+    if (smem > 48 * 1024) {
+        cudaError_t e = allow_shared_memory((const void*)top1_fused_kernel<T, VEC, WIDE>, ready);
         if (e != cudaSuccess) return e;
-        configured[dev] = smem;
     }
     // lanes per map: few enough that one pass covers all the CTA's maps (their loads are then all in flight at once)
     while (G > 1 && G * ipc > threads) G /= 2;

@@ -226,3 +226,29 @@ def test_first_call_of_a_thread(layer, dtype, kernel):
     t.join()
     assert not errors, errors[0]
     np.testing.assert_array_equal(c.logical_dw(), alone)
+
+
+def test_threads_with_layers_of_one_kernel_and_different_shared_memory():
+    """Two threads on streams of their own; the layers take the same instance of the kernel with 97 and with 217 KB of shared memory."""
+    layers = [ConvLayer("97 KB", 4, 64, 9, 24, 64, 3, 3, 1, 1), ConvLayer("217 KB", 9, 70, 12, 16, 64, 7, 3, 1, 1)]
+    calls = [GpuLayer(l, torch.bfloat16, *I.make_layer_inputs(l, torch.bfloat16, 20, i)) for i, l in enumerate(layers)]
+    alone = [c.exact() for c in calls]
+    names = [next(k for k in kernel_names(lambda: B.gaconv_dw_exact(c.x, c.dy, c.dw, c.desc)) if "cl_kernel" in k) for c in calls]
+    assert names[0] == names[1]
+    errors = []
+
+    def work(c, stream):
+        try:
+            for _ in range(4000):
+                B.gaconv_dw_exact(c.x, c.dy, c.dw, c.desc, stream)
+        except B.GaconvError as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(c, torch.cuda.Stream())) for c in calls]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
+    for c, want in zip(calls, alone):
+        np.testing.assert_array_equal(c.logical_dw(), want)
