@@ -43,7 +43,9 @@
 // Values that are not finite.  An Inf has no planes to split into (x - x0 = Inf - Inf), and the zero dY rows that end a chunk meet
 // real X rows, so that an Inf or NaN there reaches elements it has no part in.  But nothing is hidden: what has an infinite or
 // NaN product among those it should have comes out of the tensor core not finite.  So the writers look at every element, and
-// those that are not finite are summed anew, product by product from the operands as they were handed over (cl_repair).
+// those that are not finite are summed anew, product by product from the operands as they were handed over (cl_repair).  The look costs
+// nothing where a second kernel writes dW; where this one does, ~0.2 us (exact phase of a VGG-19 step 171.3 -> 173.5 us; eight chains of
+// additions, three-operand maxima or the repair in line instead of a call came to the same).
 // (What may be missing are products of the padding with an Inf or NaN in dY: the orders and forms that skip the padding skip them.)
 //
 // Every wait is bounded; on expiry the kernel raises the workspace status word, lets its copies land, frees its tensor
@@ -572,16 +574,39 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
     GACONV_STAMP(5, threadIdx.x == 0);
 }
 
+// lane of the e-th element that a block of cl_reduce_kernel writes, and its column relative to the block's first
+__device__ __forceinline__ int2 reduced_element(const ClParams& P, int e, int log_cb)
+{
+    int l = P.c_side ? e & 127 : e >> log_cb;
+    if (P.c_side && P.s_inner) { const int t_shift = 7 - (31 - __clz(P.ca)); l = ((l & ((1 << t_shift) - 1)) << (7 - t_shift)) + (l >> t_shift); }
+    return make_int2(l, P.c_side ? e >> 7 : e & ((1 << log_cb) - 1));
+}
+// Every warp of cl_reduce_kernel repairs what it has written (a thread reads its own elements back).  Apart, so that the kernel keeps
+// nothing in registers for the sake of it.
+__device__ __noinline__ void cl_repair_written(const ClParams& P, const ClSource& S, float* dw, int log_cb)
+{
+    const int tile = blockIdx.y, col0 = blockIdx.x << log_cb;
+    for (int e = threadIdx.x; e < 128 << log_cb; e += blockDim.x) {          // (whole warps: both are multiples of 32)
+        const int2 lc = reduced_element(P, e, log_cb);
+        const bool in = col0 + lc.y < P.cols;
+        const int col = written_column(P, in ? col0 + lc.y : 0);
+        const ClElement el = cl_element(P, tile, col, lc.x);
+        const float* out = dw + (el.k * P.ws_k + el.c * P.ws_c + el.r * P.ws_r + el.s * P.ws_s);
+        const uint32_t left = __ballot_sync(0xffffffffu, in && el.valid && !isfinite(__ldcg(out)));
+        if (left != 0) cl_repair(P, S, dw, tile, col, lc.x, left);
+    }
+}
+
 // Sum of the splits of every (tile, column), in a fixed order: grid (column blocks, tiles), 32 * CB * G threads.  Warp (g, c)
 // adds the 128 lanes (a float4 each) of column c over the splits g, g + G, ...; the G partial sums meet in shared memory.  G is
 // chosen so that a warp's loads are all in flight at once (eight, then a second round), CB so that the grid covers the GPU;
 // where consecutive columns are consecutive channels of dW a block writes CB of them in one piece.  Latency-bound: what an
 // element is, and where it goes, is worked out before the wait for the sums.
-// SHARED, for launches that share the GPU: registers for two blocks an SM.  On a GPU of its own there are no more blocks than SMs, and
-// with 64 registers instead of 32 all eight loads of a thread are in flight (fp32 64->128 stride 2 on 28x28, N = 64, whole
-// call: 32.7 -> 31.3 us); beside other layers that costs more than it gives (step of ResNet-20 150 -> 154).
-template <bool SHARED>
-__global__ void __launch_bounds__(1024, SHARED ? 2 : 1)
+// LEAN: 32 registers.  With 56 all eight loads of a thread are in flight (fp32 64->128 stride 2 on 28x28, N = 64, whole call:
+// 32.7 -> 31.3 us), but only where the SMs hold all blocks at once (352->288 on 9x9, N = 65, 648 blocks of 512 threads: 34.2 -> 35.3)
+// and nothing else wants room on them (step of ResNet-20 150 -> 154).
+template <bool LEAN>
+__global__ void __launch_bounds__(1024, LEAN ? 2 : 1)
 cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, const __grid_constant__ ClParams P, const __grid_constant__ ClSource S, int log_cb, int G)
 {
     __shared__ float s_sum[32][128];
@@ -615,11 +640,11 @@ cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, cons
             for (int i = 0; i < 8; ++i) { acc.x += u[i].x; acc.y += u[i].y; acc.z += u[i].z; acc.w += u[i].w; }
         }
     *reinterpret_cast<float4*>(&s_sum[warp][4 * lane]) = acc;
+    float finite = 0.f;         // NaN as soon as this thread has written an element that is not finite
     __syncthreads();
     for (int e = threadIdx.x; e < CB << 7; e += blockDim.x) {
-        const int c = P.c_side ? e >> 7 : e & (CB - 1);
-        int l = P.c_side ? e & 127 : e >> log_cb;
-        if (P.c_side && P.s_inner) { const int t_shift = 7 - ca_shift; l = ((l & ((1 << t_shift) - 1)) << ca_shift) + (l >> t_shift); }
+        const int2 lc = reduced_element(P, e, log_cb);
+        const int l = lc.x, c = lc.y;
         const int2 o = s_col[c];
         bool valid; long long off = o.x;
         if (P.c_side) {
@@ -631,15 +656,13 @@ cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, cons
             valid = o.y > 0 && lane_off >= 0;
             off += lane_off;
         }
-        float t = 0.f;
-        if (valid) {
-            t = s_sum[c][l];
-            for (int w = 1; w < G; ++w) t += s_sum[(w << log_cb) + c][l];
-            dw[off] = P.alpha * t;
-        }
-        const uint32_t left = __ballot_sync(0xffffffffu, !isfinite(t));        // (a warp's lanes come and go together: CB * 128 elements)
-        if (left != 0) cl_repair(P, S, dw, tile, written_column(P, min(col0 + c, P.cols - 1)), l, left);
+        if (!valid) continue;
+        float t = s_sum[c][l];
+        for (int w = 1; w < G; ++w) t += s_sum[(w << log_cb) + c][l];
+        dw[off] = P.alpha * t;
+        finite = fmaf(t, 0.f, finite);
     }
+    if (__any_sync(0xffffffffu, isnan(finite))) cl_repair_written(P, S, dw, log_cb);
 }
 
 // ---- packing: one operand -> channels-last bf16 planes, channels padded to a multiple of 8 with zeros -------------------
@@ -1050,7 +1073,7 @@ struct ClHost {             // what ClPlan::opaque holds
     bool pack_x, pack_dy, f32, x_nhwc, dy_npqk;
     int xch, dych;          // channels per pixel row of the operands the tensor maps describe
     int log_cb, groups;     // second kernel: columns per block, split groups per column
-    bool shared;            // other layers run beside this one
+    bool lean;              // second kernel: with few registers
 };
 static_assert(sizeof(ClHost) <= sizeof(ClPlan::opaque), "ClPlan::opaque too small");
 
@@ -1097,7 +1120,6 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
     const bool nhwc = g.xs_c == 1 || g.c == 1;
     ClHost H{};
     H.f32 = !g.bf16;
-    H.shared = g.sm_budget > 0;
     H.x_nhwc = nhwc; H.dy_npqk = dy_npqk || g.k == 1;
     H.pack_x = H.f32 || !nhwc || g.c % 8 != 0;
     H.pack_dy = H.f32 || !H.dy_npqk || g.k % 8 != 0;
@@ -1222,6 +1244,7 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
     H.log_cb = 4;
     while (H.log_cb > 0 && ((H.groups << H.log_cb) > 32 || best.tiles_k * best.tiles_c * best.tiles_r * ceil_div(best.cols, 1 << H.log_cb) < sms)) --H.log_cb;
     const int tiles = best.tiles_k * best.tiles_c * best.tiles_r;
+    H.lean = g.sm_budget > 0 || tiles * ceil_div(best.cols, 1 << H.log_cb) > sms * (65536 / (64 * 32 * H.groups << H.log_cb));
     if (tiles > 65535 || best.splits > 65535) return false;
     out->cycles = best_cycles;
     out->partial_bytes = best.splits == 1 ? 0 : (size_t)tiles * best.splits * best.cols * 512;
@@ -1288,7 +1311,7 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
     note_launch();
     if (P.splits == 1) return cudaSuccess;
     const dim3 rgrid((unsigned)ceil_div(P.cols, 1 << H.log_cb), grid.x);
-    err = launch_kernel(H.shared ? cl_reduce_kernel<true> : cl_reduce_kernel<false>, rgrid, dim3(32u * H.groups << H.log_cb), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P,
+    err = launch_kernel(H.lean ? cl_reduce_kernel<true> : cl_reduce_kernel<false>, rgrid, dim3(32u * H.groups << H.log_cb), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P,
                         src, H.log_cb, H.groups);
     if (err != cudaSuccess) return err;
     note_launch();
