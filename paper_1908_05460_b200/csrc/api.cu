@@ -105,12 +105,14 @@ private:
 };
 
 // A large dW with short sums, split over CTAs, on a GPU of its own: the channels-last kernel writes as many partial blocks as it has
-// CTAs and reads them again, the older kernel adds them inside clusters (256->256 on 8x8, N = 64 16.9 / 14.6 us, N = 128
-// 20.1 / 19.9, N = 256 26.5 / 27.1; 256->512 on 4x4, N = 128 21.0 / 19.4; 128->256 on 8x8, N = 128 15.9 / 16.6).
+// CTAs and reads them again, the older kernel adds them inside clusters.  The line is at one pixel for every hundred elements, where
+// the two meet (us, the older kernel first): 0.002 256->512 on 4x4, N = 128 18.6 / 21.9; 0.007 256->256 on 8x8, N = 64 14.5 / 15.1;
+// 0.009 the same, N = 80 15.9 / 15.7, 384->256 on 8x8 23.1 / 23.4, 192->384 on 8x8, N = 96 17.3 / 19.0; 0.0104 256->256 on 8x8, N = 96
+// 17.3 / 16.6; 0.0108 256->256 on 4x4, N = 400 21.0 / 20.8; 0.014 256->256 on 8x8, N = 128 20.0 / 18.0, 128->512 on 4x4, N = 512 25.6 / 24.0.
 bool short_sums(const Geom& g, const ClPlan& plan)
 {
     const double elements = (double)g.k * g.c * g.r * g.s;
-    return g.sm_budget == 0 && plan.partial_bytes > 0 && elements > 4e5 && (double)g.n * g.p * g.q < 0.015 * elements;
+    return g.sm_budget == 0 && plan.partial_bytes > 0 && elements > 4e5 && (double)g.n * g.p * g.q < 0.01 * elements;
 }
 
 // Small maps with many channels (up to 4x4 pixels from 128 channels, up to 8x8 from 256): the N*K patch accumulations (N*K*R*S*C FMAs on the FP32 pipes,
@@ -199,32 +201,36 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, const ClPlan& plan, bool reo
     if (g.bf16) {
         if (L.tc_ok) {
             if (!reordered && short_sums(g, plan)) return false;
-            // maps under 64 pixels: 512->512 on 4x4, N = 256 31.1 / 27.0, 128->16 on 4x8, N = 100 12.5 / 10.7; many input and few output
-            // channels (partial blocks of mostly idle lanes) 192->16 on 4x8, N = 23 8.9 / 11.6, 256->16 on 4x4, N = 200 13.3 / 15.0
+            // maps under 64 pixels: 512->512 on 4x4, N = 256 31.8 / 27.3, 128->16 on 4x8, N = 100 11.3 / 8.8; many input and few output
+            // channels (partial blocks of mostly idle lanes) 192->16 on 4x8, N = 23 7.9 / 11.3, 256->16 on 4x4, N = 200 11.5 / 13.6
             if (L.tp.reads_transposed_dy) return products > 5e6 && (g.k > 32 || g.c <= 128);
             if (products < 3e7) return false;
             if (reordered) return true;                             // 128->128 on 16x16, dY channels last 28.4 / 17.8
-            if (g.c <= 16 || (g.c < 64 && shared)) return false;    // 16->16 on 32x32 11.9 / 12.5; on 18 SMs 28 / 38
+            if (g.c <= 16 || (g.c < 64 && shared)) return false;    // 16->16 on 32x32 12.4 / 12.8; on 18 SMs 29 / 39
             // 64 channels on few SMs: the older kernel's M = 64 fits, this one's 128 lanes are half idle or its tiles shared, until the
             // main loop outweighs the rest (on 12 lanes beside copies of itself, us a layer: 64->64 on 8x8, N = 32 1.84 / 1.96,
             // N = 128 2.69 / 2.93, N = 200 3.38 / 3.45, N = 512 6.3 / 5.8; 64->40 on 16x16, N = 64 3.0 / 3.8; not with 16 outputs,
             // 64->16 on 16x16 3.8 / 3.4, nor at stride 2, 64->64 on 16x16 4.1 / 2.8; exact phase of a ResNet-20 step 77 / 80)
             if (shared && g.c <= 64 && g.k > 16 && g.k <= 64 && g.stride_h == 1 && products < 5e8) return false;
-            return g.r < 5;                                         // 5x5 64->64 on 16x16 16.1 / 17.8, 3x3 64->64 on 32x32 24.1 / 22.5
+            // Filters of five and more rows: with few input channels this kernel stacks the rows or has its M side full of shifts
+            // (5x5 on 16x16: 32->32 17.6 / 14.4, 40->64 25.0 / 18.1, 32->128 22.9 / 14.8, N = 32 32->64 18.1 / 10.4; 48->64 on 8x8 18.1 / 11.9;
+            // 7x7 32->32 on 16x16 21.0 / 14.3; 24->24 13.9 / 14.3); with 64 and more the older one is as quick or quicker (5x5 64->64 on 16x16
+            // 17.0 / 17.3, 256->256 on 8x8 50 / 55, 7x7 128->128 on 16x16 48 / 105).  3x3 64->64 on 32x32 25.0 / 23.1
+            return g.r < 5 || g.c < 64;
         }
-        if (L.stem_ok) return reordered || (!shared && g.r * g.s * g.c > 32);       // 5x5 3->64 26.4 / 22.6, 3x3 3->16 10.4 / 14.8
+        if (L.stem_ok) return reordered || (!shared && g.r * g.s * g.c > 32);       // 5x5 3->64 27.5 / 26.1, 3x3 3->16 11.1 / 16.0
     } else {
-        if (L.stem_ok) return false;                                // 3->64 on 32x32 28 / 53
+        if (L.stem_ok) return false;                                // 3->64 on 32x32 29 / 41
         // (the tensor core truncates as it adds, 1e-8 for each MMA of the other kernel's CTA: where that has more than 1,500 of them
         // its results are over 1.4e-5 away from this one's, and stay what they have been)
         if (L.tc_ok && L.tp.chain > 1500) return false;
-        if (L.tc_ok)                                                // 128->128 on 16x16 92 / 53, 64->64 on 8x8 17.1 / 18.3, on 18 SMs 44 / 32
-            return reordered || products > (g.c >= 128 ? 4e8 : shared ? 1e8 : g.c >= 64 ? 1e9 : 2e8);      // 32->32 on 16x16 18.3 / 17.1, on 18 SMs 42 / 35
-        if (direct_mma_supported(g, L.dp))                          // 16->16 on 32x32 19 / 40, 48->96 on 16x16 (N = 64) 31 / 23
-            return (g.c >= 64 && products > 4e6) || (g.c >= 24 && g.stride_h == 1 && !shared && products > 3e8);       // (N = 16) 24->16 on 32x32 10 / 14
+        if (L.tc_ok)                                                // 128->128 on 16x16 89 / 53, 64->64 on 8x8 18.0 / 19.9, on 18 SMs 45 / 35
+            return reordered || products > (g.c >= 128 ? 4e8 : shared ? 1e8 : g.c >= 64 ? 1e9 : 2e8);      // 32->32 on 16x16 19.3 / 17.7, on 18 SMs 43 / 36
+        if (direct_mma_supported(g, L.dp))                          // 16->16 on 32x32 20 / 24.5, 48->96 on 16x16 (N = 64) 31 / 25
+            return (g.c >= 64 && products > 4e6) || (g.c >= 24 && g.stride_h == 1 && !shared && products > 3e8);       // (N = 16) 24->16 on 32x32 10 / 13.5
     }
     // FP32 pipes: their one or two launches are as quick while the work is small -- longer with 3x3 filters of fp32 layers, whose
-    // operands must be packed (16->64 on 6x6, N = 30 10.3 / 12.3 us; 1x1 80->22 on 6x6, N = 105 27 / 12), and with three channels
+    // operands must be packed (16->64 on 6x6, N = 30 launched one by one 10.3 / 12.3 us; 1x1 80->22 on 6x6, N = 105 25 / 12), and with three channels
     return products > (!g.bf16 && g.r * g.s >= 9 ? 2e7 : g.c <= 4 ? 1e7 : 4e6);
 }
 struct ClRoute { bool use; ClPlan plan; size_t partial_off, x_off, dy_off, total; };

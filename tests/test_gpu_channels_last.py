@@ -252,3 +252,27 @@ def test_threads_with_layers_of_one_kernel_and_different_shared_memory():
     assert not errors, errors[0]
     for c, want in zip(calls, alone):
         np.testing.assert_array_equal(c.logical_dw(), want)
+
+
+@pytest.mark.parametrize("layer,budget,kernel", [
+    (ConvLayer("5x5, 40 channels", 16, 40, 16, 16, 64, 5, 5, 1, 2), 0, "cl_kernel"),
+    (ConvLayer("5x5, 64 channels", 16, 64, 16, 16, 64, 5, 5, 1, 2), 0, "exact_tc_kernel"),
+    (ConvLayer("7x7, 24 channels on 32x32", 9, 24, 32, 32, 16, 7, 7, 1, 3), 0, "cl_kernel"),
+    (ConvLayer("a large dW with short sums", 64, 256, 8, 8, 256, 3, 3, 1, 1), 0, "exact_tc_kernel"),
+    (ConvLayer("a large dW past the line", 96, 256, 8, 8, 256, 3, 3, 1, 1), 0, "cl_kernel"),
+    (ConvLayer("64 channels on few SMs", 32, 64, 8, 8, 64, 3, 3, 1, 1), 18, "exact_tc_kernel"),
+    (ConvLayer("64 channels on few SMs, stride 2", 32, 64, 16, 16, 64, 3, 3, 2, 1), 18, "cl_kernel"),
+    (ConvLayer("64 channels on few SMs, 230 images", 230, 64, 8, 8, 64, 3, 3, 1, 1), 18, "cl_kernel"),
+], ids=lambda v: v.name if isinstance(v, ConvLayer) else str(v))
+def test_either_side_of_a_line(layer, budget, kernel):
+    """bf16 layers that both tensor-core kernels can do, around the lines between them: the kernel, and its results on samples."""
+    x, dy = I.make_layer_inputs(layer, torch.bfloat16, 21, 0)
+    g = GpuLayer(layer, torch.bfloat16, x, dy, sm_budget=budget)
+    names = kernel_names(lambda: B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc))
+    assert any(kernel in n for n in names), names
+    got, xd, dyd = g.exact(), to_f64(x), to_f64(dy)
+    rng = np.random.default_rng(3)
+    for k, c, r, s in zip(*(rng.integers(0, m, 60).tolist() for m in (layer.k, layer.c, layer.r, layer.s))):
+        v, norm = oracle.dw_exact_at(xd, dyd, oshape(layer), k, c, r, s)
+        assert abs(got[k, c, r, s] - v) <= TOL_F32 * norm
+    assert np.all(np.isfinite(got)) and B.gaconv_poll_async_status(g.desc) == B.OK
