@@ -209,9 +209,10 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, const ClPlan& plan, bool reo
             if (g.c <= 16 || (g.c < 64 && shared)) return false;    // 16->16 on 32x32 12.4 / 12.8; on 18 SMs 29 / 39
             // 64 channels on few SMs: the older kernel's M = 64 fits, this one's 128 lanes are half idle or its tiles shared, until the
             // main loop outweighs the rest (on 12 lanes beside copies of itself, us a layer: 64->64 on 8x8, N = 32 1.84 / 1.96,
-            // N = 128 2.69 / 2.93, N = 200 3.38 / 3.45, N = 512 6.3 / 5.8; 64->40 on 16x16, N = 64 3.0 / 3.8; not with 16 outputs,
-            // 64->16 on 16x16 3.8 / 3.4, nor at stride 2, 64->64 on 16x16 4.1 / 2.8; exact phase of a ResNet-20 step 77 / 80)
-            if (shared && g.c <= 64 && g.k > 16 && g.k <= 64 && g.stride_h == 1 && products < 5e8) return false;
+            // N = 128 2.69 / 2.93, N = 256 3.90 / 3.96, N = 512 6.3 / 5.8; 64->40 on 16x16, N = 64 3.0 / 3.8; not with 16 outputs,
+            // 64->16 on 16x16 3.8 / 3.4, nor at stride 2, 64->64 on 16x16 4.1 / 2.8; exact phase of a ResNet-20 step, N = 64, 128 and
+            // 256, with the one and with the other: 55 / 60, 78 / 80, 106 / 113)
+            if (shared && g.c <= 64 && g.k > 16 && g.k <= 64 && g.stride_h == 1 && products < 1e9) return false;
             // Filters of five and more rows: with few input channels this kernel stacks the rows or has its M side full of shifts
             // (5x5 on 16x16: 32->32 17.6 / 14.4, 40->64 25.0 / 18.1, 32->128 22.9 / 14.8, N = 32 32->64 18.1 / 10.4; 48->64 on 8x8 18.1 / 11.9;
             // 7x7 32->32 on 16x16 21.0 / 14.3; 24->24 13.9 / 14.3); with 64 and more the older one is as quick or quicker (5x5 64->64 on 16x16

@@ -262,7 +262,7 @@ def test_threads_with_layers_of_one_kernel_and_different_shared_memory():
     (ConvLayer("a large dW past the line", 96, 256, 8, 8, 256, 3, 3, 1, 1), 0, "cl_kernel"),
     (ConvLayer("64 channels on few SMs", 32, 64, 8, 8, 64, 3, 3, 1, 1), 18, "exact_tc_kernel"),
     (ConvLayer("64 channels on few SMs, stride 2", 32, 64, 16, 16, 64, 3, 3, 2, 1), 18, "cl_kernel"),
-    (ConvLayer("64 channels on few SMs, 230 images", 230, 64, 8, 8, 64, 3, 3, 1, 1), 18, "cl_kernel"),
+    (ConvLayer("64 channels on few SMs, 450 images", 450, 64, 8, 8, 64, 3, 3, 1, 1), 18, "cl_kernel"),
 ], ids=lambda v: v.name if isinstance(v, ConvLayer) else str(v))
 def test_either_side_of_a_line(layer, budget, kernel):
     """bf16 layers that both tensor-core kernels can do, around the lines between them: the kernel, and its results on samples."""
