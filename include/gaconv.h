@@ -57,7 +57,7 @@ typedef enum { GACONV_METHOD_EXACT = -1, GACONV_METHOD_ZERO = 0, GACONV_METHOD_R
 /* arithmetic of the exact contraction */
 typedef enum {
     GACONV_MATH_DEFAULT = 0,   /* bf16 inputs: bf16 tensor cores, fp32 accumulate; fp32 inputs: fp32-accurate
-                                  (three TF32 tensor-core passes on split operands, or the FP32 pipes)          */
+                                  (six products of three bf16 planes or three TF32 passes on tensor cores, or the FP32 pipes) */
     GACONV_MATH_TF32 = 1       /* fp32 inputs only: one TF32 tensor-core pass (operands cut to 10 mantissa bits);
                                   GACONV_ERR_UNSUPPORTED for shapes without a tensor-core kernel                 */
 } gaconv_math_t;
