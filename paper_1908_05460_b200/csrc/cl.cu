@@ -1202,8 +1202,9 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
                                     last_bp = bp;
                                     if (!consider(ci, bp, false)) break;
                                 }
-                                // no halo columns: one MMA a k-step, of shifts alone, and a first pixel with every shift inside or to the left
-                                if (form != 1 && ci >= 16 && na == 1 && (rc == 1 || form == 2) && F.stride == 1 && g.s > 1 && g.s * F.ca <= kMaxCols && g.w >= g.s - g.pad_w && g.pad_w < g.w) {
+                                // no halo columns: one MMA a k-step, of shifts alone, a first pixel with every shift inside or to the left, and
+                                // no pixel without any (its window in the padding altogether)
+                                if (g.pad_w < g.s && form != 1 && ci >= 16 && na == 1 && (rc == 1 || form == 2) && F.stride == 1 && g.s > 1 && g.s * F.ca <= kMaxCols && g.w >= g.s - g.pad_w && g.pad_w < g.w) {
                                     last_bp = 0;
                                     for (int parts = all_rows; parts >= 1; --parts) {
                                         const int bp = ceil_div(all_rows, parts);

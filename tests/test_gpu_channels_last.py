@@ -276,3 +276,19 @@ def test_either_side_of_a_line(layer, budget, kernel):
         v, norm = oracle.dw_exact_at(xd, dyd, oshape(layer), k, c, r, s)
         assert abs(got[k, c, r, s] - v) <= TOL_F32 * norm
     assert np.all(np.isfinite(got)) and B.gaconv_poll_async_status(g.desc) == B.OK
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
+@pytest.mark.parametrize("layer", [
+    ConvLayer("two columns, padding 2", 43, 9, 8, 8, 244, 5, 2, 1, 2),
+    ConvLayer("2x2 filter, padding 2 on 4x4", 150, 118, 4, 4, 19, 2, 2, 1, 2),
+    ConvLayer("3x3 filter, padding 4 on 5x5", 150, 20, 5, 5, 26, 3, 3, 1, 4),
+], ids=lambda l: l.name)
+def test_windows_wholly_in_the_padding(layer, dtype):
+    """Output pixels that meet no pixel of X."""
+    x, dy = I.make_layer_inputs(layer, dtype, 22, 0)
+    ref, dn = oracle.dw_exact(to_f64(x), to_f64(dy), oshape(layer))
+    for kw in (*LAYOUTS.values(), dict(sm_budget=7)):
+        g = GpuLayer(layer, dtype, x, dy, **kw)
+        assert norm_err(g.exact(), ref, dn) <= TOL_F32, kw
+        assert B.gaconv_poll_async_status(g.desc) == B.OK
