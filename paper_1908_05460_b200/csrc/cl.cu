@@ -1004,7 +1004,7 @@ bool shape_chunk(ClParams& P, int ci, int bp, int order, bool bare = false)
     }
     // last X row an MMA touches: last k-step, last row and column shift, unused shifts of the c-side form
     // (kImages: in whole pixels, one more where the last k-step is half a k-step)
-    const int last = order == kFlat ? P.ksteps * 16 - 1 : ((images ? 1 : ci) - 1) * P.x_img + (bp - 1) * wp + P.q - 1 + (order == kPixels ? 8 : 0) + (images && ci % 16 != 0 ? 1 : 0);
+    const int last = order == kFlat ? P.ksteps * 16 - 1 : ((images ? 1 : ci) - 1) * P.x_img + (bp - 1) * wp + P.q - 1 + (order == kPixels ? wp - P.q + 8 : 0) + (images && ci % 16 != 0 ? 1 : 0);
     const int zeros = P.stack && images && ci == 8 && bp * P.q % 2 != 0 ? P.x_img + 1 + far_shift(P) : 0;      // pixels, see below
     P.x_pre = bare ? round_up(std::max(P.pad_w, 1) * ci * xb, 1024) : 0;
     const int far = last + halo * wp + (images ? far_shift(P) : ceil_div(P.s, st) - 1 + (P.c_side ? 128 / P.ca : 256 / P.ca));

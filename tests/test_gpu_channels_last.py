@@ -283,9 +283,11 @@ def test_either_side_of_a_line(layer, budget, kernel):
     ConvLayer("two columns, padding 2", 43, 9, 8, 8, 244, 5, 2, 1, 2),
     ConvLayer("2x2 filter, padding 2 on 4x4", 150, 118, 4, 4, 19, 2, 2, 1, 2),
     ConvLayer("3x3 filter, padding 4 on 5x5", 150, 20, 5, 5, 26, 3, 3, 1, 4),
+    ConvLayer("rows of one pixel, padding 5", 100, 79, 8, 1, 30, 4, 4, 1, 5),
+    ConvLayer("odd rows of eight, 4 outputs", 61, 159, 19, 8, 4, 3, 3, 1, 1),
 ], ids=lambda l: l.name)
 def test_windows_wholly_in_the_padding(layer, dtype):
-    """Output pixels that meet no pixel of X."""
+    """Output pixels that meet no pixel of X, and the last pairs of eight pixels of a band: nothing beyond the tiles is multiplied."""
     x, dy = I.make_layer_inputs(layer, dtype, 22, 0)
     ref, dn = oracle.dw_exact(to_f64(x), to_f64(dy), oshape(layer))
     for kw in (*LAYOUTS.values(), dict(sm_budget=7)):
