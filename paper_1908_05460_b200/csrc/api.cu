@@ -93,8 +93,10 @@ public:
         L made = build();
 #ifndef GACONV_TUNING
         std::lock_guard<std::mutex> lock(m_);
-        if (e_.size() >= kMaxEntries) e_.pop_back();
-        e_.emplace_back(key, made);
+        try {                          // (no host memory: the plan is used and not kept; nothing may throw through the C interface)
+            if (e_.size() >= kMaxEntries) e_.pop_back();
+            e_.emplace_back(key, made);
+        } catch (const std::bad_alloc&) { }
 #endif
         return made;
     }
@@ -929,17 +931,20 @@ gaconv_status_t gaconv_schedule_run_step(const gaconv_schedule_t* s, int64_t ste
         return enqueue_step(s, step, num_layers, x, dy, dw, descs, lanes, main_stream, pool, nullptr);
 
     // everything the recorded launches depend on
+    // (without host memory for it, or for the cache, a step is enqueued and not kept)
     StepKey key;
-    key.bytes.reserve((size_t)num_layers * (sizeof(gaconv_conv_desc_t) + 3 * sizeof(void*) + 4) + 64);
-    const int32_t head[3] = {pool->device, lanes, num_layers};
-    key.put(head, sizeof(head));
-    for (int l = 0; l < num_layers; ++l) {
-        const int32_t method = gaconv_schedule_method(s, l, step);
-        const void* ptrs[3] = {x[l], dy[l], dw[l]};
-        key.put(&method, sizeof(method)); key.put(ptrs, sizeof(ptrs)); key.put(descs[l], sizeof(*descs[l]));
-    }
     if (s->steps == nullptr) const_cast<gaconv_schedule*>(s)->steps = new (std::nothrow) StepCache;
     StepCache* cache = s->steps;
+    try {
+        key.bytes.reserve((size_t)num_layers * (sizeof(gaconv_conv_desc_t) + 3 * sizeof(void*) + 4) + 64);
+        const int32_t head[3] = {pool->device, lanes, num_layers};
+        key.put(head, sizeof(head));
+        for (int l = 0; l < num_layers; ++l) {
+            const int32_t method = gaconv_schedule_method(s, l, step);
+            const void* ptrs[3] = {x[l], dy[l], dw[l]};
+            key.put(&method, sizeof(method)); key.put(ptrs, sizeof(ptrs)); key.put(descs[l], sizeof(*descs[l]));
+        }
+    } catch (const std::bad_alloc&) { cache = nullptr; }
     StepGraph* g = nullptr;
     if (cache != nullptr) {
         for (StepGraph& c : cache->e)
@@ -956,9 +961,11 @@ gaconv_status_t gaconv_schedule_run_step(const gaconv_schedule_t* s, int64_t ste
                 StepCache::drop(cache->e[oldest]);
                 cache->e.erase(cache->e.begin() + oldest);
             }
-            cache->e.emplace_back();
-            cache->e.back().key = std::move(key.bytes);
-            cache->e.back().used = ++cache->clock;
+            try {
+                cache->e.emplace_back();
+                cache->e.back().key = std::move(key.bytes);
+                cache->e.back().used = ++cache->clock;
+            } catch (const std::bad_alloc&) { }
         }
         return st;
     }
@@ -966,6 +973,9 @@ gaconv_status_t gaconv_schedule_run_step(const gaconv_schedule_t* s, int64_t ste
         const uint64_t before = gaconv_launch_count();
         gaconv_status_t st = GACONV_ERR_CUDA;
         g->random.clear();
+        try { g->random.reserve(num_layers); } catch (const std::bad_alloc&) {      // (nothing is allocated while the step is recorded)
+            return enqueue_step(s, step, num_layers, x, dy, dw, descs, lanes, main_stream, pool, nullptr);
+        }
         if (cudaStreamBeginCapture(pool->record, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
             st = enqueue_step(s, step, num_layers, x, dy, dw, descs, lanes, pool->record, pool, &g->random);
             if (cudaStreamEndCapture(pool->record, &g->graph) != cudaSuccess) st = GACONV_ERR_CUDA;
