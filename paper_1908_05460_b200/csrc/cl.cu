@@ -26,7 +26,11 @@
 // A table of the plan holds the offsets of the k-steps of every order.
 //
 // Which operand is the MMA's M side:
-//   k-side  M = 128 output channels, N = consecutive column shifts x channels (up to 256).
+//   k-side  M = 128 output channels, N = consecutive column shifts x channels (up to 256).  Every MMA has the N that its shifts need: at
+//           stride 2 a 3x3 filter takes two shifts of the even columns and one of the odd, 128 + 64 accumulator columns, where two
+//           equal MMAs would overrun them (fp32 64->128 on 28x28, N = 64: bound by the operands' reads of c-side MMAs of N = 64 before,
+//           30.9 -> 27.4 us).  Filters too wide for 64 channels a tile take 32 or 16 (c-side MMAs of N = 32 to 64 before, bound the same
+//           way; bf16 5x5 72->200 on 15x15, N = 60 39 -> 29, fp32 216 -> 124, fp32 7x7 160->120 on 21x21, N = 20 466 -> 111).
 //   c-side  (few output channels) M = 128 = shifts x channels of X, N = output channels; M = 64 MMAs would take as
 //           long as M = 128 ones, so with K <= 64 this form is the faster one although one shift in four is unused.
 //   stack   (at most 64 output channels, stride 1) M = 128 = filter rows x output channels: the reduction walks over rows of X, and
@@ -87,6 +91,8 @@ enum { kFlat = 0, kPaired = 1, kPixels = 2, kImages = 3 };
 struct ClGroup {            // one MMA of a k-step
     int x_off;              // offset of its X rows inside the X region of a stage, 16-byte units
     int r, s0, cnt, cbase;  // filter row, first column shift, atoms in use, first channel (relative to the c-tile)
+    int col, n;             // its first accumulator column, and how many it has
+    uint32_t idesc;         // n in the instruction descriptor's place
 };
 
 struct ClParams {
@@ -112,7 +118,7 @@ struct ClParams {
     int stack;                      // 1: filter rows x output channels are the M side; chunks are bands of X rows
     int s_inner;                    // 1: column shifts lie next to one another in dW (K x C x R x S): columns are written shift by shift
     int merged;                     // 1: the MN atoms of an X operand are channel atoms, 0: column shifts
-    int ngroups, nmma, cols, tmem_cols;
+    int ngroups, cols, tmem_cols;
     int mma_cols;                   // columns of all MMAs of a chunk and product
     int epoch;                      // chunks of one issuer between two readings of its accumulators
     uint32_t dy_hi, x_lbo, dy_lbo, idesc;
@@ -126,13 +132,21 @@ struct ClParams {
 __device__ constexpr uint32_t prod_x(int i) { return i == 1 ? 2u : (i == 2 || i == 4) ? 1u : 0u; }
 __device__ constexpr uint32_t prod_dy(int i) { return i == 0 ? 2u : (i == 2 || i == 3) ? 1u : 0u; }
 
+// The MMA that writes a column
+__device__ __forceinline__ int group_of(const ClParams& P, int col)
+{
+    int g = 0;
+    while (g + 1 < P.ngroups && col >= P.g[g + 1].col) ++g;
+    return g;
+}
 // The e-th column of a k-side block in the order of dW: where the shifts of a channel are neighbours in memory, shift by shift,
 // so that a store of 32 lanes touches 13 sectors instead of 32 (K x C x R x S, 512->512 on 2x2 maps: the stores were 12 of 24 us).
 __device__ __forceinline__ int written_column(const ClParams& P, int e)
 {
     if (P.c_side || !P.s_inner) return e;
-    const int g = e / P.nmma, j = e - g * P.nmma, atoms = P.nmma / P.ca, c = j / atoms;
-    return g * P.nmma + (j - c * atoms) * P.ca + c;
+    const ClGroup& g = P.g[group_of(P, e)];
+    const int j = e - g.col, atoms = g.n / P.ca, c = j / atoms;
+    return g.col + (j - c * atoms) * P.ca + c;
 }
 // Element (column, lane) of a block that goes to dW directly, in words: [column][128], the lanes of a column exchanged by a key, so that neither a column's
 // lanes, nor a lane's columns, nor the shifts of a channel meet in one bank.
@@ -141,8 +155,8 @@ __device__ __forceinline__ int block_key(int col, int ca_log) { return (col + 11
 // (stack: without the filter row, which belongs to the lane)
 __device__ __forceinline__ int2 column_target(const ClParams& P, int col, int k0, int c0, int r0)
 {
-    const int gi = col / P.nmma, j = col - gi * P.nmma;
-    const ClGroup& g = P.g[gi];
+    const ClGroup& g = P.g[group_of(P, col)];
+    const int j = col - g.col;
     const int a = P.c_side || P.merged ? 0 : j / P.ca, k = P.c_side ? k0 + j : 0;
     const int c = c0 + g.cbase + (P.c_side ? 0 : P.merged ? j : j - a * P.ca);
     const bool valid = r0 + g.r < P.r && (P.c_side ? k < P.k : c < P.c && a < g.cnt);
@@ -169,8 +183,8 @@ struct ClElement { int k, c, r, s; bool valid; };
 __device__ __forceinline__ ClElement cl_element(const ClParams& P, int tile, int col, int l)
 {
     const int tr = tile / P.tiles_r, r0 = (tile - tr * P.tiles_r) * P.rc, tk = tr / P.tiles_c, k0 = tk * P.kt, c0 = (tr - tk * P.tiles_c) * P.ct;
-    const int gi = col / P.nmma, j = col - gi * P.nmma, ca_log = 31 - __clz(P.ca), ka_log = 31 - __clz(P.ka);
-    const ClGroup& g = P.g[gi];
+    const ClGroup& g = P.g[group_of(P, col)];
+    const int j = col - g.col, ca_log = 31 - __clz(P.ca), ka_log = 31 - __clz(P.ka);
     const int mn = P.c_side ? l : j, a = P.merged ? 0 : mn >> ca_log;
     ClElement e;
     e.c = c0 + g.cbase + (P.merged ? mn : mn & (P.ca - 1)); e.s = g.s0 + P.stride * a;
@@ -332,7 +346,7 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
             const int lo = max(0, (P.pad_h - r0 + P.stride - 1) / P.stride), hi = min(P.p, (P.h - 1 + P.pad_h - r0) / P.stride + 1);
             if (lo < hi) { k_first = lo * P.skip; ksteps = hi * P.skip; }       // (none: multiply the zeros)
         }
-        const uint32_t nmma = P.nmma, idesc = P.idesc;
+        const uint32_t idesc = P.idesc;
         uint32_t off[NG];
 #pragma unroll
         for (int g = 0; g < NG; ++g) off[g] = NG <= 9 || g < ngroups ? (uint32_t)P.g[g].x_off : 0u;
@@ -366,8 +380,8 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
                         for (int g = 0; g < NG; ++g)
                             if (NG <= 9 || g < ngroups) {          // (up to nine MMAs there is an instance for every count)
                                 const uint64_t ad = CSIDE ? xd + off[g] : dyd, bd = CSIDE ? dyd : xd + off[g];
-                                const uint32_t d = acc + (NG == 1 && !CSIDE ? o.w & 0xffffu : g * nmma);
-                                const uint32_t id = NG == 1 && !CSIDE ? idesc | (o.w & 0xffff0000u) : idesc;
+                                const uint32_t d = acc + (NG == 1 && !CSIDE ? o.w & 0xffffu : (uint32_t)P.g[g].col);
+                                const uint32_t id = idesc | (NG == 1 && !CSIDE ? o.w & 0xffff0000u : P.g[g].idesc);
                                 if (starts && pr == 0) umma_bf16(d, ad, bd, id, 0u);
                                 else umma_bf16_acc(d, ad, bd, id);
                             }
@@ -931,7 +945,7 @@ int shifts_of(const ClParams& P)
 // the last column shift that an MMA touches, in use or not
 int far_shift(const ClParams& P)
 {
-    const int shifts = ceil_div(P.s, P.stride), atoms = P.merged ? 1 : shifts_of(P);
+    const int shifts = ceil_div(P.s, P.stride), atoms = P.c_side && !P.merged ? shifts_of(P) : 1;
     return ceil_div(shifts, atoms) * atoms - 1;
 }
 
@@ -942,9 +956,12 @@ bool build_groups(ClParams& P)
     // atoms of one MMA on the X side: c-side exactly fills M = 128; k-side as many as N = 256 takes, the shifts of a column phase
     // shared out evenly over as few MMAs as hold them
     const int atoms = P.merged ? P.na : shifts_of(P);
+    P.cols = 0;
     auto add = [&](int tile_i, int row_px, int r, int s0, int cnt, int cbase) {
         if (P.ngroups == kMaxGroups) return false;
-        P.g[P.ngroups++] = ClGroup{(tile_i * P.x_alloc + row_px * P.px_rows * P.ca * 2) >> 4, r, s0, cnt, cbase};
+        const int n = P.c_side ? P.kt : (P.merged ? P.na : cnt) * P.ca;
+        P.g[P.ngroups++] = ClGroup{(tile_i * P.x_alloc + row_px * P.px_rows * P.ca * 2) >> 4, r, s0, cnt, cbase, P.cols, n, (uint32_t)(n >> 3) << 17};
+        P.cols += n;
         return true;
     };
     for (int rl = 0; rl < rows; ++rl)
@@ -960,9 +977,7 @@ bool build_groups(ClParams& P)
                         if (!add(base_tile + a, base_px + i, rl, ph + st * i, std::min(atoms, shifts - i), a * P.ca)) return false;
             }
         }
-    P.nmma = P.c_side ? P.kt : atoms * P.ca;
     P.s_inner = !P.merged && P.s > 1 && P.ws_s < P.ws_c;
-    P.cols = P.ngroups * P.nmma;
     if (P.cols > kMaxCols) return false;
     P.tmem_cols = 32;
     while (P.tmem_cols < 2 * P.cols) P.tmem_cols *= 2;
@@ -1061,10 +1076,10 @@ bool shape_chunk(ClParams& P, int ci, int bp, int order, bool bare = false)
     if (!build_groups(P)) return false;
     if (!P.c_side && P.ngroups == 1)
         for (int i = 0; i < P.ksteps; ++i) {
-            if (!bare || P.k_off[i].w >> 17 == 0) P.k_off[i].w = (unsigned)(P.nmma >> 3) << 17;
+            if (!bare || P.k_off[i].w >> 17 == 0) P.k_off[i].w = P.g[0].idesc;
             P.mma_cols += (P.k_off[i].w >> 17) * 8;
         }
-    else P.mma_cols = P.ksteps * P.ngroups * P.nmma;
+    else P.mma_cols = P.ksteps * P.cols;
     return true;
 }
 
@@ -1150,8 +1165,8 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
             F.ka = kw > 32 ? 64 : kw > 16 ? 32 : 16;
             F.katoms = ceil_div(kw, F.ka);
             F.tiles_k = ceil_div(g.k, F.kt);
-            // (stack: with wide filters fewer channels a tile, so that all shifts fit one MMA and the accumulators)
-            for (int ca = B.ca; ca >= (form == 2 && g.s > 3 ? 16 : B.ca); ca /= 2)
+            // (M side output channels, wide filters: fewer channels a tile, so that all shifts fit the accumulators)
+            for (int ca = B.ca; ca >= ((form == 2 && g.s > 3) || (form == 0 && g.s * B.ca > kMaxCols) ? 16 : B.ca); ca /= 2)
             for (int na = 1; na <= 4; na *= 2) {
                 F.ca = ca;
                 if (na > 1 && (F.ca < 64 || (na - 1) * 64 >= g.c)) break;
@@ -1234,8 +1249,8 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
     if (best_cycles >= 1e30) return false;
     best.chunk_base = best.chunks / best.splits;
     best.chunk_rem = best.chunks - best.chunk_base * best.splits;
-    // fp32 accumulators, bf16 operands, both MN-major (dY K-major where it is read as it lies), N, M = 128
-    best.idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | (best.c_side || best.ngroups > 1 ? (uint32_t)(best.nmma >> 3) << 17 : 0u) | (8u << 24);
+    // fp32 accumulators, bf16 operands, both MN-major (dY K-major where it is read as it lies), M = 128; N is the group's
+    best.idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | (8u << 24);
     if (best.order == kPixels) { best.idesc &= ~(best.c_side ? 1u << 16 : 1u << 15); H.pack_dy = false; }
     H.p = best;
     // second kernel: at most eight loads a thread, a block of at most 32 warps, and as many blocks as there are SMs where the

@@ -35,6 +35,10 @@ SHAPES = [
     ConvLayer("7x3 filter", 9, 70, 12, 16, 64, 7, 3, 1, 1),
     ConvLayer("odd pixels past a tile, 3 and 70 channels", 15, 3, 33, 35, 70, 3, 3, 1, 1),
     ConvLayer("odd pixels, 24 and 12 channels", 9, 24, 21, 15, 12, 5, 5, 1, 2),
+    ConvLayer("stride 2, MMAs of two column shifts and of one", 6, 70, 23, 19, 130, 3, 3, 2, 1),
+    ConvLayer("stride 3, 7x7: three shifts, two and two", 12, 30, 30, 25, 100, 7, 7, 3, 3),
+    ConvLayer("5x5, tiles of 32 of 72 channels", 5, 72, 15, 15, 136, 5, 5, 1, 2),
+    ConvLayer("7x7, tiles of 16 of 70 channels", 6, 70, 13, 10, 131, 7, 7, 1, 3),
 ]
 LAYOUTS = {"paper": {}, "nchw": dict(x_layout=B.X_NCHW, dw_layout=B.DW_KCRS),
            "nhwc": dict(dy_layout=B.DY_NPQK, dw_layout=B.DW_KCRS), "rsck": dict(x_layout=B.X_NCHW, dy_layout=B.DY_NPQK, dw_layout=B.DW_RSCK)}
