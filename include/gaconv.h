@@ -97,7 +97,8 @@ uint64_t gaconv_launch_count(void);
 /* Device scratch one call needs for `method` (GACONV_METHOD_EXACT for the exact path) with this
  * descriptor (its workspace fields are ignored).  Never fails for a valid descriptor; *bytes > 0.
  * The size has room for the copies of operands that the fastest kernel wants in another form: channels-last bf16, i.e.
- * two bytes an element of a bf16 operand and six of an fp32 one.  A call with a smaller workspace takes the kernels that need
+ * two bytes an element of a bf16 operand (whose pixels may lie up to a third further apart than its channels fill) and six of
+ * an fp32 one.  A call with a smaller workspace takes the kernels that need
  * no such copies (slower, and another rounding), down to what those need. */
 gaconv_status_t gaconv_workspace_size(const gaconv_conv_desc_t *desc, int32_t method, size_t *bytes);
 

@@ -137,7 +137,7 @@ Top1Layout build_top1_layout(const Geom& g, bool cl)
     // the contraction: by the channels-last kernel, which reads either form of the sparse tensor (256->256 on 8x8, N = 256:
     // 37 us with the other kernel, 32)
     L.cl = cl && L.dense && tensor_maps_available() && plan_cl(g, L.tp.reads_transposed_dy, &L.cp) && !short_sums(g, L.cp);
-    const size_t cl_scratch = L.cl ? L.cp.x_bytes + L.cp.dy_bytes : 0;
+    const size_t cl_scratch = L.cl ? L.cp.x_bytes[0] + L.cp.dy_bytes[0] : 0;
     const size_t maps = (size_t)g.n * g.k;
     L.idx_off = kWsDataOffset;
     L.sum_off = align_up(L.idx_off + maps * sizeof(int32_t), 256);
@@ -236,7 +236,7 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, const ClPlan& plan, bool reo
     // operands must be packed (16->64 on 6x6, N = 30 launched one by one 10.3 / 12.3 us; 1x1 80->22 on 6x6, N = 105 25 / 12), and with three channels
     return products > (!g.bf16 && g.r * g.s >= 9 ? 2e7 : g.c <= 4 ? 1e7 : 4e6);
 }
-struct ClRoute { bool use; ClPlan plan; size_t partial_off, x_off, dy_off, total; };
+struct ClRoute { bool use; ClPlan plan; size_t partial_off, x_off, dy_off[2], total[2]; };       // [0] copies packed tightly, [1] on aligned rows
 ClRoute build_cl_route(const gaconv_conv_desc_t* desc, const Geom& g)
 {
     ClRoute R{};
@@ -252,8 +252,10 @@ ClRoute build_cl_route(const gaconv_conv_desc_t* desc, const Geom& g)
 #endif
     R.partial_off = kWsDataOffset;
     R.x_off = align_up(R.partial_off + R.plan.partial_bytes, 256);
-    R.dy_off = R.x_off + R.plan.x_bytes;
-    R.total = R.dy_off + R.plan.dy_bytes;
+    for (int wide = 0; wide < 2; ++wide) {
+        R.dy_off[wide] = R.x_off + R.plan.x_bytes[wide];
+        R.total[wide] = R.dy_off[wide] + R.plan.dy_bytes[wide];
+    }
     return R;
 }
 bool cl_route(const gaconv_conv_desc_t* desc, const Geom& g, ClRoute* R)
@@ -413,13 +415,13 @@ struct gaconv_schedule {
     struct StepCache* steps = nullptr;      // repeated steps as CUDA graphs, created on first use
 };
 
-gaconv_status_t gaconv::method_workspace(const gaconv_conv_desc_t* desc, int32_t method, bool cl, size_t* bytes)
+gaconv_status_t gaconv::method_workspace(const gaconv_conv_desc_t* desc, int32_t method, bool cl, bool least, size_t* bytes)
 {
     Geom g;
     gaconv_status_t st = make_geom(desc, &g);
     if (st != GACONV_OK) return st;
     ClRoute C;
-    if (cl && method == GACONV_METHOD_EXACT && cl_route(desc, g, &C)) { *bytes = C.total; return GACONV_OK; }
+    if (cl && method == GACONV_METHOD_EXACT && cl_route(desc, g, &C)) { *bytes = C.total[!least]; return GACONV_OK; }
     const Relayout R = plan_relayout(desc, method, cl);
     if (R.move_x || R.move_dy) { *bytes = moved_ws_bytes(desc, g, R); return GACONV_OK; }
     bool ok = false;
@@ -439,12 +441,13 @@ gaconv_status_t gaconv::run_exact(const void* x, const void* dy, float* dw, cons
     if (desc->math == GACONV_MATH_TF32 && g.bf16) return GACONV_ERR_BAD_DESC;
     ClRoute C;
     // (a workspace without room for the packed operands: the kernels that need none, as far as it goes)
-    if (cl && cl_route(desc, g, &C) && (desc->workspace == nullptr || desc->workspace_bytes >= C.total)) {
-        st = check_ws(desc, C.total);
+    if (cl && cl_route(desc, g, &C) && (desc->workspace == nullptr || desc->workspace_bytes >= C.total[0])) {
+        st = check_ws(desc, C.total[0]);
         if (st != GACONV_OK) return st;
+        const bool wide = desc->workspace_bytes >= C.total[1];
         char* ws = static_cast<char*>(desc->workspace);
-        return launch_cl(x, dy, dw, reinterpret_cast<float*>(ws + C.partial_off), ws + C.x_off, ws + C.dy_off, reinterpret_cast<uint32_t*>(ws),
-                         C.plan, stream) == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
+        return launch_cl(x, dy, dw, reinterpret_cast<float*>(ws + C.partial_off), ws + C.x_off, ws + C.dy_off[wide],
+                         reinterpret_cast<uint32_t*>(ws), C.plan, wide, stream) == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
     }
     if (desc->dy_layout == GACONV_DY_NPQK && g.k > 1 && desc->algo != GACONV_ALGO_DIRECT) {
         // Small maps: the tensor-core kernel's dY operand IS the channels-last order (its pre-pass would transpose an
@@ -530,7 +533,7 @@ uint64_t gaconv_launch_count(void) { return g_launches.load(std::memory_order_re
 gaconv_status_t gaconv_workspace_size(const gaconv_conv_desc_t* desc, int32_t method, size_t* bytes)
 {
     if (bytes == nullptr) return GACONV_ERR_NULL_POINTER;
-    return method_workspace(desc, method, true, bytes);
+    return method_workspace(desc, method, true, false, bytes);
 }
 
 gaconv_status_t gaconv_workspace_init(void* workspace, size_t bytes, void* stream)
@@ -607,7 +610,7 @@ gaconv_status_t gaconv_dw_approx(int32_t method, const void* x, const void* dy, 
         if (L.cl) {
             char* packed = ws + L.scratch_off + L.tp.scratch_bytes;
             return launch_cl(x, sparse != nullptr ? sparse : ws + L.scratch_off, dw, reinterpret_cast<float*>(ws + L.partial_off), packed,
-                             packed + L.cp.x_bytes, reinterpret_cast<uint32_t*>(ws), L.cp, cs) == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
+                             packed + L.cp.x_bytes[0], reinterpret_cast<uint32_t*>(ws), L.cp, false, cs) == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
         }
         return launch_tc(x, sparse, dw, reinterpret_cast<float*>(ws + L.partial_off), ws + L.scratch_off,
                          reinterpret_cast<uint32_t*>(ws + kWsCounterOffset), reinterpret_cast<uint32_t*>(ws), L.tp,
@@ -667,8 +670,8 @@ static gaconv_status_t dw_from_host(int32_t method, const void* x_host, const vo
         if (!aligned16(x_dev) || !aligned16(dy_dev)) return GACONV_ERR_MISALIGNED;
         if (method == GACONV_METHOD_EXACT && desc->math == GACONV_MATH_TF32 && g.bf16) return GACONV_ERR_BAD_DESC;
         size_t need = 0;
-        st = method_workspace(desc, method, true, &need);
-        if (st == GACONV_OK && desc->workspace_bytes < need) st = method_workspace(desc, method, false, &need);
+        st = method_workspace(desc, method, true, true, &need);
+        if (st == GACONV_OK && desc->workspace_bytes < need) st = method_workspace(desc, method, false, true, &need);
         if (st != GACONV_OK) return st;
         st = check_ws(desc, need);
         if (st != GACONV_OK) return st;

@@ -683,7 +683,8 @@ cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, cons
 struct PackOp {
     const void* src;
     __nv_bfloat16* dst;
-    int ch, chp, px, n;         // source: n images of px pixels and ch channels; destination rows of chp channels
+    int ch, chp, px, n;         // source: n images of px pixels and ch channels; destination rows of chp channels,
+    int pitch;                  // this many apart
     int channels_last;          // source order: 1 [n][px][ch], 0 [n][ch][px]
     int px_tiles, ch_tiles;     // tiles of an image (channels-first sources): tile_px pixels x
     int ch_tile;                // at most 64 channels, a multiple of 8
@@ -770,7 +771,7 @@ pack_kernel(const PackOp x, const PackOp dy)
 #pragma unroll
                 for (int j = 0; j < 8; ++j) v[j] = c + j < o.ch ? __ldg(p + j) : E(0);
             }
-            store8(v, o.dst + (size_t)row * o.chp + c, o.plane);
+            store8(v, o.dst + (size_t)row * o.pitch + c, o.plane);
         }
         return;
     }
@@ -795,7 +796,7 @@ pack_kernel(const PackOp x, const PackOp dy)
             alignas(16) E v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) v[u] = 8 * q + u < rows ? p[u * o.px] : E(0);
-            store8(v, o.dst + ((size_t)(n0 + i) * o.px + j) * o.chp + c0 + 8 * q, o.plane);
+            store8(v, o.dst + ((size_t)(n0 + i) * o.px + j) * o.pitch + c0 + 8 * q, o.plane);
         }
         return;
     }
@@ -828,7 +829,7 @@ pack_kernel(const PackOp x, const PackOp dy)
 #pragma unroll
         for (int u = 0; u < 8; ++u) at[u] = s_tile + (r8 + u) * pitch + q * 16 + ((first_off + (r8 + u) * row_bytes) & 15);
         const int valid = rows - r8;
-        __nv_bfloat16* d = o.dst + ((size_t)n * o.px + p0) * o.chp + c0 + r8;
+        __nv_bfloat16* d = o.dst + ((size_t)n * o.px + p0) * o.pitch + c0 + r8;
 #pragma unroll 2
         for (int j = threadIdx.x >> log_q; j < left; j += 256 >> log_q) {
             alignas(16) E v[8];
@@ -838,7 +839,7 @@ pack_kernel(const PackOp x, const PackOp dy)
 #pragma unroll
                 for (int u = 0; u < 8; ++u) if (u >= valid) v[u] = E(0);
             }
-            store8(v, d + (size_t)j * o.chp, o.plane);
+            store8(v, d + (size_t)j * o.pitch, o.plane);
         }
         return;
     }
@@ -889,7 +890,7 @@ pack_kernel(const PackOp x, const PackOp dy)
             asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
                          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(tile + pl * 64 * ROW + at(row, 8 * blk8)) : "memory");
             if (px < left && c < end)
-                *reinterpret_cast<uint4*>(o.dst + pl * o.plane + ((size_t)n * o.px + p0 + px) * o.chp + c) = make_uint4(r[0], r[1], r[2], r[3]);
+                *reinterpret_cast<uint4*>(o.dst + pl * o.plane + ((size_t)n * o.px + p0 + px) * o.pitch + c) = make_uint4(r[0], r[1], r[2], r[3]);
         }
     }
 }
@@ -1086,17 +1087,28 @@ bool shape_chunk(ClParams& P, int ci, int bp, int order, bool bare = false)
 struct ClHost {             // what ClPlan::opaque holds
     ClParams p;
     bool pack_x, pack_dy, f32, x_nhwc, dy_npqk;
-    int xch, dych;          // channels per pixel row of the operands the tensor maps describe
+    int xch[2], dych[2];    // elements from one pixel of the operands to the next: packed tightly, and on aligned rows
     int log_cb, groups;     // second kernel: columns per block, split groups per column
     bool lean;              // second kernel: with few registers
 };
 static_assert(sizeof(ClHost) <= sizeof(ClPlan::opaque), "ClPlan::opaque too small");
 
-PackOp pack_op(const void* src, void* dst, int ch, int px, int n, bool last, size_t plane, int tile_px)
+// Elements from one pixel of a packed operand to the next.  64-channel boxes are read a pixel, 128 bytes, at a time: where pixels lie 240
+// bytes apart (120 channels) most reads take two lines.  So rows are spread to whole multiples of 128 bytes where that makes the operand
+// no more than a third longer (bf16 72->120 on 28x20, N = 100: main loop 27,000 -> 22,500 cycles, whole call 36.2 -> 33.9 us; 24->100 on
+// 28x28, N = 60 22.4 -> 22.0).  Not 72 channels (21,200 cycles on rows of 144 bytes against 22,500 on 256), nor the planes of fp32
+// operands, whose six products hide the reads (40->40 on 28x28, N = 60 47.0 / 52.7).
+int wide_pitch(int ch, int atom)
+{
+    const int tight = round_up(ch, 8), wide = round_up(ch, atom);
+    return atom == 64 && 3 * wide <= 4 * tight ? wide : tight;
+}
+
+PackOp pack_op(const void* src, void* dst, int ch, int pitch, int px, int n, bool last, int tile_px)
 {
     PackOp o{};
     o.src = src; o.dst = static_cast<__nv_bfloat16*>(dst);
-    o.ch = ch; o.chp = round_up(ch, 8); o.px = px; o.n = n; o.channels_last = last ? 1 : 0; o.plane = plane;
+    o.ch = ch; o.chp = round_up(ch, 8); o.pitch = pitch; o.px = px; o.n = n; o.channels_last = last ? 1 : 0; o.plane = (size_t)n * px * pitch;
     const int vec = tile_px == kPackPx<float> ? 4 : 8;
     o.ch_tiles = ceil_div(ch, 64);
     o.ch_tile = round_up(ceil_div(ch, o.ch_tiles), 8);
@@ -1138,8 +1150,7 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
     H.x_nhwc = nhwc; H.dy_npqk = dy_npqk || g.k == 1;
     H.pack_x = H.f32 || !nhwc || g.c % 8 != 0;
     H.pack_dy = H.f32 || !H.dy_npqk || g.k % 8 != 0;
-    H.xch = round_up(g.c, 8); H.dych = round_up(g.k, 8);
-    const size_t x_el = (size_t)g.n * g.h * g.w * H.xch, dy_el = (size_t)g.n * g.p * g.q * H.dych;
+    const size_t x_px = (size_t)g.n * g.h * g.w, dy_px = (size_t)g.n * g.p * g.q, x_el = x_px * round_up(g.c, 8), dy_el = dy_px * round_up(g.k, 8);
     if (x_el > ((size_t)1 << 31) || dy_el > ((size_t)1 << 31)) return false;
 
     ClParams B{};
@@ -1264,26 +1275,30 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
     if (tiles > 65535 || best.splits > 65535) return false;
     out->cycles = best_cycles;
     out->partial_bytes = best.splits == 1 ? 0 : (size_t)tiles * best.splits * best.cols * 512;
-    out->x_bytes = H.pack_x ? align_up(x_el * 2 * best.planes, 256) : 0;
-    out->dy_bytes = H.pack_dy ? align_up(dy_el * 2 * best.planes, 256) : 0;
+    for (int wide = 0; wide < 2; ++wide) {
+        H.xch[wide] = wide && H.pack_x && !H.f32 ? wide_pitch(g.c, best.ca) : round_up(g.c, 8);
+        H.dych[wide] = wide && H.pack_dy && !H.f32 ? wide_pitch(g.k, best.ka) : round_up(g.k, 8);
+        out->x_bytes[wide] = H.pack_x ? align_up(x_px * H.xch[wide] * 2 * best.planes, 256) : 0;
+        out->dy_bytes[wide] = H.pack_dy ? align_up(dy_px * H.dych[wide] * 2 * best.planes, 256) : 0;
+    }
     memcpy(out->opaque, &H, sizeof(H));
     return true;
 }
 
 cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, void* x_scratch, void* dy_scratch, uint32_t* status,
-                      const ClPlan& plan, cudaStream_t stream)
+                      const ClPlan& plan, bool wide, cudaStream_t stream)
 {
     ClHost H;
     memcpy(&H, plan.opaque, sizeof(H));
     const ClParams& P = H.p;
     cudaError_t err;
     const ClSource src{x, dy, H.f32, H.x_nhwc, H.dy_npqk};
-    const size_t x_el = (size_t)P.n * P.h * P.w * H.xch, dy_el = (size_t)P.n * P.p * P.q * H.dych;
+    const int xch = H.xch[wide], dych = H.dych[wide];
     if (H.pack_x || H.pack_dy) {
         PackOp ox{}, od{};
         const int tile_px = H.f32 ? kPackPx<float> : kPackPx<unsigned short>;
-        if (H.pack_x) ox = pack_op(x, x_scratch, P.c, P.h * P.w, P.n, H.x_nhwc, x_el, tile_px);
-        if (H.pack_dy) od = pack_op(dy, dy_scratch, P.k, P.p * P.q, P.n, H.dy_npqk, dy_el, tile_px);
+        if (H.pack_x) ox = pack_op(x, x_scratch, P.c, xch, P.h * P.w, P.n, H.x_nhwc, tile_px);
+        if (H.pack_dy) od = pack_op(dy, dy_scratch, P.k, dych, P.p * P.q, P.n, H.dy_npqk, tile_px);
         const dim3 grid((unsigned)(ox.blocks + od.blocks));
         err = H.f32 ? launch_kernel(pack_kernel<float>, grid, dim3(256), 0, stream, dim3(1, 1, 1), ox, od)
                     : launch_kernel(pack_kernel<unsigned short>, grid, dim3(256), 0, stream, dim3(1, 1, 1), ox, od);
@@ -1293,10 +1308,10 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
         if (H.pack_dy) dy = dy_scratch;
     }
     // tensor maps over (channel, column, row, image, plane), the rows of a box in the order of the reduction; box extents count the pixels stepped over at the conv stride
-    auto encode = [&](CUtensorMap* map, const void* base, int ch, int chp, int w, int h, size_t plane_el, int atom, int bw, int bh, int st) {
-        const cuuint64_t row = (cuuint64_t)chp * 2;
+    auto encode = [&](CUtensorMap* map, const void* base, int ch, int pitch, int w, int h, int atom, int bw, int bh, int st) {
+        const cuuint64_t row = (cuuint64_t)pitch * 2;
         cuuint64_t dims[5] = {(cuuint64_t)ch, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)P.n, (cuuint64_t)P.planes};
-        cuuint64_t strides[4] = {row, row * w, row * w * h, (cuuint64_t)plane_el * 2};
+        cuuint64_t strides[4] = {row, row * w, row * w * h, row * w * h * P.n};
         cuuint32_t box[5] = {(cuuint32_t)atom, (cuuint32_t)((bw - 1) * st + 1), (cuuint32_t)((bh - 1) * st + 1), (cuuint32_t)P.ci, 1};
         cuuint32_t es[5] = {1, (cuuint32_t)st, (cuuint32_t)st, 1, 1};
         if (P.order == kImages) {        // (channel, image, column, row, plane)
@@ -1314,8 +1329,8 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
         return encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(dy), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
-    if (!(P.order == kPixels ? encode_pixels(&map_dy) : encode(&map_dy, dy, P.k, H.dych, P.q, P.p, dy_el, P.ka, P.dy_pitch, P.dy_img / P.dy_pitch, 1)) ||
-        !encode(&map_x, x, P.c, H.xch, P.w, P.h, x_el, P.ca, P.x_pitch, P.x_img / P.x_pitch, P.stride))
+    if (!(P.order == kPixels ? encode_pixels(&map_dy) : encode(&map_dy, dy, P.k, dych, P.q, P.p, P.ka, P.dy_pitch, P.dy_img / P.dy_pitch, 1)) ||
+        !encode(&map_x, x, P.c, xch, P.w, P.h, P.ca, P.x_pitch, P.x_img / P.x_pitch, P.stride))
         return cudaErrorInvalidValue;
     // the stages; at the end they hold the accumulator block
     const size_t smem = std::max((size_t)P.stages * P.stage_bytes + P.slack, (size_t)P.cols * 512) + 1024;

@@ -171,18 +171,20 @@ cudaError_t launch_tc(const void* x, const void* dy, float* dw, float* partial, 
 // ---- exact filter gradient on tcgen05 with channels-last bf16 operands: any map size, channel count, stride, layout and type ----
 struct ClPlan {
     double cycles;                          // the planner's estimate of the two kernels, SM cycles
-    size_t partial_bytes, x_bytes, dy_bytes;    // workspace: accumulator blocks, packed copies of the operands (0: read in place)
+    size_t partial_bytes;                   // workspace: accumulator blocks, and
+    size_t x_bytes[2], dy_bytes[2];         // packed copies of the operands (0: read in place), [0] tightly, [1] on aligned rows
     alignas(8) unsigned char opaque[3072];  // kernel parameters, private to cl.cu
 };
 bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* plan);
 cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, void* x_scratch, void* dy_scratch, uint32_t* status,
-                      const ClPlan& plan, cudaStream_t stream);
+                      const ClPlan& plan, bool wide, cudaStream_t stream);        // wide: the copies on aligned rows
 
 int device_sms();       // SMs of the current device
 bool tensor_maps_available();       // the driver's tensor-map encoder was found
 
-// gaconv_workspace_size and gaconv_dw_exact; cl = false: without the channels-last kernel (callers whose scratch it does not fit)
-gaconv_status_t method_workspace(const gaconv_conv_desc_t* desc, int32_t method, bool cl, size_t* bytes);
+// gaconv_workspace_size and gaconv_dw_exact; cl = false: without the channels-last kernel (callers whose scratch it does not fit),
+// least: with the least scratch that it runs in
+gaconv_status_t method_workspace(const gaconv_conv_desc_t* desc, int32_t method, bool cl, bool least, size_t* bytes);
 gaconv_status_t run_exact(const void* x, const void* dy, float* dw, const gaconv_conv_desc_t* desc, cudaStream_t stream, bool cl);
 
 }  // namespace gaconv

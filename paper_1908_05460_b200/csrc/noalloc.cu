@@ -76,9 +76,9 @@ gaconv_status_t gaconv_dw_exact_static(const void* x, const void* dy, float* dw,
     if (desc == nullptr) return GACONV_ERR_NULL_POINTER;
     // the kernels of gaconv_dw_exact where their scratch fits, else those that need less of it
     size_t need = 0;
-    gaconv_status_t st = gaconv::method_workspace(desc, GACONV_METHOD_EXACT, true, &need);
+    gaconv_status_t st = gaconv::method_workspace(desc, GACONV_METHOD_EXACT, true, true, &need);
     const bool cl = st == GACONV_OK && need <= kStaticScratchBytes;
-    if (st == GACONV_OK && !cl) st = gaconv::method_workspace(desc, GACONV_METHOD_EXACT, false, &need);
+    if (st == GACONV_OK && !cl) st = gaconv::method_workspace(desc, GACONV_METHOD_EXACT, false, true, &need);
     if (st != GACONV_OK) return st;
     if (need > kStaticScratchBytes) return GACONV_ERR_WORKSPACE_TOO_SMALL;   // problem too large for the built-in scratch
     if (x == nullptr || dy == nullptr || dw == nullptr) return GACONV_ERR_NULL_POINTER;

@@ -205,6 +205,24 @@ def test_smaller_workspaces(layer, dtype, kw, method):
         assert len(accepted) > 1, (full, accepted)
 
 
+def test_packed_rows_tight_and_spread():
+    """A packed bf16 gradient of 120 channels on rows of 128, or without gaps where the workspace has no room for those: the same bits."""
+    layer = ConvLayer("28x20", 6, 72, 28, 20, 120, 3, 3, 1, 1)
+    x, dy = I.make_layer_inputs(layer, torch.bfloat16, 23, 0)
+    g = GpuLayer(layer, torch.bfloat16, x, dy, x_layout=B.X_NCHW)
+    want, full = g.exact(), B.gaconv_workspace_size(g.desc, B.METHOD_EXACT)
+    ref, dn = oracle.dw_exact(to_f64(x), to_f64(dy), oshape(layer))
+    assert norm_err(want, ref, dn) <= TOL_F32 / 2
+    tight = full - 6 * 28 * 20 * (128 - 120) * 2
+    for size, kernel in ((full, "cl_kernel"), (full - 16, "cl_kernel"), (tight, "cl_kernel"), (tight - 16, "direct_tiled_kernel")):
+        g.desc.workspace_bytes = size
+        assert any(kernel in n for n in kernel_names(lambda: B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc))), size
+        got = g.exact()
+        assert norm_err(got, ref, dn) <= TOL_F32
+        if kernel == "cl_kernel":
+            np.testing.assert_array_equal(got, want)
+
+
 @pytest.mark.parametrize("layer,dtype,kernel", [
     (ConvLayer("channels last, nothing packed", 4, 64, 9, 24, 64, 3, 3, 1, 1), torch.bfloat16, "cl_kernel"),
     (ConvLayer("older tensor-core kernel", 8, 16, 32, 32, 16, 3, 3, 1, 1), torch.bfloat16, "exact_tc_kernel"),
