@@ -217,9 +217,11 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, const ClPlan& plan, bool reo
             if (shared && g.c <= 64 && g.k > 16 && g.k <= 64 && g.stride_h == 1 && products < 1e9) return false;
             // Filters of five and more rows: with few input channels this kernel stacks the rows or has its M side full of shifts
             // (5x5 on 16x16: 32->32 17.6 / 14.4, 40->64 25.0 / 18.1, 32->128 22.9 / 14.8, N = 32 32->64 18.1 / 10.4; 48->64 on 8x8 18.1 / 11.9;
-            // 7x7 32->32 on 16x16 21.0 / 14.3; 24->24 13.9 / 14.3); with 64 and more the older one is as quick or quicker (5x5 64->64 on 16x16
-            // 17.0 / 17.3, 256->256 on 8x8 50 / 55, 7x7 128->128 on 16x16 48 / 105).  3x3 64->64 on 32x32 25.0 / 23.1
-            return g.r < 5 || g.c < 64;
+            // 7x7 32->32 on 16x16 21.0 / 14.3; 24->24 13.9 / 14.3); with 64 and more it is for 5x5 as long as most of M = 128 outputs are in use
+            // (on 16x16 64->88 17.1 / 19.0, 64->96 22.8 / 19.2, 128->128 36.5 / 28.9, on 8x8 256->256 49.0 / 35.7, N = 16 12.2 / 10.4, on 32x32
+            // 64->128, N = 64 35.2 / 28.3; but 64->64 16.2 / 18.9), while wider ones are quicker on the older (7x7 64->128 31.2 / 32.4, 128->128
+            // 47.7 / 66.3).  3x3 64->64 on 32x32 25.0 / 23.1
+            return g.r < 5 || g.c < 64 || (g.r == 5 && g.s <= 5 && g.k >= 96);
         }
         if (L.stem_ok) return reordered || (!shared && g.r * g.s * g.c > 32);       // 5x5 3->64 27.5 / 26.1, 3x3 3->16 11.1 / 16.0
     } else {

@@ -279,6 +279,9 @@ def test_threads_with_layers_of_one_kernel_and_different_shared_memory():
 @pytest.mark.parametrize("layer,budget,kernel", [
     (ConvLayer("5x5, 40 channels", 16, 40, 16, 16, 64, 5, 5, 1, 2), 0, "cl_kernel"),
     (ConvLayer("5x5, 64 channels", 16, 64, 16, 16, 64, 5, 5, 1, 2), 0, "exact_tc_kernel"),
+    (ConvLayer("5x5, 64 channels, 88 outputs", 16, 64, 16, 16, 88, 5, 5, 1, 2), 0, "exact_tc_kernel"),
+    (ConvLayer("5x5, 64 channels, 96 outputs", 16, 64, 16, 16, 96, 5, 5, 1, 2), 0, "cl_kernel"),
+    (ConvLayer("7x7, 64 channels, 128 outputs", 16, 64, 16, 16, 128, 7, 7, 1, 3), 0, "exact_tc_kernel"),
     (ConvLayer("7x7, 24 channels on 32x32", 9, 24, 32, 32, 16, 7, 7, 1, 3), 0, "cl_kernel"),
     (ConvLayer("a large dW with short sums", 64, 256, 8, 8, 256, 3, 3, 1, 1), 0, "exact_tc_kernel"),
     (ConvLayer("a large dW past the line", 96, 256, 8, 8, 256, 3, 3, 1, 1), 0, "cl_kernel"),
