@@ -28,6 +28,33 @@ template <> struct Vec<1> { float v[1]; __device__ void load(const float* p) { v
 template <> struct Vec<2> { float v[2]; __device__ void load(const float* p) { float2 t = *reinterpret_cast<const float2*>(p); v[0] = t.x; v[1] = t.y; } };
 template <> struct Vec<4> { float v[4]; __device__ void load(const float* p) { float4 t = *reinterpret_cast<const float4*>(p); v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w; } };
 
+// The CTA's threads fill `n` floats in turn, `at(i)` the address of the i-th one's source, nullptr: zero.  Eight loads a thread are under way
+// at once (few, where there is little to fill).  Bound by latency: with one load, behind two divisions by numbers that only the launch knows,
+// 16 x 512 pixels took 27 us to arrive.  (us, before / now, with the bands of plan_direct: bf16 1x1 3->80 on 36x36, N = 24 57.6 / 11.5, fp32 3->156
+// on 35x35, N = 10 44.6 / 13.3, bf16 3x3 3->16 on 33x38, N = 3 26.8 / 9.7, fp32 3->20 on 60x60, N = 6 18.0 / 12.5, 1x1 3->304 on 5x5, N = 57 16.9 / 7.3;
+// bf16 20->20 on 9x9, N = 12 11.3 / 11.6.)
+template <int U, typename T, typename At>
+__device__ __forceinline__ void fill_by(int n, At at)
+{
+    for (int i0 = threadIdx.x; i0 < n; i0 += U * kThreads) {
+        const T* src[U];
+        float* dst[U];
+        float v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) { src[u] = nullptr; dst[u] = nullptr; if (i0 + u * kThreads < n) src[u] = at(i0 + u * kThreads, dst[u]); }
+#pragma unroll
+        for (int u = 0; u < U; ++u) { v[u] = 0.f; if (src[u] != nullptr) v[u] = ldf(src[u]); }
+#pragma unroll
+        for (int u = 0; u < U; ++u) if (i0 + u * kThreads < n) *dst[u] = v[u];
+    }
+}
+template <typename T, typename At>
+__device__ __forceinline__ void fill(int n, At at)
+{
+    if (n <= 2 * kThreads) fill_by<2, T>(n, at);
+    else fill_by<8, T>(n, at);
+}
+
 // Stage one work item with the CTA's threads: dY band as [k][pixel] (row stride dys) and X window as
 // [row][col][TC], converted to fp32; four elements per load where the layout allows.
 template <typename T, bool UNUSED, int TK, int TC>
@@ -51,13 +78,16 @@ __device__ __forceinline__ void stage_item(const T* __restrict__ x, const T* __r
             *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
         }
     } else {
-        for (int i = threadIdx.x; i < TK * npx; i += kThreads) {
-            const int kk = i / npx, j = i % npx;
-            const int p = p0 + j / pl.bq, q = q0 + j % pl.bq, k = k0 + kk;
-            float v = 0.f;
-            if (k < g.k && p < g.p && q < g.q) v = ldf(dy + (((long long)n * g.k + k) * g.p + p) * g.q + q);
-            s_dy[kk * dys + j] = v;
-        }
+        const T* base = dy + ((long long)n * g.k + k0) * g.p * g.q + (long long)p0 * g.q + q0;
+        const int pq = g.p * g.q, left_k = g.k - k0, left_p = g.p - p0, left_q = g.q - q0;
+        const bool rows = pl.bq == g.q;           // (then the band's pixels lie end to end)
+        fill<T>(TK * npx, [&](int i, float*& dst) -> const T* {
+            const int kk = pl.by_npx.div(i), j = i - kk * npx;
+            dst = s_dy + kk * dys + j;
+            if (rows) return kk < left_k && j < left_p * g.q ? base + (long long)kk * pq + j : nullptr;
+            const int pp = pl.by_bq.div(j), qq = j - pp * pl.bq;
+            return kk < left_k && pp < left_p && qq < left_q ? base + (long long)kk * pq + pp * g.q + qq : nullptr;
+        });
     }
     if (pl.vec_x) {
         constexpr int CQ = TC / 4;                                // channel quads per pixel of the tile
@@ -75,14 +105,13 @@ __device__ __forceinline__ void stage_item(const T* __restrict__ x, const T* __r
             }
         }
     } else {
-        for (int i = threadIdx.x; i < win_h * win_w * TC; i += kThreads) {
-            const int cc = i % TC, pix = i / TC;
-            const int hh = h0 + pix / win_w, ww = w0 + pix % win_w, c = c0 + cc;
-            float v = 0.f;
-            if (c < g.c && hh >= 0 && hh < g.h && ww >= 0 && ww < g.w)
-                v = ldf(x + n * g.xs_n + c * g.xs_c + hh * g.xs_h + ww * g.xs_w);
-            s_x[i] = v;
-        }
+        const T* base = x + n * g.xs_n + c0 * g.xs_c + h0 * g.xs_h + w0 * g.xs_w;
+        const int left_c = g.c - c0;
+        fill<T>(win_h * win_w * TC, [&](int i, float*& dst) -> const T* {
+            const int pix = i / TC, cc = i - pix * TC, hh = pl.by_win_w.div(pix), ww = pix - hh * win_w;
+            dst = s_x + i;
+            return cc < left_c && (unsigned)(h0 + hh) < (unsigned)g.h && (unsigned)(w0 + ww) < (unsigned)g.w ? base + cc * g.xs_c + hh * g.xs_h + ww * g.xs_w : nullptr;
+        });
     }
 }
 
@@ -355,13 +384,23 @@ DirectPlan plan_direct(const Geom& g)
     const int tk = v.tkt * v.otk, tc = v.tct * v.otc;
     pl.tiles_k = (g.k + tk - 1) / tk;
     pl.tiles_c = (g.c + tc - 1) / tc;
-    pl.bq = g.q < 32 ? g.q : 32;
+    const bool narrow = g.c <= 4;
+    pl.bq = g.q <= (narrow ? 64 : 32) ? g.q : 32;         // (few channels: whole rows, which are read in runs)
     pl.bp = 1;
     // few input channels: the items are cheap and staged by the threads themselves, so a CTA takes its whole
-    // share as one or two large items (one exposed load latency instead of four)
-    const int max_px = g.c <= 4 ? 512 : 128;
-    while (pl.bp * 2 <= g.p && pl.bp * 2 * pl.bq <= max_px && smem_for(g, v, pl.bp * 2, pl.bq) <= 96 * 1024) pl.bp *= 2;
+    // share as one or two large items (one exposed load latency instead of four), as long as every SM gets one
+    // (1x1 filters: few registers, so that an SM holds six CTAs, and small items keep them all loading)
+    int max_px = narrow && g.r > 1 ? 512 : 128;
+    if (narrow)
+        while (max_px > 64 && (long long)g.n * pl.tiles_k * pl.tiles_c * ((g.p * g.q + max_px - 1) / max_px) < 148) max_px /= 2;
+    if (narrow) {          // bands of equal height
+        const int bands = (g.p * pl.bq + max_px - 1) / max_px;
+        pl.bp = (g.p + bands - 1) / bands;
+        while (pl.bp > 1 && smem_for(g, v, pl.bp, pl.bq) > 96 * 1024) pl.bp = (pl.bp + 1) / 2;
+    }
+    else while (pl.bp * 2 <= g.p && pl.bp * 2 * pl.bq <= max_px && smem_for(g, v, pl.bp * 2, pl.bq) <= 96 * 1024) pl.bp *= 2;
     while (pl.bq > 1 && smem_for(g, v, pl.bp, pl.bq) > 96 * 1024) pl.bq /= 2;
+    pl.by_npx = fast_div(pl.bp * pl.bq); pl.by_bq = fast_div(pl.bq); pl.by_win_w = fast_div((pl.bq - 1) * g.stride_w + g.s);
     pl.bands_p = (g.p + pl.bp - 1) / pl.bp;
     pl.bands_q = (g.q + pl.bq - 1) / pl.bq;
     // vector fast paths: bands of whole rows whose pixel runs start on a 4-element boundary; NHWC with
@@ -371,7 +410,7 @@ DirectPlan plan_direct(const Geom& g)
     pl.items = g.n * pl.bands_p * pl.bands_q;
     const int tiles = pl.tiles_k * pl.tiles_c;
     // one wave of two CTAs per SM (the register budget); each split's partial block is written once and read once
-    int splits = (148 * 2) / tiles;
+    int splits = 148 * (narrow && g.r == 1 ? 6 : 2) / tiles;
     if (splits < 1) splits = 1;
     if (splits > pl.items) splits = pl.items;
     const size_t out_bytes = (size_t)g.k * g.c * g.r * g.s * sizeof(float);

@@ -73,6 +73,20 @@ inline cudaError_t allow_shared_memory(const void* kernel, std::atomic<unsigned 
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// Division of 0 <= n < 2^31 by a number that the host knows: n * mul >> (32 + shift), mul = ceil(2^(31 + l) / d), l = ceil(log2 d)
+struct FastDiv {
+    unsigned d, mul, shift;
+#ifdef __CUDACC__
+    __device__ __forceinline__ int div(int n) const { return d == 1 ? n : (int)(__umulhi((unsigned)n, mul) >> shift); }
+#endif
+};
+inline FastDiv fast_div(unsigned d)
+{
+    unsigned l = 0;
+    while ((1ull << l) < d) ++l;
+    return d <= 1 ? FastDiv{1, 0, 0} : FastDiv{d, (unsigned)(((1ull << (31 + l)) + d - 1) / d), l - 1};
+}
+
 // Geometry with derived sizes and element strides of the chosen layouts.
 struct Geom {
     int n, c, h, w, k, r, s, p, q;
@@ -132,6 +146,7 @@ struct DirectPlan {
     size_t partial_bytes;
     bool tiled;             // false: filter size without a tiled instantiation -> per-element kernel
     bool vec_dy, vec_x;     // 4-element vector loads usable for the dY band / the X window
+    FastDiv by_npx, by_bq, by_win_w;        // by pixels of a band, its columns, columns of the X window
 };
 DirectPlan plan_direct(const Geom& g);
 cudaError_t launch_direct(const void* x, const void* dy, float* dw, float* partial, uint32_t* status,
