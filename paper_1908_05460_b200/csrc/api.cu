@@ -223,9 +223,14 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, const ClPlan& plan, bool reo
             // 47.7 / 66.3).  3x3 64->64 on 32x32 25.0 / 23.1
             return g.r < 5 || g.c < 64 || (g.r == 5 && g.s <= 5 && g.k >= 96);
         }
-        if (L.stem_ok) return reordered || (!shared && g.r * g.s * g.c > 32);       // 5x5 3->64 27.5 / 26.1, 3x3 3->16 11.1 / 16.0
+        // stems (on 32x32): beside others 3->64 3x3 N = 64 7.1 / 4.7, N = 256 16.7 / 13.4, 5x5 N = 16 4.2 / 2.5, but 3->16 N = 256 7.3 / 9.2; alone
+        // 3x3 3->64 N = 64 11.6 / 12.4, N = 128 15.5 / 15.1, N = 256 23.8 / 20.8, 3->16 N = 256 16.0 / 16.5, 5x5 3->64 N = 8 9.4 / 11.8, N = 32 13.7 / 12.3,
+        // N = 128 26.5 / 15.4, 3->16 N = 64 11.0 / 13.2
+        if (L.stem_ok) return reordered || (shared ? g.k > 32 && products > 5e7 : products > (g.r * g.s * g.c > 32 ? 1.2e8 : 2e8));
     } else {
-        if (L.stem_ok) return false;                                // 3->64 on 32x32 29 / 41
+        // stems on 32x32: 3x3 3->64 28.7 / 36.8; 5x5 3->64 44.2 / 37.9, N = 32 18.0 / 17.5, but 3->32 26.4 / 28.4 (beside the second layer of the
+        // two-layer CNN, N = 200, the step takes 63 / 68)
+        if (L.stem_ok) return !shared && g.r * g.s * g.c > 32 && g.k > 32 && products > 1.2e8;
         // (the tensor core truncates as it adds, 1e-8 for each MMA of the other kernel's CTA: where that has more than 1,500 of them
         // its results are over 1.4e-5 away from this one's, and stay what they have been)
         if (L.tc_ok && L.tp.chain > 1500) return false;

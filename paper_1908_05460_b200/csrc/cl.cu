@@ -33,6 +33,7 @@
 //           way; bf16 5x5 72->200 on 15x15, N = 60 39 -> 29, fp32 216 -> 124, fp32 7x7 160->120 on 21x21, N = 20 466 -> 111).
 //   c-side  (few output channels) M = 128 = shifts x channels of X, N = output channels; M = 64 MMAs would take as
 //           long as M = 128 ones, so with K <= 64 this form is the faster one although one shift in four is unused.
+//           Filters of one column have filter rows in place of the shifts (row_atoms): the X operand's atoms lie one map row apart.
 //   stack   (at most 64 output channels, stride 1) M = 128 = filter rows x output channels: the reduction walks over rows of X, and
 //           the channel atoms of the dY operand lie one map row apart, so that atom j is the gradient row that meets this X row
 //           in filter row r_hi - j.  One MMA does the work of two to eight whose M would be mostly idle.
@@ -98,6 +99,8 @@ struct ClGroup {            // one MMA of a k-step
 struct ClParams {
     int n, c, h, w, k, r, s, p, q, stride, pad_h, pad_w;
     long long ws_k, ws_c, ws_r, ws_s;
+    int vc, vw, vpad;               // few channels (vc, else 0): the problem is one of s = 1, whose c channels are the vc channels of every column
+                                    // of a window in turn; columns of X and padding as the caller has them
     float alpha;
     int tiles_k, tiles_c, tiles_r, splits, chunk_base, chunk_rem, chunks;
     int ci, bp, cpi;                // chunk = ci whole images, or bp output rows of one; chunks per image
@@ -115,6 +118,7 @@ struct ClParams {
     int skip;                       // kImages, whole maps, one filter row a tile: k-steps per map row, to leave out rows opposite the padding
     int c_side;                     // 1: X is the M side
     int slack;                      // bytes behind the last stage that MMAs may read
+    int row_atoms;                  // c-side, one column: the atoms of the X operand are filter rows, one map row apart
     int stack;                      // 1: filter rows x output channels are the M side; chunks are bands of X rows
     int s_inner;                    // 1: column shifts lie next to one another in dW (K x C x R x S): columns are written shift by shift
     int merged;                     // 1: the MN atoms of an X operand are channel atoms, 0: column shifts
@@ -151,6 +155,15 @@ __device__ __forceinline__ int written_column(const ClParams& P, int e)
 // Element (column, lane) of a block that goes to dW directly, in words: [column][128], the lanes of a column exchanged by a key, so that neither a column's
 // lanes, nor a lane's columns, nor the shifts of a channel meet in one bank.
 __device__ __forceinline__ int block_key(int col, int ca_log) { return (col + 11 * (col >> ca_log)) & 31; }
+// offset of a channel in dW
+__device__ __forceinline__ long long channel_offset(const ClParams& P, int c)
+{
+    if (P.vc == 0) return c * P.ws_c;
+    const int s = c / P.vc;
+    return (c - s * P.vc) * P.ws_c + s * P.ws_s;
+}
+// c-side: distance in dW from one atom of the M side to the next
+__device__ __forceinline__ long long atom_step(const ClParams& P) { return P.row_atoms ? P.ws_r : P.stride * P.ws_s; }
 // Column -> {offset in dW, atoms in use (0: not an element)}
 // (stack: without the filter row, which belongs to the lane)
 __device__ __forceinline__ int2 column_target(const ClParams& P, int col, int k0, int c0, int r0)
@@ -160,7 +173,7 @@ __device__ __forceinline__ int2 column_target(const ClParams& P, int col, int k0
     const int a = P.c_side || P.merged ? 0 : j / P.ca, k = P.c_side ? k0 + j : 0;
     const int c = c0 + g.cbase + (P.c_side ? 0 : P.merged ? j : j - a * P.ca);
     const bool valid = r0 + g.r < P.r && (P.c_side ? k < P.k : c < P.c && a < g.cnt);
-    return make_int2((int)(k * P.ws_k + c * P.ws_c + (P.stack ? 0 : r0 + g.r) * P.ws_r + (g.s0 + P.stride * a) * P.ws_s), valid ? g.cnt : 0);
+    return make_int2((int)(k * P.ws_k + channel_offset(P, c) + (P.stack ? 0 : r0 + g.r) * P.ws_r + (g.s0 + P.stride * a) * P.ws_s), valid ? g.cnt : 0);
 }
 
 // k-side: lane -> offset in dW, -1: not an element
@@ -187,9 +200,9 @@ __device__ __forceinline__ ClElement cl_element(const ClParams& P, int tile, int
     const int j = col - g.col, ca_log = 31 - __clz(P.ca), ka_log = 31 - __clz(P.ka);
     const int mn = P.c_side ? l : j, a = P.merged ? 0 : mn >> ca_log;
     ClElement e;
-    e.c = c0 + g.cbase + (P.merged ? mn : mn & (P.ca - 1)); e.s = g.s0 + P.stride * a;
+    e.c = c0 + g.cbase + (P.merged ? mn : mn & (P.ca - 1)); e.s = P.row_atoms ? 0 : g.s0 + P.stride * a;
     e.k = P.c_side ? k0 + j : P.stack ? l & (P.ka - 1) : k0 + l;
-    e.r = r0 + (P.stack ? P.rc - 1 - (l >> ka_log) : g.r);
+    e.r = r0 + (P.stack ? P.rc - 1 - (l >> ka_log) : P.row_atoms ? a : g.r);
     e.valid = e.k < P.k && e.c < P.c && a < g.cnt && e.r >= r0 && e.r < P.r;
     return e;
 }
@@ -205,21 +218,22 @@ __device__ __noinline__ void cl_repair(const ClParams& P, const ClSource& S, flo
         left &= left - 1;
         const int k = __shfl_sync(0xffffffffu, mine.k, owner), c = __shfl_sync(0xffffffffu, mine.c, owner);
         const int r = __shfl_sync(0xffffffffu, mine.r, owner), s = __shfl_sync(0xffffffffu, mine.s, owner);
+        const int vs = P.vc != 0 ? c / P.vc : 0, cx = c - vs * P.vc, chans = P.vc != 0 ? P.vc : P.c, cols = P.vc != 0 ? P.vw : P.w;
         double sum = 0;
         for (int base = 0; base < all; base += 32) {
             const int i = base + lane;
             if (i < all) {
                 const int n = i / px, p = (i - n * px) / P.q, q = i - n * px - p * P.q;
-                const int h = p * P.stride + r - P.pad_h, w = q * P.stride + s - P.pad_w;
-                const bool in = h >= 0 && h < P.h && w >= 0 && w < P.w;
-                const size_t xi = S.x_last ? (((size_t)n * P.h + h) * P.w + w) * P.c + c : (((size_t)n * P.c + c) * P.h + h) * P.w + w;
+                const int h = p * P.stride + r - P.pad_h, w = q * P.stride + s + vs - (P.vc != 0 ? P.vpad : P.pad_w);
+                const bool in = h >= 0 && h < P.h && w >= 0 && w < cols;
+                const size_t xi = S.x_last ? (((size_t)n * P.h + h) * cols + w) * chans + cx : (((size_t)n * chans + cx) * P.h + h) * cols + w;
                 const size_t yi = S.dy_last ? (size_t)i * P.k + k : ((size_t)n * P.k + k) * px + (i - n * px);
                 sum += (in ? cl_load(S.x, xi, S.f32) : 0.0) * cl_load(S.dy, yi, S.f32);
             }
             if (__any_sync(0xffffffffu, isnan(sum))) break;
         }
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        if (lane == 0) dw[k * P.ws_k + c * P.ws_c + r * P.ws_r + s * P.ws_s] = P.alpha * (float)sum;
+        if (lane == 0) dw[k * P.ws_k + channel_offset(P, c) + r * P.ws_r + s * P.ws_s] = P.alpha * (float)sum;
     }
 }
 
@@ -524,8 +538,8 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
             int l = threadIdx.x & 127;
             if (P.s_inner) l = ((l & ((1 << (7 - ca_log)) - 1)) << ca_log) + (l >> (7 - ca_log));
             const int a = P.merged ? 0 : l >> ca_log, cc = P.merged ? l : l & (P.ca - 1);          // this lane's atom and channel
-            float* d = dw + P.stride * a * P.ws_s + cc * P.ws_c;
-            if (c0 + cc < P.c) {
+            float* d = dw + a * atom_step(P) + channel_offset(P, cc);
+            if (c0 + cc < P.c && (!P.row_atoms || r0 + a < P.r)) {
 #pragma unroll 4
                 for (int col = third; col < cols; col += 3) {
                     const int2 o = s_col[col];
@@ -582,7 +596,7 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
         for (int e = warp; e < 4 * P.cols; e += kThreads / 32) {
             const int col = e >> 2, l = 32 * (e & 3) + lane;
             const ClElement el = cl_element(P, tile, col, l);
-            const uint32_t left = __ballot_sync(0xffffffffu, el.valid && !isfinite(__ldcg(dw + (el.k * P.ws_k + el.c * P.ws_c + el.r * P.ws_r + el.s * P.ws_s))));
+            const uint32_t left = __ballot_sync(0xffffffffu, el.valid && !isfinite(__ldcg(dw + (el.k * P.ws_k + channel_offset(P, el.c) + el.r * P.ws_r + el.s * P.ws_s))));
             if (left != 0) cl_repair(P, S, dw, tile, col, l, left);
         }
     GACONV_STAMP(5, threadIdx.x == 0);
@@ -605,7 +619,7 @@ __device__ __noinline__ void cl_repair_written(const ClParams& P, const ClSource
         const bool in = col0 + lc.y < P.cols;
         const int col = written_column(P, in ? col0 + lc.y : 0);
         const ClElement el = cl_element(P, tile, col, lc.x);
-        const float* out = dw + (el.k * P.ws_k + el.c * P.ws_c + el.r * P.ws_r + el.s * P.ws_s);
+        const float* out = dw + (el.k * P.ws_k + channel_offset(P, el.c) + el.r * P.ws_r + el.s * P.ws_s);
         const uint32_t left = __ballot_sync(0xffffffffu, in && el.valid && !isfinite(__ldcg(out)));
         if (left != 0) cl_repair(P, S, dw, tile, col, lc.x, left);
     }
@@ -663,8 +677,8 @@ cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, cons
         bool valid; long long off = o.x;
         if (P.c_side) {
             const int a = P.merged ? 0 : l >> ca_shift, ch = l & mn_mask;
-            valid = a < o.y && c0 + ch < P.c;
-            off += ch * P.ws_c + P.stride * a * P.ws_s;
+            valid = a < o.y && c0 + ch < P.c && (!P.row_atoms || r0 + a < P.r);
+            off += channel_offset(P, ch) + a * atom_step(P);
         } else {
             const int lane_off = lane_target(P, l, k0, r0);
             valid = o.y > 0 && lane_off >= 0;
@@ -686,6 +700,7 @@ struct PackOp {
     int ch, chp, px, n;         // source: n images of px pixels and ch channels; destination rows of chp channels,
     int pitch;                  // this many apart
     int channels_last;          // source order: 1 [n][px][ch], 0 [n][ch][px]
+    int vc, vw, vpad, q, h;     // ClParams::vc and so on: the destination's channels are gathered from windows of the source; its rows and columns
     int px_tiles, ch_tiles;     // tiles of an image (channels-first sources): tile_px pixels x
     int ch_tile;                // at most 64 channels, a multiple of 8
     int tile_px;                // pixels of a tile
@@ -750,6 +765,40 @@ pack_kernel(const PackOp x, const PackOp dy)
     const PackOp& o = is_x ? x : dy;
     const int blk = is_x ? blockIdx.x : blockIdx.x - x.blocks;
     const E* src = static_cast<const E*>(o.src);
+    if (o.vc) {
+        // A pixel of the destination: the channels of the columns of a window, neighbours in a channels-last row
+        const int g8 = o.chp >> 3, row_el = o.vw * o.vc;
+        const unsigned items = (unsigned)o.n * o.px * g8;
+        pdl_wait_prior_grid();
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const unsigned it = blk * 512u + i * 256 + threadIdx.x;
+            if (it >= items) return;
+            const unsigned row = it / (unsigned)g8, nh = row / (unsigned)o.q;
+            const int j0 = (int)(it - row * g8) * 8, q = (int)(row - nh * o.q);
+            alignas(16) E v[8];
+            if (o.channels_last) {
+                const int f0 = (q - o.vpad) * o.vc + j0;
+                const E* p = src + (size_t)nh * row_el;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = j0 + u < o.ch && f0 + u >= 0 && f0 + u < row_el ? __ldg(p + f0 + u) : E(0);
+            } else {
+                const unsigned n = nh / (unsigned)o.h;
+                const size_t plane = (size_t)o.h * o.vw;
+                int s = j0 / o.vc, c = j0 - s * o.vc;
+                const E* p = src + ((size_t)n * o.vc * o.h + (nh - n * o.h)) * o.vw + c * plane;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int w = q + s - o.vpad;
+                    v[u] = j0 + u < o.ch && w >= 0 && w < o.vw ? __ldg(p + w) : E(0);
+                    p += plane;
+                    if (++c == o.vc) { c = 0; ++s; p -= o.vc * plane; }
+                }
+            }
+            store8(v, o.dst + (size_t)row * o.pitch + j0, o.plane);
+        }
+        return;
+    }
     if (o.channels_last) {
         const int g8 = o.chp >> 3;
         const unsigned items = (unsigned)o.n * o.px * g8;            // (an operand has at most 2^31 elements)
@@ -953,7 +1002,7 @@ int far_shift(const ClParams& P)
 bool build_groups(ClParams& P)
 {
     P.ngroups = 0;
-    const int rows = P.stack ? 1 : P.rc, st = P.stride, wt = P.x_pitch;
+    const int rows = P.stack || P.row_atoms ? 1 : P.rc, st = P.stride, wt = P.x_pitch;
     // atoms of one MMA on the X side: c-side exactly fills M = 128; k-side as many as N = 256 takes, the shifts of a column phase
     // shared out evenly over as few MMAs as hold them
     const int atoms = P.merged ? P.na : shifts_of(P);
@@ -975,7 +1024,7 @@ bool build_groups(ClParams& P)
             } else {
                 for (int a = 0; a < P.na; ++a)
                     for (int i = 0; i < shifts; i += atoms)
-                        if (!add(base_tile + a, base_px + i, rl, ph + st * i, std::min(atoms, shifts - i), a * P.ca)) return false;
+                        if (!add(base_tile + a, base_px + i, rl, ph + st * i, P.row_atoms ? P.rc : std::min(atoms, shifts - i), a * P.ca)) return false;
             }
         }
     P.s_inner = !P.merged && P.s > 1 && P.ws_s < P.ws_c;
@@ -1023,7 +1072,7 @@ bool shape_chunk(ClParams& P, int ci, int bp, int order, bool bare = false)
     const int last = order == kFlat ? P.ksteps * 16 - 1 : ((images ? 1 : ci) - 1) * P.x_img + (bp - 1) * wp + P.q - 1 + (order == kPixels ? wp - P.q + 8 : 0) + (images && ci % 16 != 0 ? 1 : 0);
     const int zeros = P.stack && images && ci == 8 && bp * P.q % 2 != 0 ? P.x_img + 1 + far_shift(P) : 0;      // pixels, see below
     P.x_pre = bare ? round_up(std::max(P.pad_w, 1) * ci * xb, 1024) : 0;
-    const int far = last + halo * wp + (images ? far_shift(P) : ceil_div(P.s, st) - 1 + (P.c_side ? 128 / P.ca : 256 / P.ca));
+    const int far = P.row_atoms ? last + (128 / P.ca - 1) * wp : last + halo * wp + (images ? far_shift(P) : ceil_div(P.s, st) - 1 + (P.c_side ? 128 / P.ca : 256 / P.ca));
     P.x_alloc = P.x_pre + round_up(bare ? P.x_box : std::max(P.x_box, std::max(far + 1, zeros) * P.px_rows * xb), 1024);
     const int x_tiles = P.na * P.phases * P.row_tiles;
     P.x_plane = x_tiles * P.x_alloc;
@@ -1042,7 +1091,7 @@ bool shape_chunk(ClParams& P, int ci, int bp, int order, bool bare = false)
     const uint32_t x_swz = P.ca == 64 ? 2 : P.ca == 32 ? 4 : 6, dy_swz = order == kPixels || P.ka == 64 ? 2 : P.ka == 32 ? 4 : 6;
     const uint32_t dy_sbo = order == kPixels ? 8 * 128 : order == kPaired ? dy_w * db : 8 * db;
     P.dy_hi = (dy_sbo >> 4) | (1u << 14) | (dy_swz << 29);
-    P.x_lbo = (uint32_t)((P.merged ? P.x_alloc : P.px_rows * xb) >> 4) << 16;
+    P.x_lbo = (uint32_t)((P.merged ? P.x_alloc : (P.row_atoms ? wp : 1) * P.px_rows * xb) >> 4) << 16;
     // (one atom: the upper half of M repeats the lower)
     P.dy_lbo = P.stack ? (uint32_t)(dy_w * P.px_rows * db >> 4) << 16 : order == kPixels ? 1u << 16 : (uint32_t)((P.katoms > 1 ? P.dy_alloc : 0) >> 4) << 16;
     for (int i = 0; i < P.ksteps; ++i) {
@@ -1141,14 +1190,15 @@ ClKernel kernel_for(int ng, bool f32, bool c_side)
 
 }  // namespace
 
-bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
+namespace {
+bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, ClPlan* out)
 {
     if (g.stride_h != g.stride_w || g.stride_h > kMaxMapStep || g.r > 16 || g.s > 16 || !dw_offsets_fit(g)) return false;
-    const bool nhwc = g.xs_c == 1 || g.c == 1;
+    const bool nhwc = g.xs_c == 1 || (vc != 0 ? vc : g.c) == 1;
     ClHost H{};
     H.f32 = !g.bf16;
     H.x_nhwc = nhwc; H.dy_npqk = dy_npqk || g.k == 1;
-    H.pack_x = H.f32 || !nhwc || g.c % 8 != 0;
+    H.pack_x = H.f32 || !nhwc || g.c % 8 != 0 || vc != 0;
     H.pack_dy = H.f32 || !H.dy_npqk || g.k % 8 != 0;
     const size_t x_px = (size_t)g.n * g.h * g.w, dy_px = (size_t)g.n * g.p * g.q, x_el = x_px * round_up(g.c, 8), dy_el = dy_px * round_up(g.k, 8);
     if (x_el > ((size_t)1 << 31) || dy_el > ((size_t)1 << 31)) return false;
@@ -1157,6 +1207,7 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
     B.n = g.n; B.c = g.c; B.h = g.h; B.w = g.w; B.k = g.k; B.r = g.r; B.s = g.s; B.p = g.p; B.q = g.q;
     B.stride = g.stride_h; B.pad_h = g.pad_h; B.pad_w = g.pad_w; B.alpha = g.alpha;
     B.ws_k = g.ws_k; B.ws_c = g.ws_c; B.ws_r = g.ws_r; B.ws_s = g.ws_s;
+    B.vc = vc; B.vw = vw; B.vpad = vpad;
     B.planes = H.f32 ? 3 : 1; B.nprod = H.f32 ? 6 : 1;
     B.phases = std::min(g.stride_h, g.s);
     B.ca = g.c > 32 ? 64 : g.c > 16 ? 32 : 16;
@@ -1164,14 +1215,15 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
 
     ClParams best{};
     double best_cycles = 1e30;
-    for (int form = 0; form < 3; ++form) {           // k-side, c-side, stack
-        if (form == 2 && (g.k > 64 || g.r == 1 || g.stride_h != 1)) break;
+    for (int form = 0; form < 4; ++form) {           // k-side, c-side, stack, c-side with filter rows
+        if (form == 3 && (g.s != 1 || g.r == 1 || g.stride_h != 1 || B.ca > 32)) break;
+        if (form == 2 && (g.k > 64 || g.r == 1 || g.stride_h != 1)) continue;
         const int k16 = round_up(g.k, 16), all_rows = form == 2 ? g.h : g.p;
         const int kts[4] = {form == 2 ? (g.k > 32 ? 64 : k16) : form ? std::min(k16, 256) : 128, 128, 64, 32};
-        for (int ki = 0; ki < (form == 1 ? 4 : 1); ++ki) {
+        for (int ki = 0; ki < (form & 1 ? 4 : 1); ++ki) {
             if (ki > 0 && (kts[ki] >= kts[0] || kts[ki] >= k16)) continue;
             ClParams F = B;
-            F.c_side = form == 1; F.stack = form == 2; F.kt = kts[ki];
+            F.c_side = form & 1; F.row_atoms = form == 3; F.stack = form == 2; F.kt = kts[ki];
             const int kw = std::min(F.kt, k16);
             F.ka = kw > 32 ? 64 : kw > 16 ? 32 : 16;
             F.katoms = ceil_div(kw, F.ka);
@@ -1182,11 +1234,12 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
                 F.ca = ca;
                 if (na > 1 && (F.ca < 64 || (na - 1) * 64 >= g.c)) break;
                 if (form == 1 && na > 2) break;
+                if (form == 3 && na > 1) break;
                 if (form != 1 && na > 2 && g.s > 1) break;
                 F.na = na; F.ct = na * F.ca;
                 F.merged = na > 1 && (form == 1 || g.s == 1) ? 1 : 0;
                 F.tiles_c = ceil_div(g.c, F.ct);
-                for (int rc = form == 2 ? 2 : 1; rc <= (form == 2 ? std::min(g.r, 128 / F.ka) : g.r); ++rc) {
+                for (int rc = form >= 2 ? 2 : 1; rc <= (form == 2 ? std::min(g.r, 128 / F.ka) : form == 3 ? std::min(g.r, 128 / F.ca) : g.r); ++rc) {
                     F.rc = rc; F.tiles_r = ceil_div(g.r, rc);
                     if (rc > 1 && ceil_div(g.r, rc) == ceil_div(g.r, rc - 1)) continue;
                     F.row_tiles = F.stride > 1 ? rc : 1;
@@ -1284,6 +1337,28 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
     memcpy(out->opaque, &H, sizeof(H));
     return true;
 }
+}  // namespace
+
+// Few input channels (image stems) leave most of an atom of 16 idle.  With stride 1 the columns of a window can stand in for channels: the
+// packing pass, which such inputs need anyway, gathers s x c of them for every output column, and the filter becomes one of s = 1, whose
+// rows are the atoms of one c-side MMA a k-step.  (Bound by operand reads before, with one MMA a filter row; us, plain / gathered: bf16 on
+// 32x32 5x5 3->64, N = 128 25.1 / 15.4, 3x3 N = 256 23.9 / 20.8, 7x7 3->64 on 40x40, N = 50 19.2 / 15.2, fp32 5x5 3->64, N = 128 54.7 / 37.5,
+// 3x3 3->40 on 30x30, N = 40 29.3 / 19.2.)  The gathered operand is longer, and so is its pass: a tenth of the whole has to be gained by the estimate
+// (less lost: bf16 5x5 3->48 on 17x17, N = 30 12.2 / 13.1, estimated 15,300 / 14,300 cycles).
+bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
+{
+    const bool plain = plan_problem(g, dy_npqk, 0, 0, 0, out);
+    if (g.c > 4 || g.s < 2 || g.s * g.c > 32 || g.stride_h != 1 || g.stride_w != 1) return plain;
+#ifdef GACONV_TUNING
+    if (const char* e = getenv("GACONV_CL_VC")) if (atoi(e) == 0) return plain;
+#endif
+    Geom v = g;
+    v.c = g.s * g.c; v.s = 1; v.w = g.q; v.pad_w = 0;
+    ClPlan gathered;
+    if (!plan_problem(v, dy_npqk, g.c, g.w, g.pad_w, &gathered) || (plain && 10 * gathered.cycles >= 9 * out->cycles)) return plain;
+    *out = gathered;
+    return true;
+}
 
 cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, void* x_scratch, void* dy_scratch, uint32_t* status,
                       const ClPlan& plan, bool wide, cudaStream_t stream)
@@ -1298,6 +1373,10 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
         PackOp ox{}, od{};
         const int tile_px = H.f32 ? kPackPx<float> : kPackPx<unsigned short>;
         if (H.pack_x) ox = pack_op(x, x_scratch, P.c, xch, P.h * P.w, P.n, H.x_nhwc, tile_px);
+        if (P.vc != 0) {
+            ox.vc = P.vc; ox.vw = P.vw; ox.vpad = P.vpad; ox.q = P.w; ox.h = P.h;
+            ox.blocks = (int)(((size_t)P.n * P.h * P.w * (ox.chp / 8) + 511) / 512);
+        }
         if (H.pack_dy) od = pack_op(dy, dy_scratch, P.k, dych, P.p * P.q, P.n, H.dy_npqk, tile_px);
         const dim3 grid((unsigned)(ox.blocks + od.blocks));
         err = H.f32 ? launch_kernel(pack_kernel<float>, grid, dim3(256), 0, stream, dim3(1, 1, 1), ox, od)

@@ -39,6 +39,11 @@ SHAPES = [
     ConvLayer("stride 3, 7x7: three shifts, two and two", 12, 30, 30, 25, 100, 7, 7, 3, 3),
     ConvLayer("5x5, tiles of 32 of 72 channels", 5, 72, 15, 15, 136, 5, 5, 1, 2),
     ConvLayer("7x7, tiles of 16 of 70 channels", 6, 70, 13, 10, 131, 7, 7, 1, 3),
+    ConvLayer("3 channels, 5x5: windows for channels", 8, 3, 33, 40, 70, 5, 5, 1, 2),
+    ConvLayer("4 channels, 3x7, padding on one side", 13, 4, 21, 19, 100, 3, 7, 1, 2),
+    ConvLayer("2 channels, 9 rows in two tiles", 22, 2, 30, 17, 130, 9, 3, 1, 1),
+    ConvLayer("2 channels, 7x7, odd rows", 30, 2, 34, 31, 48, 7, 7, 1, 3),
+    ConvLayer("3x1 filter, 20 channels", 30, 20, 26, 16, 60, 3, 1, 1, 0),
 ]
 LAYOUTS = {"paper": {}, "nchw": dict(x_layout=B.X_NCHW, dw_layout=B.DW_KCRS),
            "nhwc": dict(dy_layout=B.DY_NPQK, dw_layout=B.DW_KCRS), "rsck": dict(x_layout=B.X_NCHW, dy_layout=B.DY_NPQK, dw_layout=B.DW_RSCK)}
@@ -283,6 +288,11 @@ def test_threads_with_layers_of_one_kernel_and_different_shared_memory():
     (ConvLayer("5x5, 64 channels, 96 outputs", 16, 64, 16, 16, 96, 5, 5, 1, 2), 0, "cl_kernel"),
     (ConvLayer("7x7, 64 channels, 128 outputs", 16, 64, 16, 16, 128, 7, 7, 1, 3), 0, "exact_tc_kernel"),
     (ConvLayer("7x7, 24 channels on 32x32", 9, 24, 32, 32, 16, 7, 7, 1, 3), 0, "cl_kernel"),
+    (ConvLayer("stem of 64 outputs, 256 images", 256, 3, 32, 32, 64, 3, 3, 1, 1), 0, "cl_kernel"),
+    (ConvLayer("stem of 64 outputs, 64 images", 64, 3, 32, 32, 64, 3, 3, 1, 1), 0, "stem_mma_kernel"),
+    (ConvLayer("stem of 64 outputs, 64 images, few SMs", 64, 3, 32, 32, 64, 3, 3, 1, 1), 37, "cl_kernel"),
+    (ConvLayer("stem of 16 outputs, few SMs", 128, 3, 32, 32, 16, 3, 3, 1, 1), 18, "stem_mma_kernel"),
+    (ConvLayer("5x5 stem, 64 images", 64, 3, 32, 32, 64, 5, 5, 1, 2), 0, "cl_kernel"),
     (ConvLayer("a large dW with short sums", 64, 256, 8, 8, 256, 3, 3, 1, 1), 0, "exact_tc_kernel"),
     (ConvLayer("a large dW past the line", 96, 256, 8, 8, 256, 3, 3, 1, 1), 0, "cl_kernel"),
     (ConvLayer("64 channels on few SMs", 32, 64, 8, 8, 64, 3, 3, 1, 1), 18, "exact_tc_kernel"),
