@@ -752,7 +752,8 @@ __device__ __forceinline__ void store8(const E (&v)[8], __nv_bfloat16* dst, size
     }
 }
 
-template <typename E>
+// WINDOWS: X is gathered from windows (PackOp::vc); apart, so that the other calls carry nothing for it.
+template <typename E, bool WINDOWS>
 __global__ void __launch_bounds__(256)
 pack_kernel(const PackOp x, const PackOp dy)
 {
@@ -765,7 +766,7 @@ pack_kernel(const PackOp x, const PackOp dy)
     const PackOp& o = is_x ? x : dy;
     const int blk = is_x ? blockIdx.x : blockIdx.x - x.blocks;
     const E* src = static_cast<const E*>(o.src);
-    if (o.vc) {
+    if (WINDOWS && is_x) {
         // A pixel of the destination: the channels of the columns of a window, neighbours in a channels-last row
         const int g8 = o.chp >> 3, row_el = o.vw * o.vc;
         const unsigned items = (unsigned)o.n * o.px * g8;
@@ -1228,8 +1229,9 @@ bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, ClPlan*
             F.ka = kw > 32 ? 64 : kw > 16 ? 32 : 16;
             F.katoms = ceil_div(kw, F.ka);
             F.tiles_k = ceil_div(g.k, F.kt);
-            // (M side output channels, wide filters: fewer channels a tile, so that all shifts fit the accumulators)
-            for (int ca = B.ca; ca >= ((form == 2 && g.s > 3) || (form == 0 && g.s * B.ca > kMaxCols) ? 16 : B.ca); ca /= 2)
+            // (M side output channels, wide filters: fewer channels a tile, so that all shifts fit the accumulators; up to 64 outputs stack:
+            // 5x5 86->37 on 10x13, N = 67 19.8 us, 21.0 without)
+            for (int ca = B.ca; ca >= ((form == 2 && g.s > 3) || (form == 0 && g.s * B.ca > kMaxCols && (g.k > 64 || g.stride_h > 1)) ? 16 : B.ca); ca /= 2)
             for (int na = 1; na <= 4; na *= 2) {
                 F.ca = ca;
                 if (na > 1 && (F.ca < 64 || (na - 1) * 64 >= g.c)) break;
@@ -1379,8 +1381,8 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
         }
         if (H.pack_dy) od = pack_op(dy, dy_scratch, P.k, dych, P.p * P.q, P.n, H.dy_npqk, tile_px);
         const dim3 grid((unsigned)(ox.blocks + od.blocks));
-        err = H.f32 ? launch_kernel(pack_kernel<float>, grid, dim3(256), 0, stream, dim3(1, 1, 1), ox, od)
-                    : launch_kernel(pack_kernel<unsigned short>, grid, dim3(256), 0, stream, dim3(1, 1, 1), ox, od);
+        auto kern = H.f32 ? (P.vc ? pack_kernel<float, true> : pack_kernel<float, false>) : (P.vc ? pack_kernel<unsigned short, true> : pack_kernel<unsigned short, false>);
+        err = launch_kernel(kern, grid, dim3(256), 0, stream, dim3(1, 1, 1), ox, od);
         if (err != cudaSuccess) return err;
         note_launch();
         if (H.pack_x) x = x_scratch;
