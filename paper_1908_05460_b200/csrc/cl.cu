@@ -96,7 +96,7 @@ struct ClGroup {            // one MMA of a k-step
     uint32_t idesc;         // n in the instruction descriptor's place
 };
 
-struct ClParams {
+struct ClShape {
     int n, c, h, w, k, r, s, p, q, stride, pad_h, pad_w;
     long long ws_k, ws_c, ws_r, ws_s;
     int vc, vw, vpad;               // few channels (vc, else 0): the problem is one of s = 1, whose c channels are the vc channels of every column
@@ -127,6 +127,8 @@ struct ClParams {
     int epoch;                      // chunks of one issuer between two readings of its accumulators
     uint32_t dy_hi, x_lbo, dy_lbo, idesc;
     ClGroup g[kMaxGroups];
+};
+struct ClParams : ClShape {
     // k-step -> offsets of its X and dY rows (16-byte units), upper word of its X descriptor, and, with one k-side MMA a k-step,
     // the first column of that MMA | its N in the instruction descriptor's place (0 << 17 in idesc)
     uint4 k_off[kMaxKsteps];
@@ -137,7 +139,7 @@ __device__ constexpr uint32_t prod_x(int i) { return i == 1 ? 2u : (i == 2 || i 
 __device__ constexpr uint32_t prod_dy(int i) { return i == 0 ? 2u : (i == 2 || i == 3) ? 1u : 0u; }
 
 // The MMA that writes a column
-__device__ __forceinline__ int group_of(const ClParams& P, int col)
+__device__ __forceinline__ int group_of(const ClShape& P, int col)
 {
     int g = 0;
     while (g + 1 < P.ngroups && col >= P.g[g + 1].col) ++g;
@@ -145,7 +147,7 @@ __device__ __forceinline__ int group_of(const ClParams& P, int col)
 }
 // The e-th column of a k-side block in the order of dW: where the shifts of a channel are neighbours in memory, shift by shift,
 // so that a store of 32 lanes touches 13 sectors instead of 32 (K x C x R x S, 512->512 on 2x2 maps: the stores were 12 of 24 us).
-__device__ __forceinline__ int written_column(const ClParams& P, int e)
+__device__ __forceinline__ int written_column(const ClShape& P, int e)
 {
     if (P.c_side || !P.s_inner) return e;
     const ClGroup& g = P.g[group_of(P, e)];
@@ -156,17 +158,17 @@ __device__ __forceinline__ int written_column(const ClParams& P, int e)
 // lanes, nor a lane's columns, nor the shifts of a channel meet in one bank.
 __device__ __forceinline__ int block_key(int col, int ca_log) { return (col + 11 * (col >> ca_log)) & 31; }
 // offset of a channel in dW
-__device__ __forceinline__ long long channel_offset(const ClParams& P, int c)
+__device__ __forceinline__ long long channel_offset(const ClShape& P, int c)
 {
     if (P.vc == 0) return c * P.ws_c;
     const int s = c / P.vc;
     return (c - s * P.vc) * P.ws_c + s * P.ws_s;
 }
 // c-side: distance in dW from one atom of the M side to the next
-__device__ __forceinline__ long long atom_step(const ClParams& P) { return P.row_atoms ? P.ws_r : P.stride * P.ws_s; }
+__device__ __forceinline__ long long atom_step(const ClShape& P) { return P.row_atoms ? P.ws_r : P.stride * P.ws_s; }
 // Column -> {offset in dW, atoms in use (0: not an element)}
 // (stack: without the filter row, which belongs to the lane)
-__device__ __forceinline__ int2 column_target(const ClParams& P, int col, int k0, int c0, int r0)
+__device__ __forceinline__ int2 column_target(const ClShape& P, int col, int k0, int c0, int r0)
 {
     const ClGroup& g = P.g[group_of(P, col)];
     const int j = col - g.col;
@@ -177,7 +179,7 @@ __device__ __forceinline__ int2 column_target(const ClParams& P, int col, int k0
 }
 
 // k-side: lane -> offset in dW, -1: not an element
-__device__ __forceinline__ int lane_target(const ClParams& P, int l, int k0, int r0)
+__device__ __forceinline__ int lane_target(const ClShape& P, int l, int k0, int r0)
 {
     if (!P.stack) return k0 + l < P.k ? (int)((k0 + l) * P.ws_k) : -1;
     const int j = l >> (31 - __clz(P.ka)), k = l & (P.ka - 1), r = r0 + P.rc - 1 - j;
@@ -193,7 +195,7 @@ __device__ __forceinline__ double cl_load(const void* p, size_t i, int f32)
 }
 // Element (column, lane) of a tile
 struct ClElement { int k, c, r, s; bool valid; };
-__device__ __forceinline__ ClElement cl_element(const ClParams& P, int tile, int col, int l)
+__device__ __forceinline__ ClElement cl_element(const ClShape& P, int tile, int col, int l)
 {
     const int tr = tile / P.tiles_r, r0 = (tile - tr * P.tiles_r) * P.rc, tk = tr / P.tiles_c, k0 = tk * P.kt, c0 = (tr - tk * P.tiles_c) * P.ct;
     const ClGroup& g = P.g[group_of(P, col)];
@@ -209,7 +211,7 @@ __device__ __forceinline__ ClElement cl_element(const ClParams& P, int tile, int
 // A warp sums the elements of the lanes in `left` anew, one by one, its lanes the output pixels in turn.  The padding counts as
 // zeros that are multiplied.  In double, so that finite sums do not depend on the order; a NaN ends the sum.
 // Never called on finite data, so that its speed is no matter.
-__device__ __noinline__ void cl_repair(const ClParams& P, const ClSource& S, float* dw, int tile, int col, int l, uint32_t left)
+__device__ __noinline__ void cl_repair(const ClShape& P, const ClSource& S, float* dw, int tile, int col, int l, uint32_t left)
 {
     const int lane = threadIdx.x & 31, px = P.p * P.q, all = P.n * px;
     const ClElement mine = cl_element(P, tile, col, l);
@@ -603,7 +605,7 @@ cl_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CU
 }
 
 // lane of the e-th element that a block of cl_reduce_kernel writes, and its column relative to the block's first
-__device__ __forceinline__ int2 reduced_element(const ClParams& P, int e, int log_cb)
+__device__ __forceinline__ int2 reduced_element(const ClShape& P, int e, int log_cb)
 {
     int l = P.c_side ? e & 127 : e >> log_cb;
     if (P.c_side && P.s_inner) { const int t_shift = 7 - (31 - __clz(P.ca)); l = ((l & ((1 << t_shift) - 1)) << (7 - t_shift)) + (l >> t_shift); }
@@ -611,7 +613,7 @@ __device__ __forceinline__ int2 reduced_element(const ClParams& P, int e, int lo
 }
 // Every warp of cl_reduce_kernel repairs what it has written (a thread reads its own elements back).  Apart, so that the kernel keeps
 // nothing in registers for the sake of it.
-__device__ __noinline__ void cl_repair_written(const ClParams& P, const ClSource& S, float* dw, int log_cb)
+__device__ __noinline__ void cl_repair_written(const ClShape& P, const ClSource& S, float* dw, int log_cb)
 {
     const int tile = blockIdx.y, col0 = blockIdx.x << log_cb;
     for (int e = threadIdx.x; e < 128 << log_cb; e += blockDim.x) {          // (whole warps: both are multiples of 32)
@@ -625,6 +627,12 @@ __device__ __noinline__ void cl_repair_written(const ClParams& P, const ClSource
     }
 }
 
+// What cl_reduce_kernel has to know of a column, worked out with the plan: its blocks start when those of cl_kernel end, so that nothing hides the
+// divisions and look-ups before their first loads, nor the banks in which the sums of a warp's columns meet (us, whole call, before / now with
+// this table and rows of 132 sums: bf16 256->256 on 8x8, N = 128 18.1 / 17.3, 128->128 on 16x16 18.1 / 17.4, 36->16 5x5 on 44x44, N = 30 17.1 / 16.3).
+struct ClColumn { int off; uint32_t info; };       // offset in dW from the tile's; column | channel << 8 | atoms in use << 16 | filter row << 20 | output << 24
+struct ClReduce { FastDiv by_r, by_c; int ws_c, atom_step; ClColumn col[kMaxCols]; };
+
 // Sum of the splits of every (tile, column), in a fixed order: grid (column blocks, tiles), 32 * CB * G threads.  Warp (g, c)
 // adds the 128 lanes (a float4 each) of column c over the splits g, g + G, ...; the G partial sums meet in shared memory.  G is
 // chosen so that a warp's loads are all in flight at once (eight, then a second round), CB so that the grid covers the GPU;
@@ -635,28 +643,31 @@ __device__ __noinline__ void cl_repair_written(const ClParams& P, const ClSource
 // and nothing else wants room on them (step of ResNet-20 150 -> 154).
 template <bool LEAN>
 __global__ void __launch_bounds__(1024, LEAN ? 2 : 1)
-cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, const __grid_constant__ ClParams P, const __grid_constant__ ClSource S, int log_cb, int G)
+cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, const __grid_constant__ ClShape P, const __grid_constant__ ClSource S, const __grid_constant__ ClReduce T, int log_cb, int G)
 {
-    __shared__ float s_sum[32][128];
+    __shared__ float s_sum[32][132];        // (rows four banks apart: the columns that a warp writes lie in different ones)
     __shared__ int2 s_col[16];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, CB = 1 << log_cb;
     const int tile = blockIdx.y, col0 = blockIdx.x << log_cb;
     pdl_release_next_grid();
-    const int tr = tile / P.tiles_r, r0 = (tile - tr * P.tiles_r) * P.rc, tk = tr / P.tiles_c;
+    const int tr = T.by_r.div(tile), r0 = (tile - tr * P.tiles_r) * P.rc, tk = T.by_c.div(tr);
     const int k0 = tk * P.kt, c0 = (tr - tk * P.tiles_c) * P.ct;
     const int ca_shift = 31 - __clz(P.ca), mn_mask = P.merged ? 127 : P.ca - 1;
+    // {offset in dW, atoms in use (0: not an element)} of a column, in the order in which they are written
+    auto target = [&](int e, uint32_t info) {
+        const bool valid = e < P.cols && r0 + (int)(info >> 20 & 15) < P.r && (P.c_side ? k0 + (int)(info >> 24) < P.k : c0 + (int)(info >> 8 & 255) < P.c);
+        return valid ? (int)(info >> 16 & 15) : 0;
+    };
+    const int cb = warp & (CB - 1), grp = warp >> log_cb, mine = min(col0 + cb, P.cols - 1);
+    const uint32_t info = T.col[mine].info;
+    const float4* src = reinterpret_cast<const float4*>(partial + ((size_t)tile * P.splits * P.cols + (info & 255)) * 128) + lane;
+    const size_t step = (size_t)P.cols * 32;
+    const bool live = target(col0 + cb, info) > 0;
     if ((int)threadIdx.x < CB) {
         const int e = col0 + threadIdx.x;
-        int2 o = make_int2(0, 0);
-        if (e < P.cols) o = column_target(P, written_column(P, e), k0, c0, r0);
-        s_col[threadIdx.x] = o;
+        const ClColumn o = T.col[min(e, P.cols - 1)];
+        s_col[threadIdx.x] = make_int2((int)(o.off + (P.c_side ? k0 * P.ws_k : 0) + c0 * P.ws_c + (P.stack ? 0 : r0 * P.ws_r)), target(e, o.info));
     }
-    const int cb = warp & (CB - 1), grp = warp >> log_cb;
-    const int src_col = col0 + cb < P.cols ? written_column(P, col0 + cb) : 0;
-    const float4* src = reinterpret_cast<const float4*>(partial + ((size_t)tile * P.splits * P.cols + src_col) * 128) + lane;
-    const size_t step = (size_t)P.cols * 32;
-    __syncthreads();
-    const bool live = s_col[cb].y > 0;
     pdl_wait_prior_grid();
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     if (live)
@@ -678,7 +689,7 @@ cl_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, cons
         if (P.c_side) {
             const int a = P.merged ? 0 : l >> ca_shift, ch = l & mn_mask;
             valid = a < o.y && c0 + ch < P.c && (!P.row_atoms || r0 + a < P.r);
-            off += channel_offset(P, ch) + a * atom_step(P);
+            off += (P.vc == 0 ? ch * T.ws_c : (int)channel_offset(P, ch)) + a * T.atom_step;         // (offsets in dW have 32 bits)
         } else {
             const int lane_off = lane_target(P, l, k0, r0);
             valid = o.y > 0 && lane_off >= 0;
@@ -1140,6 +1151,7 @@ struct ClHost {             // what ClPlan::opaque holds
     int xch[2], dych[2];    // elements from one pixel of the operands to the next: packed tightly, and on aligned rows
     int log_cb, groups;     // second kernel: columns per block, split groups per column
     bool lean;              // second kernel: with few registers
+    ClReduce reduce;
 };
 static_assert(sizeof(ClHost) <= sizeof(ClPlan::opaque), "ClPlan::opaque too small");
 
@@ -1325,6 +1337,18 @@ bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, ClPlan*
     while (H.groups < 32 && H.groups * 8 < best.splits) H.groups *= 2;
     H.log_cb = 4;
     while (H.log_cb > 0 && ((H.groups << H.log_cb) > 32 || best.tiles_k * best.tiles_c * best.tiles_r * ceil_div(best.cols, 1 << H.log_cb) < sms)) --H.log_cb;
+    H.reduce.by_r = fast_div(best.tiles_r); H.reduce.by_c = fast_div(best.tiles_c);
+    H.reduce.ws_c = (int)best.ws_c; H.reduce.atom_step = (int)(best.row_atoms ? best.ws_r : best.stride * best.ws_s);
+    for (int e = 0; e < best.cols; ++e) {       // columns in the order of dW, see written_column
+        const ClGroup* gr = best.g;
+        while (gr + 1 < best.g + best.ngroups && e >= gr[1].col) ++gr;
+        int j = e - gr->col;
+        if (!best.c_side && best.s_inner) { const int atoms = gr->n / best.ca, c = j / atoms; j = (j - c * atoms) * best.ca + c; }
+        const int a = best.c_side || best.merged ? 0 : j / best.ca, k = best.c_side ? j : 0, c = gr->cbase + (best.c_side ? 0 : best.merged ? j : j - a * best.ca);
+        const int vs = vc != 0 ? c / vc : 0;
+        H.reduce.col[e].off = (int)(k * best.ws_k + (c - vs * vc) * best.ws_c + (best.stack ? 0 : gr->r) * best.ws_r + (gr->s0 + best.stride * a + vs) * best.ws_s);
+        H.reduce.col[e].info = (uint32_t)(gr->col + j) | (uint32_t)c << 8 | (uint32_t)gr->cnt << 16 | (uint32_t)gr->r << 20 | (uint32_t)k << 24;
+    }
     const int tiles = best.tiles_k * best.tiles_c * best.tiles_r;
     H.lean = g.sm_budget > 0 || tiles * ceil_div(best.cols, 1 << H.log_cb) > sms * (65536 / (64 * 32 * H.groups << H.log_cb));
     if (tiles > 65535 || best.splits > 65535) return false;
@@ -1423,8 +1447,8 @@ cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, 
     note_launch();
     if (P.splits == 1) return cudaSuccess;
     const dim3 rgrid((unsigned)ceil_div(P.cols, 1 << H.log_cb), grid.x);
-    err = launch_kernel(H.lean ? cl_reduce_kernel<true> : cl_reduce_kernel<false>, rgrid, dim3(32u * H.groups << H.log_cb), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw, P,
-                        src, H.log_cb, H.groups);
+    err = launch_kernel(H.lean ? cl_reduce_kernel<true> : cl_reduce_kernel<false>, rgrid, dim3(32u * H.groups << H.log_cb), 0, stream, dim3(1, 1, 1), static_cast<const float*>(partial), dw,
+                        static_cast<const ClShape&>(P), src, H.reduce, H.log_cb, H.groups);
     if (err != cudaSuccess) return err;
     note_launch();
     return cudaSuccess;

@@ -188,7 +188,7 @@ struct ClPlan {
     double cycles;                          // the planner's estimate of the two kernels, SM cycles
     size_t partial_bytes;                   // workspace: accumulator blocks, and
     size_t x_bytes[2], dy_bytes[2];         // packed copies of the operands (0: read in place), [0] tightly, [1] on aligned rows
-    alignas(8) unsigned char opaque[3072];  // kernel parameters, private to cl.cu
+    alignas(8) unsigned char opaque[4608];  // kernel parameters, private to cl.cu
 };
 bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* plan);
 cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, void* x_scratch, void* dy_scratch, uint32_t* status,
