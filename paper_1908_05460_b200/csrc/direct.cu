@@ -28,13 +28,13 @@ template <> struct Vec<1> { float v[1]; __device__ void load(const float* p) { v
 template <> struct Vec<2> { float v[2]; __device__ void load(const float* p) { float2 t = *reinterpret_cast<const float2*>(p); v[0] = t.x; v[1] = t.y; } };
 template <> struct Vec<4> { float v[4]; __device__ void load(const float* p) { float4 t = *reinterpret_cast<const float4*>(p); v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w; } };
 
-// The CTA's threads fill `n` floats in turn, `at(i)` the address of the i-th one's source, nullptr: zero.  Eight loads a thread are under way
-// at once (few, where there is little to fill).  Bound by latency: with one load, behind two divisions by numbers that only the launch knows,
-// 16 x 512 pixels took 27 us to arrive.  (us, before / now, with the bands of plan_direct: bf16 1x1 3->80 on 36x36, N = 24 57.6 / 11.5, fp32 3->156
-// on 35x35, N = 10 44.6 / 13.3, bf16 3x3 3->16 on 33x38, N = 3 26.8 / 9.7, fp32 3->20 on 60x60, N = 6 18.0 / 12.5, 1x1 3->304 on 5x5, N = 57 16.9 / 7.3;
-// bf16 20->20 on 9x9, N = 12 11.3 / 11.6.)
+// The CTA's threads fill `n` floats in turn, `at(i)` the address of the i-th one's source, nullptr: zero.  U loads a thread are under way at
+// once.  Bound by latency: with one load, behind two divisions by numbers that only the launch knows, 16 x 512 pixels took 27 us to arrive.
+// (us, before / now, with the bands of plan_direct: bf16 1x1 3->80 on 36x36, N = 24 57.5 / 10.4, fp32 3->156 on 35x35, N = 10 44.5 / 13.7, bf16 3x3
+// 3->16 on 33x38, N = 3 26.0 / 9.1, fp32 3->20 on 60x60, N = 6 17.9 / 12.4, 1x1 3->304 on 5x5, N = 57 16.8 / 7.1, bf16 20->20 on 9x9, N = 12 11.3 / 11.1.
+// Eight at a time, and another form for short runs, lengthen the code: 10.9, 13.3, 9.7, 12.5, 7.3, 11.6.)
 template <int U, typename T, typename At>
-__device__ __forceinline__ void fill_by(int n, At at)
+__device__ __forceinline__ void fill(int n, At at)
 {
     for (int i0 = threadIdx.x; i0 < n; i0 += U * kThreads) {
         const T* src[U];
@@ -48,13 +48,6 @@ __device__ __forceinline__ void fill_by(int n, At at)
         for (int u = 0; u < U; ++u) if (i0 + u * kThreads < n) *dst[u] = v[u];
     }
 }
-template <typename T, typename At>
-__device__ __forceinline__ void fill(int n, At at)
-{
-    if (n <= 2 * kThreads) fill_by<2, T>(n, at);
-    else fill_by<8, T>(n, at);
-}
-
 // Stage one work item with the CTA's threads: dY band as [k][pixel] (row stride dys) and X window as
 // [row][col][TC], converted to fp32; four elements per load where the layout allows.
 template <typename T, bool UNUSED, int TK, int TC>
@@ -62,6 +55,8 @@ __device__ __forceinline__ void stage_item(const T* __restrict__ x, const T* __r
                                            const Geom& g, const DirectPlan& pl, int it, int k0, int c0, int dys,
                                            int win_h, int win_w)
 {
+    // (fp32 tiles of 16 channels leave few registers for it, and the compiler's own order of a plain loop is the quicker: 30->20 on 9x11, N = 12 11.6 / 13.0)
+    constexpr bool kPlain = sizeof(T) == 4 && TC > 4;
     const int npx = pl.bp * pl.bq;
     const int n = it / (pl.bands_p * pl.bands_q);
     const int band = it % (pl.bands_p * pl.bands_q);
@@ -77,17 +72,29 @@ __device__ __forceinline__ void stage_item(const T* __restrict__ x, const T* __r
             if (k < g.k) ld4(src, v);
             *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
         }
+    } else if constexpr (kPlain) {
+        for (int i = threadIdx.x; i < TK * npx; i += kThreads) {
+            const int kk = i / npx, j = i % npx;
+            const int p = p0 + j / pl.bq, q = q0 + j % pl.bq, k = k0 + kk;
+            float v = 0.f;
+            if (k < g.k && p < g.p && q < g.q) v = ldf(dy + (((long long)n * g.k + k) * g.p + p) * g.q + q);
+            s_dy[kk * dys + j] = v;
+        }
     } else {
         const T* base = dy + ((long long)n * g.k + k0) * g.p * g.q + (long long)p0 * g.q + q0;
         const int pq = g.p * g.q, left_k = g.k - k0, left_p = g.p - p0, left_q = g.q - q0;
         const bool rows = pl.bq == g.q;           // (then the band's pixels lie end to end)
-        fill<T>(TK * npx, [&](int i, float*& dst) -> const T* {
-            const int kk = pl.by_npx.div(i), j = i - kk * npx;
-            dst = s_dy + kk * dys + j;
-            if (rows) return kk < left_k && j < left_p * g.q ? base + (long long)kk * pq + j : nullptr;
-            const int pp = pl.by_bq.div(j), qq = j - pp * pl.bq;
-            return kk < left_k && pp < left_p && qq < left_q ? base + (long long)kk * pq + pp * g.q + qq : nullptr;
-        });
+        auto fill_dy = [&](auto image) {            // (a number that holds offsets within an image)
+            typedef decltype(image) Off;
+            fill<sizeof(Off) == 4 ? 4 : 1, T>(TK * npx, [&](int i, float*& dst) -> const T* {
+                const int kk = pl.by_npx.div(i), j = i - kk * npx;
+                dst = s_dy + kk * dys + j;
+                if (rows) return kk < left_k && j < left_p * g.q ? base + ((Off)kk * pq + j) : nullptr;
+                const int pp = pl.by_bq.div(j), qq = j - pp * pl.bq;
+                return kk < left_k && pp < left_p && qq < left_q ? base + ((Off)kk * pq + pp * g.q + qq) : nullptr;
+            });
+        };
+        if (pl.small) fill_dy(0); else fill_dy(0ll);
     }
     if (pl.vec_x) {
         constexpr int CQ = TC / 4;                                // channel quads per pixel of the tile
@@ -104,14 +111,28 @@ __device__ __forceinline__ void stage_item(const T* __restrict__ x, const T* __r
                 *reinterpret_cast<float4*>(drow + i * 4) = make_float4(v[0], v[1], v[2], v[3]);
             }
         }
+    } else if constexpr (kPlain) {
+        for (int i = threadIdx.x; i < win_h * win_w * TC; i += kThreads) {
+            const int cc = i % TC, pix = i / TC;
+            const int hh = h0 + pix / win_w, ww = w0 + pix % win_w, c = c0 + cc;
+            float v = 0.f;
+            if (c < g.c && hh >= 0 && hh < g.h && ww >= 0 && ww < g.w)
+                v = ldf(x + n * g.xs_n + c * g.xs_c + hh * g.xs_h + ww * g.xs_w);
+            s_x[i] = v;
+        }
     } else {
         const T* base = x + n * g.xs_n + c0 * g.xs_c + h0 * g.xs_h + w0 * g.xs_w;
         const int left_c = g.c - c0;
-        fill<T>(win_h * win_w * TC, [&](int i, float*& dst) -> const T* {
-            const int pix = i / TC, cc = i - pix * TC, hh = pl.by_win_w.div(pix), ww = pix - hh * win_w;
-            dst = s_x + i;
-            return cc < left_c && (unsigned)(h0 + hh) < (unsigned)g.h && (unsigned)(w0 + ww) < (unsigned)g.w ? base + cc * g.xs_c + hh * g.xs_h + ww * g.xs_w : nullptr;
-        });
+        auto fill_x = [&](auto image) {
+            typedef decltype(image) Off;
+            const Off step_c = (Off)g.xs_c, step_h = (Off)g.xs_h, step_w = (Off)g.xs_w;
+            fill<sizeof(Off) == 4 ? 4 : 1, T>(win_h * win_w * TC, [&](int i, float*& dst) -> const T* {
+                const int pix = i / TC, cc = i - pix * TC, hh = pl.by_win_w.div(pix), ww = pix - hh * win_w;
+                dst = s_x + i;
+                return cc < left_c && (unsigned)(h0 + hh) < (unsigned)g.h && (unsigned)(w0 + ww) < (unsigned)g.w ? base + (cc * step_c + hh * step_h + ww * step_w) : nullptr;
+            });
+        };
+        if (pl.small) fill_x(0); else fill_x(0ll);
     }
 }
 
@@ -400,6 +421,8 @@ DirectPlan plan_direct(const Geom& g)
     }
     else while (pl.bp * 2 <= g.p && pl.bp * 2 * pl.bq <= max_px && smem_for(g, v, pl.bp * 2, pl.bq) <= 96 * 1024) pl.bp *= 2;
     while (pl.bq > 1 && smem_for(g, v, pl.bp, pl.bq) > 96 * 1024) pl.bq /= 2;
+    // (offsets of elements in and around an image, up to a window beyond it, in 32 bits)
+    pl.small = (double)(g.c + 16) * (g.h + 1024) * (g.w + 1024) < 2e9 && (double)(g.k + 16) * g.p * g.q < 2e9;
     pl.by_npx = fast_div(pl.bp * pl.bq); pl.by_bq = fast_div(pl.bq); pl.by_win_w = fast_div((pl.bq - 1) * g.stride_w + g.s);
     pl.bands_p = (g.p + pl.bp - 1) / pl.bp;
     pl.bands_q = (g.q + pl.bq - 1) / pl.bq;

@@ -146,6 +146,7 @@ struct DirectPlan {
     size_t partial_bytes;
     bool tiled;             // false: filter size without a tiled instantiation -> per-element kernel
     bool vec_dy, vec_x;     // 4-element vector loads usable for the dY band / the X window
+    bool small;             // an image's elements are within 32-bit offsets of one another
     FastDiv by_npx, by_bq, by_win_w;        // by pixels of a band, its columns, columns of the X window
 };
 DirectPlan plan_direct(const Geom& g);
