@@ -1228,6 +1228,8 @@ bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, ClPlan*
 
     ClParams best{};
     double best_cycles = 1e30;
+    // a packing pass of dY: its launch, and its bytes twice
+    const double dy_pass = H.pack_dy ? 3500 + (double)dy_el * 2 * (1 + B.planes) / (16.0 * sms) : 0.0;
     for (int form = 0; form < 4; ++form) {           // k-side, c-side, stack, c-side with filter rows
         if (form == 3 && (g.s != 1 || g.r == 1 || g.stride_h != 1 || B.ca > 32)) break;
         if (form == 2 && (g.k > 64 || g.r == 1 || g.stride_h != 1)) continue;
@@ -1281,8 +1283,7 @@ bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, ClPlan*
 #endif
                             Cost c = cost_of(C, sms, std::min(1.0, 1.3 * share / C.cols));
                             if (form == 2) c.cycles *= 1.07;          // (by a few per cent the other forms are as quick or quicker)
-                            // a packing pass of dY: its launch, and its bytes twice
-                            if (mode != kPixels && H.pack_dy) c.cycles += 3500 + (double)dy_el * 2 * (1 + C.planes) / (16.0 * sms);
+                            if (mode != kPixels) c.cycles += dy_pass;
                             if (c.cycles < best_cycles) { best_cycles = c.cycles; C.splits = c.splits; best = C; }
                             return true;
                         };
@@ -1353,6 +1354,7 @@ bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, ClPlan*
     H.lean = g.sm_budget > 0 || tiles * ceil_div(best.cols, 1 << H.log_cb) > sms * (65536 / (64 * 32 * H.groups << H.log_cb));
     if (tiles > 65535 || best.splits > 65535) return false;
     out->cycles = best_cycles;
+    out->dy_pass = best.order == kPixels ? 0.0 : dy_pass;
     out->partial_bytes = best.splits == 1 ? 0 : (size_t)tiles * best.splits * best.cols * 512;
     for (int wide = 0; wide < 2; ++wide) {
         H.xch[wide] = wide && H.pack_x && !H.f32 ? wide_pitch(g.c, best.ca) : round_up(g.c, 8);
@@ -1369,8 +1371,10 @@ bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, ClPlan*
 // packing pass, which such inputs need anyway, gathers s x c of them for every output column, and the filter becomes one of s = 1, whose
 // rows are the atoms of one c-side MMA a k-step.  (Bound by operand reads before, with one MMA a filter row; us, plain / gathered: bf16 on
 // 32x32 5x5 3->64, N = 128 25.1 / 15.4, 3x3 N = 256 23.9 / 20.8, 7x7 3->64 on 40x40, N = 50 19.2 / 15.2, fp32 5x5 3->64, N = 128 54.7 / 37.5,
-// 3x3 3->40 on 30x30, N = 40 29.3 / 19.2.)  The gathered operand is longer, and so is its pass: a tenth of the whole has to be gained by the estimate
-// (less lost: bf16 5x5 3->48 on 17x17, N = 30 12.2 / 13.1, estimated 15,300 / 14,300 cycles).
+// 3x3 3->40 on 30x30, N = 40 29.3 / 19.2.)  The gathered operand is longer, and so is its pass: a tenth of the estimate has to be gained
+// (less lost: bf16 5x5 3->48 on 17x17, N = 30 12.2 / 13.1, estimated 11,100 / 10,100 cycles).  What both forms spend on packing dY is left out: it
+// is there or not by the memory order of dY, which must not decide how its products are summed.  (Of 60 stems for which that moves the line, N = 9
+// to 244, 36 gain more than 2 % from it, up to a quarter, 11 lose as much; geometric mean 0.96.)
 bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
 {
     const bool plain = plan_problem(g, dy_npqk, 0, 0, 0, out);
@@ -1381,7 +1385,9 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
     Geom v = g;
     v.c = g.s * g.c; v.s = 1; v.w = g.q; v.pad_w = 0;
     ClPlan gathered;
-    if (!plan_problem(v, dy_npqk, g.c, g.w, g.pad_w, &gathered) || (plain && 10 * gathered.cycles >= 9 * out->cycles)) return plain;
+    if (!plan_problem(v, dy_npqk, g.c, g.w, g.pad_w, &gathered)) return plain;
+    const double same = std::min(gathered.dy_pass, out->dy_pass);
+    if (plain && 10 * (gathered.cycles - same) >= 9 * (out->cycles - same)) return plain;
     *out = gathered;
     return true;
 }

@@ -186,7 +186,8 @@ cudaError_t launch_tc(const void* x, const void* dy, float* dw, float* partial, 
 
 // ---- exact filter gradient on tcgen05 with channels-last bf16 operands: any map size, channel count, stride, layout and type ----
 struct ClPlan {
-    double cycles;                          // the planner's estimate of the two kernels, SM cycles
+    double cycles;                          // the planner's estimate of the kernels, SM cycles,
+    double dy_pass;                         // and what of it is for a packed copy of dY
     size_t partial_bytes;                   // workspace: accumulator blocks, and
     size_t x_bytes[2], dy_bytes[2];         // packed copies of the operands (0: read in place), [0] tightly, [1] on aligned rows
     alignas(8) unsigned char opaque[4608];  // kernel parameters, private to cl.cu

@@ -44,6 +44,9 @@ SHAPES = [
     ConvLayer("2 channels, 9 rows in two tiles", 22, 2, 30, 17, 130, 9, 3, 1, 1),
     ConvLayer("2 channels, 7x7, odd rows", 30, 2, 34, 31, 48, 7, 7, 1, 3),
     ConvLayer("3x1 filter, 20 channels", 30, 20, 26, 16, 60, 3, 1, 1, 0),
+    # (the gain of gathered windows is a tenth of the estimate without the packing pass of dY, less of it with)
+    ConvLayer("windows of two channels, 224 outputs, rows of 43", 19, 2, 43, 43, 224, 3, 3, 1, 1),
+    ConvLayer("windows of four channels, 248 outputs, rows of 14", 18, 4, 14, 14, 248, 5, 5, 1, 2),
 ]
 LAYOUTS = {"paper": {}, "nchw": dict(x_layout=B.X_NCHW, dw_layout=B.DW_KCRS),
            "nhwc": dict(dy_layout=B.DY_NPQK, dw_layout=B.DW_KCRS), "rsck": dict(x_layout=B.X_NCHW, dy_layout=B.DY_NPQK, dw_layout=B.DW_RSCK)}
