@@ -98,8 +98,10 @@ uint64_t gaconv_launch_count(void);
  * descriptor (its workspace fields are ignored).  Never fails for a valid descriptor; *bytes > 0.
  * The size has room for the copies of operands that the fastest kernel wants in another form: channels-last bf16, i.e.
  * two bytes an element of a bf16 operand (whose pixels may lie up to a third further apart than its channels fill) and six of
- * an fp32 one.  A call with a smaller workspace takes the kernels that need
- * no such copies (slower, and another rounding), down to what those need. */
+ * an fp32 one.  Inputs of up to four channels at stride 1 may be copied window by window: s*c channels, rounded up to a multiple
+ * of 8, for every output column in place of c for every input column.  A call with a smaller workspace takes, as far as each goes: the
+ * same kernels with the pixels of the copies closer together (the same bits); kernels or plans that need less (slower, and another
+ * rounding).  What fits none of them is refused. */
 gaconv_status_t gaconv_workspace_size(const gaconv_conv_desc_t *desc, int32_t method, size_t *bytes);
 
 /* Prepare a workspace once after allocating it (zero-fills its control words).  Afterwards the
@@ -124,15 +126,14 @@ gaconv_status_t gaconv_dw_exact(const void *x, const void *dy, float *dw,
  * Some callers cannot give the library a workspace because they may not call cudaMalloc where they
  * run: a host framework's plugin that is handed only its inputs and outputs, a loop that was promised
  * "no allocation after warm-up", a process whose device memory pool belongs to someone else.  This
- * variant computes what gaconv_dw_exact computes, with the same kernels as far as their scratch fits (a call whose
- * repacked operands do not fit takes the kernels that need none), but keeps the scratch
- * (split partial sums, control words) in a fixed array inside the library: gaconv_static_scratch_bytes()
+ * variant computes what gaconv_dw_exact computes in a workspace of that size, and keeps the scratch
+ * (repacked operands, split partial sums, control words) in a fixed array inside the library: gaconv_static_scratch_bytes()
  * bytes (8 MiB) that every GPU loading the library holds until the process exits.  desc->workspace and
  * desc->workspace_bytes are ignored.  The call allocates nothing (no cudaMalloc, cudaFree or
  * allocating library routine).
- *   - Limit: a problem whose scratch, without repacked operands, exceeds
- *     gaconv_static_scratch_bytes() is rejected with GACONV_ERR_WORKSPACE_TOO_SMALL and nothing is
- *     enqueued; use gaconv_dw_exact with a caller-owned workspace for those.
+ *   - Limit: a problem that no kernel computes in gaconv_static_scratch_bytes() of scratch is rejected with
+ *     GACONV_ERR_WORKSPACE_TOO_SMALL and nothing is enqueued; use gaconv_dw_exact with a caller-owned
+ *     workspace for those.
  *   - The first call on each device resolves the array's device address and clears its control words
  *     on `stream`; make that first call before any stream capture begins.
  *   - All calls on a device share the one array, which keeps the previous call's contents (each call

@@ -136,7 +136,7 @@ Top1Layout build_top1_layout(const Geom& g, bool cl)
     L.dense = top1_dense_route(g, &L.tp);
     // the contraction: by the channels-last kernel, which reads either form of the sparse tensor (256->256 on 8x8, N = 256:
     // 37 us with the other kernel, 32)
-    L.cl = cl && L.dense && tensor_maps_available() && plan_cl(g, L.tp.reads_transposed_dy, &L.cp) && !short_sums(g, L.cp);
+    L.cl = cl && L.dense && tensor_maps_available() && plan_cl(g, L.tp.reads_transposed_dy, kNoLimit, &L.cp) && !short_sums(g, L.cp);
     const size_t cl_scratch = L.cl ? L.cp.x_bytes[0] + L.cp.dy_bytes[0] : 0;
     const size_t maps = (size_t)g.n * g.k;
     L.idx_off = kWsDataOffset;
@@ -243,17 +243,24 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, const ClPlan& plan, bool reo
     // operands must be packed (16->64 on 6x6, N = 30 launched one by one 10.3 / 12.3 us; 1x1 80->22 on 6x6, N = 105 25 / 12), and with three channels
     return products > (!g.bf16 && g.r * g.s >= 9 ? 2e7 : g.c <= 4 ? 1e7 : 4e6);
 }
-struct ClRoute { bool use; ClPlan plan; size_t partial_off, x_off, dy_off[2], total[2]; };       // [0] copies packed tightly, [1] on aligned rows
-ClRoute build_cl_route(const gaconv_conv_desc_t* desc, const Geom& g)
+struct ClRoute {
+    bool use;
+    bool lean_first;        // without room for it: another plan of this kernel is quicker than the other kernels
+    ClPlan plan;
+    size_t partial_off, x_off, dy_off[2], total[2];       // [0] copies packed tightly, [1] on aligned rows
+};
+ClRoute build_cl_route(const gaconv_conv_desc_t* desc, const Geom& g, size_t limit)
 {
     ClRoute R{};
-    if (!tensor_maps_available() || !plan_cl(g, desc->dy_layout == GACONV_DY_NPQK, &R.plan)) return R;
+    if (!tensor_maps_available() || limit < kWsDataOffset || !plan_cl(g, desc->dy_layout == GACONV_DY_NPQK, limit == kNoLimit ? limit : limit - kWsDataOffset, &R.plan)) return R;
     gaconv_conv_desc_t native = *desc;
     native.x_layout = GACONV_X_NHWC; native.dy_layout = GACONV_DY_NKPQ;
     Geom gn;
     if (make_geom(&native, &gn) != GACONV_OK) return R;
     const ExactLayout L = exact_layout(gn, GACONV_MATH_DEFAULT, GACONV_ALGO_AUTO);
-    R.use = prefer_cl(gn, L, R.plan, (desc->x_layout == GACONV_X_NCHW && g.c > 1) || (desc->dy_layout == GACONV_DY_NPQK && g.k > 1));
+    const bool reordered = (desc->x_layout == GACONV_X_NCHW && g.c > 1) || (desc->dy_layout == GACONV_DY_NPQK && g.k > 1);
+    R.use = limit != kNoLimit || prefer_cl(gn, L, R.plan, reordered);
+    R.lean_first = R.plan.windows && (!L.stem_ok || (g.bf16 && reordered));
 #ifdef GACONV_TUNING
     if (const char* e = getenv("GACONV_CL")) R.use = atoi(e) != 0;
 #endif
@@ -265,11 +272,30 @@ ClRoute build_cl_route(const gaconv_conv_desc_t* desc, const Geom& g)
     }
     return R;
 }
-bool cl_route(const gaconv_conv_desc_t* desc, const Geom& g, ClRoute* R)
+// limit (a multiple of 256 bytes, or kNoLimit): scratch that the route may use
+ClRoute planned_route(const gaconv_conv_desc_t* desc, const Geom& g, size_t limit)
+{
+    static PlanCache<ClRoute> cache;
+    return cache.get(plan_key(g, desc->dy_layout, limit == kNoLimit ? -1 : (int)(limit >> 8)), [&] { return build_cl_route(desc, g, limit); });
+}
+// The channels-last kernel takes a call given `given` bytes of scratch.  Where its plan does not fit, the other kernels come next, except for
+// gathered stems whose other kernels first have to transpose an operand or are the FP32 pipes: the plain form, or fewer splits, needs less (7x7
+// 2->48 on 34x31 maps, N = 30, by the estimate 1.4 times the cycles).
+bool cl_route(const gaconv_conv_desc_t* desc, const Geom& g, size_t given, ClRoute* R)
 {
     if (desc->math != GACONV_MATH_DEFAULT || desc->algo != GACONV_ALGO_AUTO) return false;
-    static PlanCache<ClRoute> cache;
-    *R = cache.get(plan_key(g, desc->dy_layout, 0), [&] { return build_cl_route(desc, g); });
+    *R = planned_route(desc, g, kNoLimit);
+    if (!R->use || given >= R->total[0]) return R->use;
+    if (!R->lean_first) return false;
+    const double most = 3 * R->plan.cycles;
+    *R = planned_route(desc, g, given & ~(size_t)255);
+    return R->use && R->plan.cycles <= most;
+}
+// Its plans that no other kernel fits beside: fewer splits, or copies of fewer bytes, in place of an error
+bool cl_last_route(const gaconv_conv_desc_t* desc, const Geom& g, size_t given, ClRoute* R)
+{
+    if (desc->math != GACONV_MATH_DEFAULT || desc->algo != GACONV_ALGO_AUTO || !planned_route(desc, g, kNoLimit).use) return false;
+    *R = planned_route(desc, g, given & ~(size_t)255);
     return R->use;
 }
 
@@ -422,13 +448,10 @@ struct gaconv_schedule {
     struct StepCache* steps = nullptr;      // repeated steps as CUDA graphs, created on first use
 };
 
-gaconv_status_t gaconv::method_workspace(const gaconv_conv_desc_t* desc, int32_t method, bool cl, bool least, size_t* bytes)
+// scratch of a call, exact ones without the channels-last kernel
+// (cl: the dense route of top-1 with it)
+static gaconv_status_t other_workspace(const gaconv_conv_desc_t* desc, const Geom& g, int32_t method, bool cl, size_t* bytes)
 {
-    Geom g;
-    gaconv_status_t st = make_geom(desc, &g);
-    if (st != GACONV_OK) return st;
-    ClRoute C;
-    if (cl && method == GACONV_METHOD_EXACT && cl_route(desc, g, &C)) { *bytes = C.total[!least]; return GACONV_OK; }
     const Relayout R = plan_relayout(desc, method, cl);
     if (R.move_x || R.move_dy) { *bytes = moved_ws_bytes(desc, g, R); return GACONV_OK; }
     bool ok = false;
@@ -438,24 +461,35 @@ gaconv_status_t gaconv::method_workspace(const gaconv_conv_desc_t* desc, int32_t
     return GACONV_OK;
 }
 
-gaconv_status_t gaconv::run_exact(const void* x, const void* dy, float* dw, const gaconv_conv_desc_t* desc, cudaStream_t stream, bool cl)
+gaconv_status_t gaconv::method_workspace(const gaconv_conv_desc_t* desc, int32_t method, size_t given, size_t* bytes)
 {
     Geom g;
     gaconv_status_t st = make_geom(desc, &g);
     if (st != GACONV_OK) return st;
-    if (x == nullptr || dy == nullptr || dw == nullptr) return GACONV_ERR_NULL_POINTER;
-    if (!aligned16(x) || !aligned16(dy) || !aligned16(dw)) return GACONV_ERR_MISALIGNED;
-    if (desc->math == GACONV_MATH_TF32 && g.bf16) return GACONV_ERR_BAD_DESC;
+    const bool exact = method == GACONV_METHOD_EXACT;
     ClRoute C;
-    // (a workspace without room for the packed operands: the kernels that need none, as far as it goes)
-    if (cl && cl_route(desc, g, &C) && (desc->workspace == nullptr || desc->workspace_bytes >= C.total[0])) {
-        st = check_ws(desc, C.total[0]);
-        if (st != GACONV_OK) return st;
-        const bool wide = desc->workspace_bytes >= C.total[1];
-        char* ws = static_cast<char*>(desc->workspace);
-        return launch_cl(x, dy, dw, reinterpret_cast<float*>(ws + C.partial_off), ws + C.x_off, ws + C.dy_off[wide],
-                         reinterpret_cast<uint32_t*>(ws), C.plan, wide, stream) == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
-    }
+    if (exact && cl_route(desc, g, given, &C)) { *bytes = C.total[given >= C.total[1]]; return GACONV_OK; }
+    st = other_workspace(desc, g, method, !exact, bytes);
+    if (st != GACONV_OK || *bytes <= given) return st;
+    if (!exact) return other_workspace(desc, g, method, false, bytes);
+    if (cl_last_route(desc, g, given, &C)) *bytes = C.total[0];
+    return GACONV_OK;
+}
+
+static gaconv_status_t run_cl(const void* x, const void* dy, float* dw, const gaconv_conv_desc_t* desc, const ClRoute& C, cudaStream_t stream)
+{
+    const gaconv_status_t st = check_ws(desc, C.total[0]);
+    if (st != GACONV_OK) return st;
+    const bool wide = desc->workspace_bytes >= C.total[1];
+    char* ws = static_cast<char*>(desc->workspace);
+    return launch_cl(x, dy, dw, reinterpret_cast<float*>(ws + C.partial_off), ws + C.x_off, ws + C.dy_off[wide],
+                     reinterpret_cast<uint32_t*>(ws), C.plan, wide, stream) == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
+}
+
+// exact dW by the kernels other than the channels-last one
+static gaconv_status_t run_others(const void* x, const void* dy, float* dw, const gaconv_conv_desc_t* desc, const Geom& g, cudaStream_t stream)
+{
+    gaconv_status_t st;
     if (desc->dy_layout == GACONV_DY_NPQK && g.k > 1 && desc->algo != GACONV_ALGO_DIRECT) {
         // Small maps: the tensor-core kernel's dY operand IS the channels-last order (its pre-pass would transpose an
         // N x K x P x Q gradient into it), so a channels-last gradient is read where it lies; only X may have to move.
@@ -483,11 +517,12 @@ gaconv_status_t gaconv::run_exact(const void* x, const void* dy, float* dw, cons
     }
     {
         gaconv_conv_desc_t inner;
+        Geom gi;
         const void *xt = nullptr, *dyt = nullptr;
         bool moved = false;
         st = relayout_operands(x, dy, desc, GACONV_METHOD_EXACT, stream, &inner, &xt, &dyt, &moved);
         if (st != GACONV_OK) return st;
-        if (moved) return run_exact(xt, dyt, dw, &inner, stream, false);
+        if (moved) return make_geom(&inner, &gi) == GACONV_OK ? run_others(xt, dyt, dw, &inner, gi, stream) : GACONV_ERR_BAD_DESC;
     }
     const ExactLayout L = exact_layout(g, desc->math, desc->algo);
     const bool mma_ok = direct_mma_supported(g, L.dp);
@@ -540,7 +575,7 @@ uint64_t gaconv_launch_count(void) { return g_launches.load(std::memory_order_re
 gaconv_status_t gaconv_workspace_size(const gaconv_conv_desc_t* desc, int32_t method, size_t* bytes)
 {
     if (bytes == nullptr) return GACONV_ERR_NULL_POINTER;
-    return method_workspace(desc, method, true, false, bytes);
+    return method_workspace(desc, method, kNoLimit, bytes);
 }
 
 gaconv_status_t gaconv_workspace_init(void* workspace, size_t bytes, void* stream)
@@ -554,7 +589,18 @@ gaconv_status_t gaconv_workspace_init(void* workspace, size_t bytes, void* strea
 
 gaconv_status_t gaconv_dw_exact(const void* x, const void* dy, float* dw, const gaconv_conv_desc_t* desc, void* stream)
 {
-    return run_exact(x, dy, dw, desc, static_cast<cudaStream_t>(stream), true);
+    Geom g;
+    gaconv_status_t st = make_geom(desc, &g);
+    if (st != GACONV_OK) return st;
+    if (x == nullptr || dy == nullptr || dw == nullptr) return GACONV_ERR_NULL_POINTER;
+    if (!aligned16(x) || !aligned16(dy) || !aligned16(dw)) return GACONV_ERR_MISALIGNED;
+    if (desc->math == GACONV_MATH_TF32 && g.bf16) return GACONV_ERR_BAD_DESC;
+    cudaStream_t cs = static_cast<cudaStream_t>(stream);
+    const size_t given = desc->workspace != nullptr ? desc->workspace_bytes : kNoLimit;
+    ClRoute C;
+    if (cl_route(desc, g, given, &C)) return run_cl(x, dy, dw, desc, C, cs);
+    st = run_others(x, dy, dw, desc, g, cs);
+    return st == GACONV_ERR_WORKSPACE_TOO_SMALL && cl_last_route(desc, g, given, &C) ? run_cl(x, dy, dw, desc, C, cs) : st;
 }
 
 gaconv_status_t gaconv_dw_approx(int32_t method, const void* x, const void* dy, float* dw,
@@ -677,8 +723,7 @@ static gaconv_status_t dw_from_host(int32_t method, const void* x_host, const vo
         if (!aligned16(x_dev) || !aligned16(dy_dev)) return GACONV_ERR_MISALIGNED;
         if (method == GACONV_METHOD_EXACT && desc->math == GACONV_MATH_TF32 && g.bf16) return GACONV_ERR_BAD_DESC;
         size_t need = 0;
-        st = method_workspace(desc, method, true, true, &need);
-        if (st == GACONV_OK && desc->workspace_bytes < need) st = method_workspace(desc, method, false, true, &need);
+        st = method_workspace(desc, method, desc->workspace_bytes, &need);
         if (st != GACONV_OK) return st;
         st = check_ws(desc, need);
         if (st != GACONV_OK) return st;

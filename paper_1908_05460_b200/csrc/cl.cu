@@ -968,7 +968,7 @@ constexpr int kStageBudget = 216 * 1024;
 // cycles of instructions each (two of either work in turn); a CTA writes its block at ~21 bytes a cycle to the workspace and at
 // ~18 to dW; start, first loads, drain and the second kernel come to a few thousand.
 struct Cost { double cycles; int splits; };
-Cost cost_of(const ClParams& P, int sms, double block_share)
+Cost cost_of(const ClParams& P, int sms, double block_share, size_t room)     // room: bytes for partial blocks
 {
     double ksteps = P.ksteps;
     if (P.skip) {       // the tile with the fewest rows left out decides
@@ -985,7 +985,7 @@ Cost cost_of(const ClParams& P, int sms, double block_share)
     const int tiles = P.tiles_k * P.tiles_c * P.tiles_r;
     const double block_bytes = (double)P.cols * 512 * block_share;
     Cost best{1e30, 1};
-    int most = std::max(1, std::min(P.chunks, sms / tiles));
+    int most = std::max(1, (int)std::min<size_t>(std::min(P.chunks, sms / tiles), room / ((size_t)tiles * P.cols * 512)));
 #ifdef GACONV_TUNING
     if (const char* e = getenv("GACONV_CL_SP")) most = std::min(most, atoi(e));
 #endif
@@ -1204,7 +1204,7 @@ ClKernel kernel_for(int ng, bool f32, bool c_side)
 }  // namespace
 
 namespace {
-bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, ClPlan* out)
+bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, size_t limit, ClPlan* out)
 {
     if (g.stride_h != g.stride_w || g.stride_h > kMaxMapStep || g.r > 16 || g.s > 16 || !dw_offsets_fit(g)) return false;
     const bool nhwc = g.xs_c == 1 || (vc != 0 ? vc : g.c) == 1;
@@ -1229,6 +1229,7 @@ bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, ClPlan*
     ClParams best{};
     double best_cycles = 1e30;
     // a packing pass of dY: its launch, and its bytes twice
+    const size_t x_copy = H.pack_x ? align_up(x_el * 2 * B.planes, 256) : 0, dy_copy = H.pack_dy ? align_up(dy_el * 2 * B.planes, 256) : 0;
     const double dy_pass = H.pack_dy ? 3500 + (double)dy_el * 2 * (1 + B.planes) / (16.0 * sms) : 0.0;
     for (int form = 0; form < 4; ++form) {           // k-side, c-side, stack, c-side with filter rows
         if (form == 3 && (g.s != 1 || g.r == 1 || g.stride_h != 1 || B.ca > 32)) break;
@@ -1281,7 +1282,9 @@ bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, ClPlan*
                             if (const char* e = getenv("GACONV_CL_BARE")) if ((C.x_pre > 0) != (atoi(e) != 0)) return true;
                             if (const char* e = getenv("GACONV_CL_NA")) if (C.na != atoi(e)) return true;
 #endif
-                            Cost c = cost_of(C, sms, std::min(1.0, 1.3 * share / C.cols));
+                            const size_t copies = x_copy + (mode == kPixels ? 0 : dy_copy);
+                            if (copies > limit) return true;
+                            Cost c = cost_of(C, sms, std::min(1.0, 1.3 * share / C.cols), limit - copies);
                             if (form == 2) c.cycles *= 1.07;          // (by a few per cent the other forms are as quick or quicker)
                             if (mode != kPixels) c.cycles += dy_pass;
                             if (c.cycles < best_cycles) { best_cycles = c.cycles; C.splits = c.splits; best = C; }
@@ -1355,6 +1358,7 @@ bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, ClPlan*
     if (tiles > 65535 || best.splits > 65535) return false;
     out->cycles = best_cycles;
     out->dy_pass = best.order == kPixels ? 0.0 : dy_pass;
+    out->windows = vc != 0;
     out->partial_bytes = best.splits == 1 ? 0 : (size_t)tiles * best.splits * best.cols * 512;
     for (int wide = 0; wide < 2; ++wide) {
         H.xch[wide] = wide && H.pack_x && !H.f32 ? wide_pitch(g.c, best.ca) : round_up(g.c, 8);
@@ -1375,9 +1379,9 @@ bool plan_problem(const Geom& g, bool dy_npqk, int vc, int vw, int vpad, ClPlan*
 // (less lost: bf16 5x5 3->48 on 17x17, N = 30 12.2 / 13.1, estimated 11,100 / 10,100 cycles).  What both forms spend on packing dY is left out: it
 // is there or not by the memory order of dY, which must not decide how its products are summed.  (Of 60 stems for which that moves the line, N = 9
 // to 244, 36 gain more than 2 % from it, up to a quarter, 11 lose as much; geometric mean 0.96.)
-bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
+bool plan_cl(const Geom& g, bool dy_npqk, size_t limit, ClPlan* out)
 {
-    const bool plain = plan_problem(g, dy_npqk, 0, 0, 0, out);
+    const bool plain = plan_problem(g, dy_npqk, 0, 0, 0, limit, out);
     if (g.c > 4 || g.s < 2 || g.s * g.c > 32 || g.stride_h != 1 || g.stride_w != 1) return plain;
 #ifdef GACONV_TUNING
     if (const char* e = getenv("GACONV_CL_VC")) if (atoi(e) == 0) return plain;
@@ -1385,7 +1389,7 @@ bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* out)
     Geom v = g;
     v.c = g.s * g.c; v.s = 1; v.w = g.q; v.pad_w = 0;
     ClPlan gathered;
-    if (!plan_problem(v, dy_npqk, g.c, g.w, g.pad_w, &gathered)) return plain;
+    if (!plan_problem(v, dy_npqk, g.c, g.w, g.pad_w, limit, &gathered)) return plain;
     const double same = std::min(gathered.dy_pass, out->dy_pass);
     if (plain && 10 * (gathered.cycles - same) >= 9 * (out->cycles - same)) return plain;
     *out = gathered;
@@ -1475,7 +1479,7 @@ extern "C" int gaconv_tuning_plan_cl(const int* v, int bf16, int x_nhwc, int npq
     g.ws_c = 1; g.ws_s = g.c; g.ws_r = g.s * g.c; g.ws_k = g.r * g.s * g.c;
     g.bf16 = bf16 != 0; g.alpha = 1.f; g.sm_budget = budget;
     ClPlan P;
-    if (!plan_cl(g, npqk != 0, &P) || size < (int)sizeof(ClHost)) return -1;
+    if (!plan_cl(g, npqk != 0, kNoLimit, &P) || size < (int)sizeof(ClHost)) return -1;
     memcpy(out, P.opaque, sizeof(ClHost));
     return (int)P.cycles;
 }

@@ -188,20 +188,21 @@ cudaError_t launch_tc(const void* x, const void* dy, float* dw, float* partial, 
 struct ClPlan {
     double cycles;                          // the planner's estimate of the kernels, SM cycles,
     double dy_pass;                         // and what of it is for a packed copy of dY
+    bool windows;                           // X is gathered from windows (stems), into a longer copy
     size_t partial_bytes;                   // workspace: accumulator blocks, and
     size_t x_bytes[2], dy_bytes[2];         // packed copies of the operands (0: read in place), [0] tightly, [1] on aligned rows
     alignas(8) unsigned char opaque[4608];  // kernel parameters, private to cl.cu
 };
-bool plan_cl(const Geom& g, bool dy_npqk, ClPlan* plan);
+constexpr size_t kNoLimit = ~(size_t)0;
+// limit: bytes for partial_bytes + x_bytes[0] + dy_bytes[0]; false where nothing fits
+bool plan_cl(const Geom& g, bool dy_npqk, size_t limit, ClPlan* plan);
 cudaError_t launch_cl(const void* x, const void* dy, float* dw, float* partial, void* x_scratch, void* dy_scratch, uint32_t* status,
                       const ClPlan& plan, bool wide, cudaStream_t stream);        // wide: the copies on aligned rows
 
 int device_sms();       // SMs of the current device
 bool tensor_maps_available();       // the driver's tensor-map encoder was found
 
-// gaconv_workspace_size and gaconv_dw_exact; cl = false: without the channels-last kernel (callers whose scratch it does not fit),
-// least: with the least scratch that it runs in
-gaconv_status_t method_workspace(const gaconv_conv_desc_t* desc, int32_t method, bool cl, bool least, size_t* bytes);
-gaconv_status_t run_exact(const void* x, const void* dy, float* dw, const gaconv_conv_desc_t* desc, cudaStream_t stream, bool cl);
+// The scratch that a call given `given` bytes of it uses; more than `given`: the call is refused.  (kNoLimit: gaconv_workspace_size.)
+gaconv_status_t method_workspace(const gaconv_conv_desc_t* desc, int32_t method, size_t given, size_t* bytes);
 
 }  // namespace gaconv

@@ -74,11 +74,8 @@ gaconv_status_t gaconv_poll_async_status_static(void* stream)
 gaconv_status_t gaconv_dw_exact_static(const void* x, const void* dy, float* dw, const gaconv_conv_desc_t* desc, void* stream)
 {
     if (desc == nullptr) return GACONV_ERR_NULL_POINTER;
-    // the kernels of gaconv_dw_exact where their scratch fits, else those that need less of it
     size_t need = 0;
-    gaconv_status_t st = gaconv::method_workspace(desc, GACONV_METHOD_EXACT, true, true, &need);
-    const bool cl = st == GACONV_OK && need <= kStaticScratchBytes;
-    if (st == GACONV_OK && !cl) st = gaconv::method_workspace(desc, GACONV_METHOD_EXACT, false, true, &need);
+    gaconv_status_t st = gaconv::method_workspace(desc, GACONV_METHOD_EXACT, kStaticScratchBytes, &need);
     if (st != GACONV_OK) return st;
     if (need > kStaticScratchBytes) return GACONV_ERR_WORKSPACE_TOO_SMALL;   // problem too large for the built-in scratch
     if (x == nullptr || dy == nullptr || dw == nullptr) return GACONV_ERR_NULL_POINTER;
@@ -88,7 +85,7 @@ gaconv_status_t gaconv_dw_exact_static(const void* x, const void* dy, float* dw,
     gaconv_conv_desc_t local = *desc;          // same problem, scratch replaced by the built-in array
     local.workspace = scratch;
     local.workspace_bytes = kStaticScratchBytes;
-    return gaconv::run_exact(x, dy, dw, &local, static_cast<cudaStream_t>(stream), cl);
+    return gaconv_dw_exact(x, dy, dw, &local, stream);
 }
 
 }  // extern "C"

@@ -102,6 +102,31 @@ def test_static_scratch_takes_the_kernels_that_fit():
     assert np.max(np.abs(got - want)) <= 1e-4 * np.abs(want).max() and B.gaconv_poll_async_status_static() == B.OK
 
 
+@pytest.mark.parametrize("layer,kw", [
+    (ConvLayer("windows of three channels", 93, 3, 49, 49, 48, 3, 3, 1, 1), {}),
+    (ConvLayer("windows of a 7x7 filter", 300, 3, 25, 25, 32, 7, 7, 1, 3), dict(x_layout=B.X_NCHW, sm_budget=18)),
+    (ConvLayer("5x5 on 3x3 maps, blocks of 5 MB", 979, 200, 3, 3, 112, 5, 5, 1, 1), dict(x_layout=B.X_NCHW)),
+], ids=lambda v: v.name if isinstance(v, ConvLayer) else "")
+def test_static_scratch_without_room_for_the_first_plan(layer, kw):
+    """What the planner likes best (gathered windows, more splits) is beyond the built-in array, and the other kernels would have to transpose
+    operands that are, too: the channels-last kernel in less scratch."""
+    x, dy = I.make_layer_inputs(layer, torch.bfloat16, 25, 0)
+    g = GpuLayer(layer, torch.bfloat16, x, dy, dy_layout=B.DY_NPQK, **kw)
+    bare = B.make_desc(layer, torch.bfloat16, dy_layout=B.DY_NPQK, **kw)
+    assert B.gaconv_workspace_size(bare, B.METHOD_EXACT) > B.gaconv_static_scratch_bytes()
+    want = g.exact()
+    g.dw.fill_(float("nan"))
+    B.gaconv_dw_exact_static(g.x, g.dy, g.dw, bare)
+    got = g.logical_dw()
+    assert B.gaconv_poll_async_status_static() == B.OK
+    assert any("cl_kernel" in k for k in kernel_names(lambda: B.gaconv_dw_exact_static(g.x, g.dy, g.dw, bare)))
+    xd, dyd, rng = to_f64(x), to_f64(dy), np.random.default_rng(4)
+    for k, c, r, s in zip(*(rng.integers(0, m, 60).tolist() for m in (layer.k, layer.c, layer.r, layer.s))):
+        v, norm = oracle.dw_exact_at(xd, dyd, oshape(layer), k, c, r, s)
+        assert abs(got[k, c, r, s] - v) <= TOL_F32 * norm and abs(want[k, c, r, s] - v) <= TOL_F32 * norm
+    assert np.all(np.isfinite(got))
+
+
 # strides and boxes beyond what a tensor map steps over (8 pixels, 256 a side): other kernels take them
 FAR = [
     ConvLayer("stride 9", 20, 64, 40, 37, 96, 3, 3, 9, 1),
@@ -177,6 +202,8 @@ def test_values_that_are_not_finite(li, dtype):
     (ConvLayer("packed planes", 24, 64, 30, 30, 64, 3, 3, 1, 1), torch.float32, {}),
     (ConvLayer("packed gradient", 20, 72, 28, 20, 120, 3, 3, 1, 1), torch.bfloat16, {}),
     (ConvLayer("packed, channels first", 20, 72, 28, 20, 120, 3, 3, 1, 1), torch.bfloat16, dict(x_layout=B.X_NCHW)),
+    (ConvLayer("packed windows", 20, 3, 33, 31, 48, 7, 7, 1, 3), torch.bfloat16, dict(x_layout=B.X_NCHW, dy_layout=B.DY_NPQK)),
+    (ConvLayer("packed windows of fp32", 40, 4, 29, 30, 40, 3, 3, 1, 1), torch.float32, dict(dy_layout=B.DY_NPQK)),
     (ConvLayer("top-1 by the dense route", 20, 256, 8, 8, 100, 3, 3, 1, 1), torch.bfloat16, dict(x_layout=B.X_NCHW, dy_layout=B.DY_NPQK)),
 ], ids=lambda v: v.name if isinstance(v, ConvLayer) else None)
 def test_smaller_workspaces(layer, dtype, kw, method):
