@@ -1,6 +1,7 @@
 // C-ABI entry points of libgaconv: argument validation, workspace planning, kernel dispatch and the
 // approximation-schedule driver (paper Section 2.5).  Every step of the path runs in this library's
 // kernels; there is no CPU or library fallback.
+#include <algorithm>
 #include <atomic>
 #include <cstdlib>
 #include <cstring>
@@ -157,7 +158,9 @@ Top1Layout top1_layout(const Geom& g, bool cl)
     return cache.get(plan_key(g, cl, 0), [&] { return build_top1_layout(g, cl); });
 }
 
-struct ExactLayout { size_t partial_off, scratch_off, total; DirectPlan dp; TcPlan tp; StemPlan sp; bool tc_ok, stem_ok; };
+// kernels other than the channels-last one; least: the scratch that the one taken cannot do without
+enum class ExactKernel { tc, stem, mma, direct };
+struct ExactLayout { size_t partial_off, scratch_off, total, least; DirectPlan dp; TcPlan tp; StemPlan sp; bool tc_ok, stem_ok, mma_ok; ExactKernel kernel; };
 // fp32 inputs take the tcgen05 kernel (TF32 MMAs on split operands) where the layer is wide enough for the
 // tensor cores to pay for the extra pass that splits the operands: 64 input channels, or 32 when the filter
 // rows share one MMA (measured: 32->32@16x16 18.7 us against 19.9 us on the warp-level path; without the
@@ -181,6 +184,12 @@ ExactLayout build_exact_layout(const Geom& g, int math, int algo)
     if (L.stem_ok && L.sp.partial_bytes > partial) partial = L.sp.partial_bytes;
     L.scratch_off = align_up(L.partial_off + partial, 256);
     L.total = align_up(L.scratch_off + (L.tc_ok ? L.tp.scratch_bytes : 0), 256);
+    L.mma_ok = direct_mma_supported(g, L.dp);
+    const bool any = algo != GACONV_ALGO_DIRECT;
+    L.kernel = L.tc_ok && any ? ExactKernel::tc : L.stem_ok && any && math == GACONV_MATH_DEFAULT ? ExactKernel::stem
+             : L.mma_ok && (any || math == GACONV_MATH_TF32) ? ExactKernel::mma : ExactKernel::direct;
+    L.least = L.kernel == ExactKernel::tc ? L.total
+            : L.partial_off + (L.kernel == ExactKernel::stem ? L.sp.partial_bytes : L.kernel == ExactKernel::mma ? L.dp.partial_bytes : 0);
     return L;
 }
 
@@ -236,7 +245,7 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, const ClPlan& plan, bool reo
         if (L.tc_ok && L.tp.chain > 1500) return false;
         if (L.tc_ok)                                                // 128->128 on 16x16 89 / 53, 64->64 on 8x8 18.0 / 19.9, on 18 SMs 45 / 35
             return reordered || products > (g.c >= 128 ? 4e8 : shared ? 1e8 : g.c >= 64 ? 1e9 : 2e8);      // 32->32 on 16x16 19.3 / 17.7, on 18 SMs 43 / 36
-        if (direct_mma_supported(g, L.dp))                          // 16->16 on 32x32 20 / 24.5, 48->96 on 16x16 (N = 64) 31 / 25
+        if (L.mma_ok)                                               // 16->16 on 32x32 20 / 24.5, 48->96 on 16x16 (N = 64) 31 / 25
             return (g.c >= 64 && products > 4e6) || (g.c >= 24 && g.stride_h == 1 && !shared && products > 3e8);       // (N = 16) 24->16 on 32x32 10 / 13.5
     }
     // FP32 pipes: their one or two launches are as quick while the work is small -- longer with 3x3 filters of fp32 layers, whose
@@ -291,10 +300,10 @@ bool cl_route(const gaconv_conv_desc_t* desc, const Geom& g, size_t given, ClRou
     *R = planned_route(desc, g, given & ~(size_t)255);
     return R->use && R->plan.cycles <= most;
 }
-// Its plans that no other kernel fits beside: fewer splits, or copies of fewer bytes, in place of an error
+// In place of an error, where no other kernel fits: fewer splits, or copies of fewer bytes
 bool cl_last_route(const gaconv_conv_desc_t* desc, const Geom& g, size_t given, ClRoute* R)
 {
-    if (desc->math != GACONV_MATH_DEFAULT || desc->algo != GACONV_ALGO_AUTO || !planned_route(desc, g, kNoLimit).use) return false;
+    if (desc->math != GACONV_MATH_DEFAULT || desc->algo != GACONV_ALGO_AUTO) return false;
     *R = planned_route(desc, g, given & ~(size_t)255);
     return R->use;
 }
@@ -343,7 +352,7 @@ uint64_t splitmix64(uint64_t x)
 // version of the problem, and read in place by the FP32-pipe and scalar-gather kernels otherwise (odd shapes,
 // GACONV_ALGO_DIRECT).  The call then continues with an inner descriptor in the kernels' layouts whose workspace is
 // the head of the caller's.
-struct Relayout { size_t inner_bytes; bool move_x, move_dy; gaconv_conv_desc_t inner; };
+struct Relayout { size_t inner_bytes, inner_least; bool move_x, move_dy; gaconv_conv_desc_t inner; };
 size_t x_bytes_of(const gaconv_conv_desc_t* d) { return (size_t)d->n * d->c * d->h * d->w * (d->in_dtype == GACONV_BF16 ? 2 : 4); }
 size_t dy_bytes_of(const Geom& g) { return (size_t)g.n * g.k * g.p * g.q * (g.bf16 ? 2 : 4); }
 
@@ -383,7 +392,7 @@ Relayout plan_relayout(const gaconv_conv_desc_t* desc, int32_t method, bool cl)
         if (make_geom(&nhwc, &gi) == GACONV_OK) {
             if (method == GACONV_METHOD_EXACT) {
                 const ExactLayout L = exact_layout(gi, desc->math, desc->algo);
-                R.move_x = L.tc_ok || L.stem_ok || direct_mma_supported(gi, L.dp);
+                R.move_x = L.tc_ok || L.stem_ok || L.mma_ok;
             } else if (method == GACONV_METHOD_TOP1) {
                 R.move_x = top1_layout(gi, cl).dense || (top1_fused_supported(gi) && gi.c % 4 == 0);
             } else {
@@ -395,17 +404,21 @@ Relayout plan_relayout(const gaconv_conv_desc_t* desc, int32_t method, bool cl)
     if (R.move_x || R.move_dy) {
         Geom gi;
         bool ok = false;
-        if (make_geom(&R.inner, &gi) == GACONV_OK) R.inner_bytes = native_ws_bytes(&R.inner, gi, method, cl, &ok);
-        if (!ok) { R.move_x = R.move_dy = false; R.inner = *desc; R.inner_bytes = 0; }
+        if (make_geom(&R.inner, &gi) == GACONV_OK) {
+            R.inner_bytes = native_ws_bytes(&R.inner, gi, method, cl, &ok);
+            R.inner_least = method == GACONV_METHOD_EXACT ? exact_layout(gi, R.inner.math, R.inner.algo).least : R.inner_bytes;
+        }
+        if (!ok) { R.move_x = R.move_dy = false; R.inner = *desc; R.inner_bytes = R.inner_least = 0; }
     }
     return R;
 }
 
 // the inner call's scratch, then the transposed copies
-size_t moved_ws_bytes(const gaconv_conv_desc_t* desc, const Geom& g, const Relayout& R)
+size_t copied_bytes(const gaconv_conv_desc_t* desc, const Geom& g, const Relayout& R)
 {
-    return align_up(R.inner_bytes, 256) + (R.move_x ? align_up(x_bytes_of(desc), 256) : 0) + (R.move_dy ? dy_bytes_of(g) : 0);
+    return (R.move_x ? align_up(x_bytes_of(desc), 256) : 0) + (R.move_dy ? dy_bytes_of(g) : 0);
 }
+size_t moved_ws_bytes(const gaconv_conv_desc_t* desc, const Geom& g, const Relayout& R) { return align_up(R.inner_bytes, 256) + copied_bytes(desc, g, R); }
 
 // Transposes what has to move into the workspace tail and hands back the inner descriptor and operand pointers.
 // *moved == false: nothing to do, the caller goes on with its own descriptor.
@@ -419,10 +432,10 @@ gaconv_status_t relayout_operands(const void* x, const void* dy, const gaconv_co
     gaconv_status_t st = make_geom(desc, &g);
     if (st != GACONV_OK) return st;
     if (desc->workspace_bytes < moved_ws_bytes(desc, g, R)) R = plan_relayout(desc, method, false);
-    const size_t head = align_up(R.inner_bytes, 256);
-    const size_t x_tail = R.move_x ? align_up(x_bytes_of(desc), 256) : 0;
-    st = check_ws(desc, moved_ws_bytes(desc, g, R));
+    const size_t x_tail = R.move_x ? align_up(x_bytes_of(desc), 256) : 0, copies = copied_bytes(desc, g, R);
+    st = check_ws(desc, align_up(R.inner_least, 256) + copies);
     if (st != GACONV_OK) return st;
+    const size_t head = std::min(align_up(R.inner_bytes, 256), (desc->workspace_bytes - copies) & ~(size_t)255);
     char* ws = static_cast<char*>(desc->workspace);
     *x_out = x; *dy_out = dy;
     if (R.move_x) {
@@ -450,14 +463,18 @@ struct gaconv_schedule {
 
 // scratch of a call, exact ones without the channels-last kernel
 // (cl: the dense route of top-1 with it)
-static gaconv_status_t other_workspace(const gaconv_conv_desc_t* desc, const Geom& g, int32_t method, bool cl, size_t* bytes)
+static gaconv_status_t other_workspace(const gaconv_conv_desc_t* desc, const Geom& g, int32_t method, bool cl, size_t given, size_t* bytes)
 {
     const Relayout R = plan_relayout(desc, method, cl);
-    if (R.move_x || R.move_dy) { *bytes = moved_ws_bytes(desc, g, R); return GACONV_OK; }
+    if (R.move_x || R.move_dy) {
+        *bytes = moved_ws_bytes(desc, g, R);
+        if (*bytes > given) *bytes = align_up(R.inner_least, 256) + copied_bytes(desc, g, R);
+        return GACONV_OK;
+    }
     bool ok = false;
     const size_t need = native_ws_bytes(desc, g, method, cl, &ok);
     if (!ok) return GACONV_ERR_BAD_DESC;
-    *bytes = need;
+    *bytes = need <= given || method != GACONV_METHOD_EXACT ? need : exact_layout(g, desc->math, desc->algo).least;
     return GACONV_OK;
 }
 
@@ -469,9 +486,9 @@ gaconv_status_t gaconv::method_workspace(const gaconv_conv_desc_t* desc, int32_t
     const bool exact = method == GACONV_METHOD_EXACT;
     ClRoute C;
     if (exact && cl_route(desc, g, given, &C)) { *bytes = C.total[given >= C.total[1]]; return GACONV_OK; }
-    st = other_workspace(desc, g, method, !exact, bytes);
+    st = other_workspace(desc, g, method, !exact, given, bytes);
     if (st != GACONV_OK || *bytes <= given) return st;
-    if (!exact) return other_workspace(desc, g, method, false, bytes);
+    if (!exact) return other_workspace(desc, g, method, false, given, bytes);
     if (cl_last_route(desc, g, given, &C)) *bytes = C.total[0];
     return GACONV_OK;
 }
@@ -525,31 +542,30 @@ static gaconv_status_t run_others(const void* x, const void* dy, float* dw, cons
         if (moved) return make_geom(&inner, &gi) == GACONV_OK ? run_others(xt, dyt, dw, &inner, gi, stream) : GACONV_ERR_BAD_DESC;
     }
     const ExactLayout L = exact_layout(g, desc->math, desc->algo);
-    const bool mma_ok = direct_mma_supported(g, L.dp);
-    if (desc->math == GACONV_MATH_TF32 && !mma_ok && !L.tc_ok) return GACONV_ERR_UNSUPPORTED;
+    if (desc->math == GACONV_MATH_TF32 && !L.mma_ok && !L.tc_ok) return GACONV_ERR_UNSUPPORTED;
     if (desc->algo == GACONV_ALGO_TENSOR && !L.tc_ok) return GACONV_ERR_UNSUPPORTED;
-    st = check_ws(desc, L.total);
+    st = check_ws(desc, L.least);
     if (st != GACONV_OK) return st;
     char* ws = static_cast<char*>(desc->workspace);
-    if (L.tc_ok && desc->algo != GACONV_ALGO_DIRECT) {
+    if (L.kernel == ExactKernel::tc) {
         cudaError_t e = launch_tc(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off), ws + L.scratch_off,
                                   reinterpret_cast<uint32_t*>(ws + kWsCounterOffset), reinterpret_cast<uint32_t*>(ws), L.tp,
                                   stream);
         return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
     }
-    if (L.stem_ok && desc->algo != GACONV_ALGO_DIRECT && desc->math == GACONV_MATH_DEFAULT) {
+    if (L.kernel == ExactKernel::stem) {
         cudaError_t e = launch_stem(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off), reinterpret_cast<uint32_t*>(ws), L.sp,
                                     stream);
         return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
     }
-    if (mma_ok && (desc->algo != GACONV_ALGO_DIRECT || desc->math == GACONV_MATH_TF32)) {
+    if (L.kernel == ExactKernel::mma) {
         cudaError_t e = launch_direct_mma(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off), reinterpret_cast<uint32_t*>(ws),
                                           g, L.dp, desc->math != GACONV_MATH_TF32, stream);
         return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
     }
-    cudaError_t e = launch_direct(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off),
-                                  reinterpret_cast<uint32_t*>(ws), g, L.dp,
-                                  stream);
+    DirectPlan dp = L.dp;
+    limit_direct(g, desc->workspace_bytes - L.partial_off, &dp);
+    cudaError_t e = launch_direct(x, dy, dw, reinterpret_cast<float*>(ws + L.partial_off), reinterpret_cast<uint32_t*>(ws), g, dp, stream);
     return e == cudaSuccess ? GACONV_OK : GACONV_ERR_CUDA;
 }
 
@@ -729,7 +745,7 @@ static gaconv_status_t dw_from_host(int32_t method, const void* x_host, const vo
         if (st != GACONV_OK) return st;
         if (method == GACONV_METHOD_EXACT) {
             const ExactLayout L = exact_layout(g, desc->math, desc->algo);
-            if (desc->math == GACONV_MATH_TF32 && !direct_mma_supported(g, L.dp) && !L.tc_ok) return GACONV_ERR_UNSUPPORTED;
+            if (desc->math == GACONV_MATH_TF32 && !L.mma_ok && !L.tc_ok) return GACONV_ERR_UNSUPPORTED;
             if (desc->algo == GACONV_ALGO_TENSOR && !L.tc_ok) return GACONV_ERR_UNSUPPORTED;
         }
         const size_t eb = g.bf16 ? 2 : 4;

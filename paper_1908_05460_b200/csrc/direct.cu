@@ -14,6 +14,8 @@
 // TKT*TCT*R*S FMAs.  At the end the pixel groups are summed (warp shuffles, then shared memory, in a
 // fixed order) and the CTA writes its block: to dW if it is the only split, else to its slot of
 // the partial buffer, which reduce_splits() adds up in split order.
+#include <algorithm>
+
 #include "gaconv_internal.h"
 #include "device_utils.cuh"
 #include "tma.cuh"
@@ -447,6 +449,15 @@ DirectPlan plan_direct(const Geom& g)
     pl.splits = splits;
     pl.partial_bytes = splits > 1 ? (size_t)splits * out_bytes : 0;
     return pl;
+}
+
+void limit_direct(const Geom& g, size_t bytes, DirectPlan* pl)
+{
+    if (pl->partial_bytes <= bytes) return;
+    const size_t out_bytes = (size_t)g.k * g.c * g.r * g.s * sizeof(float);
+    const int most = std::max(1, (int)(bytes / out_bytes)), per = (pl->items + most - 1) / most;
+    pl->splits = (pl->items + per - 1) / per;
+    pl->partial_bytes = pl->splits > 1 ? (size_t)pl->splits * out_bytes : 0;
 }
 
 cudaError_t launch_direct(const void* x, const void* dy, float* dw, float* partial, uint32_t* status,

@@ -150,6 +150,8 @@ struct DirectPlan {
     FastDiv by_npx, by_bq, by_win_w;        // by pixels of a band, its columns, columns of the X window
 };
 DirectPlan plan_direct(const Geom& g);
+// fewer splits, so that the partial blocks take no more than `bytes` (the only split writes dW itself)
+void limit_direct(const Geom& g, size_t bytes, DirectPlan* plan);
 cudaError_t launch_direct(const void* x, const void* dy, float* dw, float* partial, uint32_t* status,
                           const Geom& g, const DirectPlan& plan, cudaStream_t stream);
 

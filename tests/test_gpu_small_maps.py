@@ -49,3 +49,46 @@ def test_small_layers_on_the_fp32_pipes(layer, dtype):
         assert norm_err(got, ref, dn) <= TOL_F32, kw
         np.testing.assert_array_equal(got, g.exact())
     assert any("direct_tiled_kernel" in n for n in kernel_names(lambda: B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc)))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
+@pytest.mark.parametrize("layer,kw", [
+    (ConvLayer("1x1, 16 splits a tile and more", 24, 3, 36, 36, 80, 1, 1, 1, 0), {}),
+    (ConvLayer("1x1, an odd element count", 19, 3, 13, 13, 75, 1, 1, 1, 0), dict(dy_layout=B.DY_NPQK, dw_layout=B.DW_KCRS)),
+    (ConvLayer("5x5, four channels", 9, 4, 21, 20, 9, 5, 5, 1, 2), dict(x_layout=B.X_NCHW, dy_layout=B.DY_NPQK)),
+    (ConvLayer("3x3, 20 channels, odd rows", 5, 20, 9, 11, 20, 3, 3, 1, 1), dict(dy_layout=B.DY_NPQK, dw_layout=B.DW_RSCK)),
+], ids=lambda v: v.name if isinstance(v, ConvLayer) else "")
+def test_fewer_splits_in_smaller_workspaces(layer, kw, dtype):
+    """The FP32-pipe kernel splits as far as the workspace has room for its partial blocks, down to one split; nothing is written beyond it."""
+    x, dy = I.make_layer_inputs(layer, dtype, 26, 0)
+    ref, dn = oracle.dw_exact(to_f64(x), to_f64(dy), oshape(layer))
+    g = GpuLayer(layer, dtype, x, dy, algo=B.ALGO_DIRECT, **kw)
+    full, out = B.gaconv_workspace_size(g.desc, B.METHOD_EXACT), layer.k * layer.c * layer.r * layer.s * 4
+    copy = g.dy.numel() * g.dy.element_size() if kw.get("dy_layout") == B.DY_NPQK else 0
+    least = 17 * 1024 + copy               # (control words and a ragged end)
+    assert full > least + 4 * out
+    ws, before = torch.empty(full + 4096, dtype=torch.uint8, device="cuda"), None
+    for size in (full, full - 16, least + 4 * out, least + 2 * out, least + out, least):
+        ws.fill_(0x5a)
+        B.gaconv_workspace_init(ws, size)
+        g.desc.workspace, g.desc.workspace_bytes = ws.data_ptr(), size
+        got = g.exact()
+        assert norm_err(got, ref, dn) <= TOL_F32, size
+        assert bool((ws[size:] == 0x5a).all()), size
+        assert any("direct_tiled_kernel" in n for n in kernel_names(lambda: B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc)))
+    g.desc.workspace_bytes = 16 * 1024 + copy
+    with pytest.raises(B.GaconvError) as e:
+        B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc)
+    assert e.value.status == B.ERR_WORKSPACE_TOO_SMALL
+
+
+def test_static_scratch_full_of_a_transposed_gradient():
+    """A channels-last gradient of 8.3 MB that is transposed into the built-in array: the partial blocks take what is left."""
+    layer = ConvLayer("1x1", 164, 3, 13, 13, 75, 1, 1, 1, 0)
+    x, dy = I.make_layer_inputs(layer, torch.float32, 27, 0)
+    ref, dn = oracle.dw_exact(to_f64(x), to_f64(dy), oshape(layer))
+    g = GpuLayer(layer, torch.float32, x, dy, dy_layout=B.DY_NPQK)
+    bare = B.make_desc(layer, torch.float32, dy_layout=B.DY_NPQK)
+    assert B.gaconv_workspace_size(bare, B.METHOD_EXACT) > B.gaconv_static_scratch_bytes()
+    B.gaconv_dw_exact_static(g.x, g.dy, g.dw, bare)
+    assert norm_err(g.logical_dw(), ref, dn) <= TOL_F32 and B.gaconv_poll_async_status_static() == B.OK
