@@ -423,8 +423,9 @@ DirectPlan plan_direct(const Geom& g)
     }
     else while (pl.bp * 2 <= g.p && pl.bp * 2 * pl.bq <= max_px && smem_for(g, v, pl.bp * 2, pl.bq) <= 96 * 1024) pl.bp *= 2;
     while (pl.bq > 1 && smem_for(g, v, pl.bp, pl.bq) > 96 * 1024) pl.bq /= 2;
-    // (offsets of elements in and around an image, up to a window beyond it, in 32 bits)
-    pl.small = (double)(g.c + 16) * (g.h + 1024) * (g.w + 1024) < 2e9 && (double)(g.k + 16) * g.p * g.q < 2e9;
+    // offsets of an item's elements from its first one, in a window of X and in a band of dY, have 32 bits
+    const long long win_h = (long long)(pl.bp - 1) * g.stride_h + g.r, win_w = (long long)(pl.bq - 1) * g.stride_w + g.s;
+    pl.small = (win_h - 1) * g.xs_h + (win_w - 1) * g.xs_w + (tc - 1) * g.xs_c < (1ll << 31) && (long long)(tk - 1) * g.p * g.q + (long long)(pl.bp - 1) * g.q + pl.bq < (1ll << 31);
     pl.by_npx = fast_div(pl.bp * pl.bq); pl.by_bq = fast_div(pl.bq); pl.by_win_w = fast_div((pl.bq - 1) * g.stride_w + g.s);
     pl.bands_p = (g.p + pl.bp - 1) / pl.bp;
     pl.bands_q = (g.q + pl.bq - 1) / pl.bq;

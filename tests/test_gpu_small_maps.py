@@ -40,15 +40,37 @@ def test_matches_the_oracle(li, dtype, layout):
     ConvLayer("20 channels, odd rows", 2, 20, 9, 11, 20, 3, 3, 1, 1),
 ], ids=lambda l: l.name)
 def test_small_layers_on_the_fp32_pipes(layer, dtype):
-    """Bands and windows that are filled element by element: their edges, remainders of eight loads a thread, every memory order."""
+    """Bands and windows that are filled element by element: their edges, remainders of four loads a thread, every memory order."""
     x, dy = I.make_layer_inputs(layer, dtype, 24, 0)
     ref, dn = oracle.dw_exact(to_f64(x), to_f64(dy), oshape(layer), 0.5)
-    for kw in ({}, dict(x_layout=B.X_NCHW, dw_layout=B.DW_KCRS), dict(algo=B.ALGO_DIRECT)):
+    orders = ({}, dict(x_layout=B.X_NCHW, dw_layout=B.DW_KCRS), dict(dy_layout=B.DY_NPQK), dict(x_layout=B.X_NCHW, dy_layout=B.DY_NPQK, dw_layout=B.DW_RSCK))
+    for kw in (*orders, *(dict(o, algo=B.ALGO_DIRECT) for o in orders)):
         g = GpuLayer(layer, dtype, x, dy, alpha=0.5, **kw)
         got = g.exact()
         assert norm_err(got, ref, dn) <= TOL_F32, kw
         np.testing.assert_array_equal(got, g.exact())
-    assert any("direct_tiled_kernel" in n for n in kernel_names(lambda: B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc)))
+        if "algo" in kw:
+            assert any("direct_tiled_kernel" in n for n in kernel_names(lambda: B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc))), kw
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
+@pytest.mark.parametrize("x_layout,w", [(B.X_NHWC, 800_000), (B.X_NCHW, 2_400_000)], ids=["nhwc", "nchw"])
+@pytest.mark.parametrize("rows", [1920, 640], ids=["64-bit offsets", "32-bit offsets"])
+def test_windows_that_reach_far(rows, x_layout, w, dtype):
+    """One wide row of X in the middle of `rows` rows of padding, one column of outputs: the offset of its pixel within a window, 944 or 304 rows
+    of 2.4 million elements, takes more than 31 bits, or less."""
+    n, c, k = 2, 3, 5
+    gen = torch.Generator().manual_seed(28)
+    x, dy = torch.randn((n, c), generator=gen).to(dtype), torch.randn((n, k, 2 * rows // 16 + 1), generator=gen).to(dtype)
+    d = B.make_desc(ConvLayer("one row", n, c, 1, w, k, 1, 1, 1, 0), dtype, x_layout=x_layout, algo=B.ALGO_DIRECT)
+    d.stride_h, d.stride_w, d.pad_h = 16, w, rows                     # (one column; the pixel is the middle output's)
+    xg = torch.full((n, 1, w, c) if x_layout == B.X_NHWC else (n, c, 1, w), float("nan"), dtype=dtype, device="cuda")
+    (xg[:, 0, 0, :] if x_layout == B.X_NHWC else xg[:, :, 0, 0]).copy_(x)
+    dw, ws = torch.full((k, c), float("nan"), device="cuda"), B.attach_workspace(d, methods=(B.METHOD_EXACT,))
+    B.gaconv_dw_exact(xg, dy.cuda(), dw, d)
+    want = torch.einsum("nk,nc->kc", dy[:, :, rows // 16].double(), x.double())
+    assert float((dw.cpu().double() - want).abs().max()) <= 1e-5 and B.gaconv_poll_async_status(d) == B.OK
+    del ws
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
