@@ -711,7 +711,7 @@ struct PackOp {
     int ch, chp, px, n;         // source: n images of px pixels and ch channels; destination rows of chp channels,
     int pitch;                  // this many apart
     int channels_last;          // source order: 1 [n][px][ch], 0 [n][ch][px]
-    int vc, vw, vpad, q, h;     // ClParams::vc and so on: the destination's channels are gathered from windows of the source; its rows and columns
+    int vc, vw, vpad, q, h;     // ClShape::vc and so on: the destination's channels are gathered from windows of the source; its rows and columns
     int px_tiles, ch_tiles;     // tiles of an image (channels-first sources): tile_px pixels x
     int ch_tile;                // at most 64 channels, a multiple of 8
     int tile_px;                // pixels of a tile

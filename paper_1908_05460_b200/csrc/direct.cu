@@ -435,7 +435,10 @@ DirectPlan plan_direct(const Geom& g)
     pl.vec_x = g.xs_c == 1 && g.c % 4 == 0 && tc % 4 == 0;
     pl.items = g.n * pl.bands_p * pl.bands_q;
     const int tiles = pl.tiles_k * pl.tiles_c;
-    // one wave of two CTAs per SM (the register budget); each split's partial block is written once and read once
+    // one wave of two CTAs per SM (the register budget), six of 1x1 filters over few channels, whose loads they hide (us, two / six: bf16 3->80 on
+    // 36x36, N = 24 14.5 / 10.4, fp32 3->156 on 35x35, N = 10 20.5 / 13.8); each split's partial block is written once and read once.  An SM
+    // budget does not count here: twelve such layers beside one another take 7.0 / 7.1 and 10.4 / 10.4 us each, bf16 4->48 on 17x17, N = 64
+    // 5.9 / 6.3, and six of them beside six tensor-core layers 115 / 111 in all.
     int splits = 148 * (narrow && g.r == 1 ? 6 : 2) / tiles;
     if (splits < 1) splits = 1;
     if (splits > pl.items) splits = pl.items;

@@ -1,5 +1,6 @@
 """The channels-last tensor-core kernel (csrc/cl.cu) at the edges of its tiles, against the oracle: odd maps, channel
 counts off every tile size, strides, every packing path, several images per chunk, one split and many."""
+import re
 import threading
 
 import numpy as np
@@ -39,11 +40,12 @@ SHAPES = [
     ConvLayer("stride 3, 7x7: three shifts, two and two", 12, 30, 30, 25, 100, 7, 7, 3, 3),
     ConvLayer("5x5, tiles of 32 of 72 channels", 5, 72, 15, 15, 136, 5, 5, 1, 2),
     ConvLayer("7x7, tiles of 16 of 70 channels", 6, 70, 13, 10, 131, 7, 7, 1, 3),
-    ConvLayer("3 channels, 5x5: windows for channels", 8, 3, 33, 40, 70, 5, 5, 1, 2),
+    ConvLayer("3 channels, 5x5, rows of 40", 8, 3, 33, 40, 70, 5, 5, 1, 2),
     ConvLayer("4 channels, 3x7, padding on one side", 13, 4, 21, 19, 100, 3, 7, 1, 2),
-    ConvLayer("2 channels, 9 rows in two tiles", 22, 2, 30, 17, 130, 9, 3, 1, 1),
-    ConvLayer("2 channels, 7x7, odd rows", 30, 2, 34, 31, 48, 7, 7, 1, 3),
+    ConvLayer("windows of two channels, 9 rows in two tiles", 22, 2, 30, 17, 130, 9, 3, 1, 1),
+    ConvLayer("windows of two channels, 7x7, odd rows", 30, 2, 34, 31, 48, 7, 7, 1, 3),
     ConvLayer("3x1 filter, 20 channels", 30, 20, 26, 16, 60, 3, 1, 1, 0),
+    ConvLayer("windows of three channels, 5x5, rows of 41", 8, 3, 33, 41, 70, 5, 5, 1, 2),
     # (the gain of gathered windows is a tenth of the estimate without the packing pass of dY, less of it with)
     ConvLayer("windows of two channels, 224 outputs, rows of 43", 19, 2, 43, 43, 224, 3, 3, 1, 1),
     ConvLayer("windows of four channels, 248 outputs, rows of 14", 18, 4, 14, 14, 248, 5, 5, 1, 2),
@@ -64,7 +66,10 @@ def test_every_layout_matches_the_oracle(li, dtype):
         before = B.gaconv_launch_count()
         got = g.exact()
         assert B.gaconv_launch_count() - before <= 3, name
-        assert any("cl_kernel" in k for k in kernel_names(lambda: B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc))), name
+        names = kernel_names(lambda: B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc))
+        assert any("cl_kernel" in k for k in names), name
+        if layer.name.startswith("windows"):
+            assert any(re.search("pack_kernelI[ft]Lb1E", k) for k in names), (name, names)
         assert norm_err(got, ref, dn) <= TOL_F32 / 2, name        # bf16 products are exact in fp32 as well
         np.testing.assert_array_equal(got, g.exact())
         # the same operands, however they were handed over; only a bf16 gradient on rows of whole 16-byte pieces is read as it
