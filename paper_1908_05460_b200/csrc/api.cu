@@ -232,14 +232,18 @@ bool prefer_cl(const Geom& g, const ExactLayout& L, const ClPlan& plan, bool reo
             // 47.7 / 66.3).  3x3 64->64 on 32x32 25.0 / 23.1
             return g.r < 5 || g.c < 64 || (g.r == 5 && g.s <= 5 && g.k >= 96);
         }
-        // stems (on 32x32): beside others 3->64 3x3 N = 64 7.1 / 4.7, N = 256 16.7 / 13.4, 5x5 N = 16 4.2 / 2.5, but 3->16 N = 256 7.3 / 9.2; alone
-        // 3x3 3->64 N = 64 11.6 / 12.4, N = 128 15.5 / 15.1, N = 256 23.8 / 20.8, 3->16 N = 256 16.0 / 16.5, 5x5 3->64 N = 8 9.4 / 11.8, N = 32 13.7 / 12.3,
-        // N = 128 26.5 / 15.4, 3->16 N = 64 11.0 / 13.2
-        if (L.stem_ok) return reordered || (shared ? g.k > 32 && products > 5e7 : products > (g.r * g.s * g.c > 32 ? 1.2e8 : 2e8));
+        // stems, those whose windows are gathered (on 32x32): beside others 3->64 3x3 N = 64 7.1 / 4.7, N = 256 16.7 / 13.4, 5x5 N = 16 4.2 / 2.5, but 3->16
+        // N = 256 7.3 / 9.2; alone 3x3 3->64 N = 64 11.6 / 12.4, N = 128 15.5 / 15.1, N = 256 23.8 / 20.8, 3->16 N = 256 16.0 / 16.5, 5x5 3->64 N = 8
+        // 9.4 / 11.8, N = 32 13.7 / 12.3, N = 128 26.5 / 15.4, 3->16 N = 64 11.0 / 13.2; 3x3 on 64x64 3->32 N = 84 21.5 / 22.9, on 96x96 1->16 N = 232
+        // 39 / 54.  Not the plain form, which is left for strides: 5x5 3->40 on 64x64 at stride 2, N = 38, beside others 7.0 / 9.2, alone 1->128 on 96x96,
+        // N = 50 23.3 / 34.2.  (Of 178 stems alone 3 are more than 5 % off the better kernel, 10 % at most.)
+        if (L.stem_ok) return reordered || (plan.windows && (shared ? g.k > 32 && products > 5e7 : g.r * g.s * g.c > 32 ? products > 1.2e8 : g.k > 32 && products > 2e8));
     } else {
-        // stems on 32x32: 3x3 3->64 28.7 / 36.8; 5x5 3->64 44.2 / 37.9, N = 32 18.0 / 17.5, but 3->32 26.4 / 28.4 (beside the second layer of the
-        // two-layer CNN, N = 200, the step takes 63 / 68)
-        if (L.stem_ok) return !shared && g.r * g.s * g.c > 32 && g.k > 32 && products > 1.2e8;
+        // stems: 3x3 3->64 on 32x32 28.7 / 36.8; gathered windows of 5x5 filters of three channels 3->64 on 32x32, N = 116 44.0 / 37.2, N = 59 26.8 / 24.9,
+        // N = 23 15.3 / 16.4, on 40x40, N = 61 36.5 / 36.2, 3->96 on 32x32, N = 58 34.5 / 28.9, but 3->48, N = 38 18.6 / 18.6, 3->40 on 64x64, N = 45 44.5 / 58.3;
+        // fewer columns 4->128 3x3, N = 28 17.8 / 22.4, 2->96 5x5 on 48x48, N = 98 70 / 96; the plain form, at stride 2, 3->40 5x5 on 64x64, N = 170 60 / 138
+        // (beside the second layer of the two-layer CNN, N = 200, the step takes 63 / 68)
+        if (L.stem_ok) return !shared && plan.windows && g.r * g.s * g.c > 64 && g.k >= 64 && products > 1.2e8;
         // (the tensor core truncates as it adds, 1e-8 for each MMA of the other kernel's CTA: where that has more than 1,500 of them
         // its results are over 1.4e-5 away from this one's, and stay what they have been)
         if (L.tc_ok && L.tp.chain > 1500) return false;

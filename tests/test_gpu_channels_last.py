@@ -348,6 +348,30 @@ def test_either_side_of_a_line(layer, budget, kernel):
     assert np.all(np.isfinite(got)) and B.gaconv_poll_async_status(g.desc) == B.OK
 
 
+@pytest.mark.parametrize("layer,dtype,budget,kernel", [
+    (ConvLayer("5x5, stride 2", 60, 3, 64, 64, 40, 5, 5, 2, 2), torch.bfloat16, 18, "stem_mma_kernel"),
+    (ConvLayer("5x5, stride 2, one channel", 50, 1, 96, 96, 128, 5, 5, 2, 2), torch.bfloat16, 0, "stem_mma_kernel"),
+    (ConvLayer("5x5, windows", 60, 3, 32, 32, 40, 5, 5, 1, 2), torch.bfloat16, 18, "cl_kernel"),
+    (ConvLayer("3x3, 16 outputs", 220, 1, 96, 96, 16, 3, 3, 1, 1), torch.bfloat16, 0, "stem_mma_kernel"),
+    (ConvLayer("5x5, stride 2", 70, 3, 64, 64, 64, 5, 5, 2, 2), torch.float32, 0, "stem_mma_kernel"),
+    (ConvLayer("5x5, windows of two channels", 30, 2, 48, 48, 96, 5, 5, 1, 2), torch.float32, 0, "stem_mma_kernel"),
+    (ConvLayer("5x5, 48 outputs", 60, 3, 32, 32, 48, 5, 5, 1, 2), torch.float32, 0, "stem_mma_kernel"),
+    (ConvLayer("5x5, 64 outputs", 60, 3, 32, 32, 64, 5, 5, 1, 2), torch.float32, 0, "cl_kernel"),
+], ids=lambda v: v.name if isinstance(v, ConvLayer) else str(v))
+def test_stems_either_side_of_a_line(layer, dtype, budget, kernel):
+    """Image stems that both kernels can do: the plain form of the channels-last kernel, and its six products where few columns are in use, are slower."""
+    x, dy = I.make_layer_inputs(layer, dtype, 29, 0)
+    g = GpuLayer(layer, dtype, x, dy, sm_budget=budget)
+    names = kernel_names(lambda: B.gaconv_dw_exact(g.x, g.dy, g.dw, g.desc))
+    assert any(kernel in n for n in names), names
+    got, xd, dyd = g.exact(), to_f64(x), to_f64(dy)
+    rng = np.random.default_rng(5)
+    for k, c, r, s in zip(*(rng.integers(0, m, 40).tolist() for m in (layer.k, layer.c, layer.r, layer.s))):
+        v, norm = oracle.dw_exact_at(xd, dyd, oshape(layer), k, c, r, s)
+        assert abs(got[k, c, r, s] - v) <= TOL_F32 * norm
+    assert np.all(np.isfinite(got)) and B.gaconv_poll_async_status(g.desc) == B.OK
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
 @pytest.mark.parametrize("layer", [
     ConvLayer("two columns, padding 2", 43, 9, 8, 8, 244, 5, 2, 1, 2),
