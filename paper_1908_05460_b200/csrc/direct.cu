@@ -33,8 +33,8 @@ template <> struct Vec<4> { float v[4]; __device__ void load(const float* p) { f
 // The CTA's threads fill `n` floats in turn, `at(i)` the address of the i-th one's source, nullptr: zero.  U loads a thread are under way at
 // once.  Bound by latency: with one load, behind two divisions by numbers that only the launch knows, 16 x 512 pixels took 27 us to arrive.
 // (us, before / now, with the bands of plan_direct: bf16 1x1 3->80 on 36x36, N = 24 57.5 / 10.4, fp32 3->156 on 35x35, N = 10 44.5 / 13.7, bf16 3x3
-// 3->16 on 33x38, N = 3 26.0 / 9.1, fp32 3->20 on 60x60, N = 6 17.9 / 12.4, 1x1 3->304 on 5x5, N = 57 16.8 / 7.1, bf16 20->20 on 9x9, N = 12 11.3 / 11.1.
-// Eight at a time, and another form for short runs, lengthen the code: 10.9, 13.3, 9.7, 12.5, 7.3, 11.6.)
+// 3->16 on 33x38, N = 3 26.0 / 9.1, fp32 3->20 on 60x60, N = 6 17.9 / 12.4, 1x1 3->304 on 5x5, N = 57 16.8 / 7.1.
+// Eight at a time, and another form for short runs, lengthen the code: 10.9, 13.3, 9.7, 12.5, 7.3.)
 template <int U, typename T, typename At>
 __device__ __forceinline__ void fill(int n, At at)
 {
@@ -57,8 +57,9 @@ __device__ __forceinline__ void stage_item(const T* __restrict__ x, const T* __r
                                            const Geom& g, const DirectPlan& pl, int it, int k0, int c0, int dys,
                                            int win_h, int win_w)
 {
-    // (fp32 tiles of 16 channels leave few registers for it, and the compiler's own order of a plain loop is the quicker: 30->20 on 9x11, N = 12 11.6 / 13.0)
-    constexpr bool kPlain = sizeof(T) == 4 && TC > 4;
+    // (tiles of 16 channels leave few registers for it, and the compiler's own order of a plain loop is the quicker: fp32 30->20 on 9x11, N = 12
+    // 11.6 / 13.0, bf16 73->23 5x5 on 12x12, N = 45 20.5 / 23.2, 67->2 3x3 on 29x29, N = 3 12.5 / 13.7; of 215 bf16 layers 65 lost more than 5 % with it, 27 gained)
+    constexpr bool kPlain = TC > 4;
     const int npx = pl.bp * pl.bq;
     const int n = it / (pl.bands_p * pl.bands_q);
     const int band = it % (pl.bands_p * pl.bands_q);
